@@ -11,7 +11,7 @@
 #include <string>
 #include <vector>
 
-#include "cpm_internal.cuh"
+#include "phasor.cuh"
 
 namespace cpm {
 
@@ -140,6 +140,24 @@ int copy_out(Ctx* c, void* dst, const void* dev, size_t bytes) {
   if (dst == dev) return CPM_OK;
   return cuda_check(c, cudaMemcpyAsync(dst, dev, bytes, cudaMemcpyDeviceToHost, c->stream),
                     "copy out");
+}
+
+// Per-axis phasor tables (FP64 storage): the layout of a point's entries, and how many
+// frames' ions are tabulated at a time so that the tables stay within kAxisBytes.
+constexpr size_t kAxisBytes = 512ull << 20;
+
+AxisPhasors axis_phasors(const Ctx* c) {
+  AxisPhasors ap;
+  ap.off[0] = 0;
+  ap.off[1] = c->kmax[0] + 1;
+  ap.off[2] = ap.off[1] + c->kmax[1] + 1;
+  ap.len = ap.off[2] + c->kmax[2] + 1;
+  return ap;
+}
+
+int axis_frames(const AxisPhasors& ap, int frames, int n_ion) {
+  const size_t per = (size_t)std::max(n_ion, 1) * ap.len * sizeof(double2);
+  return (int)std::max<size_t>(1, std::min<size_t>((size_t)frames, kAxisBytes / per));
 }
 
 Geometry geometry(const Ctx* c) {
@@ -607,6 +625,10 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
   hkl.resize(3 * (size_t)c->mpad, 0);
   std::vector<double> sqw(c->mpad, 0.0);
   for (int k = 0; k < c->m; ++k) sqw[k] = sqrt(w[k]);
+  for (int d = 0; d < 3; ++d) {
+    c->kmax[d] = 0;
+    for (int k = 0; k < c->m; ++k) c->kmax[d] = std::max(c->kmax[d], std::abs(hkl[3 * (size_t)k + d]));
+  }
   c->kw.assign(c->mpad, 0.0);
   std::copy(w.begin(), w.end(), c->kw.begin());
   KPlan pl;
@@ -963,7 +985,12 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
                          ? bsol_direct_splits(n, frames, c->mpad, c->kh, std::max(dev_sms, 1))
                          : 1;
   const size_t sbytes = nsplit > 1 ? (size_t)nsplit * kbytes : 0;
-  if ((st = buf_reserve(c, &c->ws_pot, vbytes + hbytes + kbytes + ubytes + sbytes))) return st;
+  // FP64 storage: the ions' per-axis phasors, at most kAxisBytes of frames at a time
+  const AxisPhasors ap = axis_phasors(c);
+  const int fchunk = axis_frames(ap, frames, n_ion);
+  const size_t abytes = f64 ? up((size_t)fchunk * std::max(n_ion, 1) * ap.len * sizeof(double2)) : 0;
+  if ((st = buf_reserve(c, &c->ws_pot, vbytes + hbytes + kbytes + ubytes + sbytes + abytes)))
+    return st;
   if (!f64 && !c->turn.ptr) {
     if ((st = buf_alloc(c, &c->turn, 4096 * 4 * sizeof(float)))) return st;
     launch_turn_table(c->turn.ptr, s);
@@ -974,6 +1001,7 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   uint32_t* sion = (uint32_t*)((char*)c->ws_pot.ptr + vbytes + hbytes + kbytes);
   double* spart =
       nsplit > 1 ? (double*)((char*)c->ws_pot.ptr + vbytes + hbytes + kbytes + ubytes) : nullptr;
+  double2* axis = (double2*)((char*)c->ws_pot.ptr + vbytes + hbytes + kbytes + ubytes + sbytes);
   cudaEvent_t pev[4];
   for (int e = 0; e < 4; ++e) {
     while (c->ev_pot.size() < 4) {
@@ -986,9 +1014,16 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   cudaEventRecord(pev[0], s);
   if (n_ion > 0) {
     launch_ion_fixed(dx, frames, n_ion, c->p.box, sion, s);
-    launch_ion_structure_factor(f64, dx, sion, dq, frames, n_ion, (const int*)c->hkl.ptr,
-                                (const double*)c->sqw.ptr, c->mpad, c->kh, c->p.box,
-                                c->turn.ptr, v, vh, s);
+    for (int f0 = 0; f0 < frames; f0 += f64 ? fchunk : frames) {
+      const int nf = f64 ? std::min(fchunk, frames - f0) : frames;
+      if (f64)
+        launch_axis_phasors(dx + (size_t)f0 * n_ion * 3, nullptr, (int64_t)nf * n_ion, c->p.box, ap,
+                            axis, s);
+      launch_ion_structure_factor(f64, axis, ap, sion, n_ion, dq + (size_t)f0 * n_ion, nf, n_ion,
+                                  (const int*)c->hkl.ptr, (const double*)c->sqw.ptr, c->mpad,
+                                  c->kh, c->turn.ptr,
+                                  (char*)v + (size_t)f0 * 2 * c->mpad * c->esz(), vh, s);
+    }
   } else if ((st = cuda_check(c, cudaMemsetAsync(v, 0, vbytes + hbytes, s), "v zero"))) {
     return st;
   }
@@ -1037,37 +1072,61 @@ int cpm_ion_forces(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
       (st = stage_out(c, &c->ws_out0, f_out, (size_t)frames * n_ion * 3 * sizeof(double),
                       (void**)&dout)))
     return st;
-  // scratch: structure factors v [frames][2 mpad] (storage type) | v_head [frames][2 kh] |
-  //          fixed-point ion coordinates [frames][n_ion][3] | k-space gradients [frames][n_ion][3]
-  auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
-  const int kh = f64 ? c->mpad : c->kh;  // FP64 storage: every k-vector in FP64
-  const size_t vbytes = up((size_t)frames * 2 * c->mpad * c->esz());
-  const size_t hbytes = up((size_t)frames * 2 * std::max(c->kh, 1) * sizeof(double));
-  const size_t ubytes = up((size_t)frames * n_ion * 3 * sizeof(uint32_t));
-  const size_t gbytes = up((size_t)frames * n_ion * 3 * sizeof(double));
-  if ((st = buf_reserve(c, &c->ws_pot, vbytes + hbytes + ubytes + gbytes))) return st;
+  // FP64 storage takes its phasors from per-axis ones of the ions (at most kAxisBytes of
+  // frames at a time) and of the electrode
+  const AxisPhasors ap = axis_phasors(c);
+  const int fchunk = f64 ? axis_frames(ap, frames, n_ion) : frames;
+  int dev_sms = 1;
+  cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, c->device);
+  const ForceSplits sp = force_splits(f64, n, fchunk, n_ion, c->mpad, c->kh, std::max(dev_sms, 1));
+  // scratch, for the frames of one pass: structure factors v [frames][2 mpad] (storage type) |
+  // v_head [frames][2 kh] | fixed-point ion coordinates [frames][n_ion][3] | the shares'
+  // gradients [k_total + real][frames][n_ion][3] and slab sums [real][frames] | per-axis
+  // phasors of the ions and the electrode
+  size_t off = 0;
+  auto take = [&](size_t b) {
+    const size_t o = off;
+    off += (b + 255) & ~size_t(255);
+    return o;
+  };
+  const size_t gbytes = (size_t)fchunk * n_ion * 3 * sizeof(double);
+  const size_t ov = take((size_t)fchunk * 2 * c->mpad * c->esz()),
+               oh = take((size_t)fchunk * 2 * std::max(c->kh, 1) * sizeof(double)),
+               ou = take((size_t)fchunk * n_ion * 3 * sizeof(uint32_t)),
+               ok = take(sp.k_total * gbytes), orl = take(sp.real * gbytes),
+               os = take((size_t)sp.real * fchunk * sizeof(double2)),
+               oa = f64 ? take((size_t)fchunk * n_ion * ap.len * sizeof(double2)) : 0,
+               oe = f64 ? take((size_t)n * ap.len * sizeof(double2)) : 0;
+  if ((st = buf_reserve(c, &c->ws_pot, off))) return st;
   if (!f64 && !c->turn.ptr) {
     if ((st = buf_alloc(c, &c->turn, 4096 * 4 * sizeof(float)))) return st;
     launch_turn_table(c->turn.ptr, s);
   }
   char* base = (char*)c->ws_pot.ptr;
-  void* v = base;
-  double* vh = (double*)(base + vbytes);
-  uint32_t* sion = (uint32_t*)(base + vbytes + hbytes);
-  double* grad = (double*)(base + vbytes + hbytes + ubytes);
-  launch_ion_fixed(dx, frames, n_ion, c->p.box, sion, s);
-  // the electrode's charge-weighted structure factors, frame by frame: the ions' kernel
-  // run over the electrode atoms (same coordinates every frame)
-  for (int f = 0; f < frames; ++f)
-    launch_ion_structure_factor(f64, (const double*)c->xyz.ptr, (const uint32_t*)c->sfix.ptr,
-                                dqe + (size_t)f * n, 1, n, (const int*)c->hkl.ptr,
-                                (const double*)c->sqw.ptr, c->mpad, c->kh, c->p.box,
-                                c->turn.ptr, (char*)v + (size_t)f * 2 * c->mpad * c->esz(),
-                                vh + (size_t)f * 2 * std::max(c->kh, 1), s);
-  launch_ion_forces((const double*)c->xyz.ptr, (const double*)c->alpha.ptr,
-                    (const uint32_t*)c->sfix.ptr, n, dx, dq, sion, frames, n_ion, dqe,
-                    (const int*)c->hkl.ptr, (const double*)c->sqw.ptr, c->mpad, kh, geometry(c),
-                    c->turn.ptr, (const float*)v, f64 ? (const double*)v : vh, grad, dout, s);
+  void* v = base + ov;
+  double* vh = (double*)(base + oh);
+  uint32_t* sion = (uint32_t*)(base + ou);
+  double2 *ax = (double2*)(base + oa), *ax_el = (double2*)(base + oe);
+  if (f64) launch_axis_phasors((const double*)c->xyz.ptr, nullptr, n, c->p.box, ap, ax_el, s);
+  for (int f0 = 0; f0 < frames; f0 += fchunk) {
+    const int nf = std::min(fchunk, frames - f0);
+    const double* fx = dx + (size_t)f0 * n_ion * 3;
+    const double* fq = dqe + (size_t)f0 * n;
+    launch_ion_fixed(fx, nf, n_ion, c->p.box, sion, s);
+    // (the forces' ion phases are those of the fixed-point coordinates in both storages)
+    if (f64) launch_axis_phasors(fx, sion, (int64_t)nf * n_ion, c->p.box, ap, ax, s);
+    // the electrode's charge-weighted structure factors: the ions' kernel run over the
+    // electrode atoms (the same coordinates every frame)
+    launch_ion_structure_factor(f64, ax_el, ap, (const uint32_t*)c->sfix.ptr, 0, fq, nf, n,
+                                (const int*)c->hkl.ptr, (const double*)c->sqw.ptr, c->mpad, c->kh,
+                                c->turn.ptr, v, vh, s);
+    launch_ion_forces(f64, (const double*)c->xyz.ptr, (const double*)c->alpha.ptr,
+                      (const uint32_t*)c->sfix.ptr, n, fx, dq + (size_t)f0 * n_ion, sion, nf, n_ion,
+                      fq, (const int*)c->hkl.ptr, (const double*)c->sqw.ptr, c->mpad, c->kh,
+                      geometry(c), c->turn.ptr, v, vh, ax, ap, sp, (double*)(base + ok),
+                      (double*)(base + orl), (double2*)(base + os),
+                      dout + (size_t)f0 * n_ion * 3, s);
+  }
   if ((st = cuda_check(c, cudaGetLastError(), "ion forces"))) return st;
   if ((st = copy_out(c, f_out, dout, (size_t)frames * n_ion * 3 * sizeof(double)))) return st;
   return cuda_check(c, cudaStreamSynchronize(s), "ion forces sync");

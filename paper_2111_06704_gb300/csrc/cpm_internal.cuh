@@ -94,6 +94,7 @@ struct Ctx {
   int npad = 0;     // rows of A (multiple of 128), zero beyond n
   int m = 0;        // k-vectors
   int mpad = 0;     // k-vectors padded to a multiple of 64 (zero weight)
+  int kmax[3] = {0, 0, 0};  // largest |h|, |k|, |l| of the table
   int64_t ldE = 0;  // leading dimension of E (elements)
   double vol = 0;
 
@@ -252,10 +253,20 @@ void launch_get_E(bool fp64, const void* E, int n, int64_t ldE, const double* xy
 void launch_ion_fixed(const double* ion_xyz, int frames, int n_ion, const double L[3],
                       uint32_t* sion, cudaStream_t s);
 void launch_turn_table(void* T, cudaStream_t s);
-void launch_ion_structure_factor(bool fp64, const double* ion_xyz, const uint32_t* sion,
+struct AxisPhasors;
+// per-axis FP64 phasors (FP64 storage) of `count` points: out [count][ap.len] double2; from
+// the fixed-point coordinates sfix where not NULL, else from xyz
+void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
+                         const double L[3], const AxisPhasors& ap, double2* out,
+                         cudaStream_t s);
+// Structure factors of the points of `frames` frames, coord_stride points apart (0: every
+// frame has the same coordinates).  FP64 storage takes them from axis, float storage from
+// the fixed-point coordinates sion.
+void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhasors& ap,
+                                 const uint32_t* sion, int64_t coord_stride,
                                  const double* ion_q, int frames, int n_ion, const int* hkl,
-                                 const double* sqw, int mpad, int kh, const double L[3],
-                                 const void* turn, void* v, double* vhead, cudaStream_t s);
+                                 const double* sqw, int mpad, int kh, const void* turn,
+                                 void* v, double* vhead, cudaStream_t s);
 void launch_bsol_kspace(bool fp64, const void* A, const double* Ahead, int n, int mpad, int kh,
                         const void* v, const double* vhead, int frames, double* bsol,
                         const uint32_t* sfix, const int* hkl, const double* sqw,
@@ -269,12 +280,22 @@ void launch_bsol_real_and_finish(const double* xyz, const double* alpha, const u
                                  const Geometry& geo, const double* chi, const double* bsol_k,
                                  double* b_out, double* qsol, bool far_float, cudaStream_t s);
 
-void launch_ion_forces(const double* xyz, const double* alpha, const uint32_t* sfix, int n,
-                       const double* ion_xyz, const double* ion_q, const uint32_t* sion,
+// forces.cu
+struct ForceSplits {
+  int k_tail, k_total;  // shares of the k range: the tail's, and with the head's
+  int real;             // shares of the electrode atoms
+};
+ForceSplits force_splits(bool fp64, int n, int frames, int n_ion, int mpad, int kh, int sms);
+// kpart [k_total][frames][n_ion][3], rpart [real][frames][n_ion][3], slab [real][frames]:
+// scratch for the shares
+void launch_ion_forces(bool fp64, const double* xyz, const double* alpha, const uint32_t* sfix,
+                       int n, const double* ion_xyz, const double* ion_q, const uint32_t* sion,
                        int frames, int n_ion, const double* q, const int* hkl,
                        const double* sqw, int mpad, int kh, const Geometry& geo,
-                       const void* turn, const float* v, const double* vhead, double* grad,
-                       double* out, cudaStream_t s);
+                       const void* turn, const void* v, const double* vhead,
+                       const double2* ion_axis, const AxisPhasors& ap, const ForceSplits& sp,
+                       double* kpart, double* rpart, double2* slab, double* out,
+                       cudaStream_t s);
 
 // pcg.cu
 // One system of a ragged batch: a right-hand side with its own (float) matrix, size and

@@ -11,7 +11,7 @@
 
 #include <algorithm>
 
-#include "cpm_internal.cuh"
+#include "phasor.cuh"
 
 namespace cpm {
 
@@ -43,62 +43,6 @@ __global__ void k_turn_table(float4* __restrict__ T) {
   T[j] = make_float4(ch, (float)(c - ch), sh, (float)(s - sh));
 }
 
-// a * b for float pairs, to ~2^-44 relative (the lo * lo term dropped).
-__device__ __forceinline__ void ff_mul(float ah, float al, float bh, float bl, float& ph,
-                                       float& pl) {
-  ph = ah * bh;
-  pl = fmaf(ah, bh, -ph) + fmaf(ah, bl, al * bh);
-}
-
-// a + b for float pairs (two-sum of the high parts).
-__device__ __forceinline__ void ff_add(float ah, float al, float bh, float bl, float& sh,
-                                       float& sl) {
-  const float s = ah + bh;
-  const float bb = s - ah;
-  sl = ((ah - (s - bb)) + (bh - bb)) + (al + bl);
-  sh = s;
-}
-
-// exp(2 pi i ph 2^-32) as float pairs, to ~1e-13: the top 12 bits of the phase index the
-// exact table, the low 20 bits give an angle t < 2 pi 2^-12 whose sine and cosine follow
-// from their Taylor series (t - t^3/6, 1 - t^2/2 + t^4/24; the next terms are below
-// 1e-16), and the two rotations are multiplied in float pairs.
-__device__ __forceinline__ void phasor_ff(uint32_t ph, const float4* __restrict__ T, float& ch,
-                                          float& cl, float& sh, float& sl) {
-  const float4 t4 = __ldg(T + (ph >> 20));
-  const float low = (float)(ph & 0xFFFFFu);
-  constexpr float kCh = 1.462918119976564e-09f;   // 2 pi 2^-32, high part
-  constexpr float kCl = -4.070940267922164e-17f;  // and the rest
-  const float th = low * kCh;
-  const float tl = fmaf(low, kCh, -th) + low * kCl;
-  const float p = th * th;
-  const float pe = fmaf(th, th, -p) + 2.0f * th * tl;
-  // cos t = 1 - t^2/2 + t^4/24
-  const float half = 0.5f * p;
-  const float c0 = 1.0f - half;
-  const float c0l = ((1.0f - c0) - half) - 0.5f * pe + p * p * (1.0f / 24.0f);
-  // sin t = t - t^3/6
-  const float t3 = th * p * (1.0f / 6.0f);
-  const float s0 = th - t3;
-  const float s0l = ((th - s0) - t3) + tl;
-  // (Tc + i Ts)(c0 + i s0)
-  float ah, al, bh, bl;
-  ff_mul(t4.x, t4.y, c0, c0l, ah, al);
-  ff_mul(t4.z, t4.w, s0, s0l, bh, bl);
-  ff_add(ah, al, -bh, -bl, ch, cl);
-  ff_mul(t4.z, t4.w, c0, c0l, ah, al);
-  ff_mul(t4.x, t4.y, s0, s0l, bh, bl);
-  ff_add(ah, al, bh, bl, sh, sl);
-}
-
-// (h, l) += x by an error-free two-sum of the high part.
-__device__ __forceinline__ void pair_add1(float& h, float& l, float x) {
-  const float s = h + x;
-  const float bb = s - h;
-  l += (h - (s - bb)) + (x - bb);
-  h = s;
-}
-
 constexpr int kSfBlock = 8;  // ions a float block sum of the tail k-vectors holds
 
 // sin and cos of 2 pi ph 2^-32 from a 64-entry table of exp(2 pi i j / 64) (float cos and
@@ -126,7 +70,8 @@ __device__ __forceinline__ void sincos_t64(uint32_t ph, const float2* T, float* 
 // head (k < kh, the heaviest weights) takes float-pair phasors and goes out in FP64 to
 // vhead for the FP64 head contraction.
 __global__ void __launch_bounds__(kSfThreads, 8)
-k_ion_sf_f32(const uint32_t* __restrict__ sion, const double* __restrict__ ion_q, int n_ion,
+k_ion_sf_f32(const uint32_t* __restrict__ sion, int64_t coord_stride,
+             const double* __restrict__ ion_q, int n_ion,
              const int* __restrict__ hkl, const double* __restrict__ sqw, int mpad, int kh,
              const float4* __restrict__ turn, float* __restrict__ vout,
              double* __restrict__ vhead) {
@@ -135,7 +80,7 @@ k_ion_sf_f32(const uint32_t* __restrict__ sion, const double* __restrict__ ion_q
   __shared__ float2 t64[64];  // exp(2 pi i j / 64): entries 64 j of the 4,096-entry table
   const int f = blockIdx.y;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t* fx = sion + (size_t)f * n_ion * 3;
+  const uint32_t* fx = sion + (size_t)f * coord_stride * 3;
   const double* q = ion_q + (size_t)f * n_ion;
   for (int j = threadIdx.x; j < 64; j += blockDim.x) {
     const float4 e = __ldg(turn + 64 * j);
@@ -219,48 +164,64 @@ k_ion_sf_f32(const uint32_t* __restrict__ sion, const double* __restrict__ ion_q
   }
 }
 
-// FP64 storage (the plain baseline build): the same sums with FP64 phases, sincospi and
-// FP64 accumulation.
-__global__ void __launch_bounds__(kSfThreads)
-k_ion_sf_f64(const double* __restrict__ ion_xyz, const double* __restrict__ ion_q, int n_ion,
-             const int* __restrict__ hkl, const double* __restrict__ sqw, int mpad, double lx,
-             double ly, double lz, double* __restrict__ vout) {
-  __shared__ double sd[kIonChunk][3];
-  __shared__ double sq[kIonChunk];
+// exp(2 pi i j s_d) of every point and axis entry, s_d the fractional coordinate (from the
+// positions, or from fixed-point coordinates where sfix is given): one sincospi per entry, a
+// few hundred a point, instead of one per k-vector.
+__global__ void k_axis_phasors(const double* __restrict__ xyz, const uint32_t* __restrict__ sfix,
+                               int64_t count, double lx, double ly, double lz,
+                               const AxisPhasors ap, double2* __restrict__ out) {
+  const int64_t len = count * ap.len;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < len;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t pt = e / ap.len;
+    const int j = (int)(e - pt * ap.len);
+    const int d = j >= ap.off[2] ? 2 : j >= ap.off[1] ? 1 : 0;
+    double s;
+    if (sfix) {
+      s = sfix[3 * pt + d] * 0x1p-32;
+    } else {
+      s = xyz[3 * pt + d] / (d == 0 ? lx : d == 1 ? ly : lz);
+      s -= floor(s);
+    }
+    double fr = (j - ap.off[d]) * s;
+    fr -= rint(fr);
+    double sn, cs;
+    sincospi(2.0 * fr, &sn, &cs);
+    out[e] = make_double2(cs, sn);
+  }
+}
+
+// FP64 storage (the plain baseline build): the same sums in FP64, the phasors as products of
+// the points' per-axis phasors.  32 k-vectors a block (one a lane), the points dealt to its
+// eight warps, whose sums are added in warp order: with one thread a k-vector over all
+// points a 512-atom cell kept half of the chip busy.
+constexpr int kSf64Warps = 8;
+
+__global__ void __launch_bounds__(kSf64Warps * 32)
+k_ion_sf_f64(const double2* __restrict__ axis, const AxisPhasors ap, int64_t coord_stride,
+             const double* __restrict__ ion_q, int n_ion, const int* __restrict__ hkl,
+             const double* __restrict__ sqw, int mpad, double* __restrict__ vout) {
+  __shared__ double2 red[kSf64Warps][32];
   const int f = blockIdx.y;
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const double* xyz = ion_xyz + (size_t)f * n_ion * 3;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int k = blockIdx.x * 32 + lane;  // mpad is a multiple of 64
+  const double2* tab = axis + (size_t)f * coord_stride * ap.len;
   const double* q = ion_q + (size_t)f * n_ion;
-  int h = 0, kk = 0, l = 0;
-  if (k < mpad) {
-    h = hkl[3 * k];
-    kk = hkl[3 * k + 1];
-    l = hkl[3 * k + 2];
-  }
+  const int h0 = hkl[3 * k], h1 = hkl[3 * k + 1], h2 = hkl[3 * k + 2];
   double re = 0.0, im = 0.0;
-  for (int base = 0; base < n_ion; base += kIonChunk) {
-    const int cnt = min(kIonChunk, n_ion - base);
-    __syncthreads();
-    for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-      const double L[3] = {lx, ly, lz};
-      for (int d = 0; d < 3; ++d) {
-        double s = xyz[3 * (base + t) + d] / L[d];
-        sd[t][d] = s - floor(s);
-      }
-      sq[t] = q[base + t];
-    }
-    __syncthreads();
-    if (k >= mpad) continue;
-    for (int t = 0; t < cnt; ++t) {
-      double fr = h * sd[t][0] + kk * sd[t][1] + l * sd[t][2];
-      fr -= rint(fr);
-      double s, c;
-      sincospi(2.0 * fr, &s, &c);
-      re += sq[t] * c;
-      im += sq[t] * s;
-    }
+  for (int t = warp; t < n_ion; t += kSf64Warps) {
+    const double2 e = ap.phasor(tab + (size_t)t * ap.len, h0, h1, h2);
+    const double qt = q[t];
+    re += qt * e.x;
+    im += qt * e.y;
   }
-  if (k >= mpad) return;
+  red[warp][lane] = make_double2(re, im);
+  __syncthreads();
+  if (warp != 0) return;
+  for (int w = 1; w < kSf64Warps; ++w) {
+    re += red[w][lane].x;
+    im += red[w][lane].y;
+  }
   const double w = sqw[k];
   const size_t kcol = 128 * (size_t)(k >> 6) + (k & 63);
   double* v = vout + (size_t)f * 2 * mpad;
@@ -790,197 +751,6 @@ k_bsol_real(const double* __restrict__ xyz, const double* __restrict__ alpha,
   if (i == 0 && qsol) qsol[f] = qs;
 }
 
-
-// ---- forces on the ions: F_I = -q_I d/dr_I sum_i q_i e_iI (Eq. S25 inside the Ewald
-// sums of Eq. 22 / 25, the paper's form with Eq. 39) ------------------------------------
-//
-// Reciprocal part: d/dr_I cos(K.(r_i - r_I)) = sin(K.(r_i - r_I)) K, so with the
-// electrode's charge-weighted structure factors (C_K, S_K) = sum_i q_i (cos, sin)(K.r_i),
-// grad_I = sum_K W_K [S_K cos(K.r_I) - C_K sin(K.r_I)] K.  v holds sqrt(W) (C, S) in the
-// operand's column layout (the ions' structure-factor kernel run over the electrode), so
-// the term is sqrt(W_K) (v_s cos - v_c sin).  The head k-vectors (heaviest) in FP64 from
-// FP64 phasors; the tail in float from the table phasors (about one ulp) summed in
-// error-free float pairs; the integer h, k, l multiply last: K = 2 pi (h/Lx, k/Ly, l/Lz).
-constexpr int kForceChunk = 256;
-
-__global__ void __launch_bounds__(128)
-k_force_kspace(const uint32_t* __restrict__ sion, int n_ion, const int* __restrict__ hkl,
-               const double* __restrict__ sqw, int mpad, int kh,
-               const float4* __restrict__ turn, const float* __restrict__ v,
-               const double* __restrict__ vhead, double lx, double ly, double lz,
-               double* __restrict__ grad) {
-  __shared__ int sk[kForceChunk][3];
-  __shared__ double sw[kForceChunk][3];  // head: sqrt(W), v_c, v_s in FP64
-  __shared__ float swf[kForceChunk][3];  // tail: the same as floats (converted once here)
-  const int f = blockIdx.y;
-  const int I = blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t* u = sion + ((size_t)f * n_ion + (I < n_ion ? I : 0)) * 3;
-  const uint32_t u0 = u[0], u1 = u[1], u2 = u[2];
-  const float* vf = v + (size_t)f * 2 * mpad;
-  const double* vh = vhead + (size_t)f * 2 * (size_t)(kh > 0 ? kh : 1);
-  double g64[3] = {0.0, 0.0, 0.0};
-  float gh[3] = {0.f, 0.f, 0.f}, gl[3] = {0.f, 0.f, 0.f};
-  for (int k0 = 0; k0 < mpad; k0 += kForceChunk) {
-    const int cnt = min(kForceChunk, mpad - k0);
-    __syncthreads();
-    for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-      const int k = k0 + t;
-      sk[t][0] = hkl[3 * k];
-      sk[t][1] = hkl[3 * k + 1];
-      sk[t][2] = hkl[3 * k + 2];
-      const size_t kcol = 128 * (size_t)(k >> 6) + (k & 63);
-      sw[t][0] = sqw[k];
-      if (k < kh) {
-        sw[t][1] = vh[kcol];
-        sw[t][2] = vh[kcol + 64];
-      } else {
-        swf[t][0] = (float)sqw[k];
-        swf[t][1] = vf[kcol];
-        swf[t][2] = vf[kcol + 64];
-      }
-    }
-    __syncthreads();
-    if (I >= n_ion) continue;
-    for (int t = 0; t < cnt; ++t) {
-      const uint32_t ph = (uint32_t)sk[t][0] * u0 + (uint32_t)sk[t][1] * u1 +
-                          (uint32_t)sk[t][2] * u2;
-      if (k0 + t < kh) {
-        double sn, cs;
-        sincospi((double)(int32_t)ph * 0x1p-31, &sn, &cs);
-        const double term = sw[t][0] * (sw[t][2] * cs - sw[t][1] * sn);
-        g64[0] += term * sk[t][0];
-        g64[1] += term * sk[t][1];
-        g64[2] += term * sk[t][2];
-      } else {
-        float sn, cs;
-        sincos_table(ph, turn, &sn, &cs);
-        const float term = swf[t][0] * fmaf(swf[t][2], cs, -swf[t][1] * sn);
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          const float x = term * (float)sk[t][d];  // h, k, l: small integers, exact
-          const float s2 = gh[d] + x;
-          const float bb = s2 - gh[d];
-          gl[d] += (gh[d] - (s2 - bb)) + (x - bb);
-          gh[d] = s2;
-        }
-      }
-    }
-  }
-  if (I >= n_ion) return;
-  const double twopi = 2.0 * kPi, L[3] = {lx, ly, lz};
-  double* g = grad + ((size_t)f * n_ion + I) * 3;
-  for (int d = 0; d < 3; ++d) g[d] = (g64[d] + (double)gh[d] + (double)gl[d]) * twopi / L[d];
-}
-
-// d/dr [erfc(g r) / r - erfc(a r) / r] (a = INFINITY: a point charge, no Gaussian term).
-__device__ __forceinline__ double radial_derivative(double g, double a, double r) {
-  const double two_sqrtpi = 1.1283791670955126;  // 2 / sqrt(pi)
-  double num = -two_sqrtpi * g * exp(-(g * r) * (g * r));
-  double e = erfc(g * r);
-  if (isfinite(a)) {
-    num += two_sqrtpi * a * exp(-(a * r) * (a * r));
-    e -= erfc(a * r);
-  }
-  return num / r - e / (r * r);
-}
-
-// Real part and slab term, then F_I = -q_I grad_I.  One thread per ion (grid row: frame);
-// electrode atoms staged by chunks.  A pair is screened in float from the exact
-// fixed-point difference of its nearest image (0.01 A^2 band, as k_bsol_real); the pairs
-// that pass sum every image within r_c in FP64: grad -= q_i f'(r) / r (r_i - r_I + R).
-// The slab term of Eq. 39: grad_z += (4 pi / V) (sum_i q_i z_i - sum_i q_i z_I).
-__global__ void __launch_bounds__(128)
-k_force_real(const double* __restrict__ xyz, const double* __restrict__ alpha,
-             const uint32_t* __restrict__ sfix, int n, const double* __restrict__ ion_xyz,
-             const double* __restrict__ ion_q, const uint32_t* __restrict__ sion, int n_ion,
-             const double* __restrict__ q, double lx, double ly, double lz, double g,
-             double rc, const RealScreen rs, int slab, const double* __restrict__ grad_k,
-             double* __restrict__ out) {
-  __shared__ uint32_t su[kForceChunk][3];
-  __shared__ double sx[kForceChunk][5];  // x, y, z, alpha, q
-  __shared__ double red[2][128];
-  const int f = blockIdx.y;
-  const int I = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool live = I < n_ion;
-  const size_t e = (size_t)f * n_ion + (live ? I : 0);
-  const double ri[3] = {ion_xyz[3 * e], ion_xyz[3 * e + 1], ion_xyz[3 * e + 2]};
-  const uint32_t ui[3] = {sion[3 * e], sion[3 * e + 1], sion[3 * e + 2]};
-  const double* qf = q + (size_t)f * n;
-  const double L[3] = {lx, ly, lz};
-  const double invL[3] = {1.0 / lx, 1.0 / ly, 1.0 / lz};
-  const double rc2 = rc * rc;
-  double gr[3] = {0.0, 0.0, 0.0};
-  double qz = 0.0, qs = 0.0;  // this thread's share of sum q_i z_i and sum q_i
-  for (int base = 0; base < n; base += kForceChunk) {
-    const int cnt = min(kForceChunk, n - base);
-    __syncthreads();
-    for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-      const int i = base + t;
-      su[t][0] = sfix[3 * i];
-      su[t][1] = sfix[3 * i + 1];
-      su[t][2] = sfix[3 * i + 2];
-      sx[t][0] = xyz[3 * i];
-      sx[t][1] = xyz[3 * i + 1];
-      sx[t][2] = xyz[3 * i + 2];
-      sx[t][3] = alpha[i];
-      sx[t][4] = qf[i];
-      qz += qf[i] * xyz[3 * i + 2];
-      qs += qf[i];
-    }
-    __syncthreads();
-    if (!live) continue;
-    for (int t = 0; t < cnt; ++t) {
-      float m2 = 0.f;
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const float du = (float)(int32_t)(su[t][d] - ui[d]) * rs.fs[d];
-        m2 = fmaf(du, du, m2);
-      }
-      if (m2 >= rs.screen2) continue;
-      // every image of the pair within r_c
-      double d0[3];
-      int lo[3], hi[3];
-      for (int d = 0; d < 3; ++d) {
-        d0[d] = sx[t][d] - ri[d];
-        d0[d] -= L[d] * rint(d0[d] * invL[d]);
-        lo[d] = (int)ceil((-rc - d0[d]) * invL[d]);
-        hi[d] = (int)floor((rc - d0[d]) * invL[d]);
-      }
-      for (int a = lo[0]; a <= hi[0]; ++a)
-        for (int b = lo[1]; b <= hi[1]; ++b)
-          for (int c = lo[2]; c <= hi[2]; ++c) {
-            const double dx = d0[0] + a * L[0], dy = d0[1] + b * L[1], dz = d0[2] + c * L[2];
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            if (r2 >= rc2 || r2 == 0.0) continue;
-            const double r = sqrt(r2);
-            const double w = sx[t][4] * radial_derivative(g, sx[t][3], r) / r;
-            gr[0] -= w * dx;
-            gr[1] -= w * dy;
-            gr[2] -= w * dz;
-          }
-    }
-  }
-  // the frame's sum q_i z_i and sum q_i over the block's threads
-  red[0][threadIdx.x] = qz;
-  red[1][threadIdx.x] = qs;
-  __syncthreads();
-  for (int o = 64; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) {
-      red[0][threadIdx.x] += red[0][threadIdx.x + o];
-      red[1][threadIdx.x] += red[1][threadIdx.x + o];
-    }
-    __syncthreads();
-  }
-  if (!live) return;
-  const double* gk = grad_k + e * 3;
-  double gz = gr[2] + gk[2];
-  if (slab) gz += (4.0 * kPi / (lx * ly * lz)) * (red[0][0] - red[1][0] * ri[2]);
-  const double qI = ion_q[e];
-  out[3 * e] = -qI * (gr[0] + gk[0]);
-  out[3 * e + 1] = -qI * (gr[1] + gk[1]);
-  out[3 * e + 2] = -qI * gz;
-}
-
 }  // namespace
 
 void launch_ion_fixed(const double* ion_xyz, int frames, int n_ion, const double L[3],
@@ -994,18 +764,26 @@ void launch_turn_table(void* T, cudaStream_t s) {
   (k_turn_table<<<16, 256, 0, s>>>((float4*)T), note_launch());
 }
 
-void launch_ion_structure_factor(bool fp64, const double* ion_xyz, const uint32_t* sion,
+void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
+                         const double L[3], const AxisPhasors& ap, double2* out,
+                         cudaStream_t s) {
+  const int blocks = (int)std::min<int64_t>((count * ap.len + 127) / 128, 16384);
+  (k_axis_phasors<<<blocks, 128, 0, s>>>(xyz, sfix, count, L[0], L[1], L[2], ap, out), note_launch());
+}
+
+void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhasors& ap,
+                                 const uint32_t* sion, int64_t coord_stride,
                                  const double* ion_q, int frames, int n_ion, const int* hkl,
-                                 const double* sqw, int mpad, int kh, const double L[3],
-                                 const void* turn, void* v, double* vhead, cudaStream_t s) {
+                                 const double* sqw, int mpad, int kh, const void* turn,
+                                 void* v, double* vhead, cudaStream_t s) {
   if (fp64) {
-    dim3 grid((mpad + kSfThreads - 1) / kSfThreads, frames);
-    (k_ion_sf_f64<<<grid, kSfThreads, 0, s>>>(ion_xyz, ion_q, n_ion, hkl, sqw, mpad, L[0], L[1],
-                                              L[2], (double*)v), note_launch());
+    (k_ion_sf_f64<<<dim3(mpad / 32, frames), kSf64Warps * 32, 0, s>>>(
+         axis, ap, coord_stride, ion_q, n_ion, hkl, sqw, mpad, (double*)v),
+     note_launch());
   } else {
     dim3 grid((mpad + kSfThreads - 1) / kSfThreads, frames);
-    (k_ion_sf_f32<<<grid, kSfThreads, 0, s>>>(sion, ion_q, n_ion, hkl, sqw, mpad, kh,
-                                              (const float4*)turn, (float*)v, vhead),
+    (k_ion_sf_f32<<<grid, kSfThreads, 0, s>>>(sion, coord_stride, ion_q, n_ion, hkl, sqw, mpad,
+                                              kh, (const float4*)turn, (float*)v, vhead),
      note_launch());
   }
 }
@@ -1125,26 +903,6 @@ void launch_bsol_real_and_finish(const double* xyz, const double* alpha, const u
   (kernel<<<grid, kRealWarps * 32, 0, s>>>(xyz, alpha, sfix, n, ion_xyz, ion_q, sion, n_ion,
                                           geo.L[0], geo.L[1], geo.L[2], geo.g, geo.rc, rs, dip,
                                           chi, bsol_k, b_out, qsol),
-   note_launch());
-}
-
-}  // namespace cpm
-
-namespace cpm {
-
-void launch_ion_forces(const double* xyz, const double* alpha, const uint32_t* sfix, int n,
-                       const double* ion_xyz, const double* ion_q, const uint32_t* sion,
-                       int frames, int n_ion, const double* q, const int* hkl,
-                       const double* sqw, int mpad, int kh, const Geometry& geo,
-                       const void* turn, const float* v, const double* vhead, double* grad,
-                       double* out, cudaStream_t s) {
-  const dim3 grid((n_ion + 127) / 128, frames);
-  (k_force_kspace<<<grid, 128, 0, s>>>(sion, n_ion, hkl, sqw, mpad, kh, (const float4*)turn, v,
-                                       vhead, geo.L[0], geo.L[1], geo.L[2], grad),
-   note_launch());
-  (k_force_real<<<grid, 128, 0, s>>>(xyz, alpha, sfix, n, ion_xyz, ion_q, sion, n_ion, q,
-                                     geo.L[0], geo.L[1], geo.L[2], geo.g, geo.rc,
-                                     real_screen(geo, geo.rc * geo.rc), geo.slab, grad, out),
    note_launch());
 }
 
