@@ -357,7 +357,7 @@ void free_build(Ctx* c) {
                 &c->Ahead, &c->A,
                 &c->E, &c->diag,
                 &c->nbr_off, &c->nbr_idx, &c->prow, &c->d, &c->shell_off, &c->shell_members, &c->p_f32,
-                &c->turn, &c->gcd_labels, &c->gcd_a, &c->gcd_c, &c->gcd_cinv, &c->gcd_status,
+                &c->turn, &c->htab, &c->atoms, &c->gcd_labels, &c->gcd_a, &c->gcd_c, &c->gcd_cinv, &c->gcd_status,
                 &c->gcd_scratch, &c->smat};
   for (Buf* b : all) buf_free(c, b);
   release_workspace(c);
@@ -653,6 +653,8 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
   if ((st = buf_reserve(c, &c->xyz, (size_t)n * 3 * sizeof(double))) ||
       (st = buf_reserve(c, &c->alpha, (size_t)n * sizeof(double))) ||
       (st = buf_reserve(c, &c->sfix, (size_t)c->npad * 3 * sizeof(uint32_t))) ||
+      (!f64 && (st = buf_reserve(c, &c->atoms, atom_record_bytes(n)))) ||
+      (!f64 && (st = buf_reserve(c, &c->htab, h_table_bytes()))) ||
       (st = buf_reserve(c, &c->hkl, hkl.size() * sizeof(int))) ||
       (st = buf_reserve(c, &c->sqw, sqw.size() * sizeof(double))) ||
       (st = buf_reserve(c, &c->flush, fmask.size() * sizeof(uint32_t))) ||
@@ -679,6 +681,8 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
       (st = cuda_check(c, cudaMemcpyAsync(c->flush.ptr, fmask.data(), fmask.size() * sizeof(uint32_t), h2d, s), "flush")) ||
       (st = cuda_check(c, cudaMemcpyAsync(c->chunk_end.ptr, cmask.data(), cmask.size() * sizeof(uint32_t), h2d, s), "chunks")) ||
       (st = cuda_check(c, cudaMemcpyAsync(c->kexp.ptr, kexp.data(), kexp.size() * sizeof(int), h2d, s), "scales")) ||
+      (!f64 && (st = cuda_check(c, cudaMemcpyAsync(c->htab.ptr, h_table_host(), h_table_bytes(),
+                                                   h2d, s), "erfc table"))) ||
       (st = cuda_check(c, cudaMemsetAsync(c->E.ptr, 0, e_bytes, s), "E memset")) ||
       (st = cuda_check(c, cudaStreamSynchronize(s), "build upload")))
     return fail(st);
@@ -703,6 +707,9 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
   cudaEventRecord(ev[0], s);
   launch_fixed_point_coords((const double*)c->xyz.ptr, n, c->npad, c->p.box,
                             (uint32_t*)c->sfix.ptr, s);
+  if (!f64)
+    launch_atom_records((const double*)c->xyz.ptr, (const double*)c->alpha.ptr, n, geo,
+                        c->atoms.ptr, s);
   // the tensor-core workspace stays with the context for the next build (released by
   // cpm_release_workspace or cpm_destroy, and on a failed build)
   Buf* planes = c->tc_planes;
@@ -973,7 +980,8 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
     return st;
   // scratch: v [frames][2 mpad] (storage type) | v_head [frames][2 kh] | b^sol_k [frames][n]
   //          | fixed-point ion coordinates [frames][n_ion][3] | the direct sum's k-range
-  //          shares [nsplit][frames][n] (a streamed build split into more than one)
+  //          shares [nsplit][frames][n] (a streamed build split into more than one) | the
+  //          ions' per-axis phasors (FP64 storage) | the real-space part's scratch
   auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
   const size_t vbytes = up((size_t)frames * 2 * c->mpad * c->esz());
   const size_t hbytes = up((size_t)frames * 2 * std::max(c->kh, 1) * sizeof(double));
@@ -989,7 +997,8 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   const AxisPhasors ap = axis_phasors(c);
   const int fchunk = axis_frames(ap, frames, n_ion);
   const size_t abytes = f64 ? up((size_t)fchunk * std::max(n_ion, 1) * ap.len * sizeof(double2)) : 0;
-  if ((st = buf_reserve(c, &c->ws_pot, vbytes + hbytes + kbytes + ubytes + sbytes + abytes)))
+  const RealPlan rp = real_plan(n, frames, n_ion, std::max(dev_sms, 1));
+  if ((st = buf_reserve(c, &c->ws_pot, vbytes + hbytes + kbytes + ubytes + sbytes + abytes + rp.bytes)))
     return st;
   if (!f64 && !c->turn.ptr) {
     if ((st = buf_alloc(c, &c->turn, 4096 * 4 * sizeof(float)))) return st;
@@ -1002,6 +1011,7 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   double* spart =
       nsplit > 1 ? (double*)((char*)c->ws_pot.ptr + vbytes + hbytes + kbytes + ubytes) : nullptr;
   double2* axis = (double2*)((char*)c->ws_pot.ptr + vbytes + hbytes + kbytes + ubytes + sbytes);
+  void* rscratch = (char*)axis + abytes;
   cudaEvent_t pev[4];
   for (int e = 0; e < 4; ++e) {
     while (c->ev_pot.size() < 4) {
@@ -1013,7 +1023,7 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   }
   cudaEventRecord(pev[0], s);
   if (n_ion > 0) {
-    launch_ion_fixed(dx, frames, n_ion, c->p.box, sion, s);
+    launch_ion_prepare(dx, dq, frames, n_ion, geometry(c), sion, rp, rscratch, s);
     for (int f0 = 0; f0 < frames; f0 += f64 ? fchunk : frames) {
       const int nf = f64 ? std::min(fchunk, frames - f0) : frames;
       if (f64)
@@ -1033,9 +1043,9 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
                      (const double*)c->sqw.ptr, c->turn.ptr, nsplit, spart, s);
   cudaEventRecord(pev[2], s);
   launch_bsol_real_and_finish((const double*)c->xyz.ptr, (const double*)c->alpha.ptr,
-                              (const uint32_t*)c->sfix.ptr, n, dx, dq, sion, frames, n_ion,
-                              geometry(c), dchi, bk, db, dqs,
-                              c->p.precision != CPM_PREC_FP64, s);
+                              (const uint32_t*)c->sfix.ptr, c->atoms.ptr, c->htab.ptr, n, dx, dq,
+                              frames, n_ion, geometry(c), dchi, bk, db, dqs, f64, rp, rscratch,
+                              s);
   cudaEventRecord(pev[3], s);
   if ((st = cuda_check(c, cudaGetLastError(), "potential kernels"))) return st;
   if (qsol_out && n_ion == 0 &&

@@ -127,6 +127,8 @@ struct Ctx {
   double pgap = 0;
 
   // learned-guess feature geometry (frame independent, made on first use)
+  Buf htab;       // erfc(sqrt s) / sqrt s (real-space pairs of float storage)
+  Buf atoms;      // the electrode's records for the real-space pairs
   Buf turn;       // float4 [4096]: exp(2 pi i j / 4096) as float pairs (ion phasors)
   Buf shell_off;    // int64 [8n+1]: offsets of the (atom, shell 1..8) buckets in shell_members
   Buf shell_members;  // int32: members of the buckets (neighbours filed by shell)
@@ -274,11 +276,28 @@ void launch_bsol_kspace(bool fp64, const void* A, const double* Ahead, int n, in
 // shares of the k range of a streamed build's direct k-space sum (split_part then holds
 // nsplit x frames x n doubles)
 int bsol_direct_splits(int n, int frames, int mpad, int kh, int sms);
+
+// real_space.cu
+struct RealPlan {
+  int shares, grid_shares;      // shares of the ions within a block and over the grid
+  size_t o_sums, o_part, bytes; // scratch layout: ion records | block sums | partials
+};
+RealPlan real_plan(int n, int frames, int n_ion, int sms);
+size_t h_table_bytes();
+const void* h_table_host();     // erfc(sqrt s) / sqrt s, for a device copy
+size_t atom_record_bytes(int n);
+void launch_atom_records(const double* xyz, const double* alpha, int n, const Geometry& geo,
+                         void* rec, cudaStream_t s);
+// fixed-point ion coordinates (sion [frames][n_ion][3]) and the real-space part's scratch
+void launch_ion_prepare(const double* ion_xyz, const double* ion_q, int frames, int n_ion,
+                        const Geometry& geo, uint32_t* sion, const RealPlan& plan, void* scratch,
+                        cudaStream_t s);
 void launch_bsol_real_and_finish(const double* xyz, const double* alpha, const uint32_t* sfix,
-                                 int n, const double* ion_xyz, const double* ion_q,
-                                 const uint32_t* sion, int frames, int n_ion,
-                                 const Geometry& geo, const double* chi, const double* bsol_k,
-                                 double* b_out, double* qsol, bool far_float, cudaStream_t s);
+                                 const void* atoms, const void* htab, int n,
+                                 const double* ion_xyz, const double* ion_q, int frames,
+                                 int n_ion, const Geometry& geo, const double* chi,
+                                 const double* bsol_k, double* b_out, double* qsol, bool fp64,
+                                 const RealPlan& plan, void* scratch, cudaStream_t s);
 
 // forces.cu
 struct ForceSplits {

@@ -63,7 +63,7 @@ __device__ __forceinline__ void write_gradients(float2 (&gh)[kFkIons / 2][3],
 // error-free float pair); share nsplit, where there is one, the head (k < kh, the heaviest weights) in float
 // pairs throughout (~1e-13: FP64 runs at 1/64 of the float rate).  One thread per ion over
 // the whole k range, the form before, kept 16 blocks of the chip busy with 2,000 ions:
-// 30.7 ms with 217,619 k-vectors against 0.9 ms.
+// 30.7 ms with 217,619 k-vectors against 0.83 ms.
 __global__ void __launch_bounds__(kFkThreads)
 k_force_kspace(const uint32_t* __restrict__ sion, int n_ion, const int* __restrict__ hkl,
                const double* __restrict__ sqw, int mpad, int kh, int nsplit,
@@ -127,7 +127,7 @@ k_force_kspace(const uint32_t* __restrict__ sion, int n_ion, const int* __restri
         ff_add(ah, al, -bh, -bl, th, tl);
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          const float x = th * hf[d];
+          const float x = __fmul_rn(th, hf[d]);
           const float xl = fmaf(tl, hf[d], fmaf(th, hf[d], -x));
           if (t & 1) pair_add_pair(gh[t >> 1][d].y, gl[t >> 1][d].y, x, xl);
           else pair_add_pair(gh[t >> 1][d].x, gl[t >> 1][d].x, x, xl);

@@ -9,7 +9,7 @@ namespace cpm {
 // a * b for float pairs, to ~2^-44 relative (the lo * lo term dropped).
 __device__ __forceinline__ void ff_mul(float ah, float al, float bh, float bl, float& ph,
                                        float& pl) {
-  ph = ah * bh;
+  ph = __fmul_rn(ah, bh);  // not fused with the sums it enters
   pl = fmaf(ah, bh, -ph) + fmaf(ah, bl, al * bh);
 }
 

@@ -384,373 +384,6 @@ k_bsol_kspace_direct(const uint32_t* __restrict__ sfix, int n, const int* __rest
     }
 }
 
-// FP64 real-space sum of one electrode-ion pair over every image within r_c:
-// sum q_I [erfc(g r) - erfc(alpha_i r)] / r.
-// When every box edge exceeds 2 r_c only the nearest image can be in range.
-__device__ __forceinline__ double pair_images(const double* ri, double ai, const double* ion,
-                                              const double* L, const double* invL,
-                                              const bool* single, double rc, double rc2,
-                                              double g) {
-  double d[3] = {ri[0] - ion[0], ri[1] - ion[1], ri[2] - ion[2]};
-  if (single[0] && single[1] && single[2]) {
-    for (int u = 0; u < 3; ++u) d[u] -= L[u] * rint(d[u] * invL[u]);
-    const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-    if (r2 >= rc2 || r2 == 0.0) return 0.0;
-    const double r = sqrt(r2);
-    double e = erfc(g * r);
-    if (ai * r < 6.0) e -= erfc(ai * r);
-    return ion[3] * e / r;
-  }
-  int lo[3], hi[3];
-  for (int u = 0; u < 3; ++u) {
-    if (single[u]) {  // box edge above 2 rc: only the minimum image can be in range
-      d[u] -= L[u] * rint(d[u] * invL[u]);
-      lo[u] = hi[u] = 0;
-    } else {
-      lo[u] = (int)ceil((-rc - d[u]) * invL[u]);
-      hi[u] = (int)floor((rc - d[u]) * invL[u]);
-    }
-  }
-  double acc = 0.0;
-  for (int a = lo[0]; a <= hi[0]; ++a) {
-    const double x = d[0] + a * L[0];
-    for (int b = lo[1]; b <= hi[1]; ++b) {
-      const double y = d[1] + b * L[1];
-      const double xy = x * x + y * y;
-      if (xy >= rc2) continue;
-      for (int c = lo[2]; c <= hi[2]; ++c) {
-        const double z = d[2] + c * L[2];
-        const double r2 = xy + z * z;
-        if (r2 >= rc2 || r2 == 0.0) continue;
-        const double r = sqrt(r2);
-        double e = erfc(g * r);
-        // erfc(6) < 3e-17: beyond alpha r = 6 the Gaussian term is below double rounding
-        // of the erfc(g r) term
-        if (ai * r < 6.0) e -= erfc(ai * r);
-        acc += ion[3] * e / r;
-      }
-    }
-  }
-  return acc;
-}
-
-// Real-space electrode-ion sums, slab dipole term, and b = chi - k_e b^sol.
-// Four warps, 32 electrode atoms each (one a lane); ions staged through shared memory in
-// chunks.  Each lane screens its atom against every ion and every image of it that can
-// lie within r_c: the nearest image from the exact fixed-point coordinate difference,
-// plus the host's list of whole-box shifts (just the zero shift when every box edge
-// exceeds 2 r_c), in float (off by < 1e-3 A^2 in r^2, against a band of 0.01 A^2).  The
-// images that pass go to one of two per-warp queues that outlive the chunks and are
-// evaluated 32 at a time, all lanes busy, each atom then adding its queued values in
-// queue order:
-//   near images: FP64, from the FP64 coordinates kept in the queue, the image fixed by
-//     the fixed-point nearest one and the shift (so the screen and the sum agree on it);
-//   far images (r^2 >= r_split^2 where erfc(g r) / r <= 1e-4 1/A, r^2 below r_c^2 by more
-//     than the float error, alpha r >= 6 so that the Gaussian term has vanished): float,
-//     from the screen's r^2 (~1e-7 relative; the term to ~1e-6 of itself, <= 1e-10 1/A),
-//     summed in float apart and added at the end.
-// No warp runs both arithmetic paths in one pass.  A box so small that more than
-// kMaxShifts shifts would be needed takes every image of a screened pair in FP64 instead.
-// The float constants of the screen come from the host: FP64 runs at 1/64 of the float
-// rate here, and a constant formed from the FP64 parameters would otherwise be re-formed
-// inside the loop.
-constexpr int kRealWarps = 4;
-
-constexpr int kMaxShifts = 64;
-
-struct RealScreen {
-  float fs[3];    // L / 2^32: fixed-point units of each coordinate, A
-  float screen2;  // r_c^2 + 0.01
-  float cut2;     // r_c^2 (1 - 1e-5): far pairs lie below
-  float far2;     // r_split^2 (r_c^2 when no pair is far)
-  float g;        // Ewald splitting parameter, 1/A
-  int all_single; // every box edge above 2 r_c
-  int nshift;     // whole-box shifts screened (0: every image of a pair in FP64)
-  float shift[kMaxShifts][3];       // k L, A
-  signed char kshift[kMaxShifts][3];  // k
-};
-
-RealScreen real_screen(const Geometry& geo, double rsplit2) {
-  RealScreen rs;
-  for (int u = 0; u < 3; ++u) rs.fs[u] = (float)(geo.L[u] * 0x1p-32);
-  const double rc2 = geo.rc * geo.rc;
-  rs.screen2 = (float)rc2 + 0.01f;
-  rs.cut2 = (float)(rc2 * (1.0 - 1e-5));
-  rs.far2 = (float)rsplit2;
-  rs.g = (float)geo.g;
-  rs.all_single = 2.0 * geo.rc < geo.L[0] && 2.0 * geo.rc < geo.L[1] && 2.0 * geo.rc < geo.L[2];
-  // shifts k with |k| <= floor((r_c + L / 2) / L) per direction (only k = 0 where
-  // L > 2 r_c): every image within r_c of an atom, given the nearest one
-  int m[3], total = 1;
-  for (int u = 0; u < 3; ++u) {
-    m[u] = 2.0 * geo.rc < geo.L[u] ? 0 : (int)floor((geo.rc + 0.5 * geo.L[u]) / geo.L[u]);
-    total *= 2 * m[u] + 1;
-  }
-  rs.nshift = total <= kMaxShifts ? total : 0;
-  int k = 0;
-  for (int a = -m[0]; rs.nshift && a <= m[0]; ++a)
-    for (int b = -m[1]; b <= m[1]; ++b)
-      for (int c = -m[2]; c <= m[2]; ++c, ++k) {
-        const int ks[3] = {a, b, c};
-        for (int u = 0; u < 3; ++u) {
-          rs.shift[k][u] = (float)(ks[u] * geo.L[u]);
-          rs.kshift[k][u] = (signed char)ks[u];
-        }
-      }
-  return rs;
-}
-
-// Screen modes: every box edge above 2 r_c (the nearest image only, near and far queues),
-// a list of whole-box shifts (each shifted image screened, near and far queues), or every
-// image of a screened pair in FP64 (boxes needing more than kMaxShifts shifts).
-enum RealMode { kSingleImage = 0, kShiftList = 1, kAllImages = 2 };
-
-template <int kMode>
-__global__ void __launch_bounds__(kRealWarps * 32, 6)
-k_bsol_real(const double* __restrict__ xyz, const double* __restrict__ alpha,
-            const uint32_t* __restrict__ sfix, int n, const double* __restrict__ ion_xyz,
-            const double* __restrict__ ion_q, const uint32_t* __restrict__ sion, int n_ion,
-            double lx, double ly, double lz, double g, double rc, const RealScreen rs,
-            double dip, const double* __restrict__ chi, const double* __restrict__ bsol_k,
-            double* __restrict__ b_out, double* __restrict__ qsol) {
-  __shared__ double sx[kIonChunk][4];
-  __shared__ uint4 su[kIonChunk];  // fixed-point x, y, z (and a pad: one 16-byte load)
-  __shared__ double sa[kRealWarps * 32][4];   // the block's atoms: x, y, z, alpha
-  __shared__ double nq[kRealWarps][64][4];    // near queue: ion x, y, z, q,
-  constexpr int kShiftWarps = kMode == kShiftList ? kRealWarps : 1;
-  __shared__ int32_t ndl[kShiftWarps][64][3];  //   the fixed-point difference, the shift
-  __shared__ uint8_t nsh[kShiftWarps][64];
-  __shared__ float2 fq[kRealWarps][64];       // far queue: r^2, q
-  __shared__ uint8_t nlane[kRealWarps][64], flane[kRealWarps][64];
-  __shared__ double qval[kRealWarps][32];
-  __shared__ float fval[kRealWarps][32];
-  const int f = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const double* ix = ion_xyz + (size_t)f * n_ion * 3;
-  const double* iq = ion_q + (size_t)f * n_ion;
-  const uint32_t* iu = sion + (size_t)f * n_ion * 3;
-  uint32_t ui[3] = {0, 0, 0};
-  float af2 = 0.f;  // alpha^2 of the lane's atom
-  if (i < n) {
-    ui[0] = sfix[3 * i];
-    ui[1] = sfix[3 * i + 1];
-    ui[2] = sfix[3 * i + 2];
-    sa[threadIdx.x][0] = xyz[3 * i];
-    sa[threadIdx.x][1] = xyz[3 * i + 1];
-    sa[threadIdx.x][2] = xyz[3 * i + 2];
-    sa[threadIdx.x][3] = alpha[i];
-    af2 = (float)(alpha[i] * alpha[i]);
-  }
-  const double L[3] = {lx, ly, lz};
-  const double rc2 = rc * rc;
-  const double invL[3] = {1.0 / lx, 1.0 / ly, 1.0 / lz};
-  const bool single[3] = {2.0 * rc < lx, 2.0 * rc < ly, 2.0 * rc < lz};
-  // evaluates the first `cnt` queued images (one a lane); each atom adds its values in
-  // queue order
-  auto drain = [&](int cnt, double& acc) {
-    __syncwarp();
-    if (lane < cnt) {
-      const int a = nlane[warp][lane];
-      const double* at = sa[warp * 32 + a];
-      const double* ion = nq[warp][lane];
-      if constexpr (kMode == kShiftList) {
-        // the image: the fixed-point nearest one (whole boxes k from the FP64 difference)
-        // plus the queued shift (with every edge above 2 r_c the shift is zero, and the
-        // nearest image by rint below is the same but where it lies beyond r_c)
-        const int si = nsh[warp][lane];
-        double r2 = 0.0;
-#pragma unroll
-        for (int u = 0; u < 3; ++u) {
-          const double dd = at[u] - ion[u];
-          const double dfx = (double)ndl[warp][lane][u] * (L[u] * 0x1p-32);
-          const double k = rint((dd - dfx) * invL[u]) - (double)rs.kshift[si][u];
-          const double du = dd - k * L[u];
-          r2 += du * du;
-        }
-        double v = 0.0;
-        if (r2 < rc2 && r2 > 0.0) {
-          const double r = sqrt(r2);
-          double e = erfc(g * r);
-          if (at[3] * r < 6.0) e -= erfc(at[3] * r);
-          v = ion[3] * e / r;
-        }
-        qval[warp][lane] = v;
-      } else {
-        qval[warp][lane] = pair_images(at, at[3], ion, L, invL, single, rc, rc2, g);
-      }
-    }
-    __syncwarp();
-    for (int k = 0; k < cnt; ++k)
-      if (nlane[warp][k] == lane) acc += qval[warp][k];
-    __syncwarp();
-  };
-  auto drain_far = [&](int cnt, float& acc) {
-    __syncwarp();
-    if (lane < cnt) {
-      const float2 e = fq[warp][lane];
-      const float ir = rsqrtf(e.x);  // 1 / r to ~2 ulp
-      fval[warp][lane] = e.y * (erfcf(rs.g * (e.x * ir)) * ir);
-    }
-    __syncwarp();
-    for (int k = 0; k < cnt; ++k)
-      if (flane[warp][k] == lane) acc += fval[warp][k];
-    __syncwarp();
-  };
-  // sum q_I z_I and sum q_I over the frame: each thread takes the ions it stages
-  double acc = 0.0, qz = 0.0, qs = 0.0;
-  float accf = 0.f;
-  int qn = 0, fn = 0;  // queued near and far pairs of this warp (warp-uniform)
-  const unsigned below = (1u << lane) - 1u;
-  for (int base = 0; base < n_ion; base += kIonChunk) {
-    const int cnt = min(kIonChunk, n_ion - base);
-    __syncthreads();
-    for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-      sx[t][0] = ix[3 * (base + t)];
-      sx[t][1] = ix[3 * (base + t) + 1];
-      sx[t][2] = ix[3 * (base + t) + 2];
-      sx[t][3] = iq[base + t];
-      su[t] = make_uint4(iu[3 * (base + t)], iu[3 * (base + t) + 1], iu[3 * (base + t) + 2], 0u);
-      qz += sx[t][3] * sx[t][2];
-      qs += sx[t][3];
-    }
-    __syncthreads();
-    // one image of ion t (whole-box shift si) at r^2 = m2: classified, queued, and the
-    // queues drained when full (no lane's image within the screen: nothing, one vote)
-    auto place = [&](int t, int si, float m2, const int32_t (&dl)[3]) {
-      const bool inr = i < n && m2 < rs.screen2;
-      if (!__any_sync(0xffffffffu, inr)) return;
-      bool far = false;
-      if constexpr (kMode != kAllImages)
-        far = inr && m2 >= rs.far2 && m2 < rs.cut2 && af2 * m2 >= 36.0f;
-      const bool near = inr && !far;
-      const unsigned mn = __ballot_sync(0xffffffffu, near);
-      const unsigned mf = __ballot_sync(0xffffffffu, far);
-      if (near) {
-        const int at = qn + __popc(mn & below);
-        nq[warp][at][0] = sx[t][0];
-        nq[warp][at][1] = sx[t][1];
-        nq[warp][at][2] = sx[t][2];
-        nq[warp][at][3] = sx[t][3];
-        if constexpr (kMode == kShiftList) {
-          ndl[warp][at][0] = dl[0];
-          ndl[warp][at][1] = dl[1];
-          ndl[warp][at][2] = dl[2];
-          nsh[warp][at] = (uint8_t)si;
-        }
-        nlane[warp][at] = (uint8_t)lane;
-      }
-      if (far) {
-        const int at = fn + __popc(mf & below);
-        fq[warp][at] = make_float2(m2, (float)sx[t][3]);
-        flane[warp][at] = (uint8_t)lane;
-      }
-      qn += __popc(mn);
-      fn += __popc(mf);
-      if (qn >= 32) {
-        drain(32, acc);
-        if (lane < qn - 32) {
-#pragma unroll
-          for (int c = 0; c < 4; ++c) nq[warp][lane][c] = nq[warp][32 + lane][c];
-          if constexpr (kMode == kShiftList) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) ndl[warp][lane][c] = ndl[warp][32 + lane][c];
-            nsh[warp][lane] = nsh[warp][32 + lane];
-          }
-          nlane[warp][lane] = nlane[warp][32 + lane];
-        }
-        qn -= 32;
-        __syncwarp();
-      }
-      if (fn >= 32) {
-        drain_far(32, accf);
-        if (lane < fn - 32) {
-          fq[warp][lane] = fq[warp][32 + lane];
-          flane[warp][lane] = flane[warp][32 + lane];
-        }
-        fn -= 32;
-        __syncwarp();
-      }
-    };
-    // the nearest image's fixed-point difference (dl) and float components (dn)
-    auto nearest = [&](int t, int32_t (&dl)[3], float (&dn)[3]) {
-      const uint4 ut = su[t];
-      dl[0] = (int32_t)(ui[0] - ut.x);
-      dl[1] = (int32_t)(ui[1] - ut.y);
-      dl[2] = (int32_t)(ui[2] - ut.z);
-#pragma unroll
-      for (int u = 0; u < 3; ++u) dn[u] = (float)dl[u] * rs.fs[u];
-    };
-    if constexpr (kMode == kShiftList) {
-      for (int t = 0; t < cnt; ++t) {
-        int32_t dl[3] = {0, 0, 0};
-        float dn[3] = {0.f, 0.f, 0.f};
-        if (i < n) nearest(t, dl, dn);
-        for (int si = 0; si < rs.nshift; ++si) {
-          float m2 = 0.f;
-#pragma unroll
-          for (int u = 0; u < 3; ++u) {
-            const float du = dn[u] + rs.shift[si][u];
-            m2 = fmaf(du, du, m2);
-          }
-          place(t, si, m2, dl);
-        }
-      }
-    } else {
-      // two ions a step: their r^2 in paired instructions (each the scalar fma chain's
-      // value), one vote over both, then each placed in ion order
-      const int32_t dz[3] = {0, 0, 0};
-      int t = 0;
-      for (; t + 1 < cnt; t += 2) {
-        float2 m2 = make_float2(0.f, 0.f);
-        if (i < n) {
-          int32_t da[3], db[3];
-          float fa[3], fb[3];
-          nearest(t, da, fa);
-          nearest(t + 1, db, fb);
-          const float2 d0 = make_float2(fa[0], fb[0]), d1 = make_float2(fa[1], fb[1]),
-                       d2 = make_float2(fa[2], fb[2]);
-          m2 = __ffma2_rn(d0, d0, __ffma2_rn(d1, d1, __fmul2_rn(d2, d2)));
-        }
-        const bool any = i < n && fminf(m2.x, m2.y) < rs.screen2;
-        if (!__any_sync(0xffffffffu, any)) continue;
-        place(t, 0, m2.x, dz);
-        place(t + 1, 0, m2.y, dz);
-      }
-      if (t < cnt) {
-        float m2 = 0.f;
-        if (i < n) {
-          int32_t dl[3];
-          float dn[3];
-          nearest(t, dl, dn);
-          m2 = fmaf(dn[0], dn[0], fmaf(dn[1], dn[1], dn[2] * dn[2]));
-        }
-        place(t, 0, m2, dz);
-      }
-    }
-  }
-  if (qn > 0) drain(qn, acc);
-  if (fn > 0) drain_far(fn, accf);
-  acc += (double)accf;
-  __shared__ double red[2][kRealWarps];
-  for (int o = 16; o; o >>= 1) {
-    qz += __shfl_xor_sync(0xffffffffu, qz, o);
-    qs += __shfl_xor_sync(0xffffffffu, qs, o);
-  }
-  if (lane == 0) {
-    red[0][warp] = qz;
-    red[1][warp] = qs;
-  }
-  __syncthreads();
-  qz = red[0][0] + red[0][1] + red[0][2] + red[0][3];
-  qs = red[1][0] + red[1][1] + red[1][2] + red[1][3];
-  if (i < n) {
-    double bs = bsol_k[(size_t)f * n + i] + acc + dip * sa[threadIdx.x][2] * qz;
-    b_out[(size_t)f * n + i] = chi[i] - kKe * bs;
-  }
-  if (i == 0 && qsol) qsol[f] = qs;
-}
-
 }  // namespace
 
 void launch_ion_fixed(const double* ion_xyz, int frames, int n_ion, const double L[3],
@@ -874,36 +507,6 @@ void launch_bsol_kspace(bool fp64, const void* A, const double* Ahead, int n, in
                                                        bsol + (int64_t)f0 * n, 1), note_launch());
     }
   }
-}
-
-void launch_bsol_real_and_finish(const double* xyz, const double* alpha, const uint32_t* sfix,
-                                 int n, const double* ion_xyz, const double* ion_q,
-                                 const uint32_t* sion, int frames, int n_ion,
-                                 const Geometry& geo, const double* chi, const double* bsol_k,
-                                 double* b_out, double* qsol, bool far_float, cudaStream_t s) {
-  dim3 grid((n + kRealWarps * 32 - 1) / (kRealWarps * 32), frames);
-  double dip = geo.slab ? 4.0 * kPi / geo.vol : 0.0;
-  // r_split: erfc(g r) / r = 1e-4 / A (bisection); r_c (no far pairs) when the term never
-  // gets that small or the FP64 build asks for FP64 throughout
-  double lo = 1e-3, hi = geo.rc;
-  if (!far_float || erfc(geo.g * hi) / hi > 1e-4) {
-    lo = hi;
-  } else {
-    for (int it = 0; it < 60; ++it) {
-      const double mid = 0.5 * (lo + hi);
-      if (erfc(geo.g * mid) / mid > 1e-4) lo = mid;
-      else hi = mid;
-    }
-    lo = hi;
-  }
-  const RealScreen rs = real_screen(geo, lo * lo);
-  auto kernel = rs.all_single ? k_bsol_real<kSingleImage>
-                : rs.nshift   ? k_bsol_real<kShiftList>
-                              : k_bsol_real<kAllImages>;
-  (kernel<<<grid, kRealWarps * 32, 0, s>>>(xyz, alpha, sfix, n, ion_xyz, ion_q, sion, n_ion,
-                                          geo.L[0], geo.L[1], geo.L[2], geo.g, geo.rc, rs, dip,
-                                          chi, bsol_k, b_out, qsol),
-   note_launch());
 }
 
 }  // namespace cpm
