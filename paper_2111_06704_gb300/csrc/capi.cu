@@ -357,7 +357,7 @@ void free_build(Ctx* c) {
                 &c->Ahead, &c->A,
                 &c->E, &c->diag,
                 &c->nbr_off, &c->nbr_idx, &c->prow, &c->d, &c->shell_off, &c->shell_members, &c->p_f32,
-                &c->turn, &c->htab, &c->atoms, &c->gcd_labels, &c->gcd_a, &c->gcd_c, &c->gcd_cinv, &c->gcd_status,
+                &c->turn, &c->sfpairs, &c->htab, &c->atoms, &c->gcd_labels, &c->gcd_a, &c->gcd_c, &c->gcd_cinv, &c->gcd_status,
                 &c->gcd_scratch, &c->smat};
   for (Buf* b : all) buf_free(c, b);
   release_workspace(c);
@@ -701,6 +701,16 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
                                          "is not positive (INFINITY marks a point charge)"));
   }
 
+  if (!f64 && !c->sfpairs.ptr) {  // depends on the k-vector table only, as that does
+    const std::vector<SfPair> pairs = sf_pairs(hkl, c->m, c->mpad, c->kh);
+    c->n_sfpairs = (int)pairs.size();
+    if ((st = buf_reserve(c, &c->sfpairs, std::max<size_t>(pairs.size(), 1) * sizeof(SfPair))) ||
+        (st = cuda_check(c, cudaMemcpyAsync(c->sfpairs.ptr, pairs.data(),
+                                            pairs.size() * sizeof(SfPair), h2d, s), "pairs")) ||
+        (st = cuda_check(c, cudaStreamSynchronize(s), "pairs sync")))
+      return fail(st);
+  }
+
   cudaEvent_t ev[6];
   for (auto& e : ev) cudaEventCreate(&e);
   const Geometry geo = geometry(c);
@@ -1030,9 +1040,11 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
         launch_axis_phasors(dx + (size_t)f0 * n_ion * 3, nullptr, (int64_t)nf * n_ion, c->p.box, ap,
                             axis, s);
       launch_ion_structure_factor(f64, axis, ap, sion, n_ion, dq + (size_t)f0 * n_ion, nf, n_ion,
+                                  (const SfPair*)c->sfpairs.ptr, c->n_sfpairs,
                                   (const int*)c->hkl.ptr, (const double*)c->sqw.ptr, c->mpad,
                                   c->kh, c->turn.ptr,
-                                  (char*)v + (size_t)f0 * 2 * c->mpad * c->esz(), vh, s);
+                                  (char*)v + (size_t)f0 * 2 * c->mpad * c->esz(), vh,
+                                  std::max(dev_sms, 1), s);
     }
   } else if ((st = cuda_check(c, cudaMemsetAsync(v, 0, vbytes + hbytes, s), "v zero"))) {
     return st;
@@ -1128,8 +1140,9 @@ int cpm_ion_forces(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
     // the electrode's charge-weighted structure factors: the ions' kernel run over the
     // electrode atoms (the same coordinates every frame)
     launch_ion_structure_factor(f64, ax_el, ap, (const uint32_t*)c->sfix.ptr, 0, fq, nf, n,
+                                (const SfPair*)c->sfpairs.ptr, c->n_sfpairs,
                                 (const int*)c->hkl.ptr, (const double*)c->sqw.ptr, c->mpad, c->kh,
-                                c->turn.ptr, v, vh, s);
+                                c->turn.ptr, v, vh, std::max(dev_sms, 1), s);
     launch_ion_forces(f64, (const double*)c->xyz.ptr, (const double*)c->alpha.ptr,
                       (const uint32_t*)c->sfix.ptr, n, fx, dq + (size_t)f0 * n_ion, sion, nf, n_ion,
                       fq, (const int*)c->hkl.ptr, (const double*)c->sqw.ptr, c->mpad, c->kh,

@@ -127,6 +127,8 @@ struct Ctx {
   double pgap = 0;
 
   // learned-guess feature geometry (frame independent, made on first use)
+  Buf sfpairs;    // SfPair [n_sfpairs]: the tail k-vectors in pairs (float storage)
+  int n_sfpairs = 0;
   Buf htab;       // erfc(sqrt s) / sqrt s (real-space pairs of float storage)
   Buf atoms;      // the electrode's records for the real-space pairs
   Buf turn;       // float4 [4096]: exp(2 pi i j / 4096) as float pairs (ion phasors)
@@ -256,6 +258,10 @@ void launch_ion_fixed(const double* ion_xyz, int frames, int n_ion, const double
                       uint32_t* sion, cudaStream_t s);
 void launch_turn_table(void* T, cudaStream_t s);
 struct AxisPhasors;
+struct SfPair {  // two tail k-vectors (h, k, l), (h, k, l + 1): their places in the table
+  int h, k, l, k0, k1;
+};
+std::vector<SfPair> sf_pairs(const std::vector<int>& hkl, int m, int mpad, int kh);
 // per-axis FP64 phasors (FP64 storage) of `count` points: out [count][ap.len] double2; from
 // the fixed-point coordinates sfix where not NULL, else from xyz
 void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
@@ -266,9 +272,10 @@ void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
 // the fixed-point coordinates sion.
 void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhasors& ap,
                                  const uint32_t* sion, int64_t coord_stride,
-                                 const double* ion_q, int frames, int n_ion, const int* hkl,
+                                 const double* ion_q, int frames, int n_ion,
+                                 const SfPair* pairs, int npairs, const int* hkl,
                                  const double* sqw, int mpad, int kh, const void* turn,
-                                 void* v, double* vhead, cudaStream_t s);
+                                 void* v, double* vhead, int sms, cudaStream_t s);
 void launch_bsol_kspace(bool fp64, const void* A, const double* Ahead, int n, int mpad, int kh,
                         const void* v, const double* vhead, int frames, double* bsol,
                         const uint32_t* sfix, const int* hkl, const double* sqw,

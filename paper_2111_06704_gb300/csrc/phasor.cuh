@@ -62,6 +62,17 @@ __device__ __forceinline__ void pair_add1(float& h, float& l, float x) {
   h = s;
 }
 
+// (h, l) += x, two float pairs at once in paired IEEE instructions (a - b as fma(b, -1, a)):
+// the values of pair_add1 on each component.
+__device__ __forceinline__ void pair_add2(float2& h, float2& l, float2 x) {
+  const float2 m1 = make_float2(-1.f, -1.f);
+  const float2 s = __fadd2_rn(h, x);
+  const float2 bb = __ffma2_rn(h, m1, s);                       // s - h
+  const float2 a = __ffma2_rn(__ffma2_rn(bb, m1, s), m1, h);    // h - (s - bb)
+  l = __fadd2_rn(l, __fadd2_rn(a, __ffma2_rn(bb, m1, x)));      // + (x - bb)
+  h = s;
+}
+
 // (h, l) += a b, two float pairs at once in paired IEEE instructions (s - h as
 // -fma(s, -1, h)): a two-sum whose addend is the product before rounding.
 __device__ __forceinline__ void pair_fma2(float2& h, float2& l, float2 a, float2 b) {

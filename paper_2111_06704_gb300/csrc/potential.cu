@@ -10,15 +10,13 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "phasor.cuh"
 
 namespace cpm {
 
 namespace {
-
-constexpr int kSfThreads = 128;
-constexpr int kIonChunk = 256;
 
 // Fractional ion coordinates in 2^-32 fixed point, once per ion and frame: the phases of
 // every k-vector and the real-space screening use them.
@@ -43,21 +41,35 @@ __global__ void k_turn_table(float4* __restrict__ T) {
   T[j] = make_float4(ch, (float)(c - ch), sh, (float)(s - sh));
 }
 
-constexpr int kSfBlock = 8;  // ions a float block sum of the tail k-vectors holds
+constexpr int kSfWarps = 8;
+constexpr int kSfBlock = 8;   // ions a float block sum of the tail k-vectors holds
+constexpr int kIonChunk = 256;
 
-// sin and cos of 2 pi ph 2^-32 from a 64-entry table of exp(2 pi i j / 64) (float cos and
-// sin, in shared memory: 512 bytes, few bank conflicts for random entries) and the
-// remaining angle t = 2 pi (ph mod 2^26) 2^-32 < 0.099 rad by angle addition, with
+// sin and cos of 2 pi ph 2^-32 for two phases from a 64-entry table of exp(2 pi i j / 64) and
+// the remaining angle t = 2 pi (ph mod 2^26) 2^-32 < 0.099 rad by angle addition, with
 // cos t = 1 - t^2/2 + t^4/24 and sin t = t - t^3/6 + t^5/120 (the next terms, t^6/720 and
-// t^7/5040, lie below float rounding).  At most 1.5 float ulp of 1 (0.5 on average).
-__device__ __forceinline__ void sincos_t64(uint32_t ph, const float2* T, float* s, float* c) {
-  const float2 e = T[ph >> 26];
-  const float t = (float)(ph & 0x3FFFFFFu) * 1.462918119976564e-09f;  // 2 pi 2^-32
-  const float t2 = t * t;
-  const float ct = fmaf(t2, fmaf(t2, 1.0f / 24.0f, -0.5f), 1.0f);
-  const float st = t * fmaf(t2, fmaf(t2, 1.0f / 120.0f, -1.0f / 6.0f), 1.0f);
-  *c = fmaf(e.x, ct, -(e.y * st));
-  *s = fmaf(e.y, ct, e.x * st);
+// t^7/5040, lie below float rounding), in paired instructions.  At most 1.5 float ulp of 1
+// (0.5 on average).  tc and ts point at the lane's own copy of the table in shared memory
+// (entry j at [32 j]), so no two lanes meet in a bank.
+__device__ __forceinline__ void sincos_t64x2(uint32_t p0, uint32_t p1, const float* tc,
+                                             const float* ts, float2& s, float2& c) {
+  const int i0 = (int)(p0 >> 26) * 32, i1 = (int)(p1 >> 26) * 32;
+  const float2 ex = make_float2(tc[i0], tc[i1]), ey = make_float2(ts[i0], ts[i1]);
+  const float2 u = make_float2((float)(p0 & 0x3FFFFFFu), (float)(p1 & 0x3FFFFFFu));
+  const float k = 1.462918119976564e-09f;  // 2 pi 2^-32
+  const float2 t = __fmul2_rn(u, make_float2(k, k));
+  const float2 t2 = __fmul2_rn(t, t);
+  const float2 ct = __ffma2_rn(
+      t2, __ffma2_rn(t2, make_float2(1.0f / 24.0f, 1.0f / 24.0f), make_float2(-0.5f, -0.5f)),
+      make_float2(1.0f, 1.0f));
+  const float2 st = __fmul2_rn(
+      t, __ffma2_rn(t2,
+                    __ffma2_rn(t2, make_float2(1.0f / 120.0f, 1.0f / 120.0f),
+                               make_float2(-1.0f / 6.0f, -1.0f / 6.0f)),
+                    make_float2(1.0f, 1.0f)));
+  const float2 neg = make_float2(-ey.x, -ey.y);
+  c = __ffma2_rn(ex, ct, __fmul2_rn(neg, st));
+  s = __ffma2_rn(ey, ct, __fmul2_rn(ex, st));
 }
 
 // v[f][c(k)] = sqrt(W_k) sum_I q_I cos(theta_Ik), v[f][c(k) + 64] = sqrt(W_k) sum_I q_I sin,
@@ -65,102 +77,167 @@ __device__ __forceinline__ void sincos_t64(uint32_t ph, const float2* T, float* 
 // exact fixed-point phases.  Sums over the ions run in error-free float pairs (S_K is a
 // sum of O(n_ion) unit phasors whose float partial sums would lose bits; FP64 runs at
 // 1/64 of the float rate here); the tail's terms go in float blocks of kSfBlock ions, each
-// block's sum into the pair (a few ulp of a block, not of the whole sum).  The tail
-// k-vectors take float sin/cos from the phasor table (sincos_table, about one ulp); the
-// head (k < kh, the heaviest weights) takes float-pair phasors and goes out in FP64 to
-// vhead for the FP64 head contraction.
-__global__ void __launch_bounds__(kSfThreads, 8)
+// block's sum into the pair (a few ulp of a block, not of the whole sum).  The head (k < kh,
+// the heaviest weights) takes float-pair phasors and goes out in FP64 to vhead for the FP64
+// head contraction.
+//
+// Bound by issue: 4.4e9 phasors a call at 512 atoms, 2,000 ions, 256 frames.  A thread takes
+// two tail k-vectors with consecutive l (the list of pairs is the context's): one broadcast
+// load of an ion, four integer operations for both phases instead of six multiply-adds, and
+// paired float instructions throughout; the phasor table has a copy for every lane (random
+// entries of one copy conflicted in the banks).  One k-vector a thread with a shared table
+// took 3,995 us there, this form 3,473 (a phasor is 13 FMA-pipe operations, and a paired
+// FMA of three registers takes 3 cycles; 217,619 k-vectors over 12,800 points 2,752 -> 2,261 us).  Where the k-vectors do not fill the chip, the warps
+// of a block split the ions' blocks of eight between them (tail_shares).  The head's sums are chains of dependent additions (some 700
+// cycles an ion among other warps: one thread a k-vector for all ions was 60% longer than
+// the rest of the grid), so its blocks always split the ions eight ways, and come first.
+__global__ void __launch_bounds__(kSfWarps * 32)
 k_ion_sf_f32(const uint32_t* __restrict__ sion, int64_t coord_stride,
-             const double* __restrict__ ion_q, int n_ion,
-             const int* __restrict__ hkl, const double* __restrict__ sqw, int mpad, int kh,
-             const float4* __restrict__ turn, float* __restrict__ vout,
-             double* __restrict__ vhead) {
-  __shared__ uint32_t sf[kIonChunk][3];
-  __shared__ float sqh[kIonChunk], sql[kIonChunk];
-  __shared__ float2 t64[64];  // exp(2 pi i j / 64): entries 64 j of the 4,096-entry table
+             const double* __restrict__ ion_q, int n_ion, const SfPair* __restrict__ pairs,
+             int npairs, const int* __restrict__ hkl, const double* __restrict__ sqw, int mpad,
+             int kh, int tail_shares, int head_blocks, const float4* __restrict__ turn,
+             float* __restrict__ vout, double* __restrict__ vhead) {
+  __shared__ uint4 si[kIonChunk];   // fixed-point x, y, z and the charge as a float
+  __shared__ float sql[kIonChunk];  // the charges' low parts
+  __shared__ float tc[64][32], ts[64][32];  // exp(2 pi i j / 64), a copy for every lane
+  __shared__ double red[kSfWarps][32][4];
   const int f = blockIdx.y;
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool head = (int)blockIdx.x < head_blocks;
+  const int shares = head ? kSfWarps : tail_shares;
+  const int share = warp % shares, per = kSfWarps / shares;  // groups of 32 threads a block
   const uint32_t* fx = sion + (size_t)f * coord_stride * 3;
   const double* q = ion_q + (size_t)f * n_ion;
-  for (int j = threadIdx.x; j < 64; j += blockDim.x) {
-    const float4 e = __ldg(turn + 64 * j);
-    t64[j] = make_float2(e.x, e.z);
-  }
+  float* v = vout + (size_t)f * 2 * mpad;
+  const int at = ((int)blockIdx.x - (head ? 0 : head_blocks)) * per * 32 +
+                 (warp / shares) * 32 + lane;
   uint32_t h = 0, kk = 0, l = 0;
-  if (k < mpad) {
-    h = (uint32_t)hkl[3 * k];
-    kk = (uint32_t)hkl[3 * k + 1];
-    l = (uint32_t)hkl[3 * k + 2];
+  int k0 = -1, k1 = -1;
+  if (head) {
+    if (at < kh) {
+      k0 = at;
+      h = (uint32_t)hkl[3 * at];
+      kk = (uint32_t)hkl[3 * at + 1];
+      l = (uint32_t)hkl[3 * at + 2];
+    }
+  } else {
+    for (int e = threadIdx.x; e < 64 * 32; e += kSfWarps * 32) {
+      const float4 w = __ldg(turn + 64 * (e >> 5));
+      tc[e >> 5][e & 31] = w.x;
+      ts[e >> 5][e & 31] = w.z;
+    }
+    if (at < npairs) {
+      const SfPair p = pairs[at];
+      h = (uint32_t)p.h;
+      kk = (uint32_t)p.k;
+      l = (uint32_t)p.l;
+      k0 = p.k0;
+      k1 = p.k1;
+    }
   }
-  const bool head = k < kh;  // whole blocks take one branch unless they straddle kh
-  float reh = 0.f, rel = 0.f, imh = 0.f, iml = 0.f;
-  float rlo = 0.f, ilo = 0.f;  // tail: the charges' low parts times the phasors
+  const float *tcl = &tc[0][lane], *tsl = &ts[0][lane];
+  float2 reh = {0.f, 0.f}, rel = {0.f, 0.f}, imh = {0.f, 0.f}, iml = {0.f, 0.f};
+  float2 rlo = {0.f, 0.f}, ilo = {0.f, 0.f};  // tail: the charges' low parts times the phasors
   for (int base = 0; base < n_ion; base += kIonChunk) {
     const int cnt = min(kIonChunk, n_ion - base);
     __syncthreads();
-    for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-      sf[t][0] = fx[3 * (base + t)];
-      sf[t][1] = fx[3 * (base + t) + 1];
-      sf[t][2] = fx[3 * (base + t) + 2];
+    int low = 0;
+    for (int t = threadIdx.x; t < cnt; t += kSfWarps * 32) {
       const double qv = q[base + t];
-      sqh[t] = (float)qv;
-      sql[t] = (float)(qv - (double)sqh[t]);
+      const float qh = (float)qv, qlo = (float)(qv - (double)qh);
+      si[t] = make_uint4(fx[3 * (base + t)], fx[3 * (base + t) + 1], fx[3 * (base + t) + 2],
+                         __float_as_uint(qh));
+      sql[t] = qlo;
+      low |= qlo != 0.f;
+    }
+    low = __syncthreads_or(low);  // any charge that is no float
+    if (head) {
+#pragma unroll 2
+      for (int t = share; t < cnt; t += kSfWarps) {
+        const uint4 e = si[t];
+        const float qh = __uint_as_float(e.w), ql = sql[t];
+        float ch, cl, sh, sl, ph, pl;
+        phasor_ff(h * e.x + kk * e.y + l * e.z, turn, ch, cl, sh, sl);
+        ff_mul(qh, ql, ch, cl, ph, pl);
+        ff_add(reh.x, rel.x, ph, pl, reh.x, rel.x);
+        ff_mul(qh, ql, sh, sl, ph, pl);
+        ff_add(imh.x, iml.x, ph, pl, imh.x, iml.x);
+      }
+      continue;
+    }
+    const int blocks = cnt / kSfBlock;
+    auto block = [&](int b, auto lowpart) {
+      float2 br = make_float2(0.f, 0.f), bi = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < kSfBlock; ++u) {
+        const uint4 e = si[b * kSfBlock + u];
+        const uint32_t p0 = h * e.x + kk * e.y + l * e.z;
+        float2 sn, cs;
+        sincos_t64x2(p0, p0 + e.z, tcl, tsl, sn, cs);
+        const float2 qq = make_float2(__uint_as_float(e.w), __uint_as_float(e.w));
+        br = __ffma2_rn(qq, cs, br);
+        bi = __ffma2_rn(qq, sn, bi);
+        if constexpr (decltype(lowpart)::value) {
+          const float ql = sql[b * kSfBlock + u];
+          rlo = __ffma2_rn(make_float2(ql, ql), cs, rlo);
+          ilo = __ffma2_rn(make_float2(ql, ql), sn, ilo);
+        }
+      }
+      pair_add2(reh, rel, br);
+      pair_add2(imh, iml, bi);
+    };
+    if (low)
+      for (int b = share; b < blocks; b += shares) block(b, std::true_type());
+    else
+      for (int b = share; b < blocks; b += shares) block(b, std::false_type());
+    if (share == blocks % shares)  // ions past the last whole block, each into the pair
+      for (int t = blocks * kSfBlock; t < cnt; ++t) {
+        const uint4 e = si[t];
+        const uint32_t p0 = h * e.x + kk * e.y + l * e.z;
+        float2 sn, cs;
+        sincos_t64x2(p0, p0 + e.z, tcl, tsl, sn, cs);
+        const float qh = __uint_as_float(e.w), ql = sql[t];
+        pair_fma(reh.x, rel.x, qh, ql, cs.x);
+        pair_fma(reh.y, rel.y, qh, ql, cs.y);
+        pair_fma(imh.x, iml.x, qh, ql, sn.x);
+        pair_fma(imh.y, iml.y, qh, ql, sn.y);
+      }
+  }
+  double re[2] = {(double)reh.x + (double)rel.x + (double)rlo.x,
+                  (double)reh.y + (double)rel.y + (double)rlo.y};
+  double im[2] = {(double)imh.x + (double)iml.x + (double)ilo.x,
+                  (double)imh.y + (double)iml.y + (double)ilo.y};
+  if (shares > 1) {  // in share order
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      red[warp][lane][2 * u] = re[u];
+      red[warp][lane][2 * u + 1] = im[u];
     }
     __syncthreads();
-    if (k >= mpad) continue;
-    if (head) {
-      for (int t = 0; t < cnt; ++t) {
-        const uint32_t ph = h * sf[t][0] + kk * sf[t][1] + l * sf[t][2];
-        float ch, cl, sh, sl, ph_, pl_;
-        phasor_ff(ph, turn, ch, cl, sh, sl);
-        ff_mul(sqh[t], sql[t], ch, cl, ph_, pl_);
-        ff_add(reh, rel, ph_, pl_, reh, rel);
-        ff_mul(sqh[t], sql[t], sh, sl, ph_, pl_);
-        ff_add(imh, iml, ph_, pl_, imh, iml);
-      }
-    } else {
-      // blocks of kSfBlock ions summed in float, then added to the pairs by a two-sum;
-      // the charges' low parts (zero for charges that are floats) summed in float apart
-      int t = 0;
-      for (; t + kSfBlock <= cnt; t += kSfBlock) {
-        float br = 0.f, bi = 0.f;
+    if (share != 0) return;
+    for (int s = 1; s < shares; ++s)
 #pragma unroll
-        for (int u = 0; u < kSfBlock; ++u) {
-          const uint32_t ph = h * sf[t + u][0] + kk * sf[t + u][1] + l * sf[t + u][2];
-          float sn, cs;
-          sincos_t64(ph, t64, &sn, &cs);
-          br = fmaf(sqh[t + u], cs, br);
-          bi = fmaf(sqh[t + u], sn, bi);
-          rlo = fmaf(sql[t + u], cs, rlo);
-          ilo = fmaf(sql[t + u], sn, ilo);
-        }
-        pair_add1(reh, rel, br);
-        pair_add1(imh, iml, bi);
+      for (int u = 0; u < 2; ++u) {
+        re[u] += red[warp + s][lane][2 * u];
+        im[u] += red[warp + s][lane][2 * u + 1];
       }
-      for (; t < cnt; ++t) {
-        const uint32_t ph = h * sf[t][0] + kk * sf[t][1] + l * sf[t][2];
-        float sn, cs;
-        sincos_t64(ph, t64, &sn, &cs);
-        pair_fma(reh, rel, sqh[t], sql[t], cs);
-        pair_fma(imh, iml, sqh[t], sql[t], sn);
-      }
-    }
   }
-  if (k >= mpad) return;
-  const double re = (double)reh + (double)rel + (double)rlo,
-               im = (double)imh + (double)iml + (double)ilo;
-  const double w = sqw[k];
-  const size_t kcol = 128 * (size_t)(k >> 6) + (k & 63);  // operand column layout
-  float* v = vout + (size_t)f * 2 * mpad;
-  if (head) {  // FP64 values for the FP64 head contraction; zero float columns
-    double* vh = vhead + (size_t)f * 2 * kh;
-    vh[kcol] = w * re;
-    vh[kcol + 64] = w * im;
-    v[kcol] = 0.f;
-    v[kcol + 64] = 0.f;
-  } else {
-    v[kcol] = (float)(w * re);
-    v[kcol + 64] = (float)(w * im);
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int k = u == 0 ? k0 : k1;
+    if (k < 0) continue;
+    const double w = sqw[k];
+    const size_t kcol = 128 * (size_t)(k >> 6) + (k & 63);  // operand column layout
+    if (head) {  // FP64 values for the FP64 head contraction; zero float columns
+      double* vh = vhead + (size_t)f * 2 * kh;
+      vh[kcol] = w * re[u];
+      vh[kcol + 64] = w * im[u];
+      v[kcol] = 0.f;
+      v[kcol + 64] = 0.f;
+    } else {
+      v[kcol] = (float)(w * re[u]);
+      v[kcol + 64] = (float)(w * im[u]);
+    }
   }
 }
 
@@ -317,7 +394,6 @@ k_bsol_kspace_direct(const uint32_t* __restrict__ sfix, int n, const int* __rest
   float2 hi[kDirectFrames / 2], lo[kDirectFrames / 2];
 #pragma unroll
   for (int f = 0; f < kDirectFrames / 2; ++f) hi[f] = lo[f] = make_float2(0.f, 0.f);
-  const float2 m1 = make_float2(-1.f, -1.f);
   for (int k0 = kbeg; k0 < kend; k0 += kDirectChunk) {
     const int cnt = min(kDirectChunk, kend - k0);
     __syncthreads();
@@ -366,12 +442,7 @@ k_bsol_kspace_direct(const uint32_t* __restrict__ sfix, int n, const int* __rest
       }
 #pragma unroll
       for (int f = 0; f < kDirectFrames / 2; ++f) {
-        const float2 term = blk[f];
-        const float2 s2 = __fadd2_rn(hi[f], term);
-        const float2 bb = __ffma2_rn(hi[f], m1, s2);                          // s2 - hi
-        const float2 a = __ffma2_rn(__ffma2_rn(bb, m1, s2), m1, hi[f]);       // hi - (s2 - bb)
-        lo[f] = __fadd2_rn(lo[f], __fadd2_rn(a, __ffma2_rn(bb, m1, term)));   // + (term - bb)
-        hi[f] = s2;
+        pair_add2(hi[f], lo[f], blk[f]);
       }
     }
   }
@@ -397,6 +468,36 @@ void launch_turn_table(void* T, cudaStream_t s) {
   (k_turn_table<<<16, 256, 0, s>>>((float4*)T), note_launch());
 }
 
+// The tail k-vectors [kh, m) of the table hkl in pairs with equal h, k and consecutive l (a
+// k-vector without a partner alone, k1 = -1), and the table's padding [m, mpad) alone.
+std::vector<SfPair> sf_pairs(const std::vector<int>& hkl, int m, int mpad, int kh) {
+  int lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
+  for (int k = 0; k < m; ++k)
+    for (int d = 0; d < 3; ++d) {
+      lo[d] = std::min(lo[d], hkl[3 * (size_t)k + d]);
+      hi[d] = std::max(hi[d], hkl[3 * (size_t)k + d]);
+    }
+  const size_t nl = hi[2] - lo[2] + 1, nk = hi[1] - lo[1] + 1, nh = hi[0] - lo[0] + 1;
+  std::vector<int> at(nh * nk * nl, -1);  // tail k-vector at (h, k, l)
+  for (int k = kh; k < m; ++k)
+    at[((hkl[3 * (size_t)k] - lo[0]) * nk + (hkl[3 * (size_t)k + 1] - lo[1])) * nl +
+       (hkl[3 * (size_t)k + 2] - lo[2])] = k;
+  std::vector<SfPair> out;
+  out.reserve((m - kh) / 2 + (m - kh) / 16 + 64);
+  for (size_t c = 0; c < nh * nk; ++c) {
+    const int h = (int)(c / nk) + lo[0], k = (int)(c % nk) + lo[1];
+    for (size_t l = 0; l < nl; ++l) {
+      const int k0 = at[c * nl + l];
+      if (k0 < 0) continue;
+      const int k1 = l + 1 < nl ? at[c * nl + l + 1] : -1;
+      out.push_back({h, k, (int)l + lo[2], k0, k1});
+      if (k1 >= 0) ++l;
+    }
+  }
+  for (int k = std::max(kh, m); k < mpad; ++k) out.push_back({0, 0, 0, k, -1});
+  return out;
+}
+
 void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
                          const double L[3], const AxisPhasors& ap, double2* out,
                          cudaStream_t s) {
@@ -406,17 +507,26 @@ void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
 
 void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhasors& ap,
                                  const uint32_t* sion, int64_t coord_stride,
-                                 const double* ion_q, int frames, int n_ion, const int* hkl,
+                                 const double* ion_q, int frames, int n_ion,
+                                 const SfPair* pairs, int npairs, const int* hkl,
                                  const double* sqw, int mpad, int kh, const void* turn,
-                                 void* v, double* vhead, cudaStream_t s) {
+                                 void* v, double* vhead, int sms, cudaStream_t s) {
   if (fp64) {
     (k_ion_sf_f64<<<dim3(mpad / 32, frames), kSf64Warps * 32, 0, s>>>(
          axis, ap, coord_stride, ion_q, n_ion, hkl, sqw, mpad, (double*)v),
      note_launch());
   } else {
-    dim3 grid((mpad + kSfThreads - 1) / kSfThreads, frames);
-    (k_ion_sf_f32<<<grid, kSfThreads, 0, s>>>(sion, coord_stride, ion_q, n_ion, hkl, sqw, mpad,
-                                              kh, (const float4*)turn, (float*)v, vhead),
+    // warps of a block split the ions until the chip's warps are busy (24 resident an SM),
+    // each with at least four blocks of eight ions
+    const int groups = (npairs + 31) / 32;
+    int shares = 1;
+    while (shares < kSfWarps && (int64_t)groups * frames * shares < 24 * (int64_t)sms &&
+           n_ion >= 64 * shares)
+      shares *= 2;
+    const int per = 32 * (kSfWarps / shares), hb = (kh + 31) / 32;
+    (k_ion_sf_f32<<<dim3(hb + (npairs + per - 1) / per, frames), kSfWarps * 32, 0, s>>>(
+         sion, coord_stride, ion_q, n_ion, pairs, npairs, hkl, sqw, mpad, kh, shares, hb,
+         (const float4*)turn, (float*)v, vhead),
      note_launch());
   }
 }
