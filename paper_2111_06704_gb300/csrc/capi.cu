@@ -885,6 +885,7 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
     return fail(st == CPM_ECUDA && c->err.empty() ? cuda_check(c, cudaGetLastError(), "k-space GEMM") : st);
   }
   cudaEventRecord(ev[2], s);
+  if (c->kh > 0) launch_pairs_in_place((double*)c->Ahead.ptr, (int64_t)c->npad * 2 * c->kh, s);
   launch_mirror_lower(f64, c->E.ptr, n, c->ldE, s);
   launch_extract_diag(f64, c->E.ptr, n, c->ldE, (double*)c->diag.ptr, s);
   (k_inverse_tail<<<(n + 255) / 256, 256, 0, s>>>((double*)c->diag.ptr, n), note_launch());
@@ -988,7 +989,8 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   if (qsol_out && (st = stage_out(c, &c->ws_out1, qsol_out, (size_t)frames * sizeof(double),
                                   (void**)&dqs)))
     return st;
-  // scratch: v [frames][2 mpad] (storage type) | v_head [frames][2 kh] | b^sol_k [frames][n]
+  // scratch: v [frames][2 mpad] (storage type) | v_head [frames][2 kh]
+  //          (float pairs) | b^sol_k [frames][n]
   //          | fixed-point ion coordinates [frames][n_ion][3] | the direct sum's k-range
   //          shares [nsplit][frames][n] (a streamed build split into more than one) | the
   //          ions' per-axis phasors (FP64 storage) | the real-space part's scratch
@@ -1015,7 +1017,7 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
     launch_turn_table(c->turn.ptr, s);
   }
   void* v = c->ws_pot.ptr;
-  double* vh = (double*)((char*)c->ws_pot.ptr + vbytes);
+  void* vh = (char*)c->ws_pot.ptr + vbytes;
   double* bk = (double*)((char*)c->ws_pot.ptr + vbytes + hbytes);
   uint32_t* sion = (uint32_t*)((char*)c->ws_pot.ptr + vbytes + hbytes + kbytes);
   double* spart =
@@ -1050,9 +1052,9 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
     return st;
   }
   cudaEventRecord(pev[1], s);
-  launch_bsol_kspace(f64, c->A.ptr, (const double*)c->Ahead.ptr, n, c->mpad, c->kh, v, vh,
+  launch_bsol_kspace(f64, c->A.ptr, c->Ahead.ptr, n, c->mpad, c->kh, v, vh,
                      frames, bk, (const uint32_t*)c->sfix.ptr, (const int*)c->hkl.ptr,
-                     (const double*)c->sqw.ptr, c->turn.ptr, nsplit, spart, s);
+                     (const double*)c->sqw.ptr, c->turn.ptr, nsplit, spart, std::max(dev_sms, 1), s);
   cudaEventRecord(pev[2], s);
   launch_bsol_real_and_finish((const double*)c->xyz.ptr, (const double*)c->alpha.ptr,
                               (const uint32_t*)c->sfix.ptr, c->atoms.ptr, c->htab.ptr, n, dx, dq,
@@ -1126,7 +1128,7 @@ int cpm_ion_forces(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   }
   char* base = (char*)c->ws_pot.ptr;
   void* v = base + ov;
-  double* vh = (double*)(base + oh);
+  void* vh = base + oh;
   uint32_t* sion = (uint32_t*)(base + ou);
   double2 *ax = (double2*)(base + oa), *ax_el = (double2*)(base + oe);
   if (f64) launch_axis_phasors((const double*)c->xyz.ptr, nullptr, n, c->p.box, ap, ax_el, s);

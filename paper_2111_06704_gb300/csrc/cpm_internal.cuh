@@ -107,7 +107,8 @@ struct Ctx {
   Buf flush;    // uint32 [(2*mpad/16 + 31)/32]: k-steps after which float partials flush
   int heavy_steps = 0;  // leading k-steps accumulated exactly in FP64
   int kh = 0;           // head k-vectors with an FP64 operand copy (float storage only)
-  Buf Ahead;            // double [npad][2*kh], same column layout as A
+  Buf Ahead;            // float pairs [npad][2*kh] of the head columns, A's column layout
+                        // (made in FP64, turned into pairs at the end of the build)
   Buf chunk_end;        // uint32 bit per K-block of 64 columns (tensor-core build)
   Buf kexp;             // int per K-block: FP16 plane scale exponent (tensor-core build)
   bool streamed = false;  // A too large to keep: built in k-windows, potential direct
@@ -232,6 +233,8 @@ int launch_ek_simt(bool fp64, const void* A, int npad, int mpad, const double* x
                    int heavy_steps, const uint32_t* flush_mask, cudaStream_t s);
 void launch_mirror_lower(bool fp64, void* E, int n, int64_t ldE, cudaStream_t s);
 
+// x [len] doubles -> float pairs (hi, lo) in place
+void launch_pairs_in_place(double* x, int64_t len, cudaStream_t s);
 int launch_ek_head_f64(const double* Ahead, int kh, int ktot, int npad, float* hi, float* lo,
                        const double* xyz, const double* alpha, int n, const Geometry& geo,
                        float2* Ehead, int64_t ldE, cudaStream_t s);
@@ -275,11 +278,12 @@ void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhaso
                                  const double* ion_q, int frames, int n_ion,
                                  const SfPair* pairs, int npairs, const int* hkl,
                                  const double* sqw, int mpad, int kh, const void* turn,
-                                 void* v, double* vhead, int sms, cudaStream_t s);
-void launch_bsol_kspace(bool fp64, const void* A, const double* Ahead, int n, int mpad, int kh,
-                        const void* v, const double* vhead, int frames, double* bsol,
+                                 void* v, void* vhead, int sms, cudaStream_t s);
+void launch_bsol_kspace(bool fp64, const void* A, const void* Ahead, int n, int mpad, int kh,
+                        const void* v, const void* vhead, int frames, double* bsol,
                         const uint32_t* sfix, const int* hkl, const double* sqw,
-                        const void* turn, int nsplit, double* split_part, cudaStream_t s);
+                        const void* turn, int nsplit, double* split_part, int sms,
+                        cudaStream_t s);
 // shares of the k range of a streamed build's direct k-space sum (split_part then holds
 // nsplit x frames x n doubles)
 int bsol_direct_splits(int n, int frames, int mpad, int kh, int sms);
@@ -318,7 +322,7 @@ void launch_ion_forces(bool fp64, const double* xyz, const double* alpha, const 
                        int n, const double* ion_xyz, const double* ion_q, const uint32_t* sion,
                        int frames, int n_ion, const double* q, const int* hkl,
                        const double* sqw, int mpad, int kh, const Geometry& geo,
-                       const void* turn, const void* v, const double* vhead,
+                       const void* turn, const void* v, const void* vhead,
                        const double2* ion_axis, const AxisPhasors& ap, const ForceSplits& sp,
                        double* kpart, double* rpart, double2* slab, double* out,
                        cudaStream_t s);

@@ -59,8 +59,8 @@ __device__ __forceinline__ void write_gradients(float2 (&gh)[kFkIons / 2][3],
 // [ion][3].  A thread takes every 128th k-vector of the share for all 8 ions, so a
 // k-vector's index, weight and structure factors are read once for 8 phasors, and the ions
 // go in pairs through paired float instructions.  Shares 0 .. nsplit - 1 hold the tail
-// k-vectors (float phasors from the table, one ulp, each term times h, k, l exactly into an
-// error-free float pair); share nsplit, where there is one, the head (k < kh, the heaviest weights) in float
+// k-vectors (float phasors from the table, one ulp, each term times h, k, l unrounded into a
+// float pair); share nsplit, where there is one, the head (k < kh, the heaviest weights) in float
 // pairs throughout (~1e-13: FP64 runs at 1/64 of the float rate).  One thread per ion over
 // the whole k range, the form before, kept 16 blocks of the chip busy with 2,000 ions:
 // 30.7 ms with 217,619 k-vectors against 0.83 ms.
@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kFkThreads)
 k_force_kspace(const uint32_t* __restrict__ sion, int n_ion, const int* __restrict__ hkl,
                const double* __restrict__ sqw, int mpad, int kh, int nsplit,
                const float4* __restrict__ turn, const float* __restrict__ v,
-               const double* __restrict__ vhead, double* __restrict__ part) {
+               const float2* __restrict__ vhead, double* __restrict__ part) {
   const int f = blockIdx.y, frames = gridDim.y, sp = blockIdx.z;
   const int i0 = blockIdx.x * kFkIons;
   uint32_t u[kFkIons][3];
@@ -109,14 +109,17 @@ k_force_kspace(const uint32_t* __restrict__ sion, int n_ion, const int* __restri
       }
     }
   } else {
-    const double* vh = vhead + (size_t)f * 2 * kh;
+    const float2* vh = vhead + (size_t)f * 2 * kh;
     for (int k = threadIdx.x; k < kh; k += kFkThreads) {
       const uint32_t h0 = (uint32_t)hkl[3 * k], h1 = (uint32_t)hkl[3 * k + 1],
                      h2 = (uint32_t)hkl[3 * k + 2];
       const size_t kcol = 128 * (size_t)(k >> 6) + (k & 63);
-      const double wd = sqw[k], cd = wd * vh[kcol], sd = wd * vh[kcol + 64];
-      const float ch = (float)cd, cl = (float)(cd - (double)ch);
-      const float sh = (float)sd, sl = (float)(sd - (double)sh);
+      const double wd = sqw[k];
+      const float wh = (float)wd, wl = (float)(wd - (double)wh);
+      const float2 vc = vh[kcol], vs = vh[kcol + 64];
+      float ch, cl, sh, sl;
+      ff_mul(wh, wl, vc.x, vc.y, ch, cl);
+      ff_mul(wh, wl, vs.x, vs.y, sh, sl);
       const float hf[3] = {(float)(int)h0, (float)(int)h1, (float)(int)h2};
 #pragma unroll
       for (int t = 0; t < kFkIons; ++t) {
@@ -391,7 +394,7 @@ void launch_ion_forces(bool fp64, const double* xyz, const double* alpha, const 
                        int n, const double* ion_xyz, const double* ion_q, const uint32_t* sion,
                        int frames, int n_ion, const double* q, const int* hkl,
                        const double* sqw, int mpad, int kh, const Geometry& geo,
-                       const void* turn, const void* v, const double* vhead,
+                       const void* turn, const void* v, const void* vhead,
                        const double2* ion_axis, const AxisPhasors& ap, const ForceSplits& sp,
                        double* kpart, double* rpart, double2* slab, double* out,
                        cudaStream_t s) {
@@ -402,7 +405,7 @@ void launch_ion_forces(bool fp64, const double* xyz, const double* alpha, const 
   else
     (k_force_kspace<<<dim3((n_ion + kFkIons - 1) / kFkIons, frames, sp.k_total), kFkThreads, 0,
                       s>>>(sion, n_ion, hkl, sqw, mpad, kh, sp.k_tail, (const float4*)turn,
-                           (const float*)v, vhead, kpart),
+                           (const float*)v, (const float2*)vhead, kpart),
      note_launch());
   ForceScreen fs;
   for (int d = 0; d < 3; ++d) fs.fs[d] = (float)(geo.L[d] * 0x1p-32);

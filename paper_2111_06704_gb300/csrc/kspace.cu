@@ -482,6 +482,15 @@ __global__ void k_split_head(const double* __restrict__ A, int64_t lda, int rows
   }
 }
 
+__global__ void k_pairs_in_place(double* __restrict__ x, int64_t len) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < len;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const double v = x[e];
+    const float h = (float)v;
+    reinterpret_cast<float2*>(x)[e] = make_float2(h, (float)(v - (double)h));
+  }
+}
+
 template <typename T>
 __global__ void k_mirror_lower(T* __restrict__ E, int n, int64_t ldE) {
   __shared__ T tile[32][33];
@@ -612,6 +621,10 @@ int launch_ek_head_f64(const double* Ahead, int kh, int ktot, int npad, float* h
   (k_split_head<<<2048, 256, 0, s>>>(Ahead, 2 * (int64_t)kh, npad, ktot, hi, lo), note_launch());
   (k_ek_head_ff<<<tiles, 256, 0, s>>>(hi, lo, ktot, ktot, Ehead, ldE, ep), note_launch());
   return cudaGetLastError() == cudaSuccess ? CPM_OK : CPM_ECUDA;
+}
+
+void launch_pairs_in_place(double* x, int64_t len, cudaStream_t s) {
+  (k_pairs_in_place<<<2048, 256, 0, s>>>(x, len), note_launch());
 }
 
 void launch_mirror_lower(bool fp64, void* E, int n, int64_t ldE, cudaStream_t s) {

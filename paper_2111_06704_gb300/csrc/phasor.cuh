@@ -73,14 +73,30 @@ __device__ __forceinline__ void pair_add2(float2& h, float2& l, float2 x) {
   h = s;
 }
 
-// (h, l) += a b, two float pairs at once in paired IEEE instructions (s - h as
-// -fma(s, -1, h)): a two-sum whose addend is the product before rounding.
+// (h, l) += a b, two float pairs at once in paired IEEE instructions: the two-sum's form with
+// the product unrounded (s - h as -fma(s, -1, h)).  Good to ~2^-24 of h where h and a b cancel
+// (s then holds bits below both addends' ulps), so for sums whose terms are float anyway.
 __device__ __forceinline__ void pair_fma2(float2& h, float2& l, float2 a, float2 b) {
   const float2 m1 = make_float2(-1.f, -1.f);
   const float2 s = __ffma2_rn(a, b, h);
   const float2 nb = __ffma2_rn(s, m1, h);                                // h - s
   const float2 e = __ffma2_rn(__fadd2_rn(s, nb), m1, h);                 // h - (s - (s - h))
   l = __fadd2_rn(l, __fadd2_rn(e, __ffma2_rn(a, b, nb)));                // + (a b - (s - h))
+  h = s;
+}
+
+// (h, l) += (ah + al) (bh + bl), two at once: the product of the high parts split exactly
+// (two-product), its rounded part added by a two-sum, to ~2^-47.  na = -ah.
+__device__ __forceinline__ void pair_dot2(float2& h, float2& l, float2 ah, float2 na, float2 al,
+                                          float2 bh, float2 bl) {
+  const float2 m1 = make_float2(-1.f, -1.f);
+  const float2 n = __fmul2_rn(na, bh);                         // -p, p = ah bh rounded
+  const float2 pe = __ffma2_rn(ah, bh, n);                     // ah bh - p
+  const float2 s = __ffma2_rn(n, m1, h);                       // h + p
+  const float2 nb = __ffma2_rn(s, m1, h);                      // h - s
+  const float2 e = __ffma2_rn(__fadd2_rn(s, nb), m1, h);       // h - (s - (s - h))
+  const float2 q = __fadd2_rn(e, __ffma2_rn(n, m1, nb));       // + (p - (s - h))
+  l = __fadd2_rn(__ffma2_rn(ah, bl, __ffma2_rn(al, bh, l)), __fadd2_rn(q, pe));
   h = s;
 }
 

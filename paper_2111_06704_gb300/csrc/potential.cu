@@ -78,8 +78,8 @@ __device__ __forceinline__ void sincos_t64x2(uint32_t p0, uint32_t p1, const flo
 // sum of O(n_ion) unit phasors whose float partial sums would lose bits; FP64 runs at
 // 1/64 of the float rate here); the tail's terms go in float blocks of kSfBlock ions, each
 // block's sum into the pair (a few ulp of a block, not of the whole sum).  The head (k < kh,
-// the heaviest weights) takes float-pair phasors and goes out in FP64 to vhead for the FP64
-// head contraction.
+// the heaviest weights) takes float-pair phasors and goes out as float pairs to vhead for
+// the head contraction.
 //
 // Bound by issue: 4.4e9 phasors a call at 512 atoms, 2,000 ions, 256 frames.  A thread takes
 // two tail k-vectors with consecutive l (the list of pairs is the context's): one broadcast
@@ -96,7 +96,7 @@ k_ion_sf_f32(const uint32_t* __restrict__ sion, int64_t coord_stride,
              const double* __restrict__ ion_q, int n_ion, const SfPair* __restrict__ pairs,
              int npairs, const int* __restrict__ hkl, const double* __restrict__ sqw, int mpad,
              int kh, int tail_shares, int head_blocks, const float4* __restrict__ turn,
-             float* __restrict__ vout, double* __restrict__ vhead) {
+             float* __restrict__ vout, float2* __restrict__ vhead) {
   __shared__ uint4 si[kIonChunk];   // fixed-point x, y, z and the charge as a float
   __shared__ float sql[kIonChunk];  // the charges' low parts
   __shared__ float tc[64][32], ts[64][32];  // exp(2 pi i j / 64), a copy for every lane
@@ -228,10 +228,11 @@ k_ion_sf_f32(const uint32_t* __restrict__ sion, int64_t coord_stride,
     if (k < 0) continue;
     const double w = sqw[k];
     const size_t kcol = 128 * (size_t)(k >> 6) + (k & 63);  // operand column layout
-    if (head) {  // FP64 values for the FP64 head contraction; zero float columns
-      double* vh = vhead + (size_t)f * 2 * kh;
-      vh[kcol] = w * re[u];
-      vh[kcol + 64] = w * im[u];
+    if (head) {  // float pairs for the head contraction; zero float columns
+      float2* vh = vhead + (size_t)f * 2 * kh;
+      const double c = w * re[u], sn = w * im[u];
+      vh[kcol] = make_float2((float)c, (float)(c - (double)(float)c));
+      vh[kcol + 64] = make_float2((float)sn, (float)(sn - (double)(float)sn));
       v[kcol] = 0.f;
       v[kcol + 64] = 0.f;
     } else {
@@ -306,51 +307,150 @@ k_ion_sf_f64(const double2* __restrict__ axis, const AxisPhasors ap, int64_t coo
   v[kcol + 64] = w * im;
 }
 
-// b^sol_k[f][i] = sum_c A[i][c] v[f][c]: one warp per electrode row and NF frames per
-// grid row (the A row is read once per NF frames).  Float storage: 4-term float partials
-// summed in error-free float pairs; FP64 storage: FP64 throughout.
-template <typename T, int NF>
+// FP64 storage: b^sol_k[f][i] = sum_c A[i][c] v[f][c], one warp per electrode row and four
+// frames per grid row (the A row is read once for them).
+constexpr int kF64Frames = 4;
+
 __global__ void __launch_bounds__(256)
-k_bsol_kspace(const T* __restrict__ A, int n, int64_t lda, const T* __restrict__ v,
-              int frames, double* __restrict__ bsol, int accumulate) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+k_bsol_kspace_f64(const double* __restrict__ A, int n, int64_t lda, const double* __restrict__ v,
+                  int frames, double* __restrict__ bsol) {
+  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  const int f0 = blockIdx.y * NF;
-  if (warp >= n) return;
-  const T* a = A + (int64_t)warp * lda;
-  constexpr int VEC = 16 / sizeof(T);
-  T hi[NF], lo[NF];
+  const int f0 = blockIdx.y * kF64Frames;
+  if (row >= n) return;
+  const double* a = A + (int64_t)row * lda;
+  double acc[kF64Frames] = {0.0, 0.0, 0.0, 0.0};
+  for (int64_t c = lane * 2; c < lda; c += 64) {
+    const double2 av = __ldg(reinterpret_cast<const double2*>(a + c));
 #pragma unroll
-  for (int r = 0; r < NF; ++r) hi[r] = lo[r] = T(0);
-  for (int64_t c = lane * VEC; c < lda; c += 32 * VEC) {
-    T av[VEC];
-    *reinterpret_cast<float4*>(av) = __ldg(reinterpret_cast<const float4*>(a + c));
-#pragma unroll
-    for (int r = 0; r < NF; ++r) {
+    for (int r = 0; r < kF64Frames; ++r) {
       if (f0 + r >= frames) break;
-      T vv[VEC];
-      *reinterpret_cast<float4*>(vv) =
-          __ldg(reinterpret_cast<const float4*>(v + (int64_t)(f0 + r) * lda + c));
-      T s = T(0);
-#pragma unroll
-      for (int u = 0; u < VEC; ++u) s = fma(av[u], vv[u], s);
-      if constexpr (sizeof(T) == 4) {
-        const float t = hi[r] + s;
-        const float bb = t - hi[r];
-        lo[r] += (hi[r] - (t - bb)) + (s - bb);
-        hi[r] = t;
-      } else {
-        hi[r] += s;
-      }
+      const double2 vv = __ldg(reinterpret_cast<const double2*>(v + (int64_t)(f0 + r) * lda + c));
+      acc[r] += fma(av.y, vv.y, av.x * vv.x);
     }
   }
 #pragma unroll
-  for (int r = 0; r < NF; ++r) {
-    double x = (double)hi[r] + (double)lo[r];
+  for (int r = 0; r < kF64Frames; ++r) {
+    double x = acc[r];
     for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0 && f0 + r < frames) {
-      double* dst = bsol + (int64_t)(f0 + r) * n + warp;
-      *dst = accumulate ? *dst + x : x;
+    if (lane == 0 && f0 + r < frames) bsol[(int64_t)(f0 + r) * n + row] = x;
+  }
+}
+
+// Float storage: b^sol_k[f][i] = sum_c A[i][c] v[f][c] over the tail columns (c >= 2 kh), four
+// products summed in float and each four into an error-free float pair, plus the head columns
+// from float pairs of A and v (products and sums to ~1e-14; A null: the head alone, added to
+// bsol).  A block's eight warps are 8 / WS groups of four rows; the WS warps of a group split
+// the columns, and a warp takes NF frames at once, in pairs through paired instructions, so
+// each float4 of A serves NF frames and each of v four rows.
+//
+// One frame of a large electrode is bound by reading A (22.3 GB at 12,800 atoms and 217,619
+// k-vectors): one warp a row with one load in flight beside the sum's chain reached 4.4 TB/s
+// (5.08 ms); four independent rows a warp and the columns split over the block reach
+// 6.6 TB/s (3.37 ms).  Many frames are bound by the sums (eleven paired instructions for
+// eight products): 512 atoms, 256 frames 791 -> 479 us with the head.  The head in FP64 (1/64 of
+// the float rate) took 241 us more there and 778 us at 26,600 atoms and 16 frames, 157 us in
+// float pairs.  512 atoms, one frame: 43 -> 9 us in one launch instead of two.
+constexpr int kKsWarps = 8;
+constexpr int kKsRows = 4;
+
+template <int NF, int WS>
+__global__ void __launch_bounds__(kKsWarps * 32, NF == 8 ? 2 : 1)
+k_bsol_kspace_f32(const float* __restrict__ A, int64_t lda, const float2* __restrict__ Ahead,
+                  int n, int kh, const float* __restrict__ v, const float2* __restrict__ vhead,
+                  int frames, double* __restrict__ bsol, int stream) {
+  constexpr int NP = (NF + 1) / 2;  // frame pairs (one frame fills both halves of one)
+  constexpr int NV = kKsRows * 2 * NP;
+  __shared__ float2 sm[kKsWarps][NV];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int sub = warp % WS;
+  const int row0 = (blockIdx.x * (kKsWarps / WS) + warp / WS) * kKsRows;
+  const int f0 = blockIdx.y * NF;
+  int64_t arow[kKsRows];  // a row past the last repeats it and is not written
+#pragma unroll
+  for (int i = 0; i < kKsRows; ++i) arow[i] = min(row0 + i, n - 1);
+  int frame[2 * NP];
+#pragma unroll
+  for (int r = 0; r < 2 * NP; ++r) frame[r] = min(f0 + (r < NF ? r : 0), frames - 1);
+  float2 hi[kKsRows][NP], lo[kKsRows][NP];
+#pragma unroll
+  for (int i = 0; i < kKsRows; ++i)
+#pragma unroll
+    for (int p = 0; p < NP; ++p) hi[i][p] = lo[i][p] = make_float2(0.f, 0.f);
+  if (A) {
+    for (int64_t c = 2 * (int64_t)kh + (sub * 32 + lane) * 4; c < lda; c += 128 * WS) {
+      float a[kKsRows][4];
+#pragma unroll
+      for (int i = 0; i < kKsRows; ++i) {
+        const float4* p = reinterpret_cast<const float4*>(A + arow[i] * lda + c);
+        *reinterpret_cast<float4*>(a[i]) = stream ? __ldcs(p) : __ldg(p);
+      }
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        float va[4], vb[4];
+        *reinterpret_cast<float4*>(va) =
+            __ldg(reinterpret_cast<const float4*>(v + frame[2 * p] * lda + c));
+        *reinterpret_cast<float4*>(vb) =
+            NF == 1 ? *reinterpret_cast<float4*>(va)
+                    : __ldg(reinterpret_cast<const float4*>(v + frame[2 * p + 1] * lda + c));
+#pragma unroll
+        for (int i = 0; i < kKsRows; ++i) {
+          float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            s = __ffma2_rn(make_float2(a[i][u], a[i][u]), make_float2(va[u], vb[u]), s);
+          pair_add2(hi[i][p], lo[i][p], s);
+        }
+      }
+    }
+  }
+  // head: two columns a lane
+  const int64_t ldh = 2 * (int64_t)kh;
+  for (int64_t c = (sub * 32 + lane) * 2; c < ldh; c += 64 * WS) {
+    float4 a[kKsRows];  // (hi, lo) of columns c and c + 1
+#pragma unroll
+    for (int i = 0; i < kKsRows; ++i)
+      a[i] = __ldg(reinterpret_cast<const float4*>(Ahead + arow[i] * ldh + c));
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const float4 x = __ldg(reinterpret_cast<const float4*>(vhead + frame[2 * p] * ldh + c));
+      const float4 y =
+          NF == 1 ? x : __ldg(reinterpret_cast<const float4*>(vhead + frame[2 * p + 1] * ldh + c));
+#pragma unroll
+      for (int i = 0; i < kKsRows; ++i)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const float ah = u ? a[i].z : a[i].x, al = u ? a[i].w : a[i].y;
+          const float2 vh = u ? make_float2(x.z, y.z) : make_float2(x.x, y.x);
+          const float2 vl = u ? make_float2(x.w, y.w) : make_float2(x.y, y.y);
+          pair_dot2(hi[i][p], lo[i][p], make_float2(ah, ah), make_float2(-ah, -ah),
+                    make_float2(al, al), vh, vl);
+        }
+    }
+  }
+  // lanes, then the group's warps in order
+#pragma unroll
+  for (int i = 0; i < kKsRows; ++i)
+#pragma unroll
+    for (int r = 0; r < NF; ++r) {
+      float h = (r & 1) ? hi[i][r >> 1].y : hi[i][r >> 1].x;
+      float l = (r & 1) ? lo[i][r >> 1].y : lo[i][r >> 1].x;
+#pragma unroll
+      for (int o = 16; o; o >>= 1)
+        pair_add_pair(h, l, __shfl_xor_sync(0xffffffffu, h, o),
+                      __shfl_xor_sync(0xffffffffu, l, o));
+      if (lane == 0) sm[warp][i * NF + r] = make_float2(h, l);
+    }
+  __syncthreads();
+  for (int t = threadIdx.x; t < (kKsWarps / WS) * kKsRows * NF; t += kKsWarps * 32) {
+    const int g = t / (kKsRows * NF), e = t % (kKsRows * NF);
+    const int row = (blockIdx.x * (kKsWarps / WS) + g) * kKsRows + e / NF, f = f0 + e % NF;
+    double x = 0.0;
+#pragma unroll
+    for (int w = 0; w < WS; ++w) x += (double)sm[g * WS + w][e].x + (double)sm[g * WS + w][e].y;
+    if (row < n && f < frames) {
+      double* dst = bsol + (int64_t)f * n + row;
+      *dst = A ? x : *dst + x;
     }
   }
 }
@@ -510,7 +610,7 @@ void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhaso
                                  const double* ion_q, int frames, int n_ion,
                                  const SfPair* pairs, int npairs, const int* hkl,
                                  const double* sqw, int mpad, int kh, const void* turn,
-                                 void* v, double* vhead, int sms, cudaStream_t s) {
+                                 void* v, void* vhead, int sms, cudaStream_t s) {
   if (fp64) {
     (k_ion_sf_f64<<<dim3(mpad / 32, frames), kSf64Warps * 32, 0, s>>>(
          axis, ap, coord_stride, ion_q, n_ion, hkl, sqw, mpad, (double*)v),
@@ -526,7 +626,7 @@ void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhaso
     const int per = 32 * (kSfWarps / shares), hb = (kh + 31) / 32;
     (k_ion_sf_f32<<<dim3(hb + (npairs + per - 1) / per, frames), kSfWarps * 32, 0, s>>>(
          sion, coord_stride, ion_q, n_ion, pairs, npairs, hkl, sqw, mpad, kh, shares, hb,
-         (const float4*)turn, (float*)v, vhead),
+         (const float4*)turn, (float*)v, (float2*)vhead),
      note_launch());
   }
 }
@@ -566,15 +666,66 @@ int bsol_direct_splits(int n, int frames, int mpad, int kh, int sms) {
   return best;
 }
 
-// b^sol_k = A v: in float storage the head k-vectors (the heaviest weights) are
-// contracted in FP64 against an FP64 copy of their operand columns.  Without A (a streamed
+namespace {
+
+template <int NF, int WS>
+void launch_kspace_f32(const float* A, int64_t lda, const float2* Ahead, int n, int kh,
+                       const float* v, const float2* vhead, int frames, double* bsol,
+                       cudaStream_t s) {
+  constexpr int kRows = kKsRows * (kKsWarps / WS);
+  const int groups = (frames + NF - 1) / NF;
+  // A larger than half of L2 is read past it once (v and the sums' operands stay)
+  const int stream = A && (int64_t)n * lda * (int64_t)sizeof(float) > (64ll << 20);
+  for (int g0 = 0; g0 < groups; g0 += 65535) {
+    const int f0 = g0 * NF;
+    (k_bsol_kspace_f32<NF, WS><<<dim3((n + kRows - 1) / kRows, std::min(groups - g0, 65535)),
+                                 kKsWarps * 32, 0, s>>>(
+         A, lda, Ahead, n, kh, v + f0 * lda, vhead + (int64_t)f0 * 2 * kh, frames - f0,
+         bsol + (int64_t)f0 * n, stream),
+     note_launch());
+  }
+}
+
+// Eight frames at a time; fewer frames in one pass of the next larger size.  Rows share their
+// frames' v within a block (two warps a group) where that leaves two blocks an SM.
+void launch_kspace_frames(const float* A, int64_t lda, const float2* Ahead, int n, int kh,
+                          const float* v, const float2* vhead, int frames, double* bsol,
+                          int sms, cudaStream_t s) {
+  if (frames == 1)
+    launch_kspace_f32<1, 8>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, s);
+  else if (frames == 2)
+    launch_kspace_f32<2, 8>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, s);
+  else if (frames <= 4)
+    launch_kspace_f32<4, 8>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, s);
+  else if ((int64_t)((n + 15) / 16) * ((frames + 7) / 8) >= 2 * (int64_t)sms)
+    launch_kspace_f32<8, 2>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, s);
+  else
+    launch_kspace_f32<8, 8>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, s);
+}
+
+}  // namespace
+
+// b^sol_k = A v: in float storage the head k-vectors (the heaviest weights) are contracted in
+// float pairs against a float-pair copy of their operand columns.  Without A (a streamed
 // build) the float part is the direct sum over the tail k-vectors.
-void launch_bsol_kspace(bool fp64, const void* A, const double* Ahead, int n, int mpad, int kh,
-                        const void* v, const double* vhead, int frames, double* bsol,
+void launch_bsol_kspace(bool fp64, const void* A, const void* Ahead, int n, int mpad, int kh,
+                        const void* v, const void* vhead, int frames, double* bsol,
                         const uint32_t* sfix, const int* hkl, const double* sqw,
-                        const void* turn, int nsplit, double* split_part, cudaStream_t s) {
+                        const void* turn, int nsplit, double* split_part, int sms,
+                        cudaStream_t s) {
   const int64_t lda = 2 * (int64_t)mpad;
-  if (!A && !fp64) {
+  if (fp64) {
+    const int groups = (frames + kF64Frames - 1) / kF64Frames;
+    for (int g0 = 0; g0 < groups; g0 += 65535) {
+      const int f0 = kF64Frames * g0;
+      (k_bsol_kspace_f64<<<dim3((n * 32 + 255) / 256, std::min(groups - g0, 65535)), 256, 0, s>>>(
+           (const double*)A, n, lda, (const double*)v + f0 * lda, frames - f0,
+           bsol + (int64_t)f0 * n),
+       note_launch());
+    }
+    return;
+  }
+  if (!A) {
     const int fgroups = (frames + kDirectFrames - 1) / kDirectFrames;
     const int sp = split_part ? nsplit : 1;
     const int64_t stride = (int64_t)frames * n;  // between shares
@@ -591,32 +742,10 @@ void launch_bsol_kspace(bool fp64, const void* A, const double* Ahead, int n, in
       (k_sum_splits<<<(int)std::min<int64_t>((stride + 255) / 256, 8192), 256, 0, s>>>(
            split_part, sp, stride, stride, bsol),
        note_launch());
-    for (int g0 = 0; kh > 0 && g0 < (frames + 3) / 4; g0 += 65535) {
-      const int f0 = 4 * g0;
-      const dim3 grid((n * 32 + 255) / 256, std::min((frames - f0 + 3) / 4, 65535));
-      (k_bsol_kspace<double, 4><<<grid, 256, 0, s>>>(Ahead, n, 2 * (int64_t)kh,
-                                                     vhead + f0 * 2 * (int64_t)kh, frames - f0,
-                                                     bsol + (int64_t)f0 * n, 1), note_launch());
-    }
-    return;
+    if (kh == 0) return;
   }
-  for (int g0 = 0; g0 < (frames + 3) / 4; g0 += 65535) {
-    const int f0 = 4 * g0;
-    const dim3 grid((n * 32 + 255) / 256, std::min((frames - f0 + 3) / 4, 65535));
-    if (fp64) {
-      (k_bsol_kspace<double, 4><<<grid, 256, 0, s>>>((const double*)A, n, lda,
-                                                     (const double*)v + f0 * lda, frames - f0,
-                                                     bsol + (int64_t)f0 * n, 0), note_launch());
-    } else {
-      (k_bsol_kspace<float, 4><<<grid, 256, 0, s>>>((const float*)A, n, lda,
-                                                    (const float*)v + f0 * lda, frames - f0,
-                                                    bsol + (int64_t)f0 * n, 0), note_launch());
-      if (kh > 0)
-        (k_bsol_kspace<double, 4><<<grid, 256, 0, s>>>(Ahead, n, 2 * (int64_t)kh,
-                                                       vhead + f0 * 2 * (int64_t)kh, frames - f0,
-                                                       bsol + (int64_t)f0 * n, 1), note_launch());
-    }
-  }
+  launch_kspace_frames((const float*)A, lda, (const float2*)Ahead, n, kh, (const float*)v,
+                       (const float2*)vhead, frames, bsol, sms, s);
 }
 
 }  // namespace cpm
