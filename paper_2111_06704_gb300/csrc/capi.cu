@@ -654,7 +654,6 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
       (st = buf_reserve(c, &c->alpha, (size_t)n * sizeof(double))) ||
       (st = buf_reserve(c, &c->sfix, (size_t)c->npad * 3 * sizeof(uint32_t))) ||
       (!f64 && (st = buf_reserve(c, &c->atoms, atom_record_bytes(n)))) ||
-      (!f64 && (st = buf_reserve(c, &c->htab, h_table_bytes()))) ||
       (st = buf_reserve(c, &c->hkl, hkl.size() * sizeof(int))) ||
       (st = buf_reserve(c, &c->sqw, sqw.size() * sizeof(double))) ||
       (st = buf_reserve(c, &c->flush, fmask.size() * sizeof(uint32_t))) ||
@@ -681,8 +680,6 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
       (st = cuda_check(c, cudaMemcpyAsync(c->flush.ptr, fmask.data(), fmask.size() * sizeof(uint32_t), h2d, s), "flush")) ||
       (st = cuda_check(c, cudaMemcpyAsync(c->chunk_end.ptr, cmask.data(), cmask.size() * sizeof(uint32_t), h2d, s), "chunks")) ||
       (st = cuda_check(c, cudaMemcpyAsync(c->kexp.ptr, kexp.data(), kexp.size() * sizeof(int), h2d, s), "scales")) ||
-      (!f64 && (st = cuda_check(c, cudaMemcpyAsync(c->htab.ptr, h_table_host(), h_table_bytes(),
-                                                   h2d, s), "erfc table"))) ||
       (st = cuda_check(c, cudaMemsetAsync(c->E.ptr, 0, e_bytes, s), "E memset")) ||
       (st = cuda_check(c, cudaStreamSynchronize(s), "build upload")))
     return fail(st);
@@ -704,7 +701,11 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
   if (!f64 && !c->sfpairs.ptr) {  // depends on the k-vector table only, as that does
     const std::vector<SfPair> pairs = sf_pairs(hkl, c->m, c->mpad, c->kh);
     c->n_sfpairs = (int)pairs.size();
-    if ((st = buf_reserve(c, &c->sfpairs, std::max<size_t>(pairs.size(), 1) * sizeof(SfPair))) ||
+    // and the erfc table of the real-space pairs, the same for every context
+    if ((st = buf_reserve(c, &c->htab, h_table_bytes())) ||
+        (st = cuda_check(c, cudaMemcpyAsync(c->htab.ptr, h_table_host(), h_table_bytes(), h2d, s),
+                         "erfc table")) ||
+        (st = buf_reserve(c, &c->sfpairs, std::max<size_t>(pairs.size(), 1) * sizeof(SfPair))) ||
         (st = cuda_check(c, cudaMemcpyAsync(c->sfpairs.ptr, pairs.data(),
                                             pairs.size() * sizeof(SfPair), h2d, s), "pairs")) ||
         (st = cuda_check(c, cudaStreamSynchronize(s), "pairs sync")))
@@ -797,7 +798,7 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
   if (c->kh > 0)
     launch_structure_operand_head((const double*)c->xyz.ptr, c->npad, n, (const int*)c->hkl.ptr,
                                   (const double*)c->sqw.ptr, c->kh, c->p.box,
-                                  (double*)c->Ahead.ptr, s);
+                                  c->Ahead.ptr, s);
   cudaEventRecord(ev[1], s);
   if (tc) {
     // head (heaviest k-vectors, float-float) with the real-space, self and dipole terms in
@@ -807,7 +808,7 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
     cudaEventCreate(&ev_head);
     cudaEventRecord(ev_head, s);
     float* hhi = (float*)hsplit.ptr;
-    st = launch_ek_head_f64((const double*)c->Ahead.ptr, c->kh, head_cols, c->npad, hhi,
+    st = launch_ek_head_f64(c->Ahead.ptr, c->kh, head_cols, c->npad, hhi,
                             hhi + (size_t)c->npad * std::max(head_cols, 16),
                             (const double*)c->xyz.ptr, (const double*)c->alpha.ptr, n, geo,
                             (float2*)ehead.ptr, c->ldE, s);
@@ -885,7 +886,6 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
     return fail(st == CPM_ECUDA && c->err.empty() ? cuda_check(c, cudaGetLastError(), "k-space GEMM") : st);
   }
   cudaEventRecord(ev[2], s);
-  if (c->kh > 0) launch_pairs_in_place((double*)c->Ahead.ptr, (int64_t)c->npad * 2 * c->kh, s);
   launch_mirror_lower(f64, c->E.ptr, n, c->ldE, s);
   launch_extract_diag(f64, c->E.ptr, n, c->ldE, (double*)c->diag.ptr, s);
   (k_inverse_tail<<<(n + 255) / 256, 256, 0, s>>>((double*)c->diag.ptr, n), note_launch());

@@ -108,7 +108,6 @@ struct Ctx {
   int heavy_steps = 0;  // leading k-steps accumulated exactly in FP64
   int kh = 0;           // head k-vectors with an FP64 operand copy (float storage only)
   Buf Ahead;            // float pairs [npad][2*kh] of the head columns, A's column layout
-                        // (made in FP64, turned into pairs at the end of the build)
   Buf chunk_end;        // uint32 bit per K-block of 64 columns (tensor-core build)
   Buf kexp;             // int per K-block: FP16 plane scale exponent (tensor-core build)
   bool streamed = false;  // A too large to keep: built in k-windows, potential direct
@@ -226,16 +225,14 @@ void launch_structure_operand(bool fp64, const double* xyz, const uint32_t* sfix
                               int kb6, int kb3, int kb8, const int* kexp, const void* turn,
                               int kbeg, int kend, cudaStream_t s);
 void launch_structure_operand_head(const double* xyz, int npad, int n, const int* hkl,
-                                   const double* sqw, int kh, const double L[3], double* Ahead,
+                                   const double* sqw, int kh, const double L[3], void* Ahead,
                                    cudaStream_t s);
 int launch_ek_simt(bool fp64, const void* A, int npad, int mpad, const double* xyz,
                    const double* alpha, int n, const Geometry& geo, void* E, int64_t ldE,
                    int heavy_steps, const uint32_t* flush_mask, cudaStream_t s);
 void launch_mirror_lower(bool fp64, void* E, int n, int64_t ldE, cudaStream_t s);
 
-// x [len] doubles -> float pairs (hi, lo) in place
-void launch_pairs_in_place(double* x, int64_t len, cudaStream_t s);
-int launch_ek_head_f64(const double* Ahead, int kh, int ktot, int npad, float* hi, float* lo,
+int launch_ek_head_f64(const void* Ahead, int kh, int ktot, int npad, float* hi, float* lo,
                        const double* xyz, const double* alpha, int n, const Geometry& geo,
                        float2* Ehead, int64_t ldE, cudaStream_t s);
 

@@ -124,10 +124,12 @@ __global__ void k_structure_operand_f32(const uint32_t* __restrict__ sfix, int n
   }
 }
 
+// PAIRS: each value as a float pair (hi, lo) in its eight bytes instead of a double.
+template <bool PAIRS>
 __global__ void k_structure_operand_f64(const double* __restrict__ xyz, int npad, int n,
                                         const int* __restrict__ hkl,
                                         const double* __restrict__ sqw, int mpad, double lx,
-                                        double ly, double lz, double* __restrict__ A) {
+                                        double ly, double lz, void* __restrict__ out) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= mpad) return;
   const double h = hkl[3 * k], kk = hkl[3 * k + 1], l = hkl[3 * k + 2];
@@ -147,8 +149,15 @@ __global__ void k_structure_operand_f64(const double* __restrict__ xyz, int npad
       c *= w;
       s *= w;
     }
-    A[i * lda + kcol] = c;
-    A[i * lda + kcol + 64] = s;
+    if constexpr (PAIRS) {
+      float2* A = (float2*)out;
+      A[i * lda + kcol] = make_float2((float)c, (float)(c - (double)(float)c));
+      A[i * lda + kcol + 64] = make_float2((float)s, (float)(s - (double)(float)s));
+    } else {
+      double* A = (double*)out;
+      A[i * lda + kcol] = c;
+      A[i * lda + kcol + 64] = s;
+    }
   }
 }
 
@@ -467,27 +476,17 @@ k_ek_head_ff(const float* __restrict__ Ah_g, const float* __restrict__ Al_g, int
   }
 }
 
-// The head operand columns [0, ktot) of every row as float pairs x = hi + lo (exact to
-// ~2^-48), split once so the head GEMM loads floats only.
-__global__ void k_split_head(const double* __restrict__ A, int64_t lda, int rows, int ktot,
+// The head operand columns [0, ktot) of every row, float pairs x = hi + lo (exact to ~2^-48),
+// as a plane of each half: the head GEMM's loads.
+__global__ void k_split_head(const float2* __restrict__ A, int64_t lda, int rows, int ktot,
                              float* __restrict__ hi, float* __restrict__ lo) {
   const int64_t total = (int64_t)rows * ktot;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t r = e / ktot, c = e % ktot;
-    const double x = A[r * lda + c];
-    const float h = (float)x;
-    hi[e] = h;
-    lo[e] = (float)(x - (double)h);
-  }
-}
-
-__global__ void k_pairs_in_place(double* __restrict__ x, int64_t len) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < len;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const double v = x[e];
-    const float h = (float)v;
-    reinterpret_cast<float2*>(x)[e] = make_float2(h, (float)(v - (double)h));
+    const float2 x = A[r * lda + c];
+    hi[e] = x.x;
+    lo[e] = x.y;
   }
 }
 
@@ -544,11 +543,11 @@ void launch_fixed_point_coords(const double* xyz, int n, int npad, const double 
 }
 
 void launch_structure_operand_head(const double* xyz, int npad, int n, const int* hkl,
-                                   const double* sqw, int kh, const double L[3], double* Ahead,
+                                   const double* sqw, int kh, const double L[3], void* Ahead,
                                    cudaStream_t s) {
   dim3 grid((kh + 127) / 128, npad < 1024 ? npad : 1024);
-  (k_structure_operand_f64<<<grid, 128, 0, s>>>(xyz, npad, n, hkl, sqw, kh, L[0], L[1], L[2],
-                                               Ahead), note_launch());
+  (k_structure_operand_f64<true><<<grid, 128, 0, s>>>(xyz, npad, n, hkl, sqw, kh, L[0], L[1],
+                                                     L[2], Ahead), note_launch());
 }
 
 void launch_structure_operand(bool fp64, const double* xyz, const uint32_t* sfix, int npad,
@@ -560,7 +559,7 @@ void launch_structure_operand(bool fp64, const double* xyz, const uint32_t* sfix
   PlaneOut po{};
   if (fp64) {
     dim3 g64((mpad + 127) / 128, npad < 1024 ? npad : 1024);
-    (k_structure_operand_f64<<<g64, 128, 0, s>>>(xyz, npad, n, hkl, sqw, mpad, L[0], L[1],
+    (k_structure_operand_f64<false><<<g64, 128, 0, s>>>(xyz, npad, n, hkl, sqw, mpad, L[0], L[1],
                                                 L[2], (double*)A), note_launch());
   } else if (planes) {
     for (int t = 0; t < 3; ++t) po.p[t] = (uint16_t*)planes[t];
@@ -611,20 +610,16 @@ int launch_ek_simt(bool fp64, const void* A, int npad, int mpad, const double* x
 // FP64-accurate head of the k-space sum (the first ktot columns of the FP64 head operand,
 // row stride 2 kh, split into float pairs in hi/lo [npad][ktot]) plus the real-space,
 // self and dipole terms, lower triangle, into Ehead as float pairs (hi, lo).
-int launch_ek_head_f64(const double* Ahead, int kh, int ktot, int npad, float* hi, float* lo,
+int launch_ek_head_f64(const void* Ahead, int kh, int ktot, int npad, float* hi, float* lo,
                        const double* xyz, const double* alpha, int n, const Geometry& geo,
                        float2* Ehead, int64_t ldE, cudaStream_t s) {
   const Epi ep = make_epi(xyz, alpha, n, geo);
   constexpr int BM = 64;
   const int nt = (n + BM - 1) / BM;
   const int tiles = nt * (nt + 1) / 2;
-  (k_split_head<<<2048, 256, 0, s>>>(Ahead, 2 * (int64_t)kh, npad, ktot, hi, lo), note_launch());
+  (k_split_head<<<2048, 256, 0, s>>>((const float2*)Ahead, 2 * (int64_t)kh, npad, ktot, hi, lo), note_launch());
   (k_ek_head_ff<<<tiles, 256, 0, s>>>(hi, lo, ktot, ktot, Ehead, ldE, ep), note_launch());
   return cudaGetLastError() == cudaSuccess ? CPM_OK : CPM_ECUDA;
-}
-
-void launch_pairs_in_place(double* x, int64_t len, cudaStream_t s) {
-  (k_pairs_in_place<<<2048, 256, 0, s>>>(x, len), note_launch());
 }
 
 void launch_mirror_lower(bool fp64, void* E, int n, int64_t ldE, cudaStream_t s) {

@@ -9,15 +9,17 @@
 // evaluates the lists' heads together, each lane adding to its own atom's sum: no
 // compaction, no exchange of values between lanes.
 //
-// Float storage evaluates a pair in float pairs (hi + lo, ~1e-12 of the pair): the
-// difference from 64-bit fixed-point coordinates, erfc(x)/x from a table.  FP64 runs at
+// Float storage evaluates near pairs in float pairs (hi + lo, ~1e-12 of the pair: the
+// difference from 64-bit fixed-point coordinates, erfc(x)/x from a table) and far ones, where
+// erfc(g r) / r <= 1e-4 1/A, in plain float from the fixed-point difference (~1e-6 of a term,
+// <= 1e-10 1/A; three quarters of the images at a third of the instructions).  FP64 runs at
 // 1/64 of the float rate here and an FP64 erfc is some fifty operations, which is what
-// bound the kernel before: with near pairs in FP64, far ones in plain float, both through
-// queues of the warp, every ion screened by every lane, it took 16.4 ms at 26,600 atoms, 5,000
-// ions and 16 frames (r_c 24 A, 550 images an atom) against 1.77 ms; 183 against 12 us at
-// 12,800 atoms, 2,000 ions and one frame; 121 against 18 us at 512 atoms and 200 ions, where
-// four blocks held all the work; 2.57 against 1.48 ms at 512 atoms, 2,000 ions, 256 frames
-// (three images a pair).  FP64 storage evaluates every image in FP64.
+// bound the kernel before: with near pairs in FP64, both kinds through queues of the warp,
+// every ion screened by every lane, it took 16.4 ms at 26,600 atoms, 5,000 ions and 16 frames
+// (r_c 24 A, 550 images an atom) against 1.81 ms; 183 against 14 us at 12,800 atoms, 2,000
+// ions and one frame; 121 against 19 us at 512 atoms and 200 ions, where four blocks held all
+// the work; 2.57 against 1.45 ms at 512 atoms, 2,000 ions, 256 frames (three images a pair).
+// FP64 storage evaluates every image in FP64.
 #include <math.h>
 
 #include <algorithm>
@@ -90,7 +92,7 @@ __device__ __forceinline__ void h_table(const float4* __restrict__ T, float sh, 
 
 // ---- records -----------------------------------------------------------------------------
 // A point's fractional coordinates in 64-bit fixed point: x, y, z hold them rounded to
-// 2^-32, xl, yl, zl the signed rest in 2^-64.  Ions: (qh, ql) = q g as a float pair.
+// 2^-32, xl, yl, zl the signed rest in 2^-64.  Ions: (qh, ql) = q as a float pair.
 struct IonRec {
   uint32_t x, y, z;
   float qh;
@@ -124,7 +126,7 @@ constexpr int kPrepThreads = 128;
 // and the block's sums of q z and q for the dipole term and Q^sol: sums[frame][block].
 __global__ void __launch_bounds__(kPrepThreads)
 k_ion_prepare(const double* __restrict__ ion_xyz, const double* __restrict__ ion_q, int n_ion,
-              double lx, double ly, double lz, double g, uint32_t* __restrict__ sion,
+              double lx, double ly, double lz, uint32_t* __restrict__ sion,
               IonRec* __restrict__ rec, double2* __restrict__ sums) {
   __shared__ double2 red[kPrepThreads / 32];
   const int f = blockIdx.y, t = blockIdx.x * kPrepThreads + threadIdx.x;
@@ -136,7 +138,7 @@ k_ion_prepare(const double* __restrict__ ion_xyz, const double* __restrict__ ion
     fixed64(ion_xyz[3 * e], lx, r.x, r.xl);
     fixed64(ion_xyz[3 * e + 1], ly, r.y, r.yl);
     fixed64(z, lz, r.z, r.zl);
-    split(q * g, r.qh, r.ql);
+    split(q, r.qh, r.ql);
     sion[3 * e] = r.x;
     sion[3 * e + 1] = r.y;
     sion[3 * e + 2] = r.z;
@@ -179,14 +181,19 @@ __global__ void k_atom_records(const double* __restrict__ xyz, const double* __r
 
 constexpr int kMaxShifts = 64;
 constexpr int kRealWarps = 8;
-constexpr int kListDepth = 40;  // pairs a lane can hold: fewer than 32 at a look, and at
+constexpr int kListDepth = 72;  // pairs a lane can hold: fewer than 64 at a look, and at
 constexpr int kListStep = 8;    // most this many more before the next one
-constexpr int kListIonBits = 26;  // an entry: shift << 26 | ion (relative to a 2^26 base)
+// an entry of a list: shift << kIonBits | ion, the ion relative to a base moved on when full
+template <int kMode>
+constexpr int kIonBits = 16;
 
 // Screen modes: every box edge above 2 r_c (the nearest image only), a list of whole-box
 // shifts of the nearest image (each its own pair), or every image of a screened pair in FP64
 // (boxes so small that more than kMaxShifts shifts would be needed).
 enum RealMode { kSingleImage = 0, kShiftList = 1, kAllImages = 2 };
+
+template <>
+constexpr int kIonBits<kShiftList> = 10;
 
 struct RealArgs {
   const double *xyz, *alpha;   // electrode
@@ -203,7 +210,9 @@ struct RealArgs {
   float reach[3];              // L / 2 - r_c: largest half extent of a box of atoms whose
                                // ions need no wrapping (see below)
   float screen2;               // r_c^2 + 0.01
-  float rc2h, rc2l, g2h, g2l;  // r_c^2 and g^2 as float pairs
+  float far2, cut2;            // far images: r_split^2 <= r^2 < r_c^2 (1 - 1e-5)
+  float rc2h, rc2l, g2h, g2l;  // r_c^2, g^2 and g as float pairs
+  float gh, gl;
   int nshift;
   float shift[kMaxShifts][3];  // k L, the screen's
   signed char kshift[kMaxShifts][3];
@@ -278,8 +287,11 @@ __device__ __forceinline__ void finish_atom(const RealArgs& a, int f, int i, dou
 template <int kMode, bool kF64>
 __global__ void __launch_bounds__(kRealWarps * 32)
 k_bsol_real(const __grid_constant__ RealArgs a) {
-  // a lane's list, and the 32 ions of a step that the bounding box lets through
-  __shared__ uint32_t list[kRealWarps][kListDepth][32];
+  constexpr int kBits = kIonBits<kMode>;
+  constexpr bool kFar = !kF64;  // far images apart
+  // a lane's near pairs from the start of its list and its far ones from the end, and the 32
+  // ions of a step that the bounding box lets through
+  __shared__ uint16_t list[kRealWarps][kListDepth][32];
   __shared__ float4 cand[kMode == kSingleImage ? kRealWarps : 1][32];
   __shared__ double red[kRealWarps][32];
   const int f = blockIdx.y;
@@ -318,14 +330,23 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
       wrap |= half[u] > a.reach[u];
     }
   }
-  float acch = 0.f, accl = 0.f;
+  float acch = 0.f, accl = 0.f, accf = 0.f;
   double acc = 0.0;
-  int cnt = 0;  // entries of this lane's list
+  int cn = 0, cf = 0;  // near and far entries of this lane's list
   int base0 = 0;
+  // far images of this lane's atom: beyond alpha r = 6 as well
+  const float lane_far2 = kFar ? fmaxf(a.far2, 36.0f / ((float)(ai * ai))) : 0.f;
+
+  // lists the image of ion t at r^2 = m2 by the screen's float, if it is in range
+  auto put = [&](float m2, uint32_t entry) {
+    if (!live || m2 >= a.screen2) return;
+    if (kFar && m2 >= lane_far2 && m2 < a.cut2) list[warp][kListDepth - ++cf][lane] = (uint16_t)entry;
+    else list[warp][cn++][lane] = (uint16_t)entry;
+  };
 
   auto evaluate = [&](uint32_t entry) {
-    const int ion = base0 + (int)(entry & ((1u << kListIonBits) - 1));
-    const int si = kMode == kShiftList ? (int)(entry >> kListIonBits) : 0;
+    const int ion = base0 + (int)(entry & ((1u << kBits) - 1));
+    const int si = kMode == kShiftList ? (int)(entry >> kBits) : 0;
     if constexpr (kF64 || kMode == kAllImages) {
       const size_t e = (size_t)f * a.n_ion + ion;
       const double p[3] = {a.ion_xyz[3 * e], a.ion_xyz[3 * e + 1], a.ion_xyz[3 * e + 2]};
@@ -396,8 +417,9 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
             ff_add(vh, vl, ph, pl, vh, vl);
           }
           float ph, pl;
-          ff_mul(vh, vl, __uint_as_float(w0.w), __int_as_float(w1.w), ph, pl);
-          pair_add_pair(acch, accl, ph, pl);
+          ff_mul(vh, vl, a.gh, a.gl, ph, pl);
+          ff_mul(ph, pl, __uint_as_float(w0.w), __int_as_float(w1.w), vh, vl);
+          pair_add_pair(acch, accl, vh, vl);
         } else {  // an ion almost on an atom: FP64
           const double r2 = (double)sh + (double)sl;
           if (r2 > 0.0) {
@@ -410,12 +432,41 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
       }
     }
   };
+  // a far image, in plain float from the fixed-point difference of the nearest image; one
+  // that the screen's offsets took for far and this r^2 does not goes the near way
+  auto evaluate_far = [&](uint32_t entry) {
+    const uint4 w = __ldg(reinterpret_cast<const uint4*>(ions + base0 + (entry & ((1u << kBits) - 1))));
+    float d0 = (float)(int32_t)(ui[0] - w.x) * a.fs[0], d1 = (float)(int32_t)(ui[1] - w.y) * a.fs[1],
+          d2 = (float)(int32_t)(ui[2] - w.z) * a.fs[2];
+    float m2;
+    if constexpr (kMode == kShiftList) {
+      const int si = (int)(entry >> kBits);
+      d0 += a.shift[si][0];
+      d1 += a.shift[si][1];
+      d2 += a.shift[si][2];
+      m2 = fmaf(d2, d2, fmaf(d1, d1, d0 * d0));
+    } else {
+      m2 = fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
+    }
+    if (m2 >= lane_far2 && m2 < a.cut2) {
+      const float ir = rsqrtf(m2);  // 1 / r to ~2 ulp
+      accf += __uint_as_float(w.w) * (erfcf(a.gh * (m2 * ir)) * ir);
+    } else {
+      evaluate(entry);
+    }
+  };
   // evaluates every listed pair of the warp
   auto drain = [&]() {
-    const int most = __reduce_max_sync(0xffffffffu, cnt);
+    int most = __reduce_max_sync(0xffffffffu, cn);
     for (int k = 0; k < most; ++k)
-      if (k < cnt) evaluate(list[warp][k][lane]);
-    cnt = 0;
+      if (k < cn) evaluate(list[warp][k][lane]);
+    cn = 0;
+    if constexpr (kFar) {
+      most = __reduce_max_sync(0xffffffffu, cf);
+      for (int k = 1; k <= most; ++k)
+        if (k <= cf) evaluate_far(list[warp][kListDepth - k][lane]);
+      cf = 0;
+    }
   };
 
   // this warp's share of the ions
@@ -426,13 +477,13 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
   auto look = [&](int steps) {  // before screening `steps` (at most kListStep) more
     if (since + steps > kListStep) {
       since = 0;
-      if (__any_sync(0xffffffffu, cnt >= kListDepth - kListStep)) drain();
+      if (__any_sync(0xffffffffu, cn + cf >= kListDepth - kListStep)) drain();
     }
     since += steps;
   };
   if (grp * 32 < a.n)
     for (int t = t0; t < t1; t += 32) {
-      if (t - base0 >= (1 << kListIonBits) - 32) {  // the entries' range of ions
+      if (t - base0 > (1 << kBits) - 32) {  // the entries' range of ions
         drain();
         base0 = t;
       }
@@ -480,8 +531,7 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
               y = off[1] - p.y;
               z = off[2] - p.z;
             }
-            if (live && fmaf(x, x, fmaf(y, y, z * z)) < a.screen2)
-              list[warp][cnt++][lane] = (uint32_t)(__float_as_int(p.w) - base0);
+            put(fmaf(x, x, fmaf(y, y, z * z)), (uint32_t)(__float_as_int(p.w) - base0));
           }
         }
       } else {
@@ -492,8 +542,7 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
           const float z = (float)(int32_t)(ui[2] - w.z) * a.fs[2];
           if constexpr (kMode == kAllImages) {
             look(1);
-            if (live && fmaf(x, x, fmaf(y, y, z * z)) < a.screen2)
-              list[warp][cnt++][lane] = (uint32_t)(t + c - base0);
+            put(fmaf(x, x, fmaf(y, y, z * z)), (uint32_t)(t + c - base0));
           } else {
             for (int s0 = 0; s0 < a.nshift; s0 += kListStep) {
               const int s1 = min(a.nshift, s0 + kListStep);
@@ -501,9 +550,8 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
               for (int si = s0; si < s1; ++si) {
                 const float sx = x + a.shift[si][0], sy = y + a.shift[si][1],
                             sz = z + a.shift[si][2];
-                if (live && fmaf(sx, sx, fmaf(sy, sy, sz * sz)) < a.screen2)
-                  list[warp][cnt++][lane] =
-                      ((uint32_t)si << kListIonBits) | (uint32_t)(t + c - base0);
+                put(fmaf(sz, sz, fmaf(sy, sy, sx * sx)),
+                    ((uint32_t)si << kBits) | (uint32_t)(t + c - base0));
               }
             }
           }
@@ -511,6 +559,7 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
       }
     }
   drain();
+  acc += (double)accf;
   acc += (double)acch + (double)accl;
   if (a.shares > 1) {  // the block's shares of a group, in share order
     red[warp][lane] = acc;
@@ -575,7 +624,7 @@ void launch_ion_prepare(const double* ion_xyz, const double* ion_q, int frames, 
                         const Geometry& geo, uint32_t* sion, const RealPlan& plan, void* scratch,
                         cudaStream_t s) {
   (k_ion_prepare<<<dim3(prep_blocks(n_ion), frames), kPrepThreads, 0, s>>>(
-       ion_xyz, ion_q, n_ion, geo.L[0], geo.L[1], geo.L[2], geo.g, sion, (IonRec*)scratch,
+       ion_xyz, ion_q, n_ion, geo.L[0], geo.L[1], geo.L[2], sion, (IonRec*)scratch,
        (double2*)((char*)scratch + plan.o_sums)),
    note_launch());
 }
@@ -608,6 +657,18 @@ void launch_bsol_real_and_finish(const double* xyz, const double* alpha, const u
   };
   pair(a.rc2, a.rc2h, a.rc2l);
   pair(geo.g * geo.g, a.g2h, a.g2l);
+  pair(geo.g, a.gh, a.gl);
+  // r_split: erfc(g r) / r = 1e-4 / A (bisection); r_c (no far images) where the term never
+  // gets that small
+  double lo = 1e-3, hi = geo.rc;
+  if (erfc(geo.g * hi) / hi <= 1e-4)
+    for (int it = 0; it < 60; ++it) {
+      const double mid = 0.5 * (lo + hi);
+      if (erfc(geo.g * mid) / mid > 1e-4) lo = mid;
+      else hi = mid;
+    }
+  a.far2 = (float)(hi * hi);
+  a.cut2 = (float)(a.rc2 * (1.0 - 1e-5));
   // shifts k with |k| <= floor((r_c + L / 2) / L) per direction (only k = 0 where
   // L > 2 r_c): every image within r_c of an atom, given the nearest one
   int m[3], total = 1;
