@@ -345,7 +345,7 @@ void release_workspace(Ctx* c) {
   Buf* ws[] = {&c->tc_planes[0], &c->tc_planes[1], &c->tc_planes[2], &c->tc_planes[3],
                &c->tc_head, &c->tc_err,
                &c->tc_hsplit, &c->tc_scratch, &c->dc_cnt, &c->dc_pcol, &c->dc_status, &c->ws_solve, &c->ws_in0, &c->ws_in1, &c->ws_in2,
-               &c->ws_out0, &c->ws_out1, &c->ws_pot, &c->ws_guess, &c->ws_feat, &c->ws_cluster,
+               &c->ws_out0, &c->ws_out1, &c->ws_pot, &c->ws_guess, &c->ws_feat, &c->ws_grad, &c->ws_cluster,
                &c->tc_tiles};
   for (Buf* b : ws) buf_free(c, b);
   c->tc_tiles_nt = 0;

@@ -160,7 +160,7 @@ struct Ctx {
   std::vector<double> kw;  // k-vector weights W_K of the sorted table, mpad entries (0 past m)
   std::vector<int> kv_hkl;    // the k-vector table (host), made on the first build
   std::vector<double> kv_w;
-  Buf ws_solve, ws_in0, ws_in1, ws_in2, ws_out0, ws_out1, ws_pot, ws_guess, ws_feat;
+  Buf ws_solve, ws_in0, ws_in1, ws_in2, ws_out0, ws_out1, ws_pot, ws_guess, ws_feat, ws_grad;
   Buf ws_cluster;  // per-column results of the cluster-resident solve
   // the solver's online autotuner: per bucket of right-hand-side counts (1, 2-3, 4-7, ..,
   // 128+), the path found faster (0 not yet known, 1 host-driven kernels, 2 cluster-

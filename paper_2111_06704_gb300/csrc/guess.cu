@@ -11,7 +11,7 @@
 #include <algorithm>
 #include <vector>
 
-#include "cpm_internal.cuh"
+#include "phasor.cuh"
 
 namespace cpm {
 
@@ -31,10 +31,6 @@ static_assert(ob4 + 1 == kP, "parameter layout");
 // 10,497 multiply-adds otherwise.
 __device__ __forceinline__ float sigmoid(float z) { return __frcp_rn(1.0f + __expf(-z)); }
 __device__ __forceinline__ float silu(float z) { return z * sigmoid(z); }
-__device__ __forceinline__ float silu_grad(float z) {
-  const float s = sigmoid(z);
-  return s * (1.0f + z * (1.0f - s));
-}
 
 // Shell of every PCG-DC pattern entry (k - 1/2 <= r < k + 1/2, k = 1..8; 0 outside or
 // for the atom itself).  The electrode is fixed, so this geometry is found once; the host
@@ -162,13 +158,6 @@ k_guess_features(int n, int frames, const float2* __restrict__ pot,
   }
 }
 
-__device__ void load_params(const float* __restrict__ params, float* w, int bf16) {
-  for (int k = threadIdx.x; k < kP; k += blockDim.x) {
-    const float v = params[k];
-    w[k] = bf16 ? __bfloat162float(__float2bfloat16_rn(v)) : v;
-  }
-}
-
 // y[s] = net((feat[s] - mean) * inv_std), 128 samples per tile.  Weights (transposed,
 // unit index fastest) and the activations of a tile (feature-major) sit in shared memory;
 // each thread owns 8 samples x 4 units of a layer, so every float4 of weights and of
@@ -288,135 +277,311 @@ k_mlp_forward(const float* __restrict__ params, const float* __restrict__ norm, 
   }
 }
 
-// Gradient of the mean squared error (1/S) sum_s (y_s - t_s)^2 over this call's samples,
-// accumulated into grad (zeroed by the caller); loss_sum accumulates sum (y - t)^2.
-// One block = 128 samples; activations of the block in shared memory; the parameter
-// gradients are reductions over the block's samples, then one atomic add per parameter.
-constexpr int kB = 128;
-constexpr int kLd = kH + 1;  // padded row of a [sample][unit] array
+// Gradient of the mean squared error (1/S) sum_s (y_s - t_s)^2 over this call's samples and
+// sum_s (y_s - t_s)^2: every block's share into part[block][kPart], summed by k_grad_finish.
+//
+// Persistent blocks (one an SM: 222 KB of shared memory) take tiles of 128 samples.  Every
+// product of the pass is a register-tiled one on feature-major tiles with XOR-swizzled rows:
+// the forward layers and the back-propagated ones in 8 samples x 4 units a thread (as
+// k_mlp_forward; the thread that made a pre-activation also meets its gradient, so silu'
+// stays in its registers), the weight gradients in 4 x 4 outputs over the tile's samples.
+// The weight gradients of a tile are float sums over its 128 samples, added to a float pair a
+// thread keeps over its tiles; blocks are added in FP64 in a fixed order.  Bound by FP32
+// multiply-adds (29,000 a sample; 8 warps an SM).  One thread a sample with scalar loads of
+// every operand and an atomic add per parameter and 128 samples took 3,702 us for 426,000
+// samples (8% of the chip's FP32 rate); this takes 817 us.
+constexpr int kGradThreads = 256;
+constexpr int kPart = kP + 1;  // the parameters' gradients, the loss
+constexpr int oGW = kF * kH + 2 * kH * kH;   // WT1, WT2, WT3, then:
+constexpr int oGB = oGW + 2 * kH * kH;       // W2, W3 as given, then b1, b2, b3, W4, b4
+constexpr int oGX = oGB + 4 * kH + 4;        // tiles: X, H1, H2, GA, GB
+constexpr size_t kGradSmem = sizeof(float) * (oGX + kF * kTs + 4 * kH * kTs);
 
-__global__ void __launch_bounds__(kB, 1)
-k_mlp_grad(const float* __restrict__ params, const float* __restrict__ norm, int bf16,
-           int64_t samples, double inv_s, const float* __restrict__ feat,
-           const float* __restrict__ target, float* __restrict__ grad,
-           double* __restrict__ loss_sum) {
-  extern __shared__ float sm[];
-  float* w = sm;                       // kP
-  float* X = w + kP;                   // [kB][kF + 1]
-  float* Z1 = X + kB * (kF + 1);       // pre-activations, later dL/dz
-  float* Z2 = Z1 + kB * kLd;
-  float* Z3 = Z2 + kB * kLd;
-  float* H1 = Z3 + kB * kLd;           // silu(Z1)
-  float* H2 = H1 + kB * kLd;           // silu(Z2)
-  float* DY = H2 + kB * kLd;           // [kB]
-  load_params(params, w, bf16);
-  __syncthreads();
-  const int t = threadIdx.x;
-  const int64_t s = blockIdx.x * (int64_t)kB + t;
-  const bool valid = s < samples;
-  // ---- forward, one sample per thread
-  {
-    float* x = X + t * (kF + 1);
-    for (int c = 0; c < kF; ++c)
-      x[c] = valid ? (feat[s * kF + c] - norm[c]) * norm[kF + c] : 0.f;
-    for (int a = 0; a < kH; ++a) {
-      float z = w[ob1 + a];
-      for (int c = 0; c < kF; ++c) z = fmaf(w[oW1 + a * kF + c], x[c], z);
-      Z1[t * kLd + a] = z;
-      H1[t * kLd + a] = silu(z);
-    }
-    for (int a = 0; a < kH; ++a) {
-      float z = w[ob2 + a];
-      for (int c = 0; c < kH; ++c) z = fmaf(w[oW2 + a * kH + c], H1[t * kLd + c], z);
-      Z2[t * kLd + a] = z;
-      H2[t * kLd + a] = silu(z);
-    }
-    float y = w[ob4];
-    for (int a = 0; a < kH; ++a) {
-      float z = w[ob3 + a];
-      for (int c = 0; c < kH; ++c) z = fmaf(w[oW3 + a * kH + c], H2[t * kLd + c], z);
-      Z3[t * kLd + a] = z;
-      y = fmaf(w[oW4 + a], silu(z), y);
-    }
-    const float diff = valid ? y - target[s] : 0.f;
-    DY[t] = (float)(2.0 * inv_s) * diff;
-    double l = (double)diff * (double)diff;
-    for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((t & 31) == 0) atomicAdd(loss_sum, l);
+// acc[k][j] += sum_c W[c][4 ug + j] in[c][8 sg + k] over NIN rows.
+template <int NIN>
+__device__ __forceinline__ void tile_product(const float* __restrict__ W,
+                                             const float* __restrict__ in, float (&acc)[8][4],
+                                             int ug, int sg) {
+#pragma unroll 4
+  for (int c = 0; c < NIN; ++c) {
+    const float4 w = *reinterpret_cast<const float4*>(W + c * kH + 4 * ug);
+    const float4 x0 = *reinterpret_cast<const float4*>(in + act_at(c, 8 * sg));
+    const float4 x1 = *reinterpret_cast<const float4*>(in + act_at(c, 8 * sg + 4));
+    const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+    const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[k][j] = fmaf(xv[k], wv[j], acc[k][j]);
   }
-  __syncthreads();
-  // ---- output layer: dW4[a] = sum_s dy_s h3[s][a]; db4 = sum_s dy_s
-  if (t < kH) {
-    float acc = 0.f;
-    for (int q = 0; q < kB; ++q) acc = fmaf(DY[q], silu(Z3[q * kLd + t]), acc);
-    atomicAdd(&grad[oW4 + t], acc);
-  } else if (t == kH) {
-    float acc = 0.f;
-    for (int q = 0; q < kB; ++q) acc += DY[q];
-    atomicAdd(&grad[ob4], acc);
-  }
-  __syncthreads();
-  // g3 = dy W4 * silu'(z3), in place of Z3
-  for (int a = 0; a < kH; ++a) Z3[t * kLd + a] = DY[t] * w[oW4 + a] * silu_grad(Z3[t * kLd + a]);
-  __syncthreads();
-  // ---- hidden layers: dW = sum_s g_s h_in_s^T, db = sum_s g_s, then g_in = W^T g * silu'
-  auto layer = [&](float* G, const float* Hin, int nin, int ow, int ob) {
-    // 64 x nin outputs over kB threads
-    const int per = kH * nin / kB;
-    for (int u = 0; u < per; ++u) {
-      const int e = t * per + u;
-      const int a = e / nin, c = e % nin;
-      float acc = 0.f;
-      for (int q = 0; q < kB; ++q) {
-        const float hv = nin == kF ? Hin[q * (kF + 1) + c] : Hin[q * kLd + c];
-        acc = fmaf(G[q * kLd + a], hv, acc);
-      }
-      atomicAdd(&grad[ow + a * nin + c], acc);
-    }
-    if (t < kH) {
-      float acc = 0.f;
-      for (int q = 0; q < kB; ++q) acc += G[q * kLd + t];
-      atomicAdd(&grad[ob + t], acc);
-    }
-  };
-  layer(Z3, H2, kH, oW3, ob3);
-  // g2 = W3^T g3 * silu'(z2), in place of Z2
-  {
-    float g[kH];
-    for (int c = 0; c < kH; ++c) {
-      float acc = 0.f;
-      for (int a = 0; a < kH; ++a) acc = fmaf(w[oW3 + a * kH + c], Z3[t * kLd + a], acc);
-      g[c] = acc * silu_grad(Z2[t * kLd + c]);
-    }
-    __syncthreads();  // every thread has finished reading Z2 through `layer`
-    for (int c = 0; c < kH; ++c) Z2[t * kLd + c] = g[c];
-  }
-  __syncthreads();
-  layer(Z2, H1, kH, oW2, ob2);
-  {
-    float g[kH];
-    for (int c = 0; c < kH; ++c) {
-      float acc = 0.f;
-      for (int a = 0; a < kH; ++a) acc = fmaf(w[oW2 + a * kH + c], Z2[t * kLd + a], acc);
-      g[c] = acc * silu_grad(Z1[t * kLd + c]);
-    }
-    __syncthreads();
-    for (int c = 0; c < kH; ++c) Z1[t * kLd + c] = g[c];
-  }
-  __syncthreads();
-  layer(Z1, X, kF, oW1, ob1);
 }
 
-__global__ void k_adam(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
-                       const float* __restrict__ g, int n, float lr, float c1, float c2) {
+__device__ __forceinline__ void tile_store(float* __restrict__ out, const float (&v)[8][4],
+                                           int ug, int sg) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int row = 4 * ug + j;
+    *reinterpret_cast<float4*>(out + act_at(row, 8 * sg)) =
+        make_float4(v[0][j], v[1][j], v[2][j], v[3][j]);
+    *reinterpret_cast<float4*>(out + act_at(row, 8 * sg + 4)) =
+        make_float4(v[4][j], v[5][j], v[6][j], v[7][j]);
+  }
+}
+
+// (h, l)[i][j] += sum_s G[4 ua + i][s] in[NC uc + j][s] over the tile's samples.
+template <int NC>
+__device__ __forceinline__ void tile_outer(const float* __restrict__ G,
+                                           const float* __restrict__ in, float (&h)[4][NC],
+                                           float (&l)[4][NC], int ua, int uc) {
+  float acc[4][NC];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < NC; ++j) acc[i][j] = 0.f;
+#pragma unroll 2
+  for (int s = 0; s < kTs; s += 4) {
+    float4 g[4], x[NC];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      g[i] = *reinterpret_cast<const float4*>(G + act_at(4 * ua + i, s));
+#pragma unroll
+    for (int j = 0; j < NC; ++j)
+      x[j] = *reinterpret_cast<const float4*>(in + act_at(NC * uc + j, s));
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < NC; ++j)
+        acc[i][j] = fmaf(g[i].w, x[j].w,
+                         fmaf(g[i].z, x[j].z,
+                              fmaf(g[i].y, x[j].y, fmaf(g[i].x, x[j].x, acc[i][j]))));
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < NC; ++j) pair_add1(h[i][j], l[i][j], acc[i][j]);
+}
+
+__global__ void __launch_bounds__(kGradThreads, 1)
+k_mlp_grad(const float* __restrict__ params, const float* __restrict__ norm, int bf16,
+           int64_t samples, double inv_s, const float* __restrict__ feat,
+           const float* __restrict__ target, double* __restrict__ part) {
+  extern __shared__ __align__(16) float gsm[];
+  float *WT1 = gsm, *WT2 = WT1 + kF * kH, *WT3 = WT2 + kH * kH;
+  float *W2 = gsm + oGW, *W3 = W2 + kH * kH, *bv = gsm + oGB;
+  float *X = gsm + oGX, *H1 = X + kF * kTs, *H2 = H1 + kH * kTs, *GA = H2 + kH * kTs,
+        *GB = GA + kH * kTs;
+  const int t = threadIdx.x;
+  for (int e = t; e < kP; e += kGradThreads) {
+    float v = params[e];
+    if (bf16) v = __bfloat162float(__float2bfloat16_rn(v));
+    if (e < ob1) {
+      WT1[(e % kF) * kH + e / kF] = v;
+    } else if (e < oW2) {
+      bv[e - ob1] = v;
+    } else if (e < ob2) {
+      WT2[((e - oW2) % kH) * kH + (e - oW2) / kH] = v;
+      W2[e - oW2] = v;
+    } else if (e < oW3) {
+      bv[kH + e - ob2] = v;
+    } else if (e < ob3) {
+      WT3[((e - oW3) % kH) * kH + (e - oW3) / kH] = v;
+      W3[e - oW3] = v;
+    } else if (e < oW4) {
+      bv[2 * kH + e - ob3] = v;
+    } else {
+      bv[3 * kH + e - oW4] = v;  // W4, b4
+    }
+  }
+  const int ug = t & 15, sg = t >> 4;  // units 4 ug .., samples 8 sg ..; outputs 4 ug, sg too
+  float h3[4][4], l3[4][4], h2[4][4], l2[4][4], h1[4][2], l1[4][2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) h3[i][j] = l3[i][j] = h2[i][j] = l2[i][j] = 0.f;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) h1[i][j] = l1[i][j] = 0.f;
+  }
+  float b1[4] = {0, 0, 0, 0}, b2[4] = {0, 0, 0, 0}, b3[4] = {0, 0, 0, 0}, w4[4] = {0, 0, 0, 0};
+  float b4 = 0.f, lossh = 0.f, lossl = 0.f;
+  const float scale = (float)(2.0 * inv_s);
+  const int64_t tiles = (samples + kTs - 1) / kTs;
+  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int64_t s0 = tile * kTs;
+    __syncthreads();  // weights written / the previous tile's reads of X done
+    for (int e = t; e < kTs * kF; e += kGradThreads) {
+      const int s = e / kF, c = e % kF;
+      const int64_t gs = s0 + s;
+      X[act_at(c, s)] = gs < samples ? (feat[gs * kF + c] - norm[c]) * norm[kF + c] : 0.f;
+    }
+    __syncthreads();
+    float acc[8][4], d1[8][4], d2[8][4];  // d: silu' of layers 1 and 2
+    auto bias = [&](int layer) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[k][j] = bv[layer * kH + 4 * ug + j];
+    };
+    auto activate = [&](float (&d)[8][4]) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float z = acc[k][j], s = sigmoid(z);
+          d[k][j] = s * (1.0f + z * (1.0f - s));
+          acc[k][j] = z * s;
+        }
+    };
+    bias(0);
+    tile_product<kF>(WT1, X, acc, ug, sg);
+    activate(d1);
+    tile_store(H1, acc, ug, sg);
+    __syncthreads();
+    bias(1);
+    tile_product<kH>(WT2, H1, acc, ug, sg);
+    activate(d2);
+    tile_store(H2, acc, ug, sg);
+    __syncthreads();
+    bias(2);
+    tile_product<kH>(WT3, H2, acc, ug, sg);
+    // y, dL/dy and dL/dz3 of the thread's 8 samples
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      float hv[4], dv[4], y = 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float z = acc[k][j], s = sigmoid(z);
+        hv[j] = z * s;
+        dv[j] = s * (1.0f + z * (1.0f - s));
+        y = fmaf(bv[3 * kH + 4 * ug + j], hv[j], y);
+      }
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+      const int64_t gs = s0 + 8 * sg + k;
+      const float diff = gs < samples ? y + bv[4 * kH] - target[gs] : 0.f;
+      const float dy = scale * diff;
+      if (ug == 0) {
+        const float p = __fmul_rn(diff, diff);
+        pair_add1(lossh, lossl, p);
+        lossl += fmaf(diff, diff, -p);
+        b4 += dy;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        w4[j] = fmaf(dy, hv[j], w4[j]);
+        acc[k][j] = dy * bv[3 * kH + 4 * ug + j] * dv[j];
+        b3[j] += acc[k][j];
+      }
+    }
+    tile_store(GA, acc, ug, sg);
+    __syncthreads();
+    auto back = [&](const float* W, const float* G, const float (&d)[8][4], float (&b)[4]) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[k][j] = 0.f;
+      tile_product<kH>(W, G, acc, ug, sg);
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          acc[k][j] *= d[k][j];
+          b[j] += acc[k][j];
+        }
+    };
+    back(W3, GA, d2, b2);
+    tile_store(GB, acc, ug, sg);
+    tile_outer<4>(GA, H2, h3, l3, ug, sg);
+    __syncthreads();
+    back(W2, GB, d1, b1);
+    tile_store(GA, acc, ug, sg);
+    tile_outer<4>(GB, H1, h2, l2, ug, sg);
+    __syncthreads();
+    tile_outer<2>(GA, X, h1, l1, ug, sg);
+  }
+  // the block's sums: weight gradients from their threads, the others over the 16 sample groups
+  double* out = part + (int64_t)blockIdx.x * kPart;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int e = (4 * ug + i) * kH + 4 * sg + j;
+      out[oW3 + e] = (double)h3[i][j] + (double)l3[i][j];
+      out[oW2 + e] = (double)h2[i][j] + (double)l2[i][j];
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      out[oW1 + (4 * ug + i) * kF + 2 * sg + j] = (double)h1[i][j] + (double)l1[i][j];
+  }
+  __syncthreads();
+  float* red = GA;  // [4][16 sample groups][64 units]
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    red[(0 * 16 + sg) * kH + 4 * ug + j] = b1[j];
+    red[(1 * 16 + sg) * kH + 4 * ug + j] = b2[j];
+    red[(2 * 16 + sg) * kH + 4 * ug + j] = b3[j];
+    red[(3 * 16 + sg) * kH + 4 * ug + j] = w4[j];
+  }
+  double* red2 = reinterpret_cast<double*>(GB);  // [16][2]
+  if (ug == 0) {
+    red2[2 * sg] = (double)b4;
+    red2[2 * sg + 1] = (double)lossh + (double)lossl;
+  }
+  __syncthreads();
+  {
+    const int arr = t >> 6, u = t & 63;
+    double s = 0.0;
+    for (int g = 0; g < 16; ++g) s += (double)red[(arr * 16 + g) * kH + u];
+    out[(arr == 0 ? ob1 : arr == 1 ? ob2 : arr == 2 ? ob3 : oW4) + u] = s;
+    if (t < 2) {
+      s = 0.0;
+      for (int g = 0; g < 16; ++g) s += red2[2 * g + t];
+      out[t == 0 ? ob4 : kP] = s;
+    }
+  }
+}
+
+struct AdamStep {
+  float *p, *m, *v;
+  float lr, c1, c2;
+};
+
+__device__ __forceinline__ void adam_update(const AdamStep& a, int k, float gk) {
+  const float mk = 0.9f * a.m[k] + 0.1f * gk;
+  const float vk = 0.999f * a.v[k] + 0.001f * gk * gk;
+  a.m[k] = mk;
+  a.v[k] = vk;
+  a.p[k] -= a.lr * (mk * a.c1) / (sqrtf(vk * a.c2) + 1e-8f);
+}
+
+// grad = sum of the blocks' shares in block order (eight interleaved sums, added in order),
+// the loss likewise; with a.p, the Adam step on the same parameter.
+constexpr int kFinishSlices = 8;
+
+__global__ void __launch_bounds__(32 * kFinishSlices)
+k_grad_finish(const double* __restrict__ part, int blocks, float* __restrict__ grad,
+              double* __restrict__ loss, const AdamStep a) {
+  __shared__ double red[kFinishSlices][32];
+  const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
+  const int k = blockIdx.x * 32 + lane;
+  double s = 0.0;
+  if (k < kPart)
+#pragma unroll 4
+    for (int b = sl; b < blocks; b += kFinishSlices) s += part[(int64_t)b * kPart + k];
+  red[sl][lane] = s;
+  __syncthreads();
+  if (sl != 0 || k >= kPart) return;
+  for (int w = 1; w < kFinishSlices; ++w) s += red[w][lane];
+  if (k == kP) {
+    *loss = s;
+    return;
+  }
+  grad[k] = (float)s;
+  if (a.p) adam_update(a, k, (float)s);
+}
+
+__global__ void k_adam(const AdamStep a, const float* __restrict__ g) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  const float gk = g[k];
-  const float mk = 0.9f * m[k] + 0.1f * gk;
-  const float vk = 0.999f * v[k] + 0.001f * gk * gk;
-  m[k] = mk;
-  v[k] = vk;
-  p[k] -= lr * (mk * c1) / (sqrtf(vk * c2) + 1e-8f);
+  if (k < kP) adam_update(a, k, g[k]);
 }
 
 __global__ void k_guess_apply(int64_t len, const float* __restrict__ y, float scale,
@@ -428,9 +593,6 @@ __global__ void k_guess_apply(int64_t len, const float* __restrict__ y, float sc
 
 // Device memory of the context's device (or managed memory): what these kernels may use.
 bool dev_ok(const Ctx* c, const void* p) { return pointer_where(c, p) == 1; }
-
-constexpr size_t kGradSmem =
-    sizeof(float) * (kP + kB * (kF + 1) + 5 * kB * kLd + kB);
 
 }  // namespace
 }  // namespace cpm
@@ -519,6 +681,33 @@ int features_async(cpm_ctx* c, int frames, const double* b, const double* b_prev
   return cuda_check(c, cudaGetLastError(), "features");
 }
 
+// Gradient, loss and, with adam.p, the Adam step: two launches on the context's stream.
+int grad_async(cpm_ctx* c, const float* params, const float* norm, int bf16, int64_t samples,
+               const float* feat, const float* target, float* grad, double* loss,
+               const AdamStep& adam) {
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+  const int blocks = (int)std::min<int64_t>((samples + kTs - 1) / kTs, std::max(sms, 1));
+  int st = buf_reserve(c, &c->ws_grad, (size_t)blocks * kPart * sizeof(double));
+  if (!st) st = cuda_check(c, cudaFuncSetAttribute(k_mlp_grad,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)kGradSmem), "grad smem");
+  if (st) return st;
+  (k_mlp_grad<<<blocks, kGradThreads, kGradSmem, c->stream>>>(
+       params, norm, bf16, samples, 1.0 / (double)samples, feat, target,
+       (double*)c->ws_grad.ptr),
+   note_launch());
+  (k_grad_finish<<<(kPart + 31) / 32, 32 * kFinishSlices, 0, c->stream>>>(
+       (const double*)c->ws_grad.ptr, blocks, grad, loss, adam),
+   note_launch());
+  return cuda_check(c, cudaGetLastError(), "grad");
+}
+
+AdamStep adam_step(float* params, float* m, float* v, int step, float lr) {
+  return {params, m, v, lr, 1.0f / (1.0f - powf(0.9f, (float)step)),
+          1.0f / (1.0f - powf(0.999f, (float)step))};
+}
+
 }  // namespace
 
 extern "C" {
@@ -586,16 +775,8 @@ int cpm_mlp_grad(cpm_ctx* c, const float* params, const float* norm, int bf16,
   if (samples < 1 || !dev_ok(c, params) || !dev_ok(c, norm) || !dev_ok(c, feat) ||
       !dev_ok(c, target) || !dev_ok(c, grad) || !dev_ok(c, loss))
     return set_err(c, CPM_EINVAL, "cpm_mlp_grad: samples >= 1 and device arrays");
-  int st = cuda_check(c, cudaMemsetAsync(grad, 0, kP * sizeof(float), c->stream), "grad zero");
-  if (!st) st = cuda_check(c, cudaMemsetAsync(loss, 0, sizeof(double), c->stream), "loss zero");
-  if (!st) st = cuda_check(c, cudaFuncSetAttribute(k_mlp_grad,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)kGradSmem), "grad smem");
-  if (st) return st;
-  const int64_t blocks = (samples + kB - 1) / kB;
-  (k_mlp_grad<<<(unsigned)blocks, kB, kGradSmem, c->stream>>>(
-      params, norm, bf16, samples, 1.0 / (double)samples, feat, target, grad, loss), note_launch());
-  if ((st = cuda_check(c, cudaGetLastError(), "grad"))) return st;
+  const AdamStep none = {nullptr, nullptr, nullptr, 0.f, 0.f, 0.f};
+  if (int st = grad_async(c, params, norm, bf16, samples, feat, target, grad, loss, none)) return st;
   return cuda_check(c, cudaStreamSynchronize(c->stream), "grad sync");
 }
 
@@ -604,9 +785,8 @@ int cpm_mlp_adam(cpm_ctx* c, float* params, float* m, float* v, const float* gra
   if (!c) return CPM_EINVAL;
   if (step < 1 || !dev_ok(c, params) || !dev_ok(c, m) || !dev_ok(c, v) || !dev_ok(c, grad))
     return set_err(c, CPM_EINVAL, "cpm_mlp_adam: step >= 1 and device arrays");
-  const float c1 = 1.0f / (1.0f - powf(0.9f, (float)step));
-  const float c2 = 1.0f / (1.0f - powf(0.999f, (float)step));
-  (k_adam<<<(kP + 255) / 256, 256, 0, c->stream>>>(params, m, v, grad, kP, lr, c1, c2), note_launch());
+  (k_adam<<<(kP + 255) / 256, 256, 0, c->stream>>>(adam_step(params, m, v, step, lr), grad),
+   note_launch());
   return cuda_check(c, cudaGetLastError(), "adam");
 }
 
@@ -620,21 +800,9 @@ int cpm_guess_train_step(cpm_ctx* c, float* params, const float* norm, int bf16,
       !dev_ok(c, grad) || !dev_ok(c, loss))
     return set_err(c, CPM_EINVAL,
                    "cpm_guess_train_step: samples >= 1, step >= 1 and device arrays");
-  int st = cuda_check(c, cudaMemsetAsync(grad, 0, kP * sizeof(float), c->stream), "grad zero");
-  if (!st) st = cuda_check(c, cudaMemsetAsync(loss, 0, sizeof(double), c->stream), "loss zero");
-  if (!st) st = cuda_check(c, cudaFuncSetAttribute(k_mlp_grad,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)kGradSmem), "grad smem");
+  int st = grad_async(c, params, norm, bf16, samples, feat, target, grad, loss,
+                      adam_step(params, m, v, step, lr));
   if (st) return st;
-  const int64_t blocks = (samples + kB - 1) / kB;
-  (k_mlp_grad<<<(unsigned)blocks, kB, kGradSmem, c->stream>>>(
-       params, norm, bf16, samples, 1.0 / (double)samples, feat, target, grad, loss),
-   note_launch());
-  const float c1 = 1.0f / (1.0f - powf(0.9f, (float)step));
-  const float c2 = 1.0f / (1.0f - powf(0.999f, (float)step));
-  (k_adam<<<(kP + 255) / 256, 256, 0, c->stream>>>(params, m, v, grad, kP, lr, c1, c2),
-   note_launch());
-  if ((st = cuda_check(c, cudaGetLastError(), "train step"))) return st;
   if (loss_out) {
     double l = 0.0;
     if ((st = cuda_check(c, cudaMemcpyAsync(&l, loss, sizeof(double), cudaMemcpyDeviceToHost,
