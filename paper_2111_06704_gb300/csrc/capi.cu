@@ -69,6 +69,23 @@ int buf_reserve(Ctx* c, Buf* b, size_t bytes) {
   return buf_alloc(c, b, bytes);
 }
 
+int pinned_reserve(Ctx* c, size_t bytes) {
+  if (c->pinned && c->pinned_bytes >= bytes) return CPM_OK;
+  if (c->pinned) {
+    cudaStreamSynchronize(c->stream);  // a copy into it may still be queued
+    cudaFreeHost(c->pinned);
+    c->pinned = nullptr;
+  }
+  bytes = (bytes + 4095) & ~size_t(4095);
+  if (cudaHostAlloc(&c->pinned, bytes, cudaHostAllocDefault) != cudaSuccess) {
+    cudaGetLastError();  // the caller goes on without
+    c->pinned = nullptr;
+    return CPM_ENOMEM;
+  }
+  c->pinned_bytes = bytes;
+  return CPM_OK;
+}
+
 int pointer_where(const Ctx* c, const void* p) {
   if (!p) return 0;
   cudaPointerAttributes at;
@@ -348,6 +365,8 @@ void release_workspace(Ctx* c) {
                &c->ws_out0, &c->ws_out1, &c->ws_pot, &c->ws_guess, &c->ws_feat, &c->ws_grad, &c->ws_cluster,
                &c->tc_tiles};
   for (Buf* b : ws) buf_free(c, b);
+  if (c->pinned) cudaFreeHost(c->pinned);
+  c->pinned = nullptr;
   c->tc_tiles_nt = 0;
 }
 
@@ -921,6 +940,7 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
     int it = 0;
     double rr = 0;
     SolveArgs a{1, ones, 1.0, (double*)dp.ptr, false, 1e-10, 20000, &it, &rr};
+    a.ordered = true;
     const double saved_gap = c->pgap;
     c->pgap = 0.0;
     st = pcg_solve(c, a);

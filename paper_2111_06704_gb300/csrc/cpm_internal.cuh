@@ -161,6 +161,8 @@ struct Ctx {
   std::vector<int> kv_hkl;    // the k-vector table (host), made on the first build
   std::vector<double> kv_w;
   Buf ws_solve, ws_in0, ws_in1, ws_in2, ws_out0, ws_out1, ws_pot, ws_guess, ws_feat, ws_grad;
+  void* pinned = nullptr;  // host memory the solves poll into (pinned_reserve)
+  size_t pinned_bytes = 0;
   Buf ws_cluster;  // per-column results of the cluster-resident solve
   // the solver's online autotuner: per bucket of right-hand-side counts (1, 2-3, 4-7, ..,
   // 128+), the path found faster (0 not yet known, 1 host-driven kernels, 2 cluster-
@@ -204,6 +206,7 @@ long long launch_count();
 int buf_alloc(Ctx* c, Buf* b, size_t bytes);
 void buf_free(Ctx* c, Buf* b);
 int buf_reserve(Ctx* c, Buf* b, size_t bytes);  // grow-only
+int pinned_reserve(Ctx* c, size_t bytes);  // c->pinned, grow-only; CPM_ENOMEM leaves none
 int set_err(Ctx* c, int code, const std::string& msg);
 int cuda_check(Ctx* c, cudaError_t e, const char* what);
 // Where the array at p lives: 1 in device memory of the context's device (or managed
@@ -352,6 +355,7 @@ struct SolveArgs {
   void* ws = nullptr;    // optional fixed device workspace (else the context's, grown)
   size_t ws_bytes = 0;
   const SysCol* sys = nullptr;  // ragged batch: device array [nrhs], one system per column
+  bool ordered = false;          // one column: every sum in the build's fixed order
   bool timed = true;             // record the solve's device timings (events of the context)
 };
 int pcg_solve(Ctx* c, const SolveArgs& a);

@@ -40,25 +40,120 @@ __device__ __forceinline__ double warp_sum(double x) {
   return x;
 }
 
+// The warp sums of NV values: with a power of two of them, the lanes halve the values they
+// carry at each of the first steps of the butterfly (the values a lane drops go on in its
+// partner), so NV = 4 takes 6 additions a lane instead of 20 -- FP64 additions run at 1/64
+// of the float rate here and are most of the vector kernels' work.  The pairs added, and so the sums, are the butterfly's.  On return value
+// t's sum is in every lane whose top log2(NV) bits read t from the highest.
+template <int NV>
+__device__ __forceinline__ double warp_sums(const double (&v)[NV]) {
+  static_assert(NV == 1 || NV == 2 || NV == 4, "power of two");
+  const int lane = threadIdx.x & 31;
+  double w[NV];
+#pragma unroll
+  for (int t = 0; t < NV; ++t) w[t] = v[t];
+  int o = 16;
+#pragma unroll
+  for (int n = NV / 2; n >= 1; n /= 2, o /= 2) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int t = 0; t < n; ++t) {
+      const double keep = up ? w[t + n] : w[t], give = up ? w[t] : w[t + n];
+      w[t] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  double x = w[0];
+  for (; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+// The lane that holds value t after warp_sums.
+template <int NV>
+__device__ __forceinline__ constexpr int sums_lane(int t) {
+  return t * (32 / NV);
+}
+
 // Block-wide sum of NV values per thread; result valid in thread 0.
 template <int NV>
 __device__ void block_sum(double (&v)[NV], double* sm /* [32*NV] */) {
+  constexpr int NP = NV == 3 ? 4 : NV;  // three values go as four
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double w[NP];
 #pragma unroll
-  for (int t = 0; t < NV; ++t) v[t] = warp_sum(v[t]);
-  if (lane == 0)
-#pragma unroll
-    for (int t = 0; t < NV; ++t) sm[warp * NV + t] = v[t];
+  for (int t = 0; t < NP; ++t) w[t] = t < NV ? v[t] : 0.0;
+  double x = warp_sums<NP>(w);
+  if (lane % (32 / NP) == 0 && lane / (32 / NP) < NV) sm[warp * NV + lane / (32 / NP)] = x;
   __syncthreads();
   if (warp == 0) {
     const int nw = blockDim.x >> 5;
 #pragma unroll
-    for (int t = 0; t < NV; ++t) {
-      double x = lane < nw ? sm[lane * NV + t] : 0.0;
-      v[t] = warp_sum(x);
-    }
+    for (int t = 0; t < NP; ++t) w[t] = t < NV && lane < nw ? sm[lane * NV + t] : 0.0;
+    x = warp_sums<NP>(w);
+#pragma unroll
+    for (int t = 0; t < NV; ++t) v[t] = __shfl_sync(0xffffffffu, x, sums_lane<NP>(t));
   }
   __syncthreads();
+}
+
+// The sum of v[b * stride], b < count, over a warp: lane l adds b = l, l + 32, .. in order, then
+// the butterfly; sixteen loads in flight.
+__device__ __forceinline__ double lane_sum(const double* v, int count, int64_t stride) {
+  constexpr int kAhead = 16;
+  double s = 0.0;
+  for (int b = threadIdx.x & 31; b < count; b += 32 * kAhead) {
+    double x[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      x[u] = b + 32 * u < count ? v[(int64_t)(b + 32 * u) * stride] : 0.0;
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) s += x[u];
+  }
+  return s;
+}
+
+// Device time of an iteration's matvec and DC apply without events between the kernels: the
+// first block of the kernel stamps its start, that of the kernel after it adds the span (ns).
+struct Clock {
+  unsigned long long start, sum;
+};
+
+// The kernels of an iteration are launched with programmatic stream serialisation
+// (launch_next): a kernel's blocks may be set up while the one before drains, and wait here,
+// before they touch anything, until it has completed and its writes are visible.
+__device__ __forceinline__ void wait_previous(bool set_up_next = true) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (set_up_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+void launch_next(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                 A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+  note_launch();
+}
+
+__device__ __forceinline__ unsigned long long now_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+
+__device__ __forceinline__ void clock_start(Clock* c) {
+  if (c && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) c->start = now_ns();
+}
+
+__device__ __forceinline__ void clock_stop(Clock* c) {
+  if (c && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) c->sum += now_ns() - c->start;
 }
 
 // FP64 E (the plain baseline build): q[r] = E p[r] for NR columns from c0, one warp per
@@ -67,8 +162,10 @@ template <int NR>
 __global__ void __launch_bounds__(kThreads)
 k_matvec_f64(const double* __restrict__ E, int64_t ldE, int n, const double* __restrict__ pv,
              int64_t ldv, int c0, int nrhs, double* __restrict__ q,
-             double* __restrict__ pq_part, const ColState* __restrict__ st) {
+             double* __restrict__ pq_part, const ColState* __restrict__ st, Clock* clock) {
   __shared__ double sm[32 * NR];
+  wait_previous();
+  clock_start(clock);
   c0 += blockIdx.y * NR;  // one column group per grid row
   if (st) {  // converged columns are not multiplied again (uniform per block)
     bool live = false;
@@ -145,9 +242,11 @@ __global__ void __launch_bounds__(kThreads)
 k_matvec_f32(const float* __restrict__ E, int64_t ldE, int n, const float* __restrict__ pv,
              const float* __restrict__ plo, const double* __restrict__ p64, int64_t ldv,
              int c0, int nrhs, double* __restrict__ q, double* __restrict__ pq_part,
-             const ColState* __restrict__ st) {
+             const ColState* __restrict__ st, Clock* clock) {
   constexpr int RB = kMvRows;
   constexpr int RBB = RB * (kMvWarps / WS);  // rows per block
+  wait_previous(false);
+  clock_start(clock);
   c0 += blockIdx.y * NR;  // one column group per grid row
   if (st) {  // converged columns are not multiplied again (uniform per block)
     bool live = false;
@@ -277,6 +376,7 @@ struct StreamArgs {
   double* pq_part;  // [nrb][nrhs]
   const ColState* st;
   int* err;
+  Clock* clock;
 };
 
 __global__ void __launch_bounds__(kStThreads, 1)
@@ -289,6 +389,8 @@ k_matvec_stream(const __grid_constant__ CUtensorMap emap, StreamArgs a) {
   const int grp = a.g0 + blockIdx.y, c0 = grp * kFastCols;
   const int ncol = min(kFastCols, a.nrhs - c0);
   const int rb = blockIdx.x / a.splits, sp = blockIdx.x % a.splits;
+  wait_previous(false);
+  clock_start(a.clock);
   if (a.st) {  // a group with every column converged is not multiplied (uniform per grid row)
     bool live = false;
     for (int r = 0; r < ncol; ++r) live |= a.st[c0 + r].done == 0;
@@ -416,11 +518,14 @@ k_matvec_stream(const __grid_constant__ CUtensorMap emap, StreamArgs a) {
     __threadfence();
     const double* shares = a.part + ((int64_t)blockIdx.y * gridDim.x + (int64_t)rb * a.splits) * kStOut;
 #pragma unroll
-    for (int m = 0; m < kM; ++m) {
-      const int o = tid + kStWarps * 32 * m;
-      double sum = 0.0;
-      for (int s = 0; s < a.splits; ++s) sum += __ldcg(shares + (int64_t)s * kStOut + o);
-      v[m] = sum;
+    for (int m = 0; m < kM; ++m) v[m] = 0.0;
+    for (int s = 0; s < a.splits; ++s) {  // share order; a share's loads all in flight
+      double w[kM];
+#pragma unroll
+      for (int m = 0; m < kM; ++m)
+        w[m] = __ldcg(shares + (int64_t)s * kStOut + tid + kStWarps * 32 * m);
+#pragma unroll
+      for (int m = 0; m < kM; ++m) v[m] += w[m];
     }
     if (tid == 0) *counter = 0u;
   }
@@ -486,10 +591,12 @@ __global__ void __launch_bounds__(kThreads)
 k_matvec_ragged(const SysCol* __restrict__ sys, const float* __restrict__ pv,
                 const float* __restrict__ plo, const double* __restrict__ p64, int64_t ldv,
                 int nrhs, double* __restrict__ q, double* __restrict__ pq_part,
-                const ColState* __restrict__ st) {
+                const ColState* __restrict__ st, Clock* clock) {
   constexpr int RB = kMvRows;
   __shared__ float2 sm[kMvWarps][RB];
   __shared__ double spq[RB];
+  wait_previous(false);
+  clock_start(clock);
   const int c = blockIdx.y;
   const int n = (st && st[c].done) ? 0 : sys[c].n;  // converged: only the zero partial
   const int64_t ldE = sys[c].ldE;
@@ -564,156 +671,288 @@ k_matvec_ragged(const SysCol* __restrict__ sys, const float* __restrict__ pv,
   }
 }
 
-// alpha = r^T z / p^T q for every running column.
-__global__ void k_alpha(const double* __restrict__ pq_part, int nparts, int nrhs,
-                        ColState* __restrict__ st) {
-  const int col = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (col >= nrhs) return;
-  double s = 0.0;
-  for (int b = lane; b < nparts; b += 32) s += pq_part[(int64_t)b * nrhs + col];
-  s = warp_sum(s);
-  if (lane == 0) {
-    ColState& c = st[col];
-    if (c.done) {
-      c.alpha = 0.0;
-    } else if (!(s > 0.0) || !isfinite(s)) {
-      c.alpha = 0.0;
+// The column's next state from its sums r^T z_new, r^T z_old, r^T r: convergence, beta.
+__device__ __forceinline__ ColState advance(ColState c, double rz_new, double rz_old, double rr,
+                                            double tol, int flexible) {
+  if (c.done == 0) {
+    c.iter += 1;
+    c.relres = sqrt(rr / c.bb);
+    if (!isfinite(c.relres)) {
       c.done = 2;
+    } else if (c.relres <= tol) {
+      c.done = 1;
     } else {
-      c.alpha = c.rz / s;
+      c.beta = flexible ? (rz_new - rz_old) / c.rz : rz_new / c.rz;
+      c.rz = rz_new;
+      if (!isfinite(c.beta) || !(c.rz != 0.0)) c.done = 2;
     }
   }
+  return c;
 }
 
 // x += alpha p, r -= alpha q; Jacobi/none also form z; partial dots
-// [r^T z_new, r^T z_old, r^T r, sum r].
+// [r^T z_new, r^T z_old, r^T r, sum r].  alpha = r^T z / p^T q from the matvec's nparts partials
+// of p^T q: every block of a column adds them for itself (ordered: one warp, lane l partials l,
+// l + 32, .. in order, as the many-column solves and the build's do), so no launch of its own stands between the matvec and
+// the update, and the first block records it (a last-block scheme in the matvec cost as much
+// as the launch: 3,200 blocks each waiting on a fence and an atomic, 96 -> 107 us at 12,800
+// atoms).  The scalars are FP64, at 1/64 of the float rate, so with many columns a block takes
+// several of the column's ndots partials (vector_blocks).  rt (many-column float solves): r again as floats, transposed per group of 16 columns
+// for k_dc_apply_t.
 template <int PRE>
 __global__ void __launch_bounds__(kThreads)
-k_update(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st,
+k_update(int n, int64_t ldv, int nrhs, ColState* st,
          double* __restrict__ x, double* __restrict__ r, double* __restrict__ z,
          const double* __restrict__ p, const double* __restrict__ q,
          const double* __restrict__ inv_diag, double* __restrict__ dots,
-         const SysCol* __restrict__ sys) {
+         int ndots, const SysCol* __restrict__ sys, const double* __restrict__ pq_part, int nparts,
+         bool ordered, float* __restrict__ rt, Clock* mv_clock) {
   __shared__ double sm[32 * 4];
+  __shared__ double s_alpha;
+  __shared__ int s_done;
+  wait_previous();
+  clock_stop(mv_clock);
   {
     const int col = blockIdx.y;  // one right-hand side per grid row
     if (sys) {  // ragged batch: this column's system
       n = sys[col].n;
       inv_diag = sys[col].inv_diag;
+      nparts = (n + kMvRows - 1) / kMvRows;
     }
-    const double a = st[col].alpha;
-    const bool active = st[col].done == 0;
-    if (!active) return;  // converged column: its dots are not read (uniform per block)
-    double v[4] = {0, 0, 0, 0};
+    // read once a block: the first block marks a column that breaks down here, and the others
+    // may find that mark or the breakdown itself
+    if (threadIdx.x == 0) s_done = *(volatile const int*)&st[col].done;
+    __syncthreads();
+    if (s_done != 0) return;  // converged column: its dots are not read
+    double pq[1] = {0.0};
+    if (ordered) {
+      if (threadIdx.x < 32) pq[0] = warp_sum(lane_sum(pq_part + col, nparts, nrhs));
+    } else {
+#pragma unroll 8
+      for (int b = threadIdx.x; b < nparts; b += kThreads) pq[0] += pq_part[(int64_t)b * nrhs + col];
+      block_sum<1>(pq, sm);
+    }
+    if (threadIdx.x == 0) {
+      const bool broke = !(pq[0] > 0.0) || !isfinite(pq[0]);
+      s_alpha = broke ? 0.0 : st[col].rz / pq[0];
+      if (blockIdx.x == 0) {
+        st[col].alpha = s_alpha;
+        if (broke) st[col].done = 2;
+      }
+      s_done = broke;
+    }
+    __syncthreads();
+    if (s_done) return;
+    const double a = s_alpha;
     const int64_t o = (int64_t)col * ldv;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-      double ri = r[o + i];
-      if (active) {
+    float* rc = rt ? rt + ((int64_t)(col / kFastCols) * ldv * kFastCols + col % kFastCols)
+                   : nullptr;
+    for (int vb = blockIdx.x; vb < ndots; vb += gridDim.x) {
+      double v[4] = {0, 0, 0, 0};
+      for (int i = vb * blockDim.x + threadIdx.x; i < n; i += ndots * blockDim.x) {
+        double ri = r[o + i];
         x[o + i] += a * p[o + i];
         ri -= a * q[o + i];
         r[o + i] = ri;
+        if (rc) rc[(int64_t)i * kFastCols] = (float)ri;
+        if (PRE != CPM_PRECOND_DC) {
+          const double zo = z[o + i];
+          const double zn = PRE == CPM_PRECOND_JACOBI ? ri * inv_diag[i] : ri;
+          z[o + i] = zn;
+          v[0] += ri * zn;
+          v[1] += ri * zo;
+        }
+        v[2] += ri * ri;
+        v[3] += ri;
       }
-      if (PRE != CPM_PRECOND_DC) {
-        const double zo = z[o + i];
-        const double zn = PRE == CPM_PRECOND_JACOBI ? ri * inv_diag[i] : ri;
-        if (active) z[o + i] = zn;
-        v[0] += ri * zn;
-        v[1] += ri * zo;
-      }
-      v[2] += ri * ri;
-      v[3] += ri;
+      block_sum<4>(v, sm);
+      if (threadIdx.x == 0)
+        for (int t = 0; t < 4; ++t) dots[((int64_t)vb * nrhs + col) * 4 + t] = v[t];
     }
-    block_sum<4>(v, sm);
-    if (threadIdx.x == 0)
-      for (int t = 0; t < 4; ++t) dots[((int64_t)blockIdx.x * nrhs + col) * 4 + t] = v[t];
   }
 }
 
-// z = P r (+ p_gap * sum r on the complement of the pattern) for PCG-DC, one thread per
-// row; partial dots [r^T z_new, r^T z_old] into slots 0, 1.  rsum_part may be the dots
-// buffer itself: the kernel only reads its slot 3 and only writes slots 0 and 1.
+// z = P r (+ p_gap * sum r on the complement of the pattern) for PCG-DC, LR lanes a row
+// (neighbouring entries of a row, so its loads coalesce; one thread a row walked ~100 entries
+// in a chain of dependent, scattered loads: 15.2 us at 12,800 atoms against 7.4 with eight
+// lanes, 16.5 us at 512 against 4.3 with a warp); a block's partial dots [r^T z_new, r^T z_old]
+// go to wpart[column][ldv] at 2 block.  dots: of the solver's the kernel reads slot 3, the sum
+// r.  first: every column.
+template <int LR>
 __global__ void __launch_bounds__(kThreads)
 k_dc_apply(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st,
            const int64_t* __restrict__ off, const int* __restrict__ idx,
            const double* __restrict__ prow, double pgap, const double* __restrict__ r,
-           double* __restrict__ z, const double* __restrict__ rsum_part, int nparts,
-           double* __restrict__ dots, int first, const SysCol* __restrict__ sys) {
+           double* __restrict__ z, const double* __restrict__ dots, int nparts,
+           double* __restrict__ wpart, int first, const SysCol* __restrict__ sys, Clock* clock) {
   __shared__ double sm[32 * 2];
   __shared__ double s_rsum;
-  {
-    const int col = blockIdx.y;
-    if (sys) {  // ragged batch: this column's system
-      n = sys[col].n;
-      off = sys[col].nbr_off;
-      idx = sys[col].nbr_idx;
-      prow = sys[col].prow;
-      pgap = sys[col].pgap;
+  wait_previous();
+  clock_start(clock);
+  const int col = blockIdx.y;
+  if (sys) {  // ragged batch: this column's system
+    n = sys[col].n;
+    off = sys[col].nbr_off;
+    idx = sys[col].nbr_idx;
+    prow = sys[col].prow;
+    pgap = sys[col].pgap;
+  }
+  if (!first && st[col].done != 0) return;  // converged column (uniform per block)
+  if (threadIdx.x < 32) {
+    double s = 0.0;
+    if (pgap != 0.0) s = warp_sum(lane_sum(dots + (int64_t)col * 4 + 3, nparts, (int64_t)nrhs * 4));
+    if (threadIdx.x == 0) s_rsum = s;
+  }
+  const int64_t o = (int64_t)col * ldv;
+  const int sub = threadIdx.x % LR;
+  constexpr int kRows = kThreads / LR, kAhead = 4;  // entries a lane loads at once
+  double v[2] = {0, 0};
+  for (int j0 = blockIdx.x * kRows; j0 < n; j0 += gridDim.x * kRows) {
+    const int j = j0 + threadIdx.x / LR;
+    double acc = 0.0, rj = 0.0, zo = 0.0;
+    if (j < n) {
+      const int64_t e1 = off[j + 1];
+      if (sub == 0) {
+        rj = r[o + j];
+        zo = z[o + j];
+      }
+      for (int64_t e = off[j] + sub; e < e1; e += LR * kAhead) {
+        int id[kAhead];
+        double pe[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+          const bool in = e + u * LR < e1;
+          id[u] = in ? __ldg(idx + e + u * LR) : j;
+          pe[u] = in ? __ldg(prow + e + u * LR) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u)
+          if (e + u * LR < e1) acc += pe[u] * r[o + id[u]];
+      }
     }
-    const bool active = first || st[col].done == 0;
-    if (!active) return;  // converged column (uniform per block)
-    if (threadIdx.x < 32) {
-      double s = 0.0;
-      if (pgap != 0.0)
-        for (int b = threadIdx.x; b < nparts; b += 32) s += rsum_part[((int64_t)b * nrhs + col) * 4 + 3];
-      s = warp_sum(s);
-      if (threadIdx.x == 0) s_rsum = s;
-    }
-    __syncthreads();
-    const double gsum = pgap * s_rsum;
-    const int64_t o = (int64_t)col * ldv;
-    double v[2] = {0, 0};
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-      double acc = gsum;
-      for (int64_t e = off[j]; e < off[j + 1]; ++e) acc += prow[e] * r[o + idx[e]];
-      const double rj = r[o + j];
-      const double zo = z[o + j];
-      if (active) z[o + j] = acc;
+#pragma unroll
+    for (int w = LR / 2; w; w >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, w);
+    if (j0 == blockIdx.x * kRows) __syncthreads();  // s_rsum (every thread's first pass)
+    if (sub == 0 && j < n) {
+      acc += pgap * s_rsum;
+      z[o + j] = acc;
       v[0] += rj * acc;
       v[1] += rj * zo;
     }
-    block_sum<2>(v, sm);
-    if (threadIdx.x == 0) {
-      dots[((int64_t)blockIdx.x * nrhs + col) * 4 + 0] = v[0];
-      dots[((int64_t)blockIdx.x * nrhs + col) * 4 + 1] = v[1];
-    }
+  }
+  block_sum<2>(v, sm);
+  if (threadIdx.x == 0) {
+    wpart[o + 2 * blockIdx.x] = v[0];
+    wpart[o + 2 * blockIdx.x + 1] = v[1];
   }
 }
 
-// Reduce the dots, test convergence, form beta, and advance the column state.
-__global__ void k_beta(const double* __restrict__ dots, int nparts, int nrhs, double tol,
-                       int flexible, const ColState* __restrict__ cur,
-                       ColState* __restrict__ next) {
-  const int col = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (col >= nrhs) return;
-  double s[3] = {0, 0, 0};
-  for (int b = lane; b < nparts; b += 32)
-    for (int t = 0; t < 3; ++t) s[t] += dots[((int64_t)b * nrhs + col) * 4 + t];
-  for (int t = 0; t < 3; ++t) s[t] = warp_sum(s[t]);
-  if (lane == 0) {
-    ColState c = cur[col];
-    if (c.done == 0) {
-      c.iter += 1;
-      c.relres = sqrt(s[2] / c.bb);
-      if (!isfinite(c.relres)) {
-        c.done = 2;
-      } else if (c.relres <= tol) {
-        c.done = 1;
-      } else {
-        c.beta = flexible ? (s[0] - s[1]) / c.rz : s[0] / c.rz;
-        c.rz = s[0];
-        if (!isfinite(c.beta) || !(c.rz != 0.0)) c.done = 2;
+// The same with each row's entries added in their order and the dots in that of 256-row blocks:
+// the build's solve for d (SolveArgs::ordered).  d and p_gap enter every later solve, and a
+// many-column solve, whose float matvec rounds at 1e-7, turns a change of p_gap's last bits
+// into 2e-9 of its charges; with its sums in one fixed order the build repeats to the last bit
+// whatever the per-column kernel above does.  32 rows a block: the eight warps load the rows'
+// entries and the residuals they meet, coalesced, into shared memory, and one warp adds each
+// row's, a row a lane.  wpart[column][ldv] at 2 block; eight blocks make one of the solver's
+// partials (group_dot).
+constexpr int kOrdCols = 128;  // entries of a row a chunk holds
+constexpr size_t kOrdSmem = sizeof(double2) * kOrdCols * 33;
+
+__global__ void __launch_bounds__(kThreads)
+k_dc_apply_ordered(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st,
+                   const int64_t* __restrict__ off, const int* __restrict__ idx,
+                   const double* __restrict__ prow, double pgap, const double* __restrict__ r,
+                   double* __restrict__ z, const double* __restrict__ dots, int nparts,
+                   double* __restrict__ wpart, int first, Clock* clock) {
+  extern __shared__ double2 s_e[];  // [kOrdCols][33]: (P entry, r there), a row a column of it
+  __shared__ int64_t s_off[33];
+  wait_previous();
+  clock_start(clock);
+  const int col = blockIdx.y;
+  if (!first && st[col].done != 0) return;  // converged column (uniform per block)
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t o = (int64_t)col * ldv;
+  double gsum = 0.0, v[2] = {0.0, 0.0};
+  if (warp == 0 && pgap != 0.0)
+    gsum = pgap * warp_sum(lane_sum(dots + (int64_t)col * 4 + 3, nparts, (int64_t)nrhs * 4));
+  for (int j0 = blockIdx.x * 32; j0 < n; j0 += gridDim.x * 32) {
+    const int j = j0 + lane;
+    __syncthreads();  // the last rows' reads of s_off
+    if (threadIdx.x < 33) s_off[threadIdx.x] = off[min(n, j0 + (int)threadIdx.x)];
+    double rj = 0.0, zo = 0.0, acc = gsum;
+    if (warp == 0 && j < n) {
+      rj = r[o + j];
+      zo = z[o + j];
+    }
+    __syncthreads();
+    const int mine = (int)(s_off[lane + 1] - s_off[lane]);
+    const int most = __reduce_max_sync(0xffffffffu, mine);
+    for (int e0 = 0; e0 < most; e0 += kOrdCols) {
+      int id[16];
+      double pe[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {  // row 4 warp + u / 4, entries 32 (u % 4) + lane of the chunk
+        const int row = 4 * warp + (u >> 2);
+        const int64_t e = s_off[row] + e0 + 32 * (u & 3) + lane;
+        const bool in = e < s_off[row + 1];
+        id[u] = in ? __ldg(idx + e) : -1;
+        pe[u] = in ? __ldg(prow + e) : 0.0;
       }
+#pragma unroll
+      for (int u = 0; u < 16; ++u)
+        if (id[u] >= 0)
+          s_e[(32 * (u & 3) + lane) * 33 + 4 * warp + (u >> 2)] =
+              make_double2(pe[u], r[o + id[u]]);
+      __syncthreads();
+      if (warp == 0) {
+        const int cnt = min(kOrdCols, mine - e0);
+#pragma unroll 8
+        for (int e = 0; e < cnt; ++e) {
+          const double2 t = s_e[e * 33 + lane];
+          acc = fma(t.x, t.y, acc);
+        }
+      }
+      __syncthreads();
     }
-    next[col] = c;
+    if (warp == 0 && j < n) {
+      z[o + j] = acc;
+      v[0] = fma(rj, acc, v[0]);
+      v[1] = fma(rj, zo, v[1]);
+    }
   }
+  if (warp != 0) return;
+  const double x = warp_sums<2>(v);
+  if (lane % 16 == 0) wpart[o + 2 * blockIdx.x + lane / 16] = x;
 }
 
-// p = z + beta p, and the matvec's copy: the value itself in FP64 storage, a float
-// pair hi + lo (plo != nullptr) in float storage.
-// first = 2: only the columns whose residual replacement reopened them (restart flag),
-// which start again from p = z.  xt (float storage, many-column solves): the directions
+// Partial t of 256 rows' dots from k_dc_apply_ordered's eight blocks of 32, as block_sum adds
+// warps.
+__device__ __forceinline__ double group_dot(const double* w, int part, int t) {
+  const double* p = w + 16 * (int64_t)part + t;
+  return ((p[0] + p[8]) + (p[4] + p[12])) + ((p[2] + p[10]) + (p[6] + p[14]));
+}
+
+// The partials of r^T z_new (t = 0) and r^T z_old (t = 1): partial b of column c at
+// p[c * col + b * stride + t], or, grouped, the group_dot of eight.
+struct DotParts {
+  const double* p;
+  int64_t col, stride;
+  int count;
+  bool grouped;
+
+  __device__ __forceinline__ double lanes(int c, int t) const {
+    const double* w = p + c * col;
+    if (!grouped) return lane_sum(w + t, count, stride);
+    double s = 0.0;
+#pragma unroll 2
+    for (int b = threadIdx.x & 31; b < count; b += 32) s += group_dot(w, b, t);
+    return s;
+  }
+};
+
+// p = z, and the matvec's copy: the value itself in FP64 storage, a float pair hi + lo
+// (plo != nullptr) in float storage.  first = 1: every column; 2: only the columns whose
+// residual replacement reopened them (restart flag), which start again.  xt (float storage, many-column solves): the directions
 // again, transposed per group of 16 columns, [group][row][16], for k_matvec_stream.
 template <typename T>
 __global__ void k_p_update(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st,
@@ -723,19 +962,67 @@ __global__ void k_p_update(int n, int64_t ldv, int nrhs, const ColState* __restr
   {
     const int col = blockIdx.y;
     if (first == 2 && !st[col].restart) return;
-    if (first == 0 && st[col].done) return;
-    const double bta = first ? 0.0 : st[col].beta;
     const int64_t o = (int64_t)col * ldv;
     float* xc = xt ? xt + ((int64_t)(col / kFastCols) * ldv * kFastCols + col % kFastCols)
                    : nullptr;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-      const double v = z[o + i] + bta * p[o + i];
+      const double v = z[o + i];
       p[o + i] = v;
       const T hi = (T)v;
       pv[o + i] = hi;
       if (plo) plo[o + i] = (T)(v - (double)hi);
       if (xc) xc[(int64_t)i * kFastCols] = (float)v;
     }
+  }
+}
+
+// The end of an iteration: the column's next state from its sums, then p = z + beta p as
+// k_p_update.  Every block of a column adds the sums for itself, three warps in lane order, and
+// the first writes the state (no launch of its own for them).  r^T r is slot 2 of dots[nparts][nrhs][4].
+struct StepArgs {
+  const double* dots;
+  int nparts;
+  DotParts rz;
+  double tol;
+  int flexible;
+  const ColState* cur;
+  ColState* next;
+  Clock* dc_clock;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads)
+k_step(int n, int64_t ldv, int nrhs, const StepArgs a, const double* __restrict__ z,
+       double* __restrict__ p, T* __restrict__ pv, T* __restrict__ plo, float* __restrict__ xt) {
+  __shared__ ColState s_next;
+  __shared__ double s_sum[3];
+  wait_previous();
+  clock_stop(a.dc_clock);
+  const int col = blockIdx.y;
+  const int warp = threadIdx.x >> 5;
+  if (warp < 3 && a.cur[col].done == 0) {
+    const double v = warp_sum(
+        warp == 2 ? lane_sum(a.dots + (int64_t)col * 4 + 2, a.nparts, (int64_t)nrhs * 4)
+                  : a.rz.lanes(col, warp));
+    if ((threadIdx.x & 31) == 0) s_sum[warp] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_next = advance(a.cur[col], s_sum[0], s_sum[1], s_sum[2], a.tol, a.flexible);
+    if (blockIdx.x == 0) a.next[col] = s_next;
+  }
+  __syncthreads();
+  if (s_next.done) return;
+  const double bta = s_next.beta;
+  const int64_t o = (int64_t)col * ldv;
+  float* xc = xt ? xt + ((int64_t)(col / kFastCols) * ldv * kFastCols + col % kFastCols) : nullptr;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const double v = z[o + i] + bta * p[o + i];
+    p[o + i] = v;
+    const T hi = (T)v;
+    pv[o + i] = hi;
+    if (plo) plo[o + i] = (T)(v - (double)hi);
+    if (xc) xc[(int64_t)i * kFastCols] = (float)v;
   }
 }
 
@@ -781,19 +1068,29 @@ constexpr int kDcRowsPerWarp = 8;
 constexpr int kDcRowsPerBlock = kDcWarps * kDcRowsPerWarp;
 constexpr int kDcChunk = 128;  // entries loaded at once
 
-__global__ void __launch_bounds__(kDcWarps * 32, 3)
+// RW rows a warp: a block's 64 rows go to 8 warps of 8 rows each, or, where the blocks do not fill
+// the chip (512 rows, 16 groups: 128 blocks, 16.5 against 11.8 us), to 32 warps of 2; the block dots are
+// added as eight groups of eight rows either way.
+template <int RW>
+__global__ void __launch_bounds__(kDcRowsPerBlock / RW * 32, RW == kDcRowsPerWarp ? 3 : 1)
 k_dc_apply_t(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st,
              const int64_t* __restrict__ off, const int* __restrict__ idx,
              const double* __restrict__ prow, double pgap, const float* __restrict__ rt,
              const double* __restrict__ r, double* __restrict__ z,
              const double* __restrict__ rsum_part, int nparts, double* __restrict__ dpart,
-             int first) {
+             int first, Clock* clock) {
+  wait_previous();
+  clock_start(clock);
   __shared__ double s_gsum[kFastCols];
   __shared__ int s_active[kFastCols];
   __shared__ double s_red[kDcWarps][kFastCols][2];
+  // r, z_new, z_old of every row, where a group's rows are spread over warps
+  constexpr bool kSpread = RW != kDcRowsPerWarp;
+  constexpr int kWarps = kDcRowsPerBlock / RW;
+  __shared__ double s_row[kSpread ? kDcRowsPerBlock : 1][kFastCols][3];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int grp = blockIdx.y, c0 = grp * kFastCols;
-  for (int cc = warp; cc < kFastCols; cc += kDcWarps) {  // p_gap sums and active flags
+  for (int cc = warp; cc < kFastCols; cc += kWarps) {  // p_gap sums and active flags
     const int col = c0 + cc;
     double sr = 0.0;
     if (col < nrhs && pgap != 0.0)
@@ -805,6 +1102,9 @@ k_dc_apply_t(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st,
     }
   }
   __syncthreads();
+  bool live = false;  // a group with every column converged: its dots are not read
+  for (int cc = 0; cc < kFastCols; ++cc) live |= s_active[cc] != 0;
+  if (!live) return;
   const int slot = lane >> 2, cq = 4 * (lane & 3);
   // after the shuffles every lane holds its four columns' sums; lane l < 16 finishes
   // column c = 4 (l % 4) + l / 4, component l / 4 of its float4
@@ -814,9 +1114,9 @@ k_dc_apply_t(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st,
   const double gsum = fin ? s_gsum[cf] : 0.0;
   const int64_t oz = (int64_t)(c0 + cf) * ldv;
   const float* rg = rt + (int64_t)grp * ldv * kFastCols + cq;
-  const int jw = blockIdx.x * kDcRowsPerBlock + warp * kDcRowsPerWarp;
+  const int jw = blockIdx.x * kDcRowsPerBlock + warp * RW;
   double v0 = 0.0, v1 = 0.0;
-  for (int j = jw; j < min(n, jw + kDcRowsPerWarp); ++j) {
+  for (int j = jw; j < min(n, jw + RW); ++j) {
     double rj = 0.0, zo = 0.0;
     if (fin) {  // issued ahead of the gathers
       rj = r[oz + j];
@@ -859,11 +1159,32 @@ k_dc_apply_t(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st,
       const float a = comp == 0 ? acc.x : comp == 1 ? acc.y : comp == 2 ? acc.z : acc.w;
       const double zn = gsum + (double)a;
       if (act) z[oz + j] = zn;
-      v0 += rj * zn;
-      v1 += rj * zo;
+      if constexpr (kSpread) {
+        double* e = s_row[j - blockIdx.x * kDcRowsPerBlock][cf];
+        e[0] = rj;
+        e[1] = zn;
+        e[2] = zo;
+      } else {
+        v0 = fma(rj, zn, v0);
+        v1 = fma(rj, zo, v1);
+      }
     }
   }
-  if (lane < 16) {
+  if constexpr (kSpread) {
+    __syncthreads();
+    if (threadIdx.x < kDcWarps * kFastCols) {  // a group of eight rows and a column a thread
+      const int g = threadIdx.x / kFastCols, cc = threadIdx.x % kFastCols;
+      const int rows = min(kDcRowsPerWarp, n - (int)blockIdx.x * kDcRowsPerBlock - g * kDcRowsPerWarp);
+      if (c0 + cc < nrhs)
+        for (int u = 0; u < rows; ++u) {
+          const double* e = s_row[g * kDcRowsPerWarp + u][cc];
+          v0 = fma(e[0], e[1], v0);
+          v1 = fma(e[0], e[2], v1);
+        }
+      s_red[g][cc][0] = v0;
+      s_red[g][cc][1] = v1;
+    }
+  } else if (lane < 16) {
     s_red[warp][cf][0] = v0;
     s_red[warp][cf][1] = v1;
   }
@@ -965,18 +1286,14 @@ k_replace_r(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st,
 // column that had converged on its recursive residual but not on the true one runs again
 // from p = z (restart flag); every running column continues with the replaced r, z and
 // r^T z and its direction unchanged.
-__global__ void k_replace_state(const double* __restrict__ dots, int nparts, int nrhs,
-                                double tol, ColState* __restrict__ st) {
+// r^T r is slot 2 of dots[nparts][nrhs][4].
+__global__ void k_replace_state(const double* __restrict__ dots, int nparts, const DotParts rz,
+                                int nrhs, double tol, ColState* __restrict__ st) {
   const int col = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (col >= nrhs) return;
-  double s0 = 0.0, s2 = 0.0;
-  for (int b = lane; b < nparts; b += 32) {
-    s0 += dots[((int64_t)b * nrhs + col) * 4 + 0];
-    s2 += dots[((int64_t)b * nrhs + col) * 4 + 2];
-  }
-  s0 = warp_sum(s0);
-  s2 = warp_sum(s2);
+  const double s0 = warp_sum(rz.lanes(col, 0));
+  const double s2 = warp_sum(lane_sum(dots + (int64_t)col * 4 + 2, nparts, (int64_t)nrhs * 4));
   if (lane == 0) {
     ColState c = st[col];
     if (c.done != 2) {
@@ -1068,16 +1385,12 @@ __global__ void k_init_state(const double* __restrict__ dots, int nparts, int nr
   }
 }
 
-// The DC apply in the init phase writes r^T z into slot 0 of its own dots array.
-__global__ void k_init_rz_dc(const double* __restrict__ dots_dc, int nparts, int nrhs,
-                             ColState* __restrict__ st) {
+// r^T z of the first DC apply.
+__global__ void k_init_rz_dc(const DotParts rz, int nrhs, ColState* __restrict__ st) {
   const int col = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
   if (col >= nrhs) return;
-  double s = 0.0;
-  for (int b = lane; b < nparts; b += 32) s += dots_dc[((int64_t)b * nrhs + col) * 4];
-  s = warp_sum(s);
-  if (lane == 0) st[col].rz = s;
+  const double s = warp_sum(rz.lanes(col, 0));
+  if ((threadIdx.x & 31) == 0) st[col].rz = s;
 }
 
 __global__ void k_neutralize(double* __restrict__ q, int n, const double* __restrict__ d,
@@ -1144,7 +1457,7 @@ int matvec_parts(const Ctx* c) {
 template <typename T>
 void launch_matvec(const Ctx* c, const void* pv, const void* plo, const double* p64,
                    int64_t ldv, int nrhs, double* q, double* pq_part, int gm,
-                   const ColState* st);
+                   const ColState* st, Clock* clock);
 
 // Launches KERNEL<NR> over all nrhs columns: full groups of four columns as grid rows of
 // one launch, then a pair and a single column for the remainder.
@@ -1165,12 +1478,12 @@ void for_column_groups(int nrhs, Launch&& launch) {
 template <>
 void launch_matvec<double>(const Ctx* c, const void* pv, const void*, const double*,
                            int64_t ldv, int nrhs, double* q, double* pq_part, int gm,
-                           const ColState* st) {
+                           const ColState* st, Clock* clock) {
   const double* E = (const double*)c->E.ptr;
   const double* hi = (const double*)pv;
   for_column_groups(nrhs, [&](auto nr, int c0, int ny) {
-    (k_matvec_f64<decltype(nr)::value><<<dim3(gm, ny), kThreads, 0, c->stream>>>(
-         E, c->ldE, c->n, hi, ldv, c0, nrhs, q, pq_part, st), note_launch());
+    launch_next(k_matvec_f64<decltype(nr)::value>, dim3(gm, ny), kThreads, 0, c->stream, E, c->ldE,
+                c->n, hi, ldv, c0, nrhs, q, pq_part, st, c0 == 0 ? clock : nullptr);
   });
 }
 
@@ -1178,19 +1491,16 @@ void launch_matvec<double>(const Ctx* c, const void* pv, const void*, const doub
 template <>
 void launch_matvec<float>(const Ctx* c, const void* pv, const void* plo, const double* p64,
                           int64_t ldv, int nrhs, double* q, double* pq_part, int gm,
-                          const ColState* st) {
+                          const ColState* st, Clock* clock) {
   const float* E = (const float*)c->E.ptr;
   const float* hi = (const float*)pv;
   const float* lo = (const float*)plo;
   const bool split = mv_split_rows(c);
   for_column_groups(nrhs, [&](auto nr, int c0, int ny) {
     constexpr int NR = decltype(nr)::value;
-    if (split)
-      (k_matvec_f32<NR, kMvWarps><<<dim3(gm, ny), kThreads, 0, c->stream>>>(
-           E, c->ldE, c->n, hi, lo, p64, ldv, c0, nrhs, q, pq_part, st), note_launch());
-    else
-      (k_matvec_f32<NR, 1><<<dim3(gm, ny), kThreads, 0, c->stream>>>(
-           E, c->ldE, c->n, hi, lo, p64, ldv, c0, nrhs, q, pq_part, st), note_launch());
+    launch_next(split ? k_matvec_f32<NR, kMvWarps> : k_matvec_f32<NR, 1>, dim3(gm, ny), kThreads, 0,
+                c->stream, E, c->ldE, c->n, hi, lo, p64, ldv, c0, nrhs, q, pq_part, st,
+                c0 == 0 ? clock : nullptr);
   });
 }
 
@@ -1252,6 +1562,10 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
   // elementwise kernels: ge blocks per right-hand side, one grid row per right-hand side
   const int ge = std::max(1, std::min((n + kThreads - 1) / kThreads, 2 * sms));
   const dim3 g2(ge, nrhs);
+  // the iteration's vector kernels, which start with a column's scalars: about four blocks an SM
+  // over all columns (26,600 rows, 16 columns: 18.8 and 17.3 us with 105 blocks a column, 16.3
+  // and 10.6 with 38)
+  const dim3 gv(std::min(ge, std::max(1, (4 * sms + nrhs - 1) / nrhs)), nrhs);
   // p^T q partials per column: one per matvec block (the ragged kernel takes kMvRows rows
   // per block)
   const int gm_exact = a.sys ? (n + kMvRows - 1) / kMvRows : matvec_parts(c);
@@ -1280,6 +1594,12 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
   const int splits = fast ? stream_splits(gm_fast, glaunch, nst, sms) : 1;
   const size_t cnt_bytes = (size_t)glaunch * gm_fast * sizeof(unsigned);
   const int nblk_dc = (n + kDcRowsPerBlock - 1) / kDcRowsPerBlock;  // blocks of the DC apply
+  const bool dc_spread = (int64_t)nblk_dc * groups <= sms;
+  // the per-column DC apply: a warp a row while eight blocks an SM hold the rows so, else eight
+  // lanes (a ragged batch by its largest system)
+  const bool dc_warp = (int64_t)nrhs * n * 32 <= 8 * (int64_t)kThreads * sms;
+  const int dc_rows = kThreads / (dc_warp ? 32 : 8);
+  const int nz = a.ordered ? 8 * ge : std::min((n + dc_rows - 1) / dc_rows, 512);
   // layout: x r z p q (double) | pv (storage type) | [fast: xt | x hi | x lo | x - x_a |
   //         x_a | r_a | unit partials | counters, error flag] | pq_part | dots | dots_dc |
   //         states
@@ -1300,6 +1620,7 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
                            : 0,
                ocnt = fast ? take(cnt_bytes + sizeof(int)) : 0,
                odp = fast ? take((size_t)nblk_dc * nrhs * 2 * sizeof(double)) : 0,
+               ock = a.ws ? 0 : take(2 * sizeof(Clock)),
                opq = take((size_t)std::max(gm_fast, gm_exact) * nrhs * sizeof(double)),
                odt = take((size_t)ge * nrhs * 4 * sizeof(double)),
                odc = take((size_t)ge * nrhs * 4 * sizeof(double)),
@@ -1335,6 +1656,14 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
   double* xa = fast ? (double*)(base + oxa) : nullptr;  // the anchor's x and r
   double* ra = fast ? (double*)(base + ora) : nullptr;
   double* dpart = fast ? (double*)(base + odp) : nullptr;  // the DC apply's block dots
+  // the per-column DC apply's partials (2 nz <= ldv doubles a column) go where q is: nothing
+  // reads q between the update, which ends its use, and the next matvec
+  double* wpart = q;
+  const DotParts rz_col = {wpart, ldv, 2, a.ordered ? ge : nz, a.ordered};
+  const DotParts rz_dots = {dots, 4, 4 * (int64_t)nrhs, ge, false};
+  // device time of the iterations' matvecs and DC applies (not in the fixed workspace)
+  Clock* mv_clock = a.ws ? nullptr : (Clock*)(base + ock);
+  Clock* dc_clock = a.ws ? nullptr : mv_clock + 1;
   cudaStream_t s = c->stream;
   // the streamed matvec: its TMA map of E, units' partials and counters (zeroed above)
   CUtensorMap emap;
@@ -1349,14 +1678,17 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
                    "streamed matvec smem"))
       return CPM_ECUDA;
   }
-  auto stream_mv = [&](const float* xin, const ColState* cur) {
+  if (a.ordered && cuda_check(c, cudaFuncSetAttribute(k_dc_apply_ordered,
+                                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      (int)kOrdSmem), "ordered DC apply smem"))
+    return CPM_ECUDA;
+  auto stream_mv = [&](const float* xin, const ColState* cur, Clock* clock) {
     StreamArgs sa{n, nst, splits, gm_fast, xin, p, ldv, 0, nrhs, part, counts, q, pq_part, cur,
-                  mv_err};
+                  mv_err, clock};
     for (int g0 = 0; g0 < groups; g0 += 65535) {
       sa.g0 = g0;
-      (k_matvec_stream<<<dim3(gm_fast * splits, std::min(groups - g0, 65535)), kStThreads,
-                         kStSmem, s>>>(emap, sa),
-       note_launch());
+      launch_next(k_matvec_stream, dim3(gm_fast * splits, std::min(groups - g0, 65535)), kStThreads,
+                  kStSmem, s, emap, sa);
     }
   };
   // device timing of the solve's parts: event pairs from the context's pool
@@ -1372,40 +1704,47 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
     cudaEventRecord(e, c->stream);
     return e;
   };
-  std::vector<std::pair<cudaEvent_t, cudaEvent_t>> t_mv, t_rep, t_dc;
+  std::vector<std::pair<cudaEvent_t, cudaEvent_t>> t_rep, t_dc;
   const cudaEvent_t t_begin = ev();
-  // cur: the column states (converged columns are skipped), nullptr before they exist
-  // z = P r for PCG-DC: the many-column float path in one pass over P for each group of
-  // 16 columns (r first transposed to floats into the x - x_a buffer, free at this point),
-  // every other solve per column
-  auto dc_apply = [&](const ColState* cur, double* dots_out, int first) {
+  // z = P r for PCG-DC (r as floats in xdt for the many-column float path)
+  auto dc_launch = [&](const ColState* cur, int first, Clock* clock) {
+    const int64_t* off = (const int64_t*)c->nbr_off.ptr;
+    const int* idx = (const int*)c->nbr_idx.ptr;
+    const double* prow = (const double*)c->prow.ptr;
+    if (fast)
+      launch_next(dc_spread ? k_dc_apply_t<2> : k_dc_apply_t<kDcRowsPerWarp>, dim3(nblk_dc, groups),
+                  dc_spread ? 1024 : kDcWarps * 32, 0, s, n, ldv, nrhs, cur, off, idx, prow, c->pgap,
+                  xdt, r, z, dots, ge, dpart, first, clock);
+    else if (a.ordered)
+      launch_next(k_dc_apply_ordered, dim3(nz, nrhs), kThreads, kOrdSmem, s, n, ldv, nrhs, cur, off,
+                  idx, prow, c->pgap, r, z, dots, ge, wpart, first, clock);
+    else
+      launch_next(dc_warp ? k_dc_apply<32> : k_dc_apply<8>, dim3(nz, nrhs), kThreads, 0, s, n, ldv,
+                  nrhs, cur, off, idx, prow, c->pgap, r, z, dots, ge, wpart, first, a.sys, clock);
+  };
+  auto dc_dots = [&](double* dots_out) {
+    (k_dc_dots<<<(nrhs + 7) / 8, 256, 0, s>>>(dpart, nblk_dc, nrhs, dots_out, ge), note_launch());
+  };
+  // outside the iteration, for every column: the many-column float path transposes r to floats
+  // first (into the x - x_a buffer, free at this point) and leaves r^T z in slot 0 of dots_out
+  auto dc_apply = [&](const ColState* cur, double* dots_out) {
     const cudaEvent_t d0 = ev();
-    if (fast) {
-      (k_diff_t<<<g2, kThreads, 0, s>>>(n, ldv, r, nullptr, xdt), note_launch());
-      (k_dc_apply_t<<<dim3(nblk_dc, groups), kDcWarps * 32, 0, s>>>(
-           n, ldv, nrhs, cur, (const int64_t*)c->nbr_off.ptr, (const int*)c->nbr_idx.ptr,
-           (const double*)c->prow.ptr, c->pgap, xdt, r, z, dots, ge, dpart, first),
-       note_launch());
-      (k_dc_dots<<<(nrhs + 7) / 8, 256, 0, s>>>(dpart, nblk_dc, nrhs, dots_out, ge),
-       note_launch());
-    } else {
-      (k_dc_apply<<<g2, kThreads, 0, s>>>(n, ldv, nrhs, cur, (const int64_t*)c->nbr_off.ptr,
-                                         (const int*)c->nbr_idx.ptr, (const double*)c->prow.ptr,
-                                         c->pgap, r, z, dots, ge, dots_out, first, a.sys),
-       note_launch());
-    }
+    if (fast) (k_diff_t<<<g2, kThreads, 0, s>>>(n, ldv, r, nullptr, xdt), note_launch());
+    dc_launch(cur, 1, nullptr);
+    if (fast) dc_dots(dots_out);
     t_dc.emplace_back(d0, ev());
   };
-  auto matvec = [&](const ColState* cur) {
+  // cur: the column states (converged columns are skipped), nullptr before they exist
+  auto matvec = [&](const ColState* cur, Clock* clock) {
     if (fast) {  // the inner matvec of a many-column solve
-      stream_mv(xt, cur);
+      stream_mv(xt, cur, clock);
     } else if (f64) {
-      launch_matvec<double>(c, pv, nullptr, p, ldv, nrhs, q, pq_part, gm, cur);
+      launch_matvec<double>(c, pv, nullptr, p, ldv, nrhs, q, pq_part, gm, cur, clock);
     } else if (a.sys) {  // ragged batch: one system per column
-      (k_matvec_ragged<<<dim3(gm, nrhs), kThreads, 0, s>>>(a.sys, (const float*)pv, plo, p, ldv,
-                                                           nrhs, q, pq_part, cur), note_launch());
+      launch_next(k_matvec_ragged, dim3(gm, nrhs), kThreads, 0, s, a.sys, (const float*)pv, plo, p,
+                  ldv, nrhs, q, pq_part, cur, clock);
     } else {
-      launch_matvec<float>(c, pv, plo, p, ldv, nrhs, q, pq_part, gm, cur);
+      launch_matvec<float>(c, pv, plo, p, ldv, nrhs, q, pq_part, gm, cur, clock);
     }
   };
   // zero the padded vectors so the matvec can read whole padded rows
@@ -1419,8 +1758,7 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
     if (cuda_check(c, copy_cols(x, ldv, a.x, n, n, nrhs, s), "copy guess")) return CPM_ECUDA;
     if (f64) (k_p_update<double><<<g2, kThreads, 0, s>>>(n, ldv, nrhs, st, x, p, (double*)pv, nullptr, 1), note_launch());
     else (k_p_update<float><<<g2, kThreads, 0, s>>>(n, ldv, nrhs, st, x, p, (float*)pv, plo, 1, xt), note_launch());
-    if (fast) stream_mv(xt, nullptr);
-    else matvec(nullptr);
+    matvec(nullptr, nullptr);
   }
   const bool exact_r0 = !(fast && a.use_guess);
   (k_init_r<<<g2, kThreads, 0, s>>>(n, ldv, nrhs, a.b, a.bscale, q, q2, a.use_guess ? 1 : 0, r, x, z,
@@ -1429,14 +1767,28 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
   const int gcol = (nrhs + wb - 1) / wb;
   (k_init_state<<<gcol, wb * 32, 0, s>>>(dots, ge, nrhs, a.tol, pre, st), note_launch());
   if (pre == CPM_PRECOND_DC) {
-    dc_apply(st, dots_dc, 1);
-    (k_init_rz_dc<<<gcol, wb * 32, 0, s>>>(dots_dc, ge, nrhs, st), note_launch());
+    dc_apply(st, dots_dc);
+    const DotParts rz = fast ? DotParts{dots_dc, 4, 4 * (int64_t)nrhs, ge, false} : rz_col;
+    (k_init_rz_dc<<<gcol, wb * 32, 0, s>>>(rz, nrhs, st), note_launch());
   }
   if (f64) (k_p_update<double><<<g2, kThreads, 0, s>>>(n, ldv, nrhs, st, z, p, (double*)pv, nullptr, 1), note_launch());
   else (k_p_update<float><<<g2, kThreads, 0, s>>>(n, ldv, nrhs, st, z, p, (float*)pv, plo, 1, xt), note_launch());
   if (cuda_check(c, cudaGetLastError(), "pcg init")) return CPM_ECUDA;
 
-  std::vector<ColState> host(nrhs);
+  // the polled states, in pinned memory kept with the context (the fixed-workspace solve, which
+  // allocates nothing, polls into ordinary memory)
+  std::vector<ColState> plain;
+  ColState* host = nullptr;
+  int* wait_err = nullptr;  // a bounded wait of the streamed matvec ran out
+  const size_t host_bytes = (size_t)nrhs * sizeof(ColState) + sizeof(int);
+  if (!a.ws && pinned_reserve(c, host_bytes) == CPM_OK) {
+    host = (ColState*)c->pinned;
+  } else {
+    plain.resize(nrhs + 1);
+    host = plain.data();
+  }
+  wait_err = (int*)(host + nrhs);
+  *wait_err = 0;
   const int flexible = pre == CPM_PRECOND_DC ? 1 : 0;
   int it = 0;
   bool all_done = false;
@@ -1446,24 +1798,26 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
   std::vector<char> verified(nrhs, 0);
   std::vector<double> level(nrhs, 1.0);
   // state at the start of iteration `it` lives in st[(it & 1) * nrhs]
+  auto settle = [&]() {  // all_done from the polled states
+    all_done = true;
+    for (int col = 0; col < nrhs; ++col)
+      all_done &= host[col].done == 2 || (host[col].done == 1 && (!fast || verified[col]));
+  };
   auto poll = [&](int k) -> int {
     ColState* cur = st + (size_t)(k & 1) * nrhs;
-    if (cuda_check(c, cudaMemcpyAsync(host.data(), cur, nrhs * sizeof(ColState),
-                                      cudaMemcpyDeviceToHost, s),
+    if (cuda_check(c, cudaMemcpyAsync(host, cur, nrhs * sizeof(ColState), cudaMemcpyDeviceToHost,
+                                      s),
                    "poll"))
       return CPM_ECUDA;
-    int wait_err = 0;  // a bounded wait of the streamed matvec ran out
-    if (mv_err && cuda_check(c, cudaMemcpyAsync(&wait_err, mv_err, sizeof(int),
+    if (mv_err && cuda_check(c, cudaMemcpyAsync(wait_err, mv_err, sizeof(int),
                                                 cudaMemcpyDeviceToHost, s),
                              "poll"))
       return CPM_ECUDA;
     if (cuda_check(c, cudaStreamSynchronize(s), "poll sync")) return CPM_ECUDA;
-    if (wait_err)
+    if (*wait_err)
       return set_err(c, CPM_ECUDA, "streamed matvec: a copy did not land in time (code " +
-                                       std::to_string(wait_err) + ")");
-    all_done = true;
-    for (int col = 0; col < nrhs; ++col)
-      all_done &= host[col].done == 2 || (host[col].done == 1 && (!fast || verified[col]));
+                                       std::to_string(*wait_err) + ")");
+    settle();
     return CPM_OK;
   };
   // residual replacement (many-column solves): r = b - E x through the exact matvec for
@@ -1482,20 +1836,23 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
     const int gvec = (int)std::min<int64_t>((vlen + kThreads - 1) / kThreads, 4 * sms);
     if (from_anchor) {  // r = r_a - E_fast (x - x_a)
       (k_diff_t<<<g2, kThreads, 0, s>>>(n, ldv, x, xa, xdt), note_launch());
-      stream_mv(xdt, nullptr);
+      stream_mv(xdt, nullptr, nullptr);
       (k_anchor_r<<<g2, kThreads, 0, s>>>(n, ldv, nrhs, cur, ra, q, r, z, inv_diag, pre, dots),
        note_launch());
     } else {  // r = b - E x, exactly; the new anchor
       (k_split<<<gvec, kThreads, 0, s>>>(x, vlen, xhi, xlo), note_launch());
-      launch_matvec<float>(c, xhi, xlo, x, ldv, nrhs, q, pq_part, gm_exact, nullptr);
+      launch_matvec<float>(c, xhi, xlo, x, ldv, nrhs, q, pq_part, gm_exact, nullptr, nullptr);
       (k_replace_r<<<g2, kThreads, 0, s>>>(n, ldv, nrhs, cur, a.b, a.bscale, q, r, z, inv_diag,
                                            pre, dots), note_launch());
       if (cuda_check(c, cudaMemcpyAsync(xa, x, vbytes, cudaMemcpyDeviceToDevice, s), "anchor x") ||
           cuda_check(c, cudaMemcpyAsync(ra, r, vbytes, cudaMemcpyDeviceToDevice, s), "anchor r"))
         return CPM_ECUDA;
     }
-    if (pre == CPM_PRECOND_DC) dc_apply(cur, dots, 1);
-    (k_replace_state<<<gcol, wb * 32, 0, s>>>(dots, ge, nrhs, a.tol, cur), note_launch());
+    if (pre == CPM_PRECOND_DC) dc_apply(cur, dots);
+    const bool per_column = pre == CPM_PRECOND_DC && !fast;
+    (k_replace_state<<<gcol, wb * 32, 0, s>>>(dots, ge, per_column ? rz_col : rz_dots, nrhs, a.tol,
+                                             cur),
+     note_launch());
     (k_p_update<float><<<g2, kThreads, 0, s>>>(n, ldv, nrhs, cur, z, p, (float*)pv, plo, 2, xt),
      note_launch());
     t_rep.emplace_back(e0, ev());
@@ -1506,7 +1863,8 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
       verified[col] = host[col].done == 1;
       if (!from_anchor) anchor_level[col] = host[col].relres;
     }
-    return poll(k);  // all_done with the verified flags
+    settle();  // with the verified flags
+    return CPM_OK;
   };
   if ((rc = poll(0))) return rc;
   for (int col = 0; col < nrhs; ++col) {  // an exact r0 is the first anchor
@@ -1518,28 +1876,37 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
                cuda_check(c, cudaMemcpyAsync(ra, r, vbytes, cudaMemcpyDeviceToDevice, s),
                           "anchor r")))
     return CPM_ECUDA;
-  if ((rc = poll(0))) return rc;
+  settle();
   while (!all_done && it < a.maxit) {
     ColState* cur = st + (size_t)(it & 1) * nrhs;
     ColState* nxt = st + (size_t)((it + 1) & 1) * nrhs;
-    const cudaEvent_t m0 = ev();
-    matvec(cur);
-    t_mv.emplace_back(m0, ev());
-    (k_alpha<<<gcol, wb * 32, 0, s>>>(pq_part, gm, nrhs, cur), note_launch());
+    // four launches (five for a large many-column solve): the matvec, the update (with alpha),
+    // the DC apply, the next state and direction
+    matvec(cur, mv_clock);
+    float* rt = fast ? xdt : nullptr;
+    StepArgs sa = {dots, ge, rz_dots, a.tol, flexible, cur, nxt, nullptr};
+    launch_next(pre == CPM_PRECOND_DC       ? k_update<CPM_PRECOND_DC>
+                : pre == CPM_PRECOND_JACOBI ? k_update<CPM_PRECOND_JACOBI>
+                                            : k_update<CPM_PRECOND_NONE>,
+                gv, kThreads, 0, s, n, ldv, nrhs, cur, x, r, z, p, q, inv_diag, dots, ge, a.sys,
+                pq_part, gm, fast || a.ordered, rt, mv_clock);
     if (pre == CPM_PRECOND_DC) {
-      (k_update<CPM_PRECOND_DC><<<g2, kThreads, 0, s>>>(n, ldv, nrhs, cur, x, r, z, p, q,
-                                                       inv_diag, dots, a.sys), note_launch());
-      dc_apply(cur, dots, 0);
-    } else if (pre == CPM_PRECOND_JACOBI) {
-      (k_update<CPM_PRECOND_JACOBI><<<g2, kThreads, 0, s>>>(n, ldv, nrhs, cur, x, r, z, p, q,
-                                                           inv_diag, dots, a.sys), note_launch());
-    } else {
-      (k_update<CPM_PRECOND_NONE><<<g2, kThreads, 0, s>>>(n, ldv, nrhs, cur, x, r, z, p, q,
-                                                         inv_diag, dots, a.sys), note_launch());
+      dc_launch(cur, 0, dc_clock);
+      sa.dc_clock = dc_clock;
+      if (!fast) {
+        sa.rz = rz_col;
+      } else if (nblk_dc <= 512) {
+        sa.rz = {dpart, 2, 2 * (int64_t)nrhs, nblk_dc, false};
+      } else {  // many partials: added once, not by every block of the step
+        dc_dots(dots);
+      }
     }
-    (k_beta<<<gcol, wb * 32, 0, s>>>(dots, ge, nrhs, a.tol, flexible, cur, nxt), note_launch());
-    if (f64) (k_p_update<double><<<g2, kThreads, 0, s>>>(n, ldv, nrhs, nxt, z, p, (double*)pv, nullptr, 0), note_launch());
-    else (k_p_update<float><<<g2, kThreads, 0, s>>>(n, ldv, nrhs, nxt, z, p, (float*)pv, plo, 0, fast ? xt : nullptr), note_launch());
+    if (f64)
+      launch_next(k_step<double>, gv, kThreads, 0, s, n, ldv, nrhs, sa, z, p, (double*)pv, nullptr,
+                  nullptr);
+    else
+      launch_next(k_step<float>, gv, kThreads, 0, s, n, ldv, nrhs, sa, z, p, (float*)pv, plo,
+                  fast ? xt : nullptr);
     ++it;
     if (it % check_every == 0 || it == a.maxit) {
       if (cuda_check(c, cudaGetLastError(), "pcg iteration")) return CPM_ECUDA;
@@ -1571,7 +1938,15 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
     float ms = 0;
     cudaEventElapsedTime(&c->t_solve_ms, t_begin, t_end);
     c->t_solve_mv_ms = c->t_solve_rep_ms = c->t_solve_dc_ms = 0;
-    for (auto& e : t_mv) c->t_solve_mv_ms += (cudaEventElapsedTime(&ms, e.first, e.second), ms);
+    if (mv_clock) {
+      Clock h[2];
+      if (cuda_check(c, cudaMemcpyAsync(h, mv_clock, sizeof(h), cudaMemcpyDeviceToHost, s),
+                     "clocks") ||
+          cuda_check(c, cudaStreamSynchronize(s), "clocks"))
+        return CPM_ECUDA;
+      c->t_solve_mv_ms = 1e-6f * h[0].sum;
+      c->t_solve_dc_ms = 1e-6f * h[1].sum;
+    }
     for (auto& e : t_rep) c->t_solve_rep_ms += (cudaEventElapsedTime(&ms, e.first, e.second), ms);
     for (auto& e : t_dc) c->t_solve_dc_ms += (cudaEventElapsedTime(&ms, e.first, e.second), ms);
     c->solve_replacements = (int)t_rep.size();
@@ -1621,8 +1996,8 @@ int apply_E(Ctx* c, int nrhs, const double* p_in, double* q_out) {
   if (f64) (k_p_update<double><<<g2, kThreads, 0, s>>>(n, ldv, nrhs, st, zin, p, (double*)pv, nullptr, 1), note_launch());
   else (k_p_update<float><<<g2, kThreads, 0, s>>>(n, ldv, nrhs, st, zin, p, (float*)pv, plo, 1), note_launch());
   cudaEventRecord(c->ev_tc[0], s);
-  if (f64) launch_matvec<double>(c, pv, nullptr, p, ldv, nrhs, q, pq_part, gm, nullptr);
-  else launch_matvec<float>(c, pv, plo, p, ldv, nrhs, q, pq_part, gm, nullptr);
+  if (f64) launch_matvec<double>(c, pv, nullptr, p, ldv, nrhs, q, pq_part, gm, nullptr, nullptr);
+  else launch_matvec<float>(c, pv, plo, p, ldv, nrhs, q, pq_part, gm, nullptr, nullptr);
   cudaEventRecord(c->ev_tc[1], s);
   if (cuda_check(c, cudaGetLastError(), "apply_E")) return CPM_ECUDA;
   if (cuda_check(c, copy_cols(q_out, n, q, ldv, n, nrhs, s), "q out")) return CPM_ECUDA;
