@@ -376,7 +376,7 @@ void free_build(Ctx* c) {
                 &c->Ahead, &c->A,
                 &c->E, &c->diag,
                 &c->nbr_off, &c->nbr_idx, &c->prow, &c->d, &c->shell_off, &c->shell_members, &c->p_f32,
-                &c->turn, &c->sfpairs, &c->htab, &c->atoms, &c->gcd_labels, &c->gcd_a, &c->gcd_c, &c->gcd_cinv, &c->gcd_status,
+                &c->turn, &c->sflist, &c->htab, &c->atoms, &c->gcd_labels, &c->gcd_a, &c->gcd_c, &c->gcd_cinv, &c->gcd_status,
                 &c->gcd_scratch, &c->smat};
   for (Buf* b : all) buf_free(c, b);
   release_workspace(c);
@@ -717,17 +717,21 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
                                          "is not positive (INFINITY marks a point charge)"));
   }
 
-  if (!f64 && !c->sfpairs.ptr) {  // depends on the k-vector table only, as that does
-    const std::vector<SfPair> pairs = sf_pairs(hkl, c->m, c->mpad, c->kh);
-    c->n_sfpairs = (int)pairs.size();
-    // and the erfc table of the real-space pairs, the same for every context
-    if ((st = buf_reserve(c, &c->htab, h_table_bytes())) ||
-        (st = cuda_check(c, cudaMemcpyAsync(c->htab.ptr, h_table_host(), h_table_bytes(), h2d, s),
-                         "erfc table")) ||
-        (st = buf_reserve(c, &c->sfpairs, std::max<size_t>(pairs.size(), 1) * sizeof(SfPair))) ||
-        (st = cuda_check(c, cudaMemcpyAsync(c->sfpairs.ptr, pairs.data(),
-                                            pairs.size() * sizeof(SfPair), h2d, s), "pairs")) ||
-        (st = cuda_check(c, cudaStreamSynchronize(s), "pairs sync")))
+  if (!c->sflist.ptr) {  // depends on the k-vector table only, as that does
+    std::vector<SfPair> pairs;
+    std::vector<SfEntry> entries;
+    if (f64) entries = sf_entries(hkl, c->m);
+    else pairs = sf_pairs(hkl, c->m, c->mpad, c->kh);
+    const void* list = f64 ? (const void*)entries.data() : pairs.data();
+    const size_t bytes = f64 ? entries.size() * sizeof(SfEntry) : pairs.size() * sizeof(SfPair);
+    c->n_sflist = (int)(f64 ? entries.size() : pairs.size());
+    // and, for float storage, the erfc table of the real-space pairs, the same everywhere
+    if ((!f64 && ((st = buf_reserve(c, &c->htab, h_table_bytes())) ||
+                  (st = cuda_check(c, cudaMemcpyAsync(c->htab.ptr, h_table_host(), h_table_bytes(),
+                                                      h2d, s), "erfc table")))) ||
+        (st = buf_reserve(c, &c->sflist, std::max<size_t>(bytes, 1))) ||
+        (st = cuda_check(c, cudaMemcpyAsync(c->sflist.ptr, list, bytes, h2d, s), "k list")) ||
+        (st = cuda_check(c, cudaStreamSynchronize(s), "k list sync")))
       return fail(st);
   }
 
@@ -1029,7 +1033,7 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   const AxisPhasors ap = axis_phasors(c);
   const int fchunk = axis_frames(ap, frames, n_ion);
   const size_t abytes = f64 ? up((size_t)fchunk * std::max(n_ion, 1) * ap.len * sizeof(double2)) : 0;
-  const RealPlan rp = real_plan(n, frames, n_ion, std::max(dev_sms, 1));
+  const RealPlan rp = real_plan(n, frames, n_ion, geometry(c), std::max(dev_sms, 1));
   if ((st = buf_reserve(c, &c->ws_pot, vbytes + hbytes + kbytes + ubytes + sbytes + abytes + rp.bytes)))
     return st;
   if (!f64 && !c->turn.ptr) {
@@ -1062,9 +1066,8 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
         launch_axis_phasors(dx + (size_t)f0 * n_ion * 3, nullptr, (int64_t)nf * n_ion, c->p.box, ap,
                             axis, s);
       launch_ion_structure_factor(f64, axis, ap, sion, n_ion, dq + (size_t)f0 * n_ion, nf, n_ion,
-                                  (const SfPair*)c->sfpairs.ptr, c->n_sfpairs,
-                                  (const int*)c->hkl.ptr, (const double*)c->sqw.ptr, c->mpad,
-                                  c->kh, c->turn.ptr,
+                                  SfList{c->sflist.ptr, c->n_sflist}, (const int*)c->hkl.ptr,
+                                  (const double*)c->sqw.ptr, c->m, c->mpad, c->kh, c->turn.ptr,
                                   (char*)v + (size_t)f0 * 2 * c->mpad * c->esz(), vh,
                                   std::max(dev_sms, 1), s);
     }
@@ -1162,8 +1165,8 @@ int cpm_ion_forces(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
     // the electrode's charge-weighted structure factors: the ions' kernel run over the
     // electrode atoms (the same coordinates every frame)
     launch_ion_structure_factor(f64, ax_el, ap, (const uint32_t*)c->sfix.ptr, 0, fq, nf, n,
-                                (const SfPair*)c->sfpairs.ptr, c->n_sfpairs,
-                                (const int*)c->hkl.ptr, (const double*)c->sqw.ptr, c->mpad, c->kh,
+                                SfList{c->sflist.ptr, c->n_sflist}, (const int*)c->hkl.ptr,
+                                (const double*)c->sqw.ptr, c->m, c->mpad, c->kh,
                                 c->turn.ptr, v, vh, std::max(dev_sms, 1), s);
     launch_ion_forces(f64, (const double*)c->xyz.ptr, (const double*)c->alpha.ptr,
                       (const uint32_t*)c->sfix.ptr, n, fx, dq + (size_t)f0 * n_ion, sion, nf, n_ion,

@@ -127,8 +127,9 @@ struct Ctx {
   double pgap = 0;
 
   // learned-guess feature geometry (frame independent, made on first use)
-  Buf sfpairs;    // SfPair [n_sfpairs]: the tail k-vectors in pairs (float storage)
-  int n_sfpairs = 0;
+  Buf sflist;     // the k-vectors as the structure factors take them: SfPair (float
+                  // storage: the tail) or SfEntry (FP64)
+  int n_sflist = 0;
   Buf htab;       // erfc(sqrt s) / sqrt s (real-space pairs of float storage)
   Buf atoms;      // the electrode's records for the real-space pairs
   Buf turn;       // float4 [4096]: exp(2 pi i j / 4096) as float pairs (ion phasors)
@@ -265,6 +266,14 @@ struct SfPair {  // two tail k-vectors (h, k, l), (h, k, l + 1): their places in
   int h, k, l, k0, k1;
 };
 std::vector<SfPair> sf_pairs(const std::vector<int>& hkl, int m, int mpad, int kh);
+struct SfEntry {  // (h, k, l) and (h, k, -l), l >= 0: their places in the table (-1: none)
+  int h, k, l, col, kp, kn;
+};
+std::vector<SfEntry> sf_entries(const std::vector<int>& hkl, int m);
+struct SfList {  // the context's device list: SfPair (float storage) or SfEntry (FP64)
+  const void* list;
+  int entries;
+};
 // per-axis FP64 phasors (FP64 storage) of `count` points: out [count][ap.len] double2; from
 // the fixed-point coordinates sfix where not NULL, else from xyz
 void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
@@ -276,8 +285,8 @@ void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
 void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhasors& ap,
                                  const uint32_t* sion, int64_t coord_stride,
                                  const double* ion_q, int frames, int n_ion,
-                                 const SfPair* pairs, int npairs, const int* hkl,
-                                 const double* sqw, int mpad, int kh, const void* turn,
+                                 const SfList& kl, const int* hkl,
+                                 const double* sqw, int m, int mpad, int kh, const void* turn,
                                  void* v, void* vhead, int sms, cudaStream_t s);
 void launch_bsol_kspace(bool fp64, const void* A, const void* Ahead, int n, int mpad, int kh,
                         const void* v, const void* vhead, int frames, double* bsol,
@@ -293,7 +302,7 @@ struct RealPlan {
   int shares, grid_shares;      // shares of the ions within a block and over the grid
   size_t o_sums, o_part, bytes; // scratch layout: ion records | block sums | partials
 };
-RealPlan real_plan(int n, int frames, int n_ion, int sms);
+RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, int sms);
 size_t h_table_bytes();
 const void* h_table_host();     // erfc(sqrt s) / sqrt s, for a device copy
 size_t atom_record_bytes(int n);
@@ -313,7 +322,8 @@ void launch_bsol_real_and_finish(const double* xyz, const double* alpha, const u
 // forces.cu
 struct ForceSplits {
   int k_tail, k_total;  // shares of the k range: the tail's, and with the head's
-  int real;             // shares of the electrode atoms
+  int real;             // shares of the electrode atoms,
+  int real_per_warp;    //   and the atoms a warp takes of a staged chunk
 };
 ForceSplits force_splits(bool fp64, int n, int frames, int n_ion, int mpad, int kh, int sms);
 // kpart [k_total][frames][n_ion][3], rpart [real][frames][n_ion][3], slab [real][frames]:

@@ -191,7 +191,7 @@ __device__ __forceinline__ double radial_derivative(double g, double a, double r
 
 // Real part: gradients of 32 ions (one a lane) over one share of the electrode atoms,
 // part[share][frame][ion][3] and the share's slab sums slab[share][frame] = (sum q_i z_i,
-// sum q_i).  The block's eight warps take 32 atoms each of every staged chunk of 256.  A
+// sum q_i).  The block's eight warps take 4 to 32 atoms each of every staged chunk.  A
 // pair is screened in float from the exact fixed-point difference of its nearest image
 // (0.01 A^2 band, as k_bsol_real); the pairs that pass go to a queue of the warp and are
 // summed 32 at a time, all lanes busy, over every image within r_c in FP64:
@@ -212,7 +212,7 @@ k_force_real(const double* __restrict__ xyz, const double* __restrict__ alpha,
              const uint32_t* __restrict__ sfix, int n, const double* __restrict__ ion_xyz,
              const uint32_t* __restrict__ sion, int n_ion, const double* __restrict__ q,
              double lx, double ly, double lz, double g, double rc, const ForceScreen fs,
-             int nsplit, double* __restrict__ part, double2* __restrict__ slab) {
+             int nsplit, int per_warp, double* __restrict__ part, double2* __restrict__ slab) {
   __shared__ uint4 su[kFrChunk];  // fixed-point x, y, z of the staged atoms
   __shared__ double sion_xyz[32][3];
   __shared__ int qa[kFrWarps][64];       // queued pairs: atom,
@@ -272,10 +272,11 @@ k_force_real(const double* __restrict__ xyz, const double* __restrict__ alpha,
   const int a0 = (int)((int64_t)n * sp / nsplit), a1 = (int)((int64_t)n * (sp + 1) / nsplit);
   int qn = 0;
   double qz = 0.0, qs = 0.0;  // this thread's share of sum q_i z_i and sum q_i
-  for (int base = a0; base < a1; base += kFrChunk) {
+  const int chunk = kFrWarps * per_warp;
+  for (int base = a0; base < a1; base += chunk) {
     const int i = base + (int)threadIdx.x;
     __syncthreads();
-    if (i < a1) {
+    if (i < a1 && (int)threadIdx.x < chunk) {
       su[threadIdx.x] = make_uint4(sfix[3 * i], sfix[3 * i + 1], sfix[3 * i + 2], 0u);
       if (blockIdx.x == 0) {
         qz += qf[i] * xyz[3 * i + 2];
@@ -283,9 +284,9 @@ k_force_real(const double* __restrict__ xyz, const double* __restrict__ alpha,
       }
     }
     __syncthreads();
-    const int t1 = min(32, a1 - base - warp * 32);
+    const int t1 = min(per_warp, a1 - base - warp * per_warp);
     for (int t = 0; t < t1; ++t) {
-      const uint4 ua = su[warp * 32 + t];
+      const uint4 ua = su[warp * per_warp + t];
       const float dx = (float)(int32_t)(ua.x - u0) * fs.fs[0];
       const float dy = (float)(int32_t)(ua.y - u1) * fs.fs[1];
       const float dz = (float)(int32_t)(ua.z - u2) * fs.fs[2];
@@ -294,7 +295,7 @@ k_force_real(const double* __restrict__ xyz, const double* __restrict__ alpha,
       if (!m) continue;
       if (in) {
         const int at = qn + __popc(m & ((1u << lane) - 1u));
-        qa[warp][at] = base + warp * 32 + t;
+        qa[warp][at] = base + warp * per_warp + t;
         ql[warp][at] = (uint8_t)lane;
       }
       qn += __popc(m);
@@ -376,7 +377,7 @@ __global__ void k_force_finish(const double* __restrict__ ion_xyz,
 
 // Shares of the long sums: enough blocks for eight waves of `sms` SMs where the ions alone
 // do not give them (k-space: at least 1,024 k-vectors a share, so that a block's reduction
-// of its 24 sums stays small beside them; real space: at least one staged chunk of atoms).
+// of its 24 sums stays small beside them; real space: at least 32 atoms, four a warp).
 ForceSplits force_splits(bool fp64, int n, int frames, int n_ion, int mpad, int kh, int sms) {
   ForceSplits s;
   const int64_t want = 8 * (int64_t)sms;
@@ -386,7 +387,10 @@ ForceSplits force_splits(bool fp64, int n, int frames, int n_ion, int mpad, int 
   s.k_total = s.k_tail + (!fp64 && kh > 0 ? 1 : 0);
   const int64_t rblocks = (int64_t)frames * ((n_ion + 31) / 32);
   s.real = (int)std::max<int64_t>(1, std::min<int64_t>((want + rblocks - 1) / rblocks,
-                                                       (n + kFrChunk - 1) / kFrChunk));
+                                                       (n + 31) / 32));
+  // a share in whole chunks where it has several, else as evenly as its warps can
+  const int share = (n + s.real - 1) / s.real;
+  s.real_per_warp = std::max(4, std::min(32, (share + kFrWarps - 1) / kFrWarps));
   return s;
 }
 
@@ -412,7 +416,7 @@ void launch_ion_forces(bool fp64, const double* xyz, const double* alpha, const 
   fs.screen2 = (float)(geo.rc * geo.rc) + 0.01f;
   (k_force_real<<<dim3((n_ion + 31) / 32, frames, sp.real), kFrWarps * 32, 0, s>>>(
        xyz, alpha, sfix, n, ion_xyz, sion, n_ion, q, geo.L[0], geo.L[1], geo.L[2], geo.g, geo.rc,
-       fs, sp.real, rpart, slab),
+       fs, sp.real, sp.real_per_warp, rpart, slab),
    note_launch());
   const double twopi = 2.0 * kPi;
   const int64_t len = 3 * (int64_t)frames * n_ion;

@@ -270,71 +270,136 @@ __global__ void k_axis_phasors(const double* __restrict__ xyz, const uint32_t* _
 }
 
 // FP64 storage (the plain baseline build): the same sums in FP64, the phasors as products of
-// the points' per-axis phasors.  32 k-vectors a block (one a lane), the points dealt to its
-// eight warps, whose sums are added in warp order: with one thread a k-vector over all
-// points a 512-atom cell kept half of the chip busy.
+// the points' per-axis phasors.  A lane takes an entry, the k-vectors (h, k, l) and (h, k, -l):
+// with q exp(i (h x + k y)) = a + i b and exp(i l z) = c + i d the four sums of a c, b d, a d and
+// b c over the points give both, two FP64 operations a k-vector and point.  a + i b is formed
+// once a point and column (h, k) of the block's entries (32, sorted by column) and shared.
+// The points are dealt to the block's eight warps, whose sums are added in warp order.  Bound by
+// the FP64 pipe (two lanes a clock and SM): 84 us at 512 points, 8,645 k-vectors with ten
+// operations a k-vector and point, 20 us so.
 constexpr int kSf64Warps = 8;
+constexpr int kSf64Batch = 8;  // points a warp takes at a time
 
 __global__ void __launch_bounds__(kSf64Warps * 32)
 k_ion_sf_f64(const double2* __restrict__ axis, const AxisPhasors ap, int64_t coord_stride,
-             const double* __restrict__ ion_q, int n_ion, const int* __restrict__ hkl,
-             const double* __restrict__ sqw, int mpad, double* __restrict__ vout) {
-  __shared__ double2 red[kSf64Warps][32];
+             const double* __restrict__ ion_q, int n_ion, const SfEntry* __restrict__ entries,
+             int nentries, const double* __restrict__ sqw, int m, int mpad,
+             double* __restrict__ vout) {
+  __shared__ double2 s_ab[kSf64Warps][32][kSf64Batch];
+  __shared__ double red[kSf64Warps][32][4];
+  __shared__ int2 s_hk[32];  // the block's columns
   const int f = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int k = blockIdx.x * 32 + lane;  // mpad is a multiple of 64
+  double* v = vout + (size_t)f * 2 * mpad;
+  if (blockIdx.x == 0)  // the table's padding
+    for (int k = m + (int)threadIdx.x; k < mpad; k += kSf64Warps * 32) {
+      const size_t kcol = 128 * (size_t)(k >> 6) + (k & 63);
+      v[kcol] = v[kcol + 64] = 0.0;
+    }
+  if (nentries == 0) return;
+  const int e0 = blockIdx.x * 32;
+  const SfEntry en = entries[min(e0 + lane, nentries - 1)];
+  const int c0 = __shfl_sync(0xffffffffu, en.col, 0);
+  const int ncol = __shfl_sync(0xffffffffu, en.col, 31) - c0 + 1, mine = en.col - c0;
+  if (warp == 0) s_hk[mine] = make_int2(en.h, en.k);
+  __syncthreads();
   const double2* tab = axis + (size_t)f * coord_stride * ap.len;
   const double* q = ion_q + (size_t)f * n_ion;
-  const int h0 = hkl[3 * k], h1 = hkl[3 * k + 1], h2 = hkl[3 * k + 2];
-  double re = 0.0, im = 0.0;
-  for (int t = warp; t < n_ion; t += kSf64Warps) {
-    const double2 e = ap.phasor(tab + (size_t)t * ap.len, h0, h1, h2);
-    const double qt = q[t];
-    re += qt * e.x;
-    im += qt * e.y;
+  double ac = 0.0, bd = 0.0, ad = 0.0, bc = 0.0;
+  for (int t0 = warp * kSf64Batch; t0 < n_ion; t0 += kSf64Warps * kSf64Batch) {
+    const int cnt = min(kSf64Batch, n_ion - t0);
+    __syncwarp();
+    for (int e = lane; e < ncol * kSf64Batch; e += 32) {
+      const int c = e / kSf64Batch, t = e % kSf64Batch;
+      if (t >= cnt) continue;
+      const double2* row = tab + (size_t)(t0 + t) * ap.len;
+      const int2 hk = s_hk[c];
+      double2 x = __ldg(row + ap.off[0] + abs(hk.x)), y = __ldg(row + ap.off[1] + abs(hk.y));
+      if (hk.x < 0) x.y = -x.y;
+      if (hk.y < 0) y.y = -y.y;
+      const double qt = q[t0 + t];
+      s_ab[warp][c][t] = make_double2(qt * (x.x * y.x - x.y * y.y), qt * (x.x * y.y + x.y * y.x));
+    }
+    __syncwarp();
+#pragma unroll 4
+    for (int t = 0; t < cnt; ++t) {
+      const double2 z = __ldg(tab + (size_t)(t0 + t) * ap.len + ap.off[2] + en.l);
+      const double2 w = s_ab[warp][mine][t];
+      ac = fma(w.x, z.x, ac);
+      bd = fma(w.y, z.y, bd);
+      ad = fma(w.x, z.y, ad);
+      bc = fma(w.y, z.x, bc);
+    }
   }
-  red[warp][lane] = make_double2(re, im);
+  red[warp][lane][0] = ac;
+  red[warp][lane][1] = bd;
+  red[warp][lane][2] = ad;
+  red[warp][lane][3] = bc;
   __syncthreads();
-  if (warp != 0) return;
+  if (warp != 0 || e0 + lane >= nentries) return;
   for (int w = 1; w < kSf64Warps; ++w) {
-    re += red[w][lane].x;
-    im += red[w][lane].y;
+    ac += red[w][lane][0];
+    bd += red[w][lane][1];
+    ad += red[w][lane][2];
+    bc += red[w][lane][3];
   }
-  const double w = sqw[k];
-  const size_t kcol = 128 * (size_t)(k >> 6) + (k & 63);
-  double* v = vout + (size_t)f * 2 * mpad;
-  v[kcol] = w * re;
-  v[kcol + 64] = w * im;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {  // +l, -l
+    const int k = u == 0 ? en.kp : en.kn;
+    if (k < 0) continue;
+    const double w = sqw[k];
+    const size_t kcol = 128 * (size_t)(k >> 6) + (k & 63);
+    v[kcol] = w * (u == 0 ? ac - bd : ac + bd);
+    v[kcol + 64] = w * (u == 0 ? ad + bc : bc - ad);
+  }
 }
 
-// FP64 storage: b^sol_k[f][i] = sum_c A[i][c] v[f][c], one warp per electrode row and four
-// frames per grid row (the A row is read once for them).
+// FP64 storage: b^sol_k[f][i] = sum_c A[i][c] v[f][c], two electrode rows a block, whose eight
+// warps split the columns, and four frames per grid row (the rows are read once for them).  One
+// warp a row left 512 rows on 64 blocks: 90 us against 21.
 constexpr int kF64Frames = 4;
+constexpr int kF64Rows = 2;
 
 __global__ void __launch_bounds__(256)
 k_bsol_kspace_f64(const double* __restrict__ A, int n, int64_t lda, const double* __restrict__ v,
                   int frames, double* __restrict__ bsol) {
-  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int f0 = blockIdx.y * kF64Frames;
-  if (row >= n) return;
-  const double* a = A + (int64_t)row * lda;
-  double acc[kF64Frames] = {0.0, 0.0, 0.0, 0.0};
-  for (int64_t c = lane * 2; c < lda; c += 64) {
-    const double2 av = __ldg(reinterpret_cast<const double2*>(a + c));
+  __shared__ double red[8][kF64Rows * kF64Frames];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row0 = blockIdx.x * kF64Rows;
+  const int f0 = blockIdx.y * kF64Frames, nf = min(kF64Frames, frames - f0);
+  const double* a[kF64Rows];
+#pragma unroll
+  for (int i = 0; i < kF64Rows; ++i) a[i] = A + (int64_t)min(row0 + i, n - 1) * lda;
+  double acc[kF64Rows][kF64Frames] = {};
+#pragma unroll 2
+  for (int64_t c = threadIdx.x * 2; c < lda; c += 512) {
+    double2 av[kF64Rows];
+#pragma unroll
+    for (int i = 0; i < kF64Rows; ++i) av[i] = __ldg(reinterpret_cast<const double2*>(a[i] + c));
 #pragma unroll
     for (int r = 0; r < kF64Frames; ++r) {
-      if (f0 + r >= frames) break;
+      if (r >= nf) break;
       const double2 vv = __ldg(reinterpret_cast<const double2*>(v + (int64_t)(f0 + r) * lda + c));
-      acc[r] += fma(av.y, vv.y, av.x * vv.x);
+#pragma unroll
+      for (int i = 0; i < kF64Rows; ++i)
+        acc[i][r] = fma(av[i].y, vv.y, fma(av[i].x, vv.x, acc[i][r]));
     }
   }
 #pragma unroll
-  for (int r = 0; r < kF64Frames; ++r) {
-    double x = acc[r];
-    for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0 && f0 + r < frames) bsol[(int64_t)(f0 + r) * n + row] = x;
-  }
+  for (int i = 0; i < kF64Rows; ++i)
+#pragma unroll
+    for (int r = 0; r < kF64Frames; ++r) {
+      if (r >= nf) break;
+      double x = acc[i][r];
+      for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      if (lane == 0) red[warp][i * kF64Frames + r] = x;
+    }
+  __syncthreads();
+  const int i = threadIdx.x / kF64Frames, r = threadIdx.x % kF64Frames;
+  if (i >= kF64Rows || row0 + i >= n || r >= nf) return;
+  double x = 0.0;
+  for (int w = 0; w < 8; ++w) x += red[w][threadIdx.x];
+  bsol[(int64_t)(f0 + r) * n + row0 + i] = x;
 }
 
 // Float storage: b^sol_k[f][i] = sum_c A[i][c] v[f][c] over the tail columns (c >= 2 kh), four
@@ -598,6 +663,39 @@ std::vector<SfPair> sf_pairs(const std::vector<int>& hkl, int m, int mpad, int k
   return out;
 }
 
+// The k-vectors of the table hkl [0, m) in entries of equal h, k and opposite l, column by column
+// ((h, k) pairs), with |l| running up within a column.
+std::vector<SfEntry> sf_entries(const std::vector<int>& hkl, int m) {
+  int lo[2] = {0, 0}, hi[2] = {0, 0}, lmax = 0;
+  for (int k = 0; k < m; ++k) {
+    for (int d = 0; d < 2; ++d) {
+      lo[d] = std::min(lo[d], hkl[3 * (size_t)k + d]);
+      hi[d] = std::max(hi[d], hkl[3 * (size_t)k + d]);
+    }
+    lmax = std::max(lmax, std::abs(hkl[3 * (size_t)k + 2]));
+  }
+  const size_t nk = hi[1] - lo[1] + 1, nc = (hi[0] - lo[0] + 1) * nk, nl = lmax + 1;
+  std::vector<int> at(2 * nc * nl, -1);  // places of (h, k, l) and (h, k, -l)
+  for (int k = 0; k < m; ++k) {
+    const int* p = &hkl[3 * (size_t)k];
+    at[2 * (((p[0] - lo[0]) * nk + (p[1] - lo[1])) * nl + std::abs(p[2])) + (p[2] < 0)] = k;
+  }
+  std::vector<SfEntry> out;
+  out.reserve(m / 2 + m / 16 + 64);
+  int col = -1;
+  for (size_t c = 0; c < nc; ++c) {
+    bool first = true;
+    for (size_t l = 0; l < nl; ++l) {
+      const int kp = at[2 * (c * nl + l)], kn = at[2 * (c * nl + l) + 1];
+      if (kp < 0 && kn < 0) continue;
+      if (first) ++col;
+      first = false;
+      out.push_back({(int)(c / nk) + lo[0], (int)(c % nk) + lo[1], (int)l, col, kp, kn});
+    }
+  }
+  return out;
+}
+
 void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
                          const double L[3], const AxisPhasors& ap, double2* out,
                          cudaStream_t s) {
@@ -608,16 +706,19 @@ void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
 void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhasors& ap,
                                  const uint32_t* sion, int64_t coord_stride,
                                  const double* ion_q, int frames, int n_ion,
-                                 const SfPair* pairs, int npairs, const int* hkl,
-                                 const double* sqw, int mpad, int kh, const void* turn,
+                                 const SfList& kl, const int* hkl,
+                                 const double* sqw, int m, int mpad, int kh, const void* turn,
                                  void* v, void* vhead, int sms, cudaStream_t s) {
   if (fp64) {
-    (k_ion_sf_f64<<<dim3(mpad / 32, frames), kSf64Warps * 32, 0, s>>>(
-         axis, ap, coord_stride, ion_q, n_ion, hkl, sqw, mpad, (double*)v),
+    (k_ion_sf_f64<<<dim3(std::max(1, (kl.entries + 31) / 32), frames), kSf64Warps * 32, 0, s>>>(
+         axis, ap, coord_stride, ion_q, n_ion, (const SfEntry*)kl.list, kl.entries, sqw, m, mpad,
+         (double*)v),
      note_launch());
   } else {
     // warps of a block split the ions until the chip's warps are busy (24 resident an SM),
     // each with at least four blocks of eight ions
+    const SfPair* pairs = (const SfPair*)kl.list;
+    const int npairs = kl.entries;
     const int groups = (npairs + 31) / 32;
     int shares = 1;
     while (shares < kSfWarps && (int64_t)groups * frames * shares < 24 * (int64_t)sms &&
@@ -718,7 +819,8 @@ void launch_bsol_kspace(bool fp64, const void* A, const void* Ahead, int n, int 
     const int groups = (frames + kF64Frames - 1) / kF64Frames;
     for (int g0 = 0; g0 < groups; g0 += 65535) {
       const int f0 = kF64Frames * g0;
-      (k_bsol_kspace_f64<<<dim3((n * 32 + 255) / 256, std::min(groups - g0, 65535)), 256, 0, s>>>(
+      (k_bsol_kspace_f64<<<dim3((n + kF64Rows - 1) / kF64Rows, std::min(groups - g0, 65535)), 256, 0,
+                          s>>>(
            (const double*)A, n, lda, (const double*)v + f0 * lda, frames - f0,
            bsol + (int64_t)f0 * n),
        note_launch());

@@ -17,7 +17,7 @@
 // bound the kernel before: with near pairs in FP64, both kinds through queues of the warp,
 // every ion screened by every lane, it took 16.4 ms at 26,600 atoms, 5,000 ions and 16 frames
 // (r_c 24 A, 550 images an atom) against 1.81 ms; 183 against 14 us at 12,800 atoms, 2,000
-// ions and one frame; 121 against 19 us at 512 atoms and 200 ions, where four blocks held all
+// ions and one frame; 121 against 12 us at 512 atoms and 200 ions, where four blocks held all
 // the work; 2.57 against 1.45 ms at 512 atoms, 2,000 ions, 256 frames (three images a pair).
 // FP64 storage evaluates every image in FP64.
 #include <math.h>
@@ -604,15 +604,19 @@ void launch_atom_records(const double* xyz, const double* alpha, int n, const Ge
 // Scratch of the real-space part: ion records, block sums, and the grid shares' partials.
 // Warps of a block split the ions of one group of atoms until the chip's warps are busy (24
 // resident an SM); where eight shares leave SMs without a block, the grid splits them
-// further (each share at least 32 ions, the step of a warp).
-RealPlan real_plan(int n, int frames, int n_ion, int sms) {
+// further: shares of at least 32 ions, the step of a warp, or, where the images of every ion
+// are screened one by one (a box edge below 2 r_c), of eight (512 atoms, 200 ions: 18.9 us
+// in 16 blocks, 9.2 in 48 and 3.3 for adding their shares).
+RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, int sms) {
   RealPlan p;
   const int64_t groups = (int64_t)((n + 31) / 32) * frames;
   p.shares = 1;
   while (p.shares < kRealWarps && groups * p.shares < 24 * (int64_t)sms) p.shares *= 2;
   const int64_t blocks = (groups * p.shares + kRealWarps - 1) / kRealWarps;
+  bool single = true;
+  for (int u = 0; u < 3; ++u) single &= 2.0 * geo.rc < geo.L[u];
   p.grid_shares = (int)std::max<int64_t>(
-      1, std::min<int64_t>((sms + blocks - 1) / blocks, n_ion / (32 * p.shares)));
+      1, std::min<int64_t>((sms + blocks - 1) / blocks, n_ion / ((single ? 32 : 8) * p.shares)));
   auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
   p.o_sums = up((size_t)frames * std::max(n_ion, 1) * sizeof(IonRec));
   p.o_part = p.o_sums + up((size_t)frames * std::max(prep_blocks(n_ion), 1) * sizeof(double2));
