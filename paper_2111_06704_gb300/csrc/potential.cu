@@ -521,26 +521,44 @@ k_bsol_kspace_f32(const float* __restrict__ A, int64_t lda, const float2* __rest
 }
 
 // Streamed builds keep no A: b^sol_k[f][i] = sum_{k >= kh} sqrt(W_k) [cos(K.r_i) v_c +
-// sin(K.r_i) v_s] with the electrode phases formed on the fly (fixed point, sincos_table);
-// the terms of kDirectBlock consecutive k-vectors are summed in float, and each block's
-// sum goes into an error-free float pair (a two-sum), so the rounding of the plain sums
+// sin(K.r_i) v_s] with the electrode phases formed on the fly (fixed point, the arithmetic of
+// sincos_table); the terms of kDirectBlock consecutive k-vectors are summed in float, and each
+// block's sum goes into an error-free float pair (a two-sum), so the rounding of the plain sums
 // grows with the block, not with the ~10^5 k-vectors.  One thread per electrode atom and up to
 // kDirectFrames frames per block: each phasor is formed once and used for every frame of
 // the block; the k-vectors of a chunk and their structure factors are staged in shared
 // memory.  Frames go in pairs through paired float instructions (two IEEE results an
 // instruction, a - b as fma(b, -1, a)): the values are those of one frame at a time.
+//
+// Bound by the load unit: a phasor's 16-byte table entry is a random one.  From the 4,096-entry
+// table in L1 that took about ten wavefronts a warp (78% of the load unit's time, 2.32 ms at
+// 26,600 atoms, 22,700 k-vectors, 16 frames); the first quadrant of it (1,024 entries, the
+// others by symmetry: exact swaps and signs) fits shared memory eight times, once for every
+// 16-byte bank group, so that the eight lanes of a quarter warp never meet: four wavefronts,
+// 1.84 ms.  128 KB of table leave one block of 512 threads an SM.
 constexpr int kDirectChunk = 128;
 constexpr int kDirectFrames = 16;
 constexpr int kDirectBlock = 8;  // divides every chunk: head and table ends are multiples of 16
+constexpr int kDirectThreads = 512;
+constexpr int kQuadrant = 1024;
 
-__global__ void __launch_bounds__(128, 4)
+struct DirectSmem {
+  float4 table[kQuadrant][8];
+  // sqrt(W) (v_cos, v_sin) of frames 2 p and 2 p + 1: (c_2p, c_2p+1, s_2p, s_2p+1)
+  float4 sv[kDirectChunk][kDirectFrames / 2];
+  uint4 sh[kDirectChunk];  // h, k, l
+};
+
+__global__ void __launch_bounds__(kDirectThreads, 1)
 k_bsol_kspace_direct(const uint32_t* __restrict__ sfix, int n, const int* __restrict__ hkl,
                      const double* __restrict__ sqw, int mpad, int kh,
                      const float4* __restrict__ turn, const float* __restrict__ v, int frames,
                      double* __restrict__ bsol, int nsplit, int64_t split_stride) {
-  __shared__ uint32_t sh[kDirectChunk][3];
-  // sqrt(W) (v_cos, v_sin) of frames 2 p and 2 p + 1: (c_2p, c_2p+1, s_2p, s_2p+1)
-  __shared__ float4 sv[kDirectChunk][kDirectFrames / 2];
+  extern __shared__ __align__(16) unsigned char direct_smem[];
+  DirectSmem& sm = *reinterpret_cast<DirectSmem*>(direct_smem);
+  for (int e = threadIdx.x; e < kQuadrant * 8; e += kDirectThreads)
+    sm.table[e >> 3][e & 7] = __ldg(turn + (e >> 3));
+  const float4* tab = &sm.table[0][threadIdx.x & 7];
   const int f0 = blockIdx.y * kDirectFrames;
   const int nf = min(kDirectFrames, frames - f0);
   // block = atom block + nblk x share: share sp takes chunks [c0, c1) of the k range
@@ -564,12 +582,12 @@ k_bsol_kspace_direct(const uint32_t* __restrict__ sfix, int n, const int* __rest
     __syncthreads();
     for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
       const int k = k0 + t;
-      sh[t][0] = (uint32_t)hkl[3 * k];
-      sh[t][1] = (uint32_t)hkl[3 * k + 1];
-      sh[t][2] = (uint32_t)hkl[3 * k + 2];
+      sm.sh[t] = make_uint4((uint32_t)hkl[3 * k], (uint32_t)hkl[3 * k + 1],
+                            (uint32_t)hkl[3 * k + 2], 0u);
     }
     for (int e = threadIdx.x; e < cnt * (kDirectFrames / 2); e += blockDim.x) {
-      const int t = e / (kDirectFrames / 2), fp = e % (kDirectFrames / 2);
+      const int t = e % kDirectChunk, fp = e / kDirectChunk;
+      if (t >= cnt) continue;
       const int k = k0 + t;
       const size_t kcol = 128 * (size_t)(k >> 6) + (k & 63);
       const float w = (float)sqw[k];
@@ -584,7 +602,7 @@ k_bsol_kspace_direct(const uint32_t* __restrict__ sfix, int n, const int* __rest
         val.y = w * vf[kcol];
         val.w = w * vf[kcol + 64];
       }
-      sv[t][fp] = val;
+      sm.sv[t][fp] = val;
     }
     __syncthreads();
     if (i >= n) continue;
@@ -595,20 +613,25 @@ k_bsol_kspace_direct(const uint32_t* __restrict__ sfix, int n, const int* __rest
 #pragma unroll 2
       for (int tt = 0; tt < kDirectBlock; ++tt) {
         const int t = tb + tt;
-        float sn, cs;
-        sincos_table(sh[t][0] * u0 + sh[t][1] * u1 + sh[t][2] * u2, turn, &sn, &cs);
+        const uint4 hk = sm.sh[t];
+        const uint32_t ph = hk.x * u0 + hk.y * u1 + hk.z * u2;
+        float s0, c0;
+        sincos_entry(tab[8 * ((ph >> 20) & (kQuadrant - 1))], ph, &s0, &c0);
+        // quadrants 1 and 3 swap; the cosine's sign is set in 1 and 2, the sine's in 2 and 3
+        const bool swap = (ph & 0x40000000u) != 0;
+        const float cs = __uint_as_float(__float_as_uint(swap ? s0 : c0) ^
+                                         ((ph + 0x40000000u) & 0x80000000u));
+        const float sn = __uint_as_float(__float_as_uint(swap ? c0 : s0) ^ (ph & 0x80000000u));
         const float2 sn2 = make_float2(sn, sn), cs2 = make_float2(cs, cs);
 #pragma unroll
         for (int f = 0; f < kDirectFrames / 2; ++f) {
-          const float4 vv = sv[t][f];
+          const float4 vv = sm.sv[t][f];
           blk[f] = __ffma2_rn(sn2, make_float2(vv.z, vv.w),
                               __ffma2_rn(cs2, make_float2(vv.x, vv.y), blk[f]));
         }
       }
 #pragma unroll
-      for (int f = 0; f < kDirectFrames / 2; ++f) {
-        pair_add2(hi[f], lo[f], blk[f]);
-      }
+      for (int f = 0; f < kDirectFrames / 2; ++f) pair_add2(hi[f], lo[f], blk[f]);
     }
   }
   if (i < n)
@@ -747,18 +770,19 @@ __global__ void k_sum_splits(const double* __restrict__ part, int nsplit, int64_
 
 }  // namespace
 
-// Shares of the k range for the direct sum: the atom blocks of kDirectFrames-frame groups
-// (four resident an SM) times the shares fill whole waves of `sms` SMs best (a larger
-// count only where it fills 2% more of the last wave).
+// Shares of the k range for the direct sum: the atom blocks of kDirectFrames-frame groups (one
+// resident an SM) times the shares fill whole waves of `sms` SMs best (a larger count only
+// where it fills 2% more of the last wave; at least eight chunks a share, against the 128 KB
+// of table a block writes first).
 int bsol_direct_splits(int n, int frames, int mpad, int kh, int sms) {
-  const int64_t blocks = (int64_t)((n + 127) / 128) * ((frames + kDirectFrames - 1) / kDirectFrames);
+  const int64_t blocks = (int64_t)((n + kDirectThreads - 1) / kDirectThreads) *
+                         ((frames + kDirectFrames - 1) / kDirectFrames);
   const int nch = (mpad - kh + kDirectChunk - 1) / kDirectChunk;
-  const int64_t cap = 4 * (int64_t)sms;
   int best = 1;
   double best_eff = -1.0;
-  for (int sp = 1; sp <= std::min(4, std::max(1, nch)); ++sp) {
-    const int64_t units = blocks * sp, waves = (units + cap - 1) / cap;
-    const double eff = (double)units / (double)(waves * cap);
+  for (int sp = 1; sp <= std::min(24, std::max(1, nch / 8)); ++sp) {
+    const int64_t units = blocks * sp, waves = (units + sms - 1) / sms;
+    const double eff = (double)units / (double)(waves * sms);
     if (eff > best_eff + 0.02) {
       best_eff = eff;
       best = sp;
@@ -832,12 +856,15 @@ void launch_bsol_kspace(bool fp64, const void* A, const void* Ahead, int n, int 
     const int sp = split_part ? nsplit : 1;
     const int64_t stride = (int64_t)frames * n;  // between shares
     double* dst = sp > 1 ? split_part : bsol;
+    cudaFuncSetAttribute(k_bsol_kspace_direct, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sizeof(DirectSmem));  // a failure shows at the launch
     for (int g0 = 0; g0 < fgroups; g0 += 65535) {
       const int f0 = g0 * kDirectFrames;
-      (k_bsol_kspace_direct<<<dim3(sp * ((n + 127) / 128), std::min(fgroups - g0, 65535)), 128,
-                              0, s>>>(sfix, n, hkl, sqw, mpad, kh, (const float4*)turn,
-                                      (const float*)v + f0 * lda, frames - f0,
-                                      dst + (int64_t)f0 * n, sp, stride),
+      const int nblk = (n + kDirectThreads - 1) / kDirectThreads;
+      (k_bsol_kspace_direct<<<dim3(sp * nblk, std::min(fgroups - g0, 65535)), kDirectThreads,
+                              sizeof(DirectSmem), s>>>(
+           sfix, n, hkl, sqw, mpad, kh, (const float4*)turn, (const float*)v + f0 * lda,
+           frames - f0, dst + (int64_t)f0 * n, sp, stride),
        note_launch());
     }
     if (sp > 1)
