@@ -367,6 +367,7 @@ struct SolveArgs {
   const SysCol* sys = nullptr;  // ragged batch: device array [nrhs], one system per column
   bool ordered = false;          // one column: every sum in the build's fixed order
   bool timed = true;             // record the solve's device timings (events of the context)
+  cudaEvent_t begin = nullptr;   // the cluster path records it right before its launch
 };
 int pcg_solve(Ctx* c, const SolveArgs& a);
 // pcg_cluster.cu: the whole solve in one launch, one cluster per right-hand side

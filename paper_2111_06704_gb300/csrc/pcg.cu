@@ -1533,7 +1533,12 @@ int pcg_solve(Ctx* c, const SolveArgs& a) {
     cudaEventCreate(&e1);
     cudaEventRecord(e0, c->stream);
   }
-  int st = path == 2 ? pcg_solve_cluster(c, a) : pcg_solve_kernels(c, a);
+  // (the cluster path is tried first, and its kernel's first use in a process has to load it: its
+  // time starts at the launch.  Counted, that made a 336-atom cell take the other path, 369 us a
+  // solve for 330)
+  SolveArgs t = a;
+  if (path == 2) t.begin = e0;
+  int st = path == 2 ? pcg_solve_cluster(c, t) : pcg_solve_kernels(c, a);
   c->last_solve_path = path;
   if (tuning) {
     cudaEventRecord(e1, c->stream);

@@ -365,6 +365,7 @@ int pcg_solve_cluster(Ctx* c, const SolveArgs& a) {
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  if (a.begin) cudaEventRecord(a.begin, c->stream);
   if ((st = cuda_check(c, cudaLaunchKernelEx(&cfg, k_pcg_cluster, ca), "cluster pcg")))
     return st;
   note_launch();
