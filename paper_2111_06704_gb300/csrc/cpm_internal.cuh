@@ -192,7 +192,6 @@ struct Ctx {
   // last cpm_potential: the ions' structure factors, the k-space contraction, the real
   // space with the finish (device time)
   float t_pot_sf_ms = 0, t_pot_kspace_ms = 0, t_pot_real_ms = 0;
-  std::vector<cudaEvent_t> ev_pot;
   cudaEvent_t ev_tc[3] = {nullptr, nullptr, nullptr};
 
   bool fp64() const { return p.precision == CPM_PREC_FP64; }
@@ -281,18 +280,21 @@ void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
                          cudaStream_t s);
 // Structure factors of the points of `frames` frames, coord_stride points apart (0: every
 // frame has the same coordinates).  FP64 storage takes them from axis, float storage from
-// the fixed-point coordinates sion.
+// the fixed-point coordinates sion.  late: the kernel before is launched by launch_next and
+// waits for all that this one reads, so that the two may run side by side.  stamp (if not NULL):
+// the time at its start.
 void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhasors& ap,
                                  const uint32_t* sion, int64_t coord_stride,
                                  const double* ion_q, int frames, int n_ion,
                                  const SfList& kl, const int* hkl,
                                  const double* sqw, int m, int mpad, int kh, const void* turn,
-                                 void* v, void* vhead, int sms, cudaStream_t s);
+                                 void* v, void* vhead, int sms, bool late,
+                                 unsigned long long* stamp, cudaStream_t s);
 void launch_bsol_kspace(bool fp64, const void* A, const void* Ahead, int n, int mpad, int kh,
                         const void* v, const void* vhead, int frames, double* bsol,
                         const uint32_t* sfix, const int* hkl, const double* sqw,
                         const void* turn, int nsplit, double* split_part, int sms,
-                        cudaStream_t s);
+                        unsigned long long* stamp, cudaStream_t s);
 // shares of the k range of a streamed build's direct k-space sum (split_part then holds
 // nsplit x frames x n doubles)
 int bsol_direct_splits(int n, int frames, int mpad, int kh, int sms);
@@ -311,13 +313,16 @@ void launch_atom_records(const double* xyz, const double* alpha, int n, const Ge
 // fixed-point ion coordinates (sion [frames][n_ion][3]) and the real-space part's scratch
 void launch_ion_prepare(const double* ion_xyz, const double* ion_q, int frames, int n_ion,
                         const Geometry& geo, uint32_t* sion, const RealPlan& plan, void* scratch,
+                        unsigned long long* stamp, cudaStream_t s);
+void launch_bsol_real(const double* xyz, const double* alpha, const uint32_t* sfix,
+                      const void* atoms, const void* htab, int n, const double* ion_xyz,
+                      const double* ion_q, int frames, int n_ion, const Geometry& geo, bool fp64,
+                      const RealPlan& plan, void* scratch, cudaStream_t s);
+// stamp (if not NULL): the times at its start and end
+void launch_bsol_finish(const double* xyz, int n, int frames, int n_ion, const Geometry& geo,
+                        const double* chi, const double* bsol_k, double* b_out, double* qsol,
+                        const RealPlan& plan, void* scratch, unsigned long long* stamp,
                         cudaStream_t s);
-void launch_bsol_real_and_finish(const double* xyz, const double* alpha, const uint32_t* sfix,
-                                 const void* atoms, const void* htab, int n,
-                                 const double* ion_xyz, const double* ion_q, int frames,
-                                 int n_ion, const Geometry& geo, const double* chi,
-                                 const double* bsol_k, double* b_out, double* qsol, bool fp64,
-                                 const RealPlan& plan, void* scratch, cudaStream_t s);
 
 // forces.cu
 struct ForceSplits {
@@ -328,14 +333,17 @@ struct ForceSplits {
 ForceSplits force_splits(bool fp64, int n, int frames, int n_ion, int mpad, int kh, int sms);
 // kpart [k_total][frames][n_ion][3], rpart [real][frames][n_ion][3], slab [real][frames]:
 // scratch for the shares
-void launch_ion_forces(bool fp64, const double* xyz, const double* alpha, const uint32_t* sfix,
-                       int n, const double* ion_xyz, const double* ion_q, const uint32_t* sion,
-                       int frames, int n_ion, const double* q, const int* hkl,
-                       const double* sqw, int mpad, int kh, const Geometry& geo,
-                       const void* turn, const void* v, const void* vhead,
-                       const double2* ion_axis, const AxisPhasors& ap, const ForceSplits& sp,
-                       double* kpart, double* rpart, double2* slab, double* out,
-                       cudaStream_t s);
+void launch_force_real(const double* xyz, const double* alpha, const uint32_t* sfix, int n,
+                       const double* ion_xyz, const uint32_t* sion, int frames, int n_ion,
+                       const double* q, const Geometry& geo, const ForceSplits& sp, double* rpart,
+                       double2* slab, bool beside, cudaStream_t s);
+void launch_force_kspace_and_finish(bool fp64, const double* ion_xyz, const double* ion_q,
+                                    const uint32_t* sion, int frames, int n_ion, const int* hkl,
+                                    const double* sqw, int mpad, int kh, const Geometry& geo,
+                                    const void* turn, const void* v, const void* vhead,
+                                    const double2* ion_axis, const AxisPhasors& ap,
+                                    const ForceSplits& sp, double* kpart, const double* rpart,
+                                    const double2* slab, double* out, cudaStream_t s);
 
 // pcg.cu
 // One system of a ragged batch: a right-hand side with its own (float) matrix, size and

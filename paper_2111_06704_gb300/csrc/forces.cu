@@ -16,6 +16,7 @@
 #include <algorithm>
 
 #include "phasor.cuh"
+#include "programmatic.cuh"
 
 namespace cpm {
 
@@ -69,6 +70,10 @@ k_force_kspace(const uint32_t* __restrict__ sion, int n_ion, const int* __restri
                const double* __restrict__ sqw, int mpad, int kh, int nsplit,
                const float4* __restrict__ turn, const float* __restrict__ v,
                const float2* __restrict__ vhead, double* __restrict__ part) {
+  wait_previous(false);
+  sion = fresh(sion);
+  v = fresh(v);
+  vhead = fresh(vhead);
   const int f = blockIdx.y, frames = gridDim.y, sp = blockIdx.z;
   const int i0 = blockIdx.x * kFkIons;
   uint32_t u[kFkIons][3];
@@ -149,6 +154,9 @@ k_force_kspace_f64(const double2* __restrict__ axis, AxisPhasors ap, int n_ion,
                    const int* __restrict__ hkl, const double* __restrict__ sqw, int mpad,
                    int nsplit, const double* __restrict__ v, double* __restrict__ part) {
   __shared__ double red[kFkThreads / 32][3];
+  wait_previous(false);
+  axis = fresh(axis);
+  v = fresh(v);
   const int f = blockIdx.y, frames = gridDim.y, sp = blockIdx.z, ion = blockIdx.x;
   const double2* row = axis + ((size_t)f * n_ion + ion) * ap.len;
   const double* vf = v + (size_t)f * 2 * mpad;
@@ -212,13 +220,16 @@ k_force_real(const double* __restrict__ xyz, const double* __restrict__ alpha,
              const uint32_t* __restrict__ sfix, int n, const double* __restrict__ ion_xyz,
              const uint32_t* __restrict__ sion, int n_ion, const double* __restrict__ q,
              double lx, double ly, double lz, double g, double rc, const ForceScreen fs,
-             int nsplit, int per_warp, double* __restrict__ part, double2* __restrict__ slab) {
+             int nsplit, int per_warp, double* __restrict__ part, double2* __restrict__ slab,
+             bool beside) {
   __shared__ uint4 su[kFrChunk];  // fixed-point x, y, z of the staged atoms
   __shared__ double sion_xyz[32][3];
   __shared__ int qa[kFrWarps][64];       // queued pairs: atom,
   __shared__ uint8_t ql[kFrWarps][64];   //   lane of the ion
   __shared__ double qv[kFrWarps][32][3];
   __shared__ double red[kFrWarps][32][3];
+  wait_previous(beside);
+  sion = fresh(sion);
   const int f = blockIdx.y, frames = gridDim.y, sp = blockIdx.z;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int I = blockIdx.x * 32 + lane;
@@ -350,6 +361,10 @@ __global__ void k_force_finish(const double* __restrict__ ion_xyz,
                                const double* __restrict__ rpart, const double2* __restrict__ slab,
                                int nr, double3 kscale, double slab_factor,
                                double* __restrict__ out) {
+  wait_previous(false);
+  kpart = fresh(kpart);
+  rpart = fresh(rpart);
+  slab = fresh(slab);
   const int64_t count = (int64_t)frames * n_ion;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 3 * count;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -394,37 +409,40 @@ ForceSplits force_splits(bool fp64, int n, int frames, int n_ion, int mpad, int 
   return s;
 }
 
-void launch_ion_forces(bool fp64, const double* xyz, const double* alpha, const uint32_t* sfix,
-                       int n, const double* ion_xyz, const double* ion_q, const uint32_t* sion,
-                       int frames, int n_ion, const double* q, const int* hkl,
-                       const double* sqw, int mpad, int kh, const Geometry& geo,
-                       const void* turn, const void* v, const void* vhead,
-                       const double2* ion_axis, const AxisPhasors& ap, const ForceSplits& sp,
-                       double* kpart, double* rpart, double2* slab, double* out,
-                       cudaStream_t s) {
-  if (fp64)
-    (k_force_kspace_f64<<<dim3(n_ion, frames, sp.k_tail), kFkThreads, 0, s>>>(
-         ion_axis, ap, n_ion, hkl, sqw, mpad, sp.k_tail, (const double*)v, kpart),
-     note_launch());
-  else
-    (k_force_kspace<<<dim3((n_ion + kFkIons - 1) / kFkIons, frames, sp.k_total), kFkThreads, 0,
-                      s>>>(sion, n_ion, hkl, sqw, mpad, kh, sp.k_tail, (const float4*)turn,
-                           (const float*)v, (const float2*)vhead, kpart),
-     note_launch());
+// Launched after the ions' fixed-point coordinates, which it waits for; beside: what comes after
+// may start beside it.
+void launch_force_real(const double* xyz, const double* alpha, const uint32_t* sfix, int n,
+                       const double* ion_xyz, const uint32_t* sion, int frames, int n_ion,
+                       const double* q, const Geometry& geo, const ForceSplits& sp, double* rpart,
+                       double2* slab, bool beside, cudaStream_t s) {
   ForceScreen fs;
   for (int d = 0; d < 3; ++d) fs.fs[d] = (float)(geo.L[d] * 0x1p-32);
   fs.screen2 = (float)(geo.rc * geo.rc) + 0.01f;
-  (k_force_real<<<dim3((n_ion + 31) / 32, frames, sp.real), kFrWarps * 32, 0, s>>>(
-       xyz, alpha, sfix, n, ion_xyz, sion, n_ion, q, geo.L[0], geo.L[1], geo.L[2], geo.g, geo.rc,
-       fs, sp.real, sp.real_per_warp, rpart, slab),
-   note_launch());
+  launch_next(k_force_real, dim3((n_ion + 31) / 32, frames, sp.real), kFrWarps * 32, 0, s, xyz, alpha,
+              sfix, n, ion_xyz, sion, n_ion, q, geo.L[0], geo.L[1], geo.L[2], geo.g, geo.rc, fs,
+              sp.real, sp.real_per_warp, rpart, slab, beside);
+}
+
+void launch_force_kspace_and_finish(bool fp64, const double* ion_xyz, const double* ion_q,
+                                    const uint32_t* sion, int frames, int n_ion, const int* hkl,
+                                    const double* sqw, int mpad, int kh, const Geometry& geo,
+                                    const void* turn, const void* v, const void* vhead,
+                                    const double2* ion_axis, const AxisPhasors& ap,
+                                    const ForceSplits& sp, double* kpart, const double* rpart,
+                                    const double2* slab, double* out, cudaStream_t s) {
+  if (fp64)
+    launch_next(k_force_kspace_f64, dim3(n_ion, frames, sp.k_tail), kFkThreads, 0, s, ion_axis, ap,
+                n_ion, hkl, sqw, mpad, sp.k_tail, (const double*)v, kpart);
+  else
+    launch_next(k_force_kspace, dim3((n_ion + kFkIons - 1) / kFkIons, frames, sp.k_total), kFkThreads,
+                0, s, sion, n_ion, hkl, sqw, mpad, kh, sp.k_tail, (const float4*)turn,
+                (const float*)v, (const float2*)vhead, kpart);
   const double twopi = 2.0 * kPi;
   const int64_t len = 3 * (int64_t)frames * n_ion;
-  (k_force_finish<<<(int)std::min<int64_t>((len + 127) / 128, 8192), 128, 0, s>>>(
-       ion_xyz, ion_q, frames, n_ion, kpart, sp.k_total, rpart, slab, sp.real,
-       make_double3(twopi / geo.L[0], twopi / geo.L[1], twopi / geo.L[2]),
-       geo.slab ? 4.0 * kPi / (geo.L[0] * geo.L[1] * geo.L[2]) : 0.0, out),
-   note_launch());
+  launch_next(k_force_finish, dim3((int)std::min<int64_t>((len + 127) / 128, 8192)), 128, 0, s,
+              ion_xyz, ion_q, frames, n_ion, (const double*)kpart, sp.k_total, rpart, slab, sp.real,
+              make_double3(twopi / geo.L[0], twopi / geo.L[1], twopi / geo.L[2]),
+              geo.slab ? 4.0 * kPi / (geo.L[0] * geo.L[1] * geo.L[2]) : 0.0, out);
 }
 
 }  // namespace cpm

@@ -15,6 +15,7 @@
 
 #include "async_copy.cuh"
 #include "cpm_internal.cuh"
+#include "programmatic.cuh"
 
 namespace cpm {
 
@@ -116,37 +117,6 @@ __device__ __forceinline__ double lane_sum(const double* v, int count, int64_t s
 struct Clock {
   unsigned long long start, sum;
 };
-
-// The kernels of an iteration are launched with programmatic stream serialisation
-// (launch_next): a kernel's blocks may be set up while the one before drains, and wait here,
-// before they touch anything, until it has completed and its writes are visible.
-__device__ __forceinline__ void wait_previous(bool set_up_next = true) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (set_up_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-template <typename... P, typename... A>
-void launch_next(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
-                 A&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
-  note_launch();
-}
-
-__device__ __forceinline__ unsigned long long now_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
 
 __device__ __forceinline__ void clock_start(Clock* c) {
   if (c && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) c->start = now_ns();

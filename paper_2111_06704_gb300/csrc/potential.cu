@@ -13,6 +13,7 @@
 #include <type_traits>
 
 #include "phasor.cuh"
+#include "programmatic.cuh"
 
 namespace cpm {
 
@@ -22,6 +23,7 @@ namespace {
 // every k-vector and the real-space screening use them.
 __global__ void k_ion_fixed(const double* __restrict__ ion_xyz, int64_t count, double lx,
                             double ly, double lz, uint32_t* __restrict__ sion) {
+  set_up_next();
   const double L[3] = {lx, ly, lz};
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 3 * count;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -96,11 +98,16 @@ k_ion_sf_f32(const uint32_t* __restrict__ sion, int64_t coord_stride,
              const double* __restrict__ ion_q, int n_ion, const SfPair* __restrict__ pairs,
              int npairs, const int* __restrict__ hkl, const double* __restrict__ sqw, int mpad,
              int kh, int tail_shares, int head_blocks, const float4* __restrict__ turn,
-             float* __restrict__ vout, float2* __restrict__ vhead) {
+             float* __restrict__ vout, float2* __restrict__ vhead, bool late,
+             unsigned long long* stamp) {
   __shared__ uint4 si[kIonChunk];   // fixed-point x, y, z and the charge as a float
   __shared__ float sql[kIonChunk];  // the charges' low parts
   __shared__ float tc[64][32], ts[64][32];  // exp(2 pi i j / 64), a copy for every lane
   __shared__ double red[kSfWarps][32][4];
+  if (!late) wait_previous(false);
+  stamp_time(stamp);
+  sion = fresh(sion);
+  ion_q = fresh(ion_q);
   const int f = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool head = (int)blockIdx.x < head_blocks;
@@ -240,6 +247,7 @@ k_ion_sf_f32(const uint32_t* __restrict__ sion, int64_t coord_stride,
       v[kcol + 64] = (float)(w * im[u]);
     }
   }
+  end_after_previous(late);  // (warp 0 comes here: its share is the first)
 }
 
 // exp(2 pi i j s_d) of every point and axis entry, s_d the fractional coordinate (from the
@@ -248,6 +256,8 @@ k_ion_sf_f32(const uint32_t* __restrict__ sion, int64_t coord_stride,
 __global__ void k_axis_phasors(const double* __restrict__ xyz, const uint32_t* __restrict__ sfix,
                                int64_t count, double lx, double ly, double lz,
                                const AxisPhasors ap, double2* __restrict__ out) {
+  wait_previous(false);
+  sfix = fresh(sfix);
   const int64_t len = count * ap.len;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < len;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -284,10 +294,13 @@ __global__ void __launch_bounds__(kSf64Warps * 32)
 k_ion_sf_f64(const double2* __restrict__ axis, const AxisPhasors ap, int64_t coord_stride,
              const double* __restrict__ ion_q, int n_ion, const SfEntry* __restrict__ entries,
              int nentries, const double* __restrict__ sqw, int m, int mpad,
-             double* __restrict__ vout) {
+             double* __restrict__ vout, bool late, unsigned long long* stamp) {
   __shared__ double2 s_ab[kSf64Warps][32][kSf64Batch];
   __shared__ double red[kSf64Warps][32][4];
   __shared__ int2 s_hk[32];  // the block's columns
+  if (!late) wait_previous(false);
+  stamp_time(stamp);
+  axis = fresh(axis);
   const int f = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double* v = vout + (size_t)f * 2 * mpad;
@@ -296,7 +309,7 @@ k_ion_sf_f64(const double2* __restrict__ axis, const AxisPhasors ap, int64_t coo
       const size_t kcol = 128 * (size_t)(k >> 6) + (k & 63);
       v[kcol] = v[kcol + 64] = 0.0;
     }
-  if (nentries == 0) return;
+  if (nentries == 0) return end_after_previous(late);
   const int e0 = blockIdx.x * 32;
   const SfEntry en = entries[min(e0 + lane, nentries - 1)];
   const int c0 = __shfl_sync(0xffffffffu, en.col, 0);
@@ -336,7 +349,8 @@ k_ion_sf_f64(const double2* __restrict__ axis, const AxisPhasors ap, int64_t coo
   red[warp][lane][2] = ad;
   red[warp][lane][3] = bc;
   __syncthreads();
-  if (warp != 0 || e0 + lane >= nentries) return;
+  if (warp != 0) return;
+  if (e0 + lane >= nentries) return end_after_previous(late);
   for (int w = 1; w < kSf64Warps; ++w) {
     ac += red[w][lane][0];
     bd += red[w][lane][1];
@@ -352,6 +366,7 @@ k_ion_sf_f64(const double2* __restrict__ axis, const AxisPhasors ap, int64_t coo
     v[kcol] = w * (u == 0 ? ac - bd : ac + bd);
     v[kcol + 64] = w * (u == 0 ? ad + bc : bc - ad);
   }
+  end_after_previous(late);
 }
 
 // FP64 storage: b^sol_k[f][i] = sum_c A[i][c] v[f][c], two electrode rows a block, whose eight
@@ -362,8 +377,11 @@ constexpr int kF64Rows = 2;
 
 __global__ void __launch_bounds__(256)
 k_bsol_kspace_f64(const double* __restrict__ A, int n, int64_t lda, const double* __restrict__ v,
-                  int frames, double* __restrict__ bsol) {
+                  int frames, double* __restrict__ bsol, unsigned long long* stamp) {
   __shared__ double red[8][kF64Rows * kF64Frames];
+  wait_previous(false);
+  stamp_time(stamp);
+  v = fresh(v);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row0 = blockIdx.x * kF64Rows;
   const int f0 = blockIdx.y * kF64Frames, nf = min(kF64Frames, frames - f0);
@@ -423,10 +441,15 @@ template <int NF, int WS>
 __global__ void __launch_bounds__(kKsWarps * 32, NF == 8 ? 2 : 1)
 k_bsol_kspace_f32(const float* __restrict__ A, int64_t lda, const float2* __restrict__ Ahead,
                   int n, int kh, const float* __restrict__ v, const float2* __restrict__ vhead,
-                  int frames, double* __restrict__ bsol, int stream) {
+                  int frames, double* __restrict__ bsol, int stream,
+                  unsigned long long* stamp) {
   constexpr int NP = (NF + 1) / 2;  // frame pairs (one frame fills both halves of one)
   constexpr int NV = kKsRows * 2 * NP;
   __shared__ float2 sm[kKsWarps][NV];
+  wait_previous(false);
+  stamp_time(stamp);
+  v = fresh(v);
+  vhead = fresh(vhead);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sub = warp % WS;
   const int row0 = (blockIdx.x * (kKsWarps / WS) + warp / WS) * kKsRows;
@@ -553,8 +576,10 @@ __global__ void __launch_bounds__(kDirectThreads, 1)
 k_bsol_kspace_direct(const uint32_t* __restrict__ sfix, int n, const int* __restrict__ hkl,
                      const double* __restrict__ sqw, int mpad, int kh,
                      const float4* __restrict__ turn, const float* __restrict__ v, int frames,
-                     double* __restrict__ bsol, int nsplit, int64_t split_stride) {
+                     double* __restrict__ bsol, int nsplit, int64_t split_stride,
+                     unsigned long long* stamp) {
   extern __shared__ __align__(16) unsigned char direct_smem[];
+  stamp_time(stamp);
   DirectSmem& sm = *reinterpret_cast<DirectSmem*>(direct_smem);
   for (int e = threadIdx.x; e < kQuadrant * 8; e += kDirectThreads)
     sm.table[e >> 3][e & 7] = __ldg(turn + (e >> 3));
@@ -723,7 +748,8 @@ void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
                          const double L[3], const AxisPhasors& ap, double2* out,
                          cudaStream_t s) {
   const int blocks = (int)std::min<int64_t>((count * ap.len + 127) / 128, 16384);
-  (k_axis_phasors<<<blocks, 128, 0, s>>>(xyz, sfix, count, L[0], L[1], L[2], ap, out), note_launch());
+  launch_next(k_axis_phasors, dim3(blocks), 128, 0, s, xyz, sfix, count, L[0], L[1], L[2], ap,
+              out);
 }
 
 void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhasors& ap,
@@ -731,12 +757,12 @@ void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhaso
                                  const double* ion_q, int frames, int n_ion,
                                  const SfList& kl, const int* hkl,
                                  const double* sqw, int m, int mpad, int kh, const void* turn,
-                                 void* v, void* vhead, int sms, cudaStream_t s) {
+                                 void* v, void* vhead, int sms, bool late,
+                                 unsigned long long* stamp, cudaStream_t s) {
   if (fp64) {
-    (k_ion_sf_f64<<<dim3(std::max(1, (kl.entries + 31) / 32), frames), kSf64Warps * 32, 0, s>>>(
-         axis, ap, coord_stride, ion_q, n_ion, (const SfEntry*)kl.list, kl.entries, sqw, m, mpad,
-         (double*)v),
-     note_launch());
+    launch_next(k_ion_sf_f64, dim3(std::max(1, (kl.entries + 31) / 32), frames), kSf64Warps * 32, 0,
+                s, axis, ap, coord_stride, ion_q, n_ion, (const SfEntry*)kl.list, kl.entries, sqw, m,
+                mpad, (double*)v, late, stamp);
   } else {
     // warps of a block split the ions until the chip's warps are busy (24 resident an SM),
     // each with at least four blocks of eight ions
@@ -748,10 +774,9 @@ void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhaso
            n_ion >= 64 * shares)
       shares *= 2;
     const int per = 32 * (kSfWarps / shares), hb = (kh + 31) / 32;
-    (k_ion_sf_f32<<<dim3(hb + (npairs + per - 1) / per, frames), kSfWarps * 32, 0, s>>>(
-         sion, coord_stride, ion_q, n_ion, pairs, npairs, hkl, sqw, mpad, kh, shares, hb,
-         (const float4*)turn, (float*)v, (float2*)vhead),
-     note_launch());
+    launch_next(k_ion_sf_f32, dim3(hb + (npairs + per - 1) / per, frames), kSfWarps * 32, 0, s, sion,
+                coord_stride, ion_q, n_ion, pairs, npairs, hkl, sqw, mpad, kh, shares, hb,
+                (const float4*)turn, (float*)v, (float2*)vhead, late, stamp);
   }
 }
 
@@ -796,18 +821,17 @@ namespace {
 template <int NF, int WS>
 void launch_kspace_f32(const float* A, int64_t lda, const float2* Ahead, int n, int kh,
                        const float* v, const float2* vhead, int frames, double* bsol,
-                       cudaStream_t s) {
+                       unsigned long long* stamp, cudaStream_t s) {
   constexpr int kRows = kKsRows * (kKsWarps / WS);
   const int groups = (frames + NF - 1) / NF;
   // A larger than half of L2 is read past it once (v and the sums' operands stay)
   const int stream = A && (int64_t)n * lda * (int64_t)sizeof(float) > (64ll << 20);
   for (int g0 = 0; g0 < groups; g0 += 65535) {
     const int f0 = g0 * NF;
-    (k_bsol_kspace_f32<NF, WS><<<dim3((n + kRows - 1) / kRows, std::min(groups - g0, 65535)),
-                                 kKsWarps * 32, 0, s>>>(
-         A, lda, Ahead, n, kh, v + f0 * lda, vhead + (int64_t)f0 * 2 * kh, frames - f0,
-         bsol + (int64_t)f0 * n, stream),
-     note_launch());
+    launch_next(k_bsol_kspace_f32<NF, WS>, dim3((n + kRows - 1) / kRows, std::min(groups - g0, 65535)),
+                kKsWarps * 32, 0, s, A, lda, Ahead, n, kh, v + f0 * lda,
+                vhead + (int64_t)f0 * 2 * kh, frames - f0, bsol + (int64_t)f0 * n, stream,
+                g0 == 0 ? stamp : nullptr);
   }
 }
 
@@ -815,17 +839,17 @@ void launch_kspace_f32(const float* A, int64_t lda, const float2* Ahead, int n, 
 // frames' v within a block (two warps a group) where that leaves two blocks an SM.
 void launch_kspace_frames(const float* A, int64_t lda, const float2* Ahead, int n, int kh,
                           const float* v, const float2* vhead, int frames, double* bsol,
-                          int sms, cudaStream_t s) {
+                          int sms, unsigned long long* stamp, cudaStream_t s) {
   if (frames == 1)
-    launch_kspace_f32<1, 8>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, s);
+    launch_kspace_f32<1, 8>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, stamp, s);
   else if (frames == 2)
-    launch_kspace_f32<2, 8>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, s);
+    launch_kspace_f32<2, 8>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, stamp, s);
   else if (frames <= 4)
-    launch_kspace_f32<4, 8>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, s);
+    launch_kspace_f32<4, 8>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, stamp, s);
   else if ((int64_t)((n + 15) / 16) * ((frames + 7) / 8) >= 2 * (int64_t)sms)
-    launch_kspace_f32<8, 2>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, s);
+    launch_kspace_f32<8, 2>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, stamp, s);
   else
-    launch_kspace_f32<8, 8>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, s);
+    launch_kspace_f32<8, 8>(A, lda, Ahead, n, kh, v, vhead, frames, bsol, stamp, s);
 }
 
 }  // namespace
@@ -837,17 +861,15 @@ void launch_bsol_kspace(bool fp64, const void* A, const void* Ahead, int n, int 
                         const void* v, const void* vhead, int frames, double* bsol,
                         const uint32_t* sfix, const int* hkl, const double* sqw,
                         const void* turn, int nsplit, double* split_part, int sms,
-                        cudaStream_t s) {
+                        unsigned long long* stamp, cudaStream_t s) {
   const int64_t lda = 2 * (int64_t)mpad;
   if (fp64) {
     const int groups = (frames + kF64Frames - 1) / kF64Frames;
     for (int g0 = 0; g0 < groups; g0 += 65535) {
       const int f0 = kF64Frames * g0;
-      (k_bsol_kspace_f64<<<dim3((n + kF64Rows - 1) / kF64Rows, std::min(groups - g0, 65535)), 256, 0,
-                          s>>>(
-           (const double*)A, n, lda, (const double*)v + f0 * lda, frames - f0,
-           bsol + (int64_t)f0 * n),
-       note_launch());
+      launch_next(k_bsol_kspace_f64, dim3((n + kF64Rows - 1) / kF64Rows, std::min(groups - g0, 65535)),
+                  256, 0, s, (const double*)A, n, lda, (const double*)v + f0 * lda, frames - f0,
+                  bsol + (int64_t)f0 * n, g0 == 0 ? stamp : nullptr);
     }
     return;
   }
@@ -864,7 +886,7 @@ void launch_bsol_kspace(bool fp64, const void* A, const void* Ahead, int n, int 
       (k_bsol_kspace_direct<<<dim3(sp * nblk, std::min(fgroups - g0, 65535)), kDirectThreads,
                               sizeof(DirectSmem), s>>>(
            sfix, n, hkl, sqw, mpad, kh, (const float4*)turn, (const float*)v + f0 * lda,
-           frames - f0, dst + (int64_t)f0 * n, sp, stride),
+           frames - f0, dst + (int64_t)f0 * n, sp, stride, g0 == 0 ? stamp : nullptr),
        note_launch());
     }
     if (sp > 1)
@@ -874,7 +896,7 @@ void launch_bsol_kspace(bool fp64, const void* A, const void* Ahead, int n, int 
     if (kh == 0) return;
   }
   launch_kspace_frames((const float*)A, lda, (const float2*)Ahead, n, kh, (const float*)v,
-                       (const float2*)vhead, frames, bsol, sms, s);
+                       (const float2*)vhead, frames, bsol, sms, A ? stamp : nullptr, s);
 }
 
 }  // namespace cpm

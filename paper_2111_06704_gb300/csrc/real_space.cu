@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "phasor.cuh"
+#include "programmatic.cuh"
 
 namespace cpm {
 
@@ -127,8 +128,10 @@ constexpr int kPrepThreads = 128;
 __global__ void __launch_bounds__(kPrepThreads)
 k_ion_prepare(const double* __restrict__ ion_xyz, const double* __restrict__ ion_q, int n_ion,
               double lx, double ly, double lz, uint32_t* __restrict__ sion,
-              IonRec* __restrict__ rec, double2* __restrict__ sums) {
+              IonRec* __restrict__ rec, double2* __restrict__ sums, unsigned long long* stamp) {
   __shared__ double2 red[kPrepThreads / 32];
+  set_up_next();
+  stamp_time(stamp);
   const int f = blockIdx.y, t = blockIdx.x * kPrepThreads + threadIdx.x;
   double qz = 0.0, qs = 0.0;
   if (t < n_ion) {
@@ -216,12 +219,7 @@ struct RealArgs {
   int nshift;
   float shift[kMaxShifts][3];  // k L, the screen's
   signed char kshift[kMaxShifts][3];
-  double dip;                  // 4 pi / V, or 0
-  const double2* sums;         // [frame][nsum]: sum q z, sum q
-  int nsum;
-  const double *chi, *bsol_k;
-  double *b_out, *qsol;
-  double* part;                // [gridDim.z][frames][n] when gridDim.z > 1
+  double* part;                // [gridDim.z][frames][n]
 };
 
 // FP64 sum of one electrode-ion pair over every image within r_c.
@@ -262,28 +260,6 @@ __device__ __forceinline__ double pair_images(const double* ri, double ai, const
   return acc;
 }
 
-// b = chi - k_e (b^sol_k + real + dipole term) of atom i in frame f; every thread of the
-// warp adds the frame's block sums.
-__device__ __forceinline__ void finish_atom(const RealArgs& a, int f, int i, double real) {
-  const int lane = threadIdx.x & 31;
-  double qz = 0.0, qs = 0.0;
-  for (int s = lane; s < a.nsum; s += 32) {
-    const double2 v = a.sums[(size_t)f * a.nsum + s];
-    qz += v.x;
-    qs += v.y;
-  }
-  for (int o = 16; o; o >>= 1) {
-    qz += __shfl_xor_sync(0xffffffffu, qz, o);
-    qs += __shfl_xor_sync(0xffffffffu, qs, o);
-  }
-  if (i < a.n) {
-    const size_t e = (size_t)f * a.n + i;
-    const double bs = a.bsol_k[e] + real + a.dip * a.xyz[3 * i + 2] * qz;
-    a.b_out[e] = a.chi[i] - kKe * bs;
-  }
-  if (i == 0 && a.qsol) a.qsol[f] = qs;
-}
-
 template <int kMode, bool kF64>
 __global__ void __launch_bounds__(kRealWarps * 32)
 k_bsol_real(const __grid_constant__ RealArgs a) {
@@ -300,7 +276,8 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
   const int grp = blockIdx.x * per + warp / a.shares;
   const int i = grp * 32 + lane;
   const bool live = i < a.n;
-  const IonRec* ions = a.ions + (size_t)f * a.n_ion;
+  wait_previous();
+  const IonRec* ions = fresh(a.ions) + (size_t)f * a.n_ion;
   uint32_t ui[3] = {0, 0, 0};
   AtomRec at = {};
   double ri[3] = {0.0, 0.0, 0.0}, ai = 0.0;
@@ -567,19 +544,52 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
     if (warp % a.shares != 0) return;
     for (int s = 1; s < a.shares; ++s) acc += red[warp + s][lane];
   }
-  if (gridDim.z > 1) {
-    if (live) a.part[((size_t)blockIdx.z * gridDim.y + f) * a.n + i] = acc;
-  } else {
-    finish_atom(a, f, i, acc);
-  }
+  if (live) a.part[((size_t)blockIdx.z * gridDim.y + f) * a.n + i] = acc;
 }
 
-__global__ void __launch_bounds__(128) k_bsol_finish(const __grid_constant__ RealArgs a, int nz) {
+struct FinishArgs {
+  const double* part;  // [shares][frames][n] real-space sums
+  int shares, n;
+  const double2* sums;  // [frames][nsum] (sum q z, sum q)
+  int nsum;
+  const double* xyz;
+  double dip;  // 4 pi / V in slab geometry
+  const double *chi, *bsol_k;
+  double *b_out, *qsol;
+  unsigned long long* stamp;  // start and end
+};
+
+// b = chi - k_e (b^sol_k + real + dipole term), the real-space shares in share order; every warp
+// adds the frame's block sums.
+__global__ void __launch_bounds__(128) k_bsol_finish(const __grid_constant__ FinishArgs a) {
+  wait_previous();
+  stamp_time(a.stamp);
   const int f = blockIdx.y, i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const double* part = fresh(a.part);
+  const double2* sums = fresh(a.sums);
+  const double* bsol_k = fresh(a.bsol_k);
   double real = 0.0;
   if (i < a.n)
-    for (int z = 0; z < nz; ++z) real += a.part[((size_t)z * gridDim.y + f) * a.n + i];
-  finish_atom(a, f, i, real);
+    for (int z = 0; z < a.shares; ++z) real += part[((size_t)z * gridDim.y + f) * a.n + i];
+  double qz = 0.0, qs = 0.0;
+  for (int s = lane; s < a.nsum; s += 32) {
+    const double2 v = sums[(size_t)f * a.nsum + s];
+    qz += v.x;
+    qs += v.y;
+  }
+  for (int o = 16; o; o >>= 1) {
+    qz += __shfl_xor_sync(0xffffffffu, qz, o);
+    qs += __shfl_xor_sync(0xffffffffu, qs, o);
+  }
+  if (i < a.n) {
+    const size_t e = (size_t)f * a.n + i;
+    const double bs = bsol_k[e] + real + a.dip * a.xyz[3 * i + 2] * qz;
+    a.b_out[e] = a.chi[i] - kKe * bs;
+  }
+  if (i == 0 && a.qsol) a.qsol[f] = qs;
+  if (a.stamp && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && threadIdx.x == 0)
+    a.stamp[1] = now_ns();
 }
 
 int prep_blocks(int n_ion) { return (n_ion + kPrepThreads - 1) / kPrepThreads; }
@@ -606,7 +616,7 @@ void launch_atom_records(const double* xyz, const double* alpha, int n, const Ge
 // resident an SM); where eight shares leave SMs without a block, the grid splits them
 // further: shares of at least 32 ions, the step of a warp, or, where the images of every ion
 // are screened one by one (a box edge below 2 r_c), of eight (512 atoms, 200 ions: 18.9 us
-// in 16 blocks, 9.2 in 48 and 3.3 for adding their shares).
+// in 16 blocks, 9.2 in 48).
 RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, int sms) {
   RealPlan p;
   const int64_t groups = (int64_t)((n + 31) / 32) * frames;
@@ -620,25 +630,24 @@ RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, int sms) {
   auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
   p.o_sums = up((size_t)frames * std::max(n_ion, 1) * sizeof(IonRec));
   p.o_part = p.o_sums + up((size_t)frames * std::max(prep_blocks(n_ion), 1) * sizeof(double2));
-  p.bytes = p.o_part + (p.grid_shares > 1 ? up((size_t)p.grid_shares * frames * n * sizeof(double)) : 0);
+  p.bytes = p.o_part + up((size_t)p.grid_shares * frames * n * sizeof(double));
   return p;
 }
 
 void launch_ion_prepare(const double* ion_xyz, const double* ion_q, int frames, int n_ion,
                         const Geometry& geo, uint32_t* sion, const RealPlan& plan, void* scratch,
-                        cudaStream_t s) {
+                        unsigned long long* stamp, cudaStream_t s) {
   (k_ion_prepare<<<dim3(prep_blocks(n_ion), frames), kPrepThreads, 0, s>>>(
        ion_xyz, ion_q, n_ion, geo.L[0], geo.L[1], geo.L[2], sion, (IonRec*)scratch,
-       (double2*)((char*)scratch + plan.o_sums)),
+       (double2*)((char*)scratch + plan.o_sums), stamp),
    note_launch());
 }
 
-void launch_bsol_real_and_finish(const double* xyz, const double* alpha, const uint32_t* sfix,
-                                 const void* atoms, const void* htab, int n,
-                                 const double* ion_xyz, const double* ion_q, int frames,
-                                 int n_ion, const Geometry& geo, const double* chi,
-                                 const double* bsol_k, double* b_out, double* qsol, bool fp64,
-                                 const RealPlan& plan, void* scratch, cudaStream_t s) {
+// Launched after the ions' preparation, which it waits for; what comes after may start beside it.
+void launch_bsol_real(const double* xyz, const double* alpha, const uint32_t* sfix,
+                      const void* atoms, const void* htab, int n, const double* ion_xyz,
+                      const double* ion_q, int frames, int n_ion, const Geometry& geo, bool fp64,
+                      const RealPlan& plan, void* scratch, cudaStream_t s) {
   RealArgs a;
   a.xyz = xyz;
   a.alpha = alpha;
@@ -699,23 +708,33 @@ void launch_bsol_real_and_finish(const double* xyz, const double* alpha, const u
           a.kshift[k][u] = (signed char)ks[u];
         }
       }
-  a.dip = geo.slab ? 4.0 * kPi / geo.vol : 0.0;
-  a.sums = (const double2*)((char*)scratch + plan.o_sums);
-  a.nsum = prep_blocks(n_ion);
-  a.chi = chi;
-  a.bsol_k = bsol_k;
-  a.b_out = b_out;
-  a.qsol = qsol;
   a.part = (double*)((char*)scratch + plan.o_part);
   const int groups = (n + 31) / 32, per = kRealWarps / plan.shares;
   const dim3 grid((groups + per - 1) / per, frames, plan.grid_shares);
   auto kernel = all_single ? (fp64 ? k_bsol_real<kSingleImage, true> : k_bsol_real<kSingleImage, false>)
                 : a.nshift ? (fp64 ? k_bsol_real<kShiftList, true> : k_bsol_real<kShiftList, false>)
                            : k_bsol_real<kAllImages, true>;
-  (kernel<<<grid, kRealWarps * 32, 0, s>>>(a), note_launch());
-  if (plan.grid_shares > 1)
-    (k_bsol_finish<<<dim3((n + 127) / 128, frames), 128, 0, s>>>(a, plan.grid_shares),
-     note_launch());
+  launch_next(kernel, grid, kRealWarps * 32, 0, s, a);
+}
+
+void launch_bsol_finish(const double* xyz, int n, int frames, int n_ion, const Geometry& geo,
+                        const double* chi, const double* bsol_k, double* b_out, double* qsol,
+                        const RealPlan& plan, void* scratch, unsigned long long* stamp,
+                        cudaStream_t s) {
+  FinishArgs a;
+  a.part = (const double*)((char*)scratch + plan.o_part);
+  a.shares = plan.grid_shares;
+  a.n = n;
+  a.sums = (const double2*)((char*)scratch + plan.o_sums);
+  a.nsum = prep_blocks(n_ion);
+  a.xyz = xyz;
+  a.dip = geo.slab ? 4.0 * kPi / geo.vol : 0.0;
+  a.chi = chi;
+  a.bsol_k = bsol_k;
+  a.b_out = b_out;
+  a.qsol = qsol;
+  a.stamp = stamp;
+  launch_next(k_bsol_finish, dim3((n + 127) / 128, frames), 128, 0, s, a);
 }
 
 }  // namespace cpm
