@@ -113,14 +113,16 @@ void launch_neighbours(const double* xyz, int n, const double* L, double rc2, in
 // erfc(g r_cut)) / r, zero for the atom itself and at r = r_cut.  Every local matrix
 // M_tau only holds pairs within r_cut of each other, i.e. pattern entries, so the FP64
 // erfc runs once per entry instead of once per entry of every local matrix.
+// One warp a row of the pattern (one thread a row, ~140 erfc in a chain, took 446 us at 800
+// atoms, 38 us so).
 __global__ void k_dc_pairs(const double* __restrict__ xyz, int n, double lx, double ly,
                            double lz, double g, double rcut, const int64_t* __restrict__ off,
                            const int* __restrict__ idx, double* __restrict__ val) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   if (j >= n) return;
   const double erfc_rc = erfc(g * rcut);
   const double rc2 = rcut * rcut;
-  for (int64_t e = off[j]; e < off[j + 1]; ++e) {
+  for (int64_t e = off[j] + (threadIdx.x & 31); e < off[j + 1]; e += 32) {
     const int k = idx[e];
     double v = 0.0;
     if (k != j) {
@@ -135,18 +137,26 @@ __global__ void k_dc_pairs(const double* __restrict__ xyz, int n, double lx, dou
 }
 
 // Column tau of M_tau^-1 (Eq. 36), written to pcol[off[tau] .. off[tau+1]).  One block
-// per atom.  The symmetric local matrix is filled in FP64 from the pattern's pair values
-// (a pair of tau's neighbours closer than r_cut is an entry of the first one's pattern
-// row: each warp walks a neighbour's row, coalesced, and finds each entry's position in
-// tau's list, held in shared memory, by binary search) and kept as its packed upper
-// triangle.  A float copy is factored P M = L U with partial pivoting (FP64 runs at 1/64
-// of the float rate here, and the factorisation is m^3 / 3 multiply-adds), and the
+// per atom.  The symmetric local matrix is made of the pattern's FP64 pair values: a pair of
+// tau's neighbours closer than r_cut is an entry of both their pattern rows, and a warp walks a
+// neighbour's row, coalesced, and finds each entry's position in tau's list, held in shared
+// memory, by binary search.  A float copy is factored P M = L U with partial pivoting (FP64
+// runs at 1/64 of the float rate here, and the factorisation is m^3 / 3 multiply-adds), and the
 // solution is refined against the FP64 matrix: x += (LU)^-1 P (e_tau - M x), residuals in
 // FP64.  Each step shrinks the error by about kappa(M) 2^-24 (~1e-5 here), so the error
 // left after adding a correction d is about that times |d|: refinement stops once
 // |d| <= 1e-9 |x| (error ~1e-13 even at kappa(M) 2^-24 = 1e-4; typically after the
 // second correction).
-constexpr int kDcThreads = 128;
+//
+// The chains in k bind it: m pivot steps, and two triangular solves of m steps for each
+// correction.  Eight warps a block or more (32 an SM) share the row updates; a step's update
+// leaves the next step's pivot candidates behind, a barrier a step where no rows are exchanged;
+// the row multipliers come from one load a warp; and the solves keep the vector in one warp's
+// registers.  Every element of the factors and of
+// the vectors is one thread's chain in k, whatever the split.  12,800 atoms, neighbourhoods of
+// 79: 8.2 ms with four warps, three barriers a step and the vectors in shared memory, 4.3 ms so (4 or
+// 16 warps a block: 5.2, 6.4 ms); issue 55%, FP64 residuals a quarter of the FP64 pipe.
+constexpr int kDcMaxThreads = 512;
 constexpr int kDcMaxRefine = 6;
 
 __device__ __forceinline__ int sym_index(int a, int b, int m) {  // packed upper, a <= b
@@ -156,17 +166,17 @@ __device__ __forceinline__ int sym_index(int a, int b, int m) {  // packed upper
 // shared memory of k_dc_local for a neighbourhood of m atoms
 size_t dc_local_smem(int m) {
   return (size_t)m * (m + 1) / 2 * sizeof(double) + 2 * (size_t)m * sizeof(double) +
-         (size_t)m * (m + 1) * sizeof(float) + (size_t)m * sizeof(float) +
-         2 * (size_t)m * sizeof(int) + 16;
+         (size_t)m * (m + 1) * sizeof(float) + 2 * (size_t)m * sizeof(int);
 }
 
-__global__ void __launch_bounds__(kDcThreads)
+// SEGS: 32-element segments of the longest row
+template <int SEGS>
+__global__ void __launch_bounds__(kDcMaxThreads, 2)
 k_dc_local(const double* __restrict__ alpha, const int64_t* __restrict__ off,
-           const int* __restrict__ idx,
-           const double* __restrict__ pval, double* __restrict__ pcol,
-           int* __restrict__ status) {
+           const int* __restrict__ idx, const double* __restrict__ pval,
+           double* __restrict__ pcol, int* __restrict__ status) {
   extern __shared__ double sm[];
-  constexpr int kWarps = kDcThreads / 32;
+  const int warps = blockDim.x >> 5;
   const int tau = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t o = off[tau];
@@ -176,87 +186,98 @@ k_dc_local(const double* __restrict__ alpha, const int64_t* __restrict__ off,
   double* x = S + (size_t)m * (m + 1) / 2;     // solution (FP64)
   double* r = x + m;                           // residual (FP64)
   float* F = reinterpret_cast<float*>(r + m);  // [m][ld]: L (unit, below) and U
-  float* y = F + (size_t)m * ld;               // correction (float)
-  int* piv = reinterpret_cast<int*>(y + m);    // row exchanged with row k at step k
-  int* list = piv + m;                         // tau's neighbours (ascending)
-  __shared__ int s_piv, s_pos, s_done;
-  __shared__ float s_val;
+  int* perm = reinterpret_cast<int*>(F + (size_t)m * ld);  // row of M at each row of L U
+  int* list = perm + m;                        // tau's neighbours (ascending)
+  __shared__ uint2 cand[2][kDcMaxThreads / 32];  // pivot candidates: |value|'s bits, row
+  __shared__ int s_pos, s_done;
   for (int e = threadIdx.x; e < m * (m + 1) / 2; e += blockDim.x) S[e] = 0.0;
+  for (int e = threadIdx.x; e < m * ld; e += blockDim.x) F[e] = 0.f;
   for (int a = threadIdx.x; a < m; a += blockDim.x) {
     const int j = idx[o + a];
     list[a] = j;
+    perm[a] = a;
     if (j == tau) s_pos = a;
   }
   __syncthreads();
-  for (int a = threadIdx.x; a < m; a += blockDim.x) {
-    const double al = alpha[list[a]];
-    S[sym_index(a, a, m)] = isinf(al) ? 0.0 : 0.7978845608028654 * al;  // sqrt(2/pi) alpha_i
-  }
-  for (int a = warp; a < m; a += kWarps) {
+  for (int a = warp; a < m; a += warps) {
     const int ja = list[a];
     for (int64_t e = off[ja] + lane; e < off[ja + 1]; e += 32) {
       const int jb = idx[e];
-      int lo = 0, hi = m;  // position of jb in tau's list, if there
+      int lo = a + 1, hi = m;  // position of jb in tau's list, if there and after a
       while (lo < hi) {
         const int mid = (lo + hi) >> 1;
         if (list[mid] < jb) lo = mid + 1;
         else hi = mid;
       }
-      if (lo < m && list[lo] == jb && lo > a) S[sym_index(a, lo, m)] = pval[e];
+      if (lo < m && list[lo] == jb) {
+        const double v = pval[e];
+        S[sym_index(a, lo, m)] = v;
+        F[a * ld + lo] = F[lo * ld + a] = (float)v;
+      }
+    }
+    if (lane == 0) {
+      const double al = alpha[ja], v = isinf(al) ? 0.0 : 0.7978845608028654 * al;  // sqrt(2/pi)
+      S[sym_index(a, a, m)] = v;
+      F[a * ld + a] = (float)v;
     }
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-    const int a = e / m, b = e - a * m;
-    F[a * ld + b] = (float)S[a <= b ? sym_index(a, b, m) : sym_index(b, a, m)];
-  }
+  // ---- P M = L U in float, partial pivoting (largest, then first), whole rows exchanged -----
+  auto bits = [](float v) { v = fabsf(v); return v == v ? __float_as_uint(v) : 0u; };
+  // lane l looks after the warp's l-th row past k (never more than 32: sixteen warps take up to
+  // kMaxLocal atoms, four at most 96)
+  auto candidate = [&](int a, int k) {  // the warp's largest of column k, rows a of its lanes
+    const unsigned v = a < m ? bits(F[a * ld + k]) : 0u;
+    const unsigned mx = __reduce_max_sync(0xffffffffu, v);
+    const int bi = __reduce_min_sync(0xffffffffu, v == mx ? a : INT_MAX);
+    if (lane == 0) cand[k & 1][warp] = make_uint2(mx, (unsigned)bi);
+  };
+  candidate(warp + warps * lane, 0);
   __syncthreads();
-  // ---- P M = L U in float, partial pivoting, whole rows exchanged ---------------------
   for (int k = 0; k < m; ++k) {
-    if (warp == 0) {
-      float best = -1.f;
-      int bi = k;
-      for (int a = k + lane; a < m; a += 32) {
-        const float v = fabsf(F[a * ld + k]);
-        if (v > best) {
-          best = v;
-          bi = a;
-        }
-      }
-      for (int sh = 16; sh; sh >>= 1) {
-        const float ob = __shfl_xor_sync(0xffffffffu, best, sh);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, sh);
-        if (ob > best || (ob == best && oi < bi)) {
-          best = ob;
-          bi = oi;
-        }
-      }
-      if (lane == 0) {
-        s_piv = bi;
-        s_val = best;
-        piv[k] = bi;
-      }
-    }
-    __syncthreads();
-    if (!(s_val > 0.f)) {
+    const uint2 c = lane < warps ? cand[k & 1][lane] : make_uint2(0u, (unsigned)INT_MAX);
+    const unsigned mx = __reduce_max_sync(0xffffffffu, c.x);
+    const int pv = __reduce_min_sync(0xffffffffu, c.x == mx ? (int)c.y : INT_MAX);
+    if (mx == 0u) {
       if (threadIdx.x == 0) atomicExch(status, 1);
       return;  // singular local matrix (whole block leaves together)
     }
-    const int pv = s_piv;
-    if (pv != k)
+    if (pv != k) {
       for (int b = threadIdx.x; b < m; b += blockDim.x) {
         const float t = F[k * ld + b];
         F[k * ld + b] = F[pv * ld + b];
         F[pv * ld + b] = t;
       }
-    __syncthreads();
-    const float inv = 1.f / F[k * ld + k];
-    for (int a = k + 1 + warp; a < m; a += kWarps) {
-      const float f = F[a * ld + k] * inv;
-      for (int b = k + 1 + lane; b < m; b += 32) F[a * ld + b] -= f * F[k * ld + b];
-      __syncwarp();
-      if (lane == 0) F[a * ld + k] = f;
+      if (threadIdx.x == 0) {
+        const int t = perm[k];
+        perm[k] = perm[pv];
+        perm[pv] = t;
+      }
+      __syncthreads();
     }
+    const float inv = 1.f / F[k * ld + k];
+    const int a0 = k + 1 + warp, al = a0 + warps * lane;
+    const float fl = al < m ? F[al * ld + k] * inv : 0.f;
+    float u[SEGS];  // row k of U
+    bool on[SEGS];
+#pragma unroll
+    for (int i = 0; i < SEGS; ++i) {
+      const int b = lane + 32 * i;
+      on[i] = b > k && b < m;
+      u[i] = on[i] ? F[k * ld + b] : 0.f;
+    }
+    float* Fa = F + a0 * ld + lane;
+    for (int a = a0, l = 0; a < m; a += warps, ++l, Fa += warps * ld) {
+      const float f = __shfl_sync(0xffffffffu, fl, l);
+#pragma unroll
+      for (int i = 0; i < SEGS; ++i) {
+        if (32 * i + 31 <= k) continue;
+        if (on[i]) Fa[32 * i] = fmaf(-f, u[i], Fa[32 * i]);
+      }
+    }
+    __syncwarp();
+    if (al < m) F[al * ld + k] = fl;
+    if (k + 1 < m) candidate(al, k + 1);
     __syncthreads();
   }
   // ---- x = 0, r = e_tau; x += (LU)^-1 P r; r = e_tau - M x (FP64) ------------------------
@@ -268,32 +289,51 @@ k_dc_local(const double* __restrict__ alpha, const int64_t* __restrict__ off,
   __syncthreads();
   for (int it = 0; it < kDcMaxRefine && !s_done; ++it) {
     if (warp == 0) {
-      for (int a = lane; a < m; a += 32) y[a] = (float)r[a];
-      __syncwarp();
-      if (lane == 0)
-        for (int k = 0; k < m; ++k)
-          if (piv[k] != k) {
-            const float t = y[k];
-            y[k] = y[piv[k]];
-            y[piv[k]] = t;
-          }
-      __syncwarp();
-      for (int k = 0; k < m; ++k) {  // forward: unit lower L
-        const float yk = y[k];
-        for (int a = k + 1 + lane; a < m; a += 32) y[a] -= F[a * ld + k] * yk;
-        __syncwarp();
+      // element a = lane + 32 i of the vector in y[i]; lanes past m compute and are not read
+      float y[SEGS];
+      const float* Fr[SEGS];
+#pragma unroll
+      for (int i = 0; i < SEGS; ++i) {
+        const int a = min(lane + 32 * i, m - 1);
+        y[i] = (float)r[perm[a]];
+        Fr[i] = F + a * ld;
       }
-      for (int k = m - 1; k >= 0; --k) {  // back: U
-        const float yk = y[k] / F[k * ld + k];
-        __syncwarp();
-        if (lane == 0) y[k] = yk;
-        for (int a = lane; a < k; a += 32) y[a] -= F[a * ld + k] * yk;
-        __syncwarp();
+#pragma unroll
+      for (int ib = 0; ib < SEGS; ++ib) {  // forward: unit lower L
+        const int n = min(32, m - 32 * ib);
+#pragma unroll 4
+        for (int kk = 0; kk < n; ++kk) {
+          const int k = 32 * ib + kk;
+          const float yk = __shfl_sync(0xffffffffu, y[ib], kk);
+#pragma unroll
+          for (int i = ib; i < SEGS; ++i) {
+            const float t = fmaf(-Fr[i][k], yk, y[i]);
+            if (i > ib || lane > kk) y[i] = t;
+          }
+        }
+      }
+#pragma unroll
+      for (int ib = SEGS - 1; ib >= 0; --ib) {  // back: U
+        const int n = min(32, m - 32 * ib);
+#pragma unroll 4
+        for (int kk = n - 1; kk >= 0; --kk) {
+          const int k = 32 * ib + kk;
+          const float yk = __shfl_sync(0xffffffffu, y[ib], kk) / F[k * ld + k];
+#pragma unroll
+          for (int i = 0; i <= ib; ++i) {
+            const float t = fmaf(-Fr[i][k], yk, y[i]);
+            if (i < ib || lane < kk) y[i] = t;
+          }
+          if (lane == kk) y[ib] = yk;
+        }
       }
       double dmax = 0.0, xmax = 0.0;
-      for (int a = lane; a < m; a += 32) {
-        x[a] += (double)y[a];
-        dmax = fmax(dmax, fabs((double)y[a]));
+#pragma unroll
+      for (int i = 0; i < SEGS; ++i) {
+        const int a = lane + 32 * i;
+        if (a >= m) continue;
+        x[a] += (double)y[i];
+        dmax = fmax(dmax, fabs((double)y[i]));
         xmax = fmax(xmax, fabs(x[a]));
       }
       for (int sh = 16; sh; sh >>= 1) {
@@ -304,7 +344,7 @@ k_dc_local(const double* __restrict__ alpha, const int64_t* __restrict__ off,
     }
     __syncthreads();
     if (s_done) break;
-    for (int a = warp; a < m; a += kWarps) {  // r = e_tau - M x, one warp per row
+    for (int a = warp; a < m; a += warps) {  // r = e_tau - M x, one warp per row
       double s = 0.0;
       for (int b = lane; b < m; b += 32)
         s += S[a <= b ? sym_index(a, b, m) : sym_index(b, a, m)] * x[b];
@@ -408,16 +448,24 @@ int build_dc_preconditioner(Ctx* c) {
     launch_neighbours((const double*)c->xyz.ptr, n, L, rc * rc, nullptr,
                       (const int64_t*)c->nbr_off.ptr, (int*)c->nbr_idx.ptr, 1, 0, s);
     const size_t smem = dc_local_smem(mx);
-    st = cuda_check(c, cudaFuncSetAttribute(k_dc_local, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    // about 32 warps an SM, at least four and at most sixteen a block
+    const int fit = (int)(((size_t)227 << 10) / (smem + 1024));
+    const int warps = fit <= 2 ? 16 : fit <= 5 ? 8 : 4;
+    auto local = mx <= 32   ? k_dc_local<1>
+                 : mx <= 64 ? k_dc_local<2>
+                 : mx <= 96 ? k_dc_local<3>
+                 : mx <= 128 ? k_dc_local<4>
+                             : k_dc_local<kMaxLocal / 32>;
+    st = cuda_check(c, cudaFuncSetAttribute(local, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)smem), "dc smem");
     if (!st) {
       // pair values of the pattern, held in prow until the transpose overwrites it
-      (k_dc_pairs<<<(n + 127) / 128, 128, 0, s>>>((const double*)c->xyz.ptr, n, L[0], L[1],
+      (k_dc_pairs<<<(n + 3) / 4, 128, 0, s>>>((const double*)c->xyz.ptr, n, L[0], L[1],
                                                   L[2], c->p.g_dc, rc,
                                                   (const int64_t*)c->nbr_off.ptr,
                                                   (const int*)c->nbr_idx.ptr,
                                                   (double*)c->prow.ptr), note_launch());
-      (k_dc_local<<<n, kDcThreads, smem, s>>>((const double*)c->alpha.ptr,
+      (local<<<n, warps * 32, smem, s>>>((const double*)c->alpha.ptr,
                                               (const int64_t*)c->nbr_off.ptr,
                                               (const int*)c->nbr_idx.ptr,
                                               (const double*)c->prow.ptr, (double*)pcol.ptr,
