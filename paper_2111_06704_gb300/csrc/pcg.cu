@@ -555,8 +555,12 @@ bool make_stream_map(CUtensorMap* m, const float* E, int n, int64_t ldE) {
 }
 
 // Ragged batch: column c is system c with its own float E (ld, n); one column per grid
-// row, the same arithmetic as k_matvec_f32<1>.  Row blocks past the system's n write a
-// zero partial.
+// row, the products and lanes' sums of k_matvec_f32<1>.  Row blocks past the system's n write a
+// zero partial.  Rows are short (8,000 columns are eight groups a warp), so a warp loads its
+// next group while it multiplies one, and sums its four rows' lanes together, each exchange
+// halving what a lane holds (six float-pair additions for twenty).  Eight systems of 500 to 8,000
+// atoms: 107 -> 92 us (6.1 TB/s).  (Loading ahead costs k_matvec_f32 more in blocks an SM than it
+// gives: 97 -> 122 us at 12,800 atoms.)
 __global__ void __launch_bounds__(kThreads)
 k_matvec_ragged(const SysCol* __restrict__ sys, const float* __restrict__ pv,
                 const float* __restrict__ plo, const double* __restrict__ p64, int64_t ldv,
@@ -586,15 +590,26 @@ k_matvec_ragged(const SysCol* __restrict__ sys, const float* __restrict__ pv,
   for (int i = 0; i < RB; ++i) part[i] = perr[i] = 0.f;
   const float* ph = pv + (int64_t)c * ldv;
   const float* pl = plo + (int64_t)c * ldv;
-  for (int g = warp; g < ngroups; g += kMvWarps) {
+  float nx[RB][4], nh[4], nl[4];  // the next group
+  auto load = [&](int g) {
     const int64_t cc = (int64_t)g * 128 + lane * 4;
-    float ev[RB][4];
 #pragma unroll
     for (int i = 0; i < RB; ++i)
-      *reinterpret_cast<float4*>(ev[i]) = __ldcs(reinterpret_cast<const float4*>(erow[i] + cc));
-    float hv[4], lv[4];
-    *reinterpret_cast<float4*>(hv) = __ldg(reinterpret_cast<const float4*>(ph + cc));
-    *reinterpret_cast<float4*>(lv) = __ldg(reinterpret_cast<const float4*>(pl + cc));
+      *reinterpret_cast<float4*>(nx[i]) = __ldcs(reinterpret_cast<const float4*>(erow[i] + cc));
+    *reinterpret_cast<float4*>(nh) = __ldg(reinterpret_cast<const float4*>(ph + cc));
+    *reinterpret_cast<float4*>(nl) = __ldg(reinterpret_cast<const float4*>(pl + cc));
+  };
+  if (warp < ngroups) load(warp);
+  for (int g = warp; g < ngroups; g += kMvWarps) {
+    float ev[RB][4], hv[4], lv[4];
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+#pragma unroll
+      for (int i = 0; i < RB; ++i) ev[i][w] = nx[i][w];
+      hv[w] = nh[w];
+      lv[w] = nl[w];
+    }
+    if (g + kMvWarps < ngroups) load(g + kMvWarps);
 #pragma unroll
     for (int i = 0; i < RB; ++i)
 #pragma unroll
@@ -608,18 +623,30 @@ k_matvec_ragged(const SysCol* __restrict__ sys, const float* __restrict__ pv,
         part[i] = s;
       }
   }
+  static_assert(RB == 4, "two halvings");
+  const bool up = lane & 16, up2 = lane & 8;
 #pragma unroll
-  for (int i = 0; i < RB; ++i) {
-    float h = part[i], l = perr[i];
-#pragma unroll
-    for (int o = 16; o; o >>= 1)
-      pair_add(h, l, __shfl_xor_sync(0xffffffffu, h, o), __shfl_xor_sync(0xffffffffu, l, o));
-    if (lane == 0) sm[warp][i] = make_float2(h, l);
+  for (int i = 0; i < 2; ++i) {
+    const float gh = up ? part[i] : part[i + 2], gl = up ? perr[i] : perr[i + 2];
+    if (up) {
+      part[i] = part[i + 2];
+      perr[i] = perr[i + 2];
+    }
+    pair_add(part[i], perr[i], __shfl_xor_sync(0xffffffffu, gh, 16),
+             __shfl_xor_sync(0xffffffffu, gl, 16));
   }
+  float h = up2 ? part[1] : part[0], l = up2 ? perr[1] : perr[0];
+  pair_add(h, l, __shfl_xor_sync(0xffffffffu, up2 ? part[0] : part[1], 8),
+           __shfl_xor_sync(0xffffffffu, up2 ? perr[0] : perr[1], 8));
+#pragma unroll
+  for (int o = 4; o; o >>= 1)
+    pair_add(h, l, __shfl_xor_sync(0xffffffffu, h, o), __shfl_xor_sync(0xffffffffu, l, o));
+  if ((lane & 7) == 0) sm[warp][lane >> 3] = make_float2(h, l);  // row lane / 8
   __syncthreads();
   const int t = threadIdx.x;
   if (t < RB) {
-    float h = sm[0][t].x, l = sm[0][t].y;
+    h = sm[0][t].x;
+    l = sm[0][t].y;
 #pragma unroll
     for (int w = 1; w < kMvWarps; ++w) pair_add(h, l, sm[w][t].x, sm[w][t].y);
     const int row = row0 + t;
@@ -1574,7 +1601,10 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a) {
   // lanes (a ragged batch by its largest system)
   const bool dc_warp = (int64_t)nrhs * n * 32 <= 8 * (int64_t)kThreads * sms;
   const int dc_rows = kThreads / (dc_warp ? 32 : 8);
-  const int nz = a.ordered ? 8 * ge : std::min((n + dc_rows - 1) / dc_rows, 512);
+  // (at most six blocks an SM over all columns: the blocks' dots, FP64 at 1/64 of the float rate,
+  // were a third of eight systems' 25 us; 22 so)
+  const int nz_cap = dc_warp ? 512 : std::max(1, 6 * sms / nrhs);
+  const int nz = a.ordered ? 8 * ge : std::min((n + dc_rows - 1) / dc_rows, std::min(nz_cap, 512));
   // layout: x r z p q (double) | pv (storage type) | [fast: xt | x hi | x lo | x - x_a |
   //         x_a | r_a | unit partials | counters, error flag] | pq_part | dots | dots_dc |
   //         states
