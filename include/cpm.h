@@ -120,7 +120,7 @@ typedef struct cpm_params {
   /* How a solve runs.  0 (default): chosen per context by its online autotuner for each
      bucket of right-hand-side counts (1, 2-3, 4-7, .., 128 and more): the first eligible
      solve of a bucket runs on the cluster path, the next on the kernel path, each timed
-     per iteration on the device, and later solves take the faster (a build resets it).
+     on the device, and later solves take the faster (a build resets it).
      1: the kernel path: a few kernels an iteration, the host polling convergence every
      four iterations (every size, every precision, ragged batches).  2: the cluster path:
      the whole solve in one launch, one thread-block cluster of 8 CTAs per right-hand

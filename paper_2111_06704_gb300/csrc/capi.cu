@@ -387,7 +387,7 @@ void free_build(Ctx* c) {
   c->smat_ready = false;
   for (int b = 0; b < 8; ++b) {  // the solver's autotuner starts again with the next build
     c->tune_path[b] = 0;
-    c->tune_cost[b][0] = c->tune_cost[b][1] = 0.f;
+    c->tune_fixed[b] = c->tune_iter[b] = 0.f;
   }
 }
 
@@ -618,7 +618,7 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
   c->solve_only = false;
   for (int b = 0; b < 8; ++b) {  // the solver's autotuner starts again for this electrode
     c->tune_path[b] = 0;
-    c->tune_cost[b][0] = c->tune_cost[b][1] = 0.f;
+    c->tune_fixed[b] = c->tune_iter[b] = 0.f;
   }
   if (n < 1 || !xyz || !alpha) return set_err(c, CPM_EINVAL, "cpm_build_E: n >= 1 and arrays required");
   // buffers of the previous build are reused where large enough (reserve), not freed

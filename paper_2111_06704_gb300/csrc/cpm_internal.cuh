@@ -167,9 +167,10 @@ struct Ctx {
   Buf ws_cluster;  // per-column results of the cluster-resident solve
   // the solver's online autotuner: per bucket of right-hand-side counts (1, 2-3, 4-7, ..,
   // 128+), the path found faster (0 not yet known, 1 host-driven kernels, 2 cluster-
-  // resident) and the measured device time per iteration of each path (reset by a build)
+  // resident) and the cluster path's measured device time, without its iterations and for one
+  // iteration (reset by a build)
   int tune_path[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  float tune_cost[8][2] = {};
+  float tune_fixed[8] = {}, tune_iter[8] = {};
   int last_solve_path = 0;
   // tensor-core build workspace, kept for the next build: operand planes, the FP64
   // head matrix, the error flag, the head's float pairs, the per-SM hi / lo scratch
@@ -375,7 +376,9 @@ struct SolveArgs {
   const SysCol* sys = nullptr;  // ragged batch: device array [nrhs], one system per column
   bool ordered = false;          // one column: every sum in the build's fixed order
   bool timed = true;             // record the solve's device timings (events of the context)
-  cudaEvent_t begin = nullptr;   // the cluster path records it right before its launch
+  // cluster path: an event to record right before its launch, and its iterations' time
+  cudaEvent_t begin = nullptr;
+  float* loop_ms = nullptr;
 };
 int pcg_solve(Ctx* c, const SolveArgs& a);
 // pcg_cluster.cu: the whole solve in one launch, one cluster per right-hand side

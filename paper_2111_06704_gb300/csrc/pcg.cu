@@ -1510,8 +1510,10 @@ int pcg_solve_kernels(Ctx* c, const SolveArgs& a);
 // The solve: the cluster-resident kernel (small electrodes) or the host-driven kernels.
 // With solver_path 0 the choice is the context's online autotuner's: for each bucket of
 // right-hand-side counts, the first eligible solve runs on the cluster path and the next
-// on the host-driven one, each timed per iteration on the device; later solves of that
-// bucket take the faster.  Both give the same iteration on the same matrix.
+// on the host-driven one, each timed on the device; later solves of that bucket take the
+// faster for the second's number of iterations (the first is the build's, a few iterations: by
+// its time per iteration alone a 320-atom cell took the kernels, 383 us a solve for 330).  Both
+// give the same iteration on the same matrix.
 int pcg_solve(Ctx* c, const SolveArgs& a) {
   const bool eligible = !c->fp64() && !a.sys && !a.ws && c->n <= cluster_solve_max_atoms() &&
                         c->p.solver_path != 1;
@@ -1521,7 +1523,7 @@ int pcg_solve(Ctx* c, const SolveArgs& a) {
   if (eligible) {
     if (c->p.solver_path == 2) path = 2;
     else if (c->tune_path[bucket]) path = c->tune_path[bucket];
-    else path = c->tune_cost[bucket][1] > 0.f ? 1 : 2;  // try the cluster path first
+    else path = c->tune_iter[bucket] > 0.f ? 1 : 2;  // try the cluster path first
   }
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   const bool tuning = eligible && c->p.solver_path == 0 && !c->tune_path[bucket];
@@ -1534,7 +1536,11 @@ int pcg_solve(Ctx* c, const SolveArgs& a) {
   // time starts at the launch.  Counted, that made a 336-atom cell take the other path, 369 us a
   // solve for 330)
   SolveArgs t = a;
-  if (path == 2) t.begin = e0;
+  float loop_ms = 0.f;
+  if (path == 2 && tuning) {
+    t.begin = e0;
+    t.loop_ms = &loop_ms;
+  }
   int st = path == 2 ? pcg_solve_cluster(c, t) : pcg_solve_kernels(c, a);
   c->last_solve_path = path;
   if (tuning) {
@@ -1545,9 +1551,14 @@ int pcg_solve(Ctx* c, const SolveArgs& a) {
     int iters = 1;
     for (int col = 0; a.iters && col < a.nrhs; ++col) iters = std::max(iters, a.iters[col]);
     if (st == CPM_OK || st == CPM_ENOCONV) {
-      c->tune_cost[bucket][path - 1] = ms / iters;
-      if (c->tune_cost[bucket][0] > 0.f && c->tune_cost[bucket][1] > 0.f)
-        c->tune_path[bucket] = c->tune_cost[bucket][1] < c->tune_cost[bucket][0] ? 2 : 1;
+      if (path == 2) {
+        loop_ms = std::min(loop_ms, ms);
+        c->tune_fixed[bucket] = ms - loop_ms;
+        c->tune_iter[bucket] = std::max(loop_ms / iters, 1e-6f);
+      } else {  // against the cluster path over as many iterations
+        const float cluster = c->tune_fixed[bucket] + iters * c->tune_iter[bucket];
+        c->tune_path[bucket] = cluster < ms ? 2 : 1;
+      }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
