@@ -173,7 +173,42 @@ __device__ __forceinline__ int act_at(int row, int s) {
   return row * kTs + 4 * ((s >> 2) ^ ((row >> 2) & 7)) + (s & 3);
 }
 
-// out[a][s] = silu(bias[a] + sum_c WT[c][a] in[c][s]) for this thread's 8 x 4 block.
+// acc[k][j] += sum_c W[c][4 ug + j] in[c][8 sg + k] over NIN rows, two samples a paired FMA
+// (half the issue slots of scalar ones: 426,000 samples, forward pass 296 -> 290 us, gradient
+// 812 -> 781).
+template <int NIN>
+__device__ __forceinline__ void tile_product(const float* __restrict__ W,
+                                             const float* __restrict__ in, float (&acc)[8][4],
+                                             int ug, int sg) {
+  float2 a[4][4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a[k][j] = make_float2(acc[2 * k][j], acc[2 * k + 1][j]);
+#pragma unroll 4
+  for (int c = 0; c < NIN; ++c) {
+    const float4 w = *reinterpret_cast<const float4*>(W + c * kH + 4 * ug);
+    const float4 x0 = *reinterpret_cast<const float4*>(in + act_at(c, 8 * sg));
+    const float4 x1 = *reinterpret_cast<const float4*>(in + act_at(c, 8 * sg + 4));
+    const float2 xv[4] = {make_float2(x0.x, x0.y), make_float2(x0.z, x0.w),
+                          make_float2(x1.x, x1.y), make_float2(x1.z, x1.w)};
+    const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        a[k][j] = __ffma2_rn(xv[k], make_float2(wv[j], wv[j]), a[k][j]);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      acc[2 * k][j] = a[k][j].x;
+      acc[2 * k + 1][j] = a[k][j].y;
+    }
+}
+
+// acc = bias[a] + sum_c WT[c][a] in[c][s] for this thread's 8 x 4 block.
 template <int NIN>
 __device__ __forceinline__ void fwd_layer(const float* __restrict__ WT,
                                           const float* __restrict__ bias,
@@ -183,18 +218,7 @@ __device__ __forceinline__ void fwd_layer(const float* __restrict__ WT,
   for (int k = 0; k < 8; ++k)
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[k][j] = bias[4 * ug + j];
-#pragma unroll 8
-  for (int c = 0; c < NIN; ++c) {
-    const float4 w = *reinterpret_cast<const float4*>(WT + c * kH + 4 * ug);
-    const float4 x0 = *reinterpret_cast<const float4*>(in + act_at(c, 8 * sg));
-    const float4 x1 = *reinterpret_cast<const float4*>(in + act_at(c, 8 * sg + 4));
-    const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-    const float wv[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[k][j] = fmaf(xv[k], wv[j], acc[k][j]);
-  }
+  tile_product<NIN>(WT, in, acc, ug, sg);
 }
 
 __device__ __forceinline__ void fwd_store(float* __restrict__ out, const float (&acc)[8][4],
@@ -289,32 +313,14 @@ k_mlp_forward(const float* __restrict__ params, const float* __restrict__ norm, 
 // thread keeps over its tiles; blocks are added in FP64 in a fixed order.  Bound by FP32
 // multiply-adds (29,000 a sample; 8 warps an SM).  One thread a sample with scalar loads of
 // every operand and an atomic add per parameter and 128 samples took 3,702 us for 426,000
-// samples (8% of the chip's FP32 rate); this takes 817 us.
+// samples (8% of the chip's FP32 rate); this takes 781 us (the sigmoids' exponentials and
+// divisions issue as much as the products).
 constexpr int kGradThreads = 256;
 constexpr int kPart = kP + 1;  // the parameters' gradients, the loss
 constexpr int oGW = kF * kH + 2 * kH * kH;   // WT1, WT2, WT3, then:
 constexpr int oGB = oGW + 2 * kH * kH;       // W2, W3 as given, then b1, b2, b3, W4, b4
 constexpr int oGX = oGB + 4 * kH + 4;        // tiles: X, H1, H2, GA, GB
 constexpr size_t kGradSmem = sizeof(float) * (oGX + kF * kTs + 4 * kH * kTs);
-
-// acc[k][j] += sum_c W[c][4 ug + j] in[c][8 sg + k] over NIN rows.
-template <int NIN>
-__device__ __forceinline__ void tile_product(const float* __restrict__ W,
-                                             const float* __restrict__ in, float (&acc)[8][4],
-                                             int ug, int sg) {
-#pragma unroll 4
-  for (int c = 0; c < NIN; ++c) {
-    const float4 w = *reinterpret_cast<const float4*>(W + c * kH + 4 * ug);
-    const float4 x0 = *reinterpret_cast<const float4*>(in + act_at(c, 8 * sg));
-    const float4 x1 = *reinterpret_cast<const float4*>(in + act_at(c, 8 * sg + 4));
-    const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-    const float wv[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[k][j] = fmaf(xv[k], wv[j], acc[k][j]);
-  }
-}
 
 __device__ __forceinline__ void tile_store(float* __restrict__ out, const float (&v)[8][4],
                                            int ug, int sg) {
@@ -333,11 +339,11 @@ template <int NC>
 __device__ __forceinline__ void tile_outer(const float* __restrict__ G,
                                            const float* __restrict__ in, float (&h)[4][NC],
                                            float (&l)[4][NC], int ua, int uc) {
-  float acc[4][NC];
+  float2 acc[4][NC];  // even samples, odd samples
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < NC; ++j) acc[i][j] = 0.f;
+    for (int j = 0; j < NC; ++j) acc[i][j] = make_float2(0.f, 0.f);
 #pragma unroll 2
   for (int s = 0; s < kTs; s += 4) {
     float4 g[4], x[NC];
@@ -351,14 +357,14 @@ __device__ __forceinline__ void tile_outer(const float* __restrict__ G,
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < NC; ++j)
-        acc[i][j] = fmaf(g[i].w, x[j].w,
-                         fmaf(g[i].z, x[j].z,
-                              fmaf(g[i].y, x[j].y, fmaf(g[i].x, x[j].x, acc[i][j]))));
+        acc[i][j] = __ffma2_rn(make_float2(g[i].z, g[i].w), make_float2(x[j].z, x[j].w),
+                               __ffma2_rn(make_float2(g[i].x, g[i].y),
+                                          make_float2(x[j].x, x[j].y), acc[i][j]));
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < NC; ++j) pair_add1(h[i][j], l[i][j], acc[i][j]);
+    for (int j = 0; j < NC; ++j) pair_add1(h[i][j], l[i][j], acc[i][j].x + acc[i][j].y);
 }
 
 __global__ void __launch_bounds__(kGradThreads, 1)
