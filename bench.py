@@ -1371,7 +1371,7 @@ def run_scale_point(args, rank, world, local_rank):
                  "traffic": (stream_tb * n * n) if stream_tb else None,
                  "kernel": "k_matvec_stream (16-column float matvec of the PCG iterations, E "
                            "streamed by TMA once per iteration)",
-                 "timed_region": "the timed steps: CUDA events around each iteration's matvec "
+                 "timed_region": "the timed steps: device-clock stamps around each iteration's matvec "
                                  "launch on the solve stream (last step's solve)",
                  "work": "algorithmic bytes per launch: N^2 x 4 (E) + 16 N x 4 (float "
                          "directions) + 16 N x 8 (FP64 products)",
@@ -1433,7 +1433,7 @@ def run_scale_point(args, rank, world, local_rank):
             "gbs": e_bytes / (solve_parts["matvec_ms"] / max(1, solve_parts["max_iterations"])
                               * 1e-3) / 1e9,
             "note": "matvec_ms: the iterations' matvec launches (one per iteration for the "
-                    "group of 16 columns), events around each"},
+                    "group of 16 columns), by stamps of the device clock"},
         "mean_iters": statistics.mean(iters),
         "previous_step_guess_iters": float(np.mean(it_prev)),
         "q_rel_err_vs_tight_solve": q_err,

@@ -238,7 +238,7 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
  * ion_q[frames*n_ion] (e), q[frames*n] the electrode charges (e, e.g. cpm_neutralize's),
  * f_out[frames*n_ion*3] in e^2/A^2 (times k_e = 14.399645478 for eV/A).  Real space in
  * FP64 over every image within r_c; the reciprocal part from the electrode's
- * charge-weighted structure factors (head k-vectors in FP64, the rest in float phasors
+ * charge-weighted structure factors (head k-vectors in float pairs, the rest in float phasors
  * with error-free float-pair sums).  Not a step of the charge solve: what the charges do to
  * the ions in an MD step (Supplementary Note, Eq. S25).
  */
@@ -463,10 +463,11 @@ typedef struct cpm_info_t {
                            build makes each window's operand planes inside it, so there
                            t_tc_ms (the tensor-core launches alone) is the smaller */
   double t_solve_ms;         /* last PCG solve on this context: device time */
-  double t_solve_matvec_ms;  /* ... of its matvec launches (inner and error-free) */
+  double t_solve_matvec_ms;  /* ... of its iterations' matvecs (device clock) */
   double t_solve_replace_ms; /* ... of its residual replacements (many-column solves) */
   int solve_replacements;    /* ... and their count */
-  double t_pot_sf_ms;        /* last cpm_potential: the ions' structure factors, */
+  double t_pot_sf_ms;        /* last cpm_potential: the ions' structure factors (from the
+                                start of their blocks, beside the last of the real space), */
   double t_pot_kspace_ms;    /* the k-space contraction with the electrode operand, */
   double t_pot_real_ms;      /* the real-space sums and b = chi - k_e b^sol (device time) */
   int solve_path;            /* path of the last solve: 1 kernels, 2 cluster-resident */
