@@ -1032,7 +1032,7 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   const AxisPhasors ap = axis_phasors(c);
   const int fchunk = axis_frames(ap, frames, n_ion);
   const size_t abytes = f64 ? up((size_t)fchunk * std::max(n_ion, 1) * ap.len * sizeof(double2)) : 0;
-  const RealPlan rp = real_plan(n, frames, n_ion, geometry(c), std::max(dev_sms, 1));
+  const RealPlan rp = real_plan(n, frames, n_ion, geometry(c), f64, std::max(dev_sms, 1));
   if ((st = buf_reserve(c, &c->ws_pot, vbytes + hbytes + kbytes + ubytes + sbytes + abytes + rp.bytes)))
     return st;
   if (!f64 && !c->turn.ptr) {

@@ -303,9 +303,10 @@ int bsol_direct_splits(int n, int frames, int mpad, int kh, int sms);
 // real_space.cu
 struct RealPlan {
   int shares, grid_shares;      // shares of the ions within a block and over the grid
+  int warps;                    // of a block
   size_t o_sums, o_part, bytes; // scratch layout: ion records | block sums | partials
 };
-RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, int sms);
+RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, bool fp64, int sms);
 size_t h_table_bytes();
 const void* h_table_host();     // erfc(sqrt s) / sqrt s, for a device copy
 size_t atom_record_bytes(int n);

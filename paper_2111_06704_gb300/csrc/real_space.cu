@@ -272,7 +272,7 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
   __shared__ double red[kRealWarps][32];
   const int f = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int per = kRealWarps / a.shares;  // groups of 32 atoms a block
+  const int per = (blockDim.x >> 5) / a.shares;  // groups of 32 atoms a block
   const int grp = blockIdx.x * per + warp / a.shares;
   const int i = grp * 32 + lane;
   const bool live = i < a.n;
@@ -617,16 +617,28 @@ void launch_atom_records(const double* xyz, const double* alpha, int n, const Ge
 // further: shares of at least 32 ions, the step of a warp, or, where the images of every ion
 // are screened one by one (a box edge below 2 r_c), of eight (512 atoms, 200 ions: 18.9 us
 // in 16 blocks, 9.2 in 48).
-RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, int sms) {
+// Float storage adds an atom's far images in one float chain, in the ions' order; its rounding is
+// most of the real-space error where the ions are many (1e-9 of b at 5,000 ions in a small box),
+// and shares of the ions would exchange it for another, so that b would move by as much with the
+// number of frames.  Above kRealChainIons the ions stay together, in blocks of fewer warps where
+// the groups would leave SMs without one.
+constexpr int kRealChainIons = 1200;
+
+RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, bool fp64, int sms) {
   RealPlan p;
   const int64_t groups = (int64_t)((n + 31) / 32) * frames;
-  p.shares = 1;
-  while (p.shares < kRealWarps && groups * p.shares < 24 * (int64_t)sms) p.shares *= 2;
-  const int64_t blocks = (groups * p.shares + kRealWarps - 1) / kRealWarps;
-  bool single = true;
-  for (int u = 0; u < 3; ++u) single &= 2.0 * geo.rc < geo.L[u];
-  p.grid_shares = (int)std::max<int64_t>(
-      1, std::min<int64_t>((sms + blocks - 1) / blocks, n_ion / ((single ? 32 : 8) * p.shares)));
+  p.shares = p.grid_shares = 1;
+  p.warps = kRealWarps;
+  if (!fp64 && n_ion > kRealChainIons) {
+    p.warps = (int)std::max<int64_t>(1, std::min<int64_t>(kRealWarps, groups / (2 * (int64_t)sms)));
+  } else {
+    while (p.shares < kRealWarps && groups * p.shares < 24 * (int64_t)sms) p.shares *= 2;
+    const int64_t blocks = (groups * p.shares + kRealWarps - 1) / kRealWarps;
+    bool single = true;
+    for (int u = 0; u < 3; ++u) single &= 2.0 * geo.rc < geo.L[u];
+    p.grid_shares = (int)std::max<int64_t>(
+        1, std::min<int64_t>((sms + blocks - 1) / blocks, n_ion / ((single ? 32 : 8) * p.shares)));
+  }
   auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
   p.o_sums = up((size_t)frames * std::max(n_ion, 1) * sizeof(IonRec));
   p.o_part = p.o_sums + up((size_t)frames * std::max(prep_blocks(n_ion), 1) * sizeof(double2));
@@ -709,12 +721,12 @@ void launch_bsol_real(const double* xyz, const double* alpha, const uint32_t* sf
         }
       }
   a.part = (double*)((char*)scratch + plan.o_part);
-  const int groups = (n + 31) / 32, per = kRealWarps / plan.shares;
+  const int groups = (n + 31) / 32, per = plan.warps / plan.shares;
   const dim3 grid((groups + per - 1) / per, frames, plan.grid_shares);
   auto kernel = all_single ? (fp64 ? k_bsol_real<kSingleImage, true> : k_bsol_real<kSingleImage, false>)
                 : a.nshift ? (fp64 ? k_bsol_real<kShiftList, true> : k_bsol_real<kShiftList, false>)
                            : k_bsol_real<kAllImages, true>;
-  launch_next(kernel, grid, kRealWarps * 32, 0, s, a);
+  launch_next(kernel, grid, plan.warps * 32, 0, s, a);
 }
 
 void launch_bsol_finish(const double* xyz, int n, int frames, int n_ion, const Geometry& geo,
