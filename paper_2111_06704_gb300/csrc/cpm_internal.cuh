@@ -304,7 +304,9 @@ int bsol_direct_splits(int n, int frames, int mpad, int kh, int sms);
 struct RealPlan {
   int shares, grid_shares;      // shares of the ions within a block and over the grid
   int warps;                    // of a block
-  size_t o_sums, o_part, bytes; // scratch layout: ion records | block sums | partials
+  int far_cap;                  // far terms of an atom and share kept for the finish, or 0
+  // scratch layout: ion records | block sums | partials | far terms | their counts
+  size_t o_sums, o_part, o_far, o_far_count, bytes;
 };
 RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, bool fp64, int sms);
 size_t h_table_bytes();

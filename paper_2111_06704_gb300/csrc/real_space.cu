@@ -220,6 +220,10 @@ struct RealArgs {
   float shift[kMaxShifts][3];  // k L, the screen's
   signed char kshift[kMaxShifts][3];
   double* part;                // [gridDim.z][frames][n]
+  // far terms of a share in the ions' order, far_cap an atom (0: summed by the share):
+  float* far;                  // [share][frame][far_cap][n]
+  int* far_count;              // [share][frame][n]
+  int far_cap;
 };
 
 // FP64 sum of one electrode-ion pair over every image within r_c.
@@ -308,6 +312,10 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
     }
   }
   float acch = 0.f, accl = 0.f, accf = 0.f;
+  const int sh = blockIdx.z * a.shares + warp % a.shares;
+  const size_t at_share = (size_t)sh * gridDim.y + f;
+  float* far = a.far + at_share * a.far_cap * a.n + i;
+  int nfar = 0;
   double acc = 0.0;
   int cn = 0, cf = 0;  // near and far entries of this lane's list
   int base0 = 0;
@@ -427,7 +435,9 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
     }
     if (m2 >= lane_far2 && m2 < a.cut2) {
       const float ir = rsqrtf(m2);  // 1 / r to ~2 ulp
-      accf += __uint_as_float(w.w) * (erfcf(a.gh * (m2 * ir)) * ir);
+      const float q = __uint_as_float(w.w), e = erfcf(a.gh * (m2 * ir)) * ir;
+      if (nfar < a.far_cap) far[(size_t)nfar++ * a.n] = q * e;
+      else accf += q * e;
     } else {
       evaluate(entry);
     }
@@ -447,7 +457,7 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
   };
 
   // this warp's share of the ions
-  const int nsh = a.shares * gridDim.z, sh = blockIdx.z * a.shares + warp % a.shares;
+  const int nsh = a.shares * gridDim.z;
   const int t0 = (int)((int64_t)a.n_ion * sh / nsh), t1 = (int)((int64_t)a.n_ion * (sh + 1) / nsh);
   base0 = t0;
   int since = 0;  // screened since the lists were last looked at
@@ -538,6 +548,7 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
   drain();
   acc += (double)accf;
   acc += (double)acch + (double)accl;
+  if (a.far_cap > 0 && live) a.far_count[at_share * a.n + i] = nfar;
   if (a.shares > 1) {  // the block's shares of a group, in share order
     red[warp][lane] = acc;
     __syncthreads();
@@ -550,6 +561,9 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
 struct FinishArgs {
   const double* part;  // [shares][frames][n] real-space sums
   int shares, n;
+  const float* far;  // far terms [far_shares][frame][far_cap][n] (far_cap 0: none)
+  const int* far_count;
+  int far_shares, far_cap;
   const double2* sums;  // [frames][nsum] (sum q z, sum q)
   int nsum;
   const double* xyz;
@@ -572,6 +586,25 @@ __global__ void __launch_bounds__(128) k_bsol_finish(const __grid_constant__ Fin
   double real = 0.0;
   if (i < a.n)
     for (int z = 0; z < a.shares; ++z) real += part[((size_t)z * gridDim.y + f) * a.n + i];
+  if (a.far_cap > 0 && i < a.n) {  // one float chain over the shares, as one warp adds them
+    const float* far = fresh(a.far);
+    const int* count = fresh(a.far_count);
+    float c = 0.f;
+    for (int z = 0; z < a.far_shares; ++z) {
+      const size_t at = (size_t)z * gridDim.y + f;
+      const float* t = far + at * a.far_cap * a.n + i;
+      const int m = count[at * a.n + i];
+      for (int k0 = 0; k0 < m; k0 += 16) {
+        float x[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) x[k] = k0 + k < m ? t[(size_t)(k0 + k) * a.n] : 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          if (k0 + k < m) c += x[k];
+      }
+    }
+    real += (double)c;
+  }
   double qz = 0.0, qs = 0.0;
   for (int s = lane; s < a.nsum; s += 32) {
     const double2 v = sums[(size_t)f * a.nsum + s];
@@ -619,30 +652,48 @@ void launch_atom_records(const double* xyz, const double* alpha, int n, const Ge
 // in 16 blocks, 9.2 in 48).
 // Float storage adds an atom's far images in one float chain, in the ions' order; its rounding is
 // most of the real-space error where the ions are many (1e-9 of b at 5,000 ions in a small box),
-// and shares of the ions would exchange it for another, so that b would move by as much with the
-// number of frames.  Above kRealChainIons the ions stay together, in blocks of fewer warps where
-// the groups would leave SMs without one.
+// and sums by shares would exchange it for another, so that b would move by as much with the
+// number of frames.  Above kRealChainIons the shares therefore leave their far terms in scratch,
+// four times the mean number of images within r_c of an atom (ions fill part of the box; a term
+// too many is added by its share), and the finish adds them in order.  Where that takes more
+// than kRealFarBytes the ions stay together, in blocks of fewer warps.  One frame of 2,000 ions, 320
+// atoms: 209 us a call so, 110 with sums by shares, 1,800 with the ions together; 5,341 atoms,
+// 5,000 ions, two frames: 963, 767 and 1,958.
 constexpr int kRealChainIons = 1200;
+constexpr size_t kRealFarBytes = (size_t)192 << 20;
 
 RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, bool fp64, int sms) {
   RealPlan p;
   const int64_t groups = (int64_t)((n + 31) / 32) * frames;
   p.shares = p.grid_shares = 1;
   p.warps = kRealWarps;
-  if (!fp64 && n_ion > kRealChainIons) {
-    p.warps = (int)std::max<int64_t>(1, std::min<int64_t>(kRealWarps, groups / (2 * (int64_t)sms)));
-  } else {
-    while (p.shares < kRealWarps && groups * p.shares < 24 * (int64_t)sms) p.shares *= 2;
-    const int64_t blocks = (groups * p.shares + kRealWarps - 1) / kRealWarps;
-    bool single = true;
-    for (int u = 0; u < 3; ++u) single &= 2.0 * geo.rc < geo.L[u];
-    p.grid_shares = (int)std::max<int64_t>(
-        1, std::min<int64_t>((sms + blocks - 1) / blocks, n_ion / ((single ? 32 : 8) * p.shares)));
+  p.far_cap = 0;
+  while (p.shares < kRealWarps && groups * p.shares < 24 * (int64_t)sms) p.shares *= 2;
+  const int64_t blocks = (groups * p.shares + kRealWarps - 1) / kRealWarps;
+  bool single = true;
+  for (int u = 0; u < 3; ++u) single &= 2.0 * geo.rc < geo.L[u];
+  p.grid_shares = (int)std::max<int64_t>(
+      1, std::min<int64_t>((sms + blocks - 1) / blocks, n_ion / ((single ? 32 : 8) * p.shares)));
+  if (!fp64 && n_ion > kRealChainIons && p.shares * p.grid_shares > 1) {
+    const int nsh = p.shares * p.grid_shares;
+    const double mean = n_ion * (4.0 / 3.0 * kPi * geo.rc * geo.rc * geo.rc) /
+                        (geo.L[0] * geo.L[1] * geo.L[2]);
+    const double cap = 4.0 * mean / nsh + 16.0;
+    if (cap * nsh * frames * n * sizeof(float) <= (double)kRealFarBytes) {
+      p.far_cap = (int)cap;
+    } else {
+      p.shares = p.grid_shares = 1;
+      p.warps =
+          (int)std::max<int64_t>(1, std::min<int64_t>(kRealWarps, groups / (2 * (int64_t)sms)));
+    }
   }
   auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
   p.o_sums = up((size_t)frames * std::max(n_ion, 1) * sizeof(IonRec));
   p.o_part = p.o_sums + up((size_t)frames * std::max(prep_blocks(n_ion), 1) * sizeof(double2));
-  p.bytes = p.o_part + up((size_t)p.grid_shares * frames * n * sizeof(double));
+  p.o_far = p.o_part + up((size_t)p.grid_shares * frames * n * sizeof(double));
+  const size_t lists = (size_t)p.shares * p.grid_shares * frames * n;
+  p.o_far_count = p.o_far + up(lists * p.far_cap * sizeof(float));
+  p.bytes = p.o_far_count + (p.far_cap > 0 ? up(lists * sizeof(int)) : 0);
   return p;
 }
 
@@ -721,6 +772,9 @@ void launch_bsol_real(const double* xyz, const double* alpha, const uint32_t* sf
         }
       }
   a.part = (double*)((char*)scratch + plan.o_part);
+  a.far = (float*)((char*)scratch + plan.o_far);
+  a.far_count = (int*)((char*)scratch + plan.o_far_count);
+  a.far_cap = plan.far_cap;
   const int groups = (n + 31) / 32, per = plan.warps / plan.shares;
   const dim3 grid((groups + per - 1) / per, frames, plan.grid_shares);
   auto kernel = all_single ? (fp64 ? k_bsol_real<kSingleImage, true> : k_bsol_real<kSingleImage, false>)
@@ -736,6 +790,10 @@ void launch_bsol_finish(const double* xyz, int n, int frames, int n_ion, const G
   FinishArgs a;
   a.part = (const double*)((char*)scratch + plan.o_part);
   a.shares = plan.grid_shares;
+  a.far = (const float*)((char*)scratch + plan.o_far);
+  a.far_count = (const int*)((char*)scratch + plan.o_far_count);
+  a.far_shares = plan.shares * plan.grid_shares;
+  a.far_cap = plan.far_cap;
   a.n = n;
   a.sums = (const double2*)((char*)scratch + plan.o_sums);
   a.nsum = prep_blocks(n_ion);
