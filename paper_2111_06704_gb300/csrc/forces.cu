@@ -81,7 +81,7 @@ k_force_kspace(const uint32_t* __restrict__ sion, int n_ion, const int* __restri
   for (int t = 0; t < kFkIons; ++t) {  // an ion past the last repeats it and is not written
     const uint32_t* p = sion + ((size_t)f * n_ion + min(i0 + t, n_ion - 1)) * 3;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) u[t][d] = __ldg(p + d);
+    for (int d = 0; d < 3; ++d) u[t][d] = __ldca(p + d);
   }
   float2 gh[kFkIons / 2][3], gl[kFkIons / 2][3];
 #pragma unroll

@@ -135,6 +135,8 @@ k_matvec_f64(const double* __restrict__ E, int64_t ldE, int n, const double* __r
              double* __restrict__ pq_part, const ColState* __restrict__ st, Clock* clock) {
   __shared__ double sm[32 * NR];
   wait_previous();
+  pv = fresh(pv);
+  st = fresh(st);
   clock_start(clock);
   c0 += blockIdx.y * NR;  // one column group per grid row
   if (st) {  // converged columns are not multiplied again (uniform per block)
@@ -216,6 +218,10 @@ k_matvec_f32(const float* __restrict__ E, int64_t ldE, int n, const float* __res
   constexpr int RB = kMvRows;
   constexpr int RBB = RB * (kMvWarps / WS);  // rows per block
   wait_previous(false);
+  pv = fresh(pv);
+  plo = fresh(plo);
+  p64 = fresh(p64);
+  st = fresh(st);
   clock_start(clock);
   c0 += blockIdx.y * NR;  // one column group per grid row
   if (st) {  // converged columns are not multiplied again (uniform per block)
@@ -251,8 +257,8 @@ k_matvec_f32(const float* __restrict__ E, int64_t ldE, int n, const float* __res
     for (int r = 0; r < NR; ++r) {
       const int64_t o = (int64_t)(c0 + r) * ldv + cc;
       float hv[4], lv[4];
-      *reinterpret_cast<float4*>(hv) = __ldg(reinterpret_cast<const float4*>(pv + o));
-      *reinterpret_cast<float4*>(lv) = __ldg(reinterpret_cast<const float4*>(plo + o));
+      *reinterpret_cast<float4*>(hv) = __ldca(reinterpret_cast<const float4*>(pv + o));
+      *reinterpret_cast<float4*>(lv) = __ldca(reinterpret_cast<const float4*>(plo + o));
 #pragma unroll
       for (int i = 0; i < RB; ++i)
 #pragma unroll
@@ -360,6 +366,9 @@ k_matvec_stream(const __grid_constant__ CUtensorMap emap, StreamArgs a) {
   const int ncol = min(kFastCols, a.nrhs - c0);
   const int rb = blockIdx.x / a.splits, sp = blockIdx.x % a.splits;
   wait_previous(false);
+  a.xt = fresh(a.xt);
+  a.p64 = fresh(a.p64);
+  a.st = fresh(a.st);
   clock_start(a.clock);
   if (a.st) {  // a group with every column converged is not multiplied (uniform per grid row)
     bool live = false;
@@ -570,6 +579,10 @@ k_matvec_ragged(const SysCol* __restrict__ sys, const float* __restrict__ pv,
   __shared__ float2 sm[kMvWarps][RB];
   __shared__ double spq[RB];
   wait_previous(false);
+  pv = fresh(pv);
+  plo = fresh(plo);
+  p64 = fresh(p64);
+  st = fresh(st);
   clock_start(clock);
   const int c = blockIdx.y;
   const int n = (st && st[c].done) ? 0 : sys[c].n;  // converged: only the zero partial
@@ -596,8 +609,8 @@ k_matvec_ragged(const SysCol* __restrict__ sys, const float* __restrict__ pv,
 #pragma unroll
     for (int i = 0; i < RB; ++i)
       *reinterpret_cast<float4*>(nx[i]) = __ldcs(reinterpret_cast<const float4*>(erow[i] + cc));
-    *reinterpret_cast<float4*>(nh) = __ldg(reinterpret_cast<const float4*>(ph + cc));
-    *reinterpret_cast<float4*>(nl) = __ldg(reinterpret_cast<const float4*>(pl + cc));
+    *reinterpret_cast<float4*>(nh) = __ldca(reinterpret_cast<const float4*>(ph + cc));
+    *reinterpret_cast<float4*>(nl) = __ldca(reinterpret_cast<const float4*>(pl + cc));
   };
   if (warp < ngroups) load(warp);
   for (int g = warp; g < ngroups; g += kMvWarps) {
@@ -708,6 +721,13 @@ k_update(int n, int64_t ldv, int nrhs, ColState* st,
   __shared__ double s_alpha;
   __shared__ int s_done;
   wait_previous();
+  st = fresh(st);
+  x = fresh(x);
+  r = fresh(r);
+  z = fresh(z);
+  p = fresh(p);
+  q = fresh(q);
+  pq_part = fresh(pq_part);
   clock_stop(mv_clock);
   {
     const int col = blockIdx.y;  // one right-hand side per grid row
@@ -785,6 +805,10 @@ k_dc_apply(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st,
   __shared__ double sm[32 * 2];
   __shared__ double s_rsum;
   wait_previous();
+  st = fresh(st);
+  r = fresh(r);
+  z = fresh(z);
+  dots = fresh(dots);
   clock_start(clock);
   const int col = blockIdx.y;
   if (sys) {  // ragged batch: this column's system
@@ -864,6 +888,10 @@ k_dc_apply_ordered(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st
   extern __shared__ double2 s_e[];  // [kOrdCols][33]: (P entry, r there), a row a column of it
   __shared__ int64_t s_off[33];
   wait_previous();
+  st = fresh(st);
+  r = fresh(r);
+  z = fresh(z);
+  dots = fresh(dots);
   clock_start(clock);
   const int col = blockIdx.y;
   if (!first && st[col].done != 0) return;  // converged column (uniform per block)
@@ -989,11 +1017,16 @@ struct StepArgs {
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
-k_step(int n, int64_t ldv, int nrhs, const StepArgs a, const double* __restrict__ z,
+k_step(int n, int64_t ldv, int nrhs, StepArgs a, const double* __restrict__ z,
        double* __restrict__ p, T* __restrict__ pv, T* __restrict__ plo, float* __restrict__ xt) {
   __shared__ ColState s_next;
   __shared__ double s_sum[3];
   wait_previous();
+  a.dots = fresh(a.dots);
+  a.rz.p = fresh(a.rz.p);
+  a.cur = fresh(a.cur);
+  z = fresh(z);
+  p = fresh(p);
   clock_stop(a.dc_clock);
   const int col = blockIdx.y;
   const int warp = threadIdx.x >> 5;
@@ -1077,6 +1110,11 @@ k_dc_apply_t(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st,
              const double* __restrict__ rsum_part, int nparts, double* __restrict__ dpart,
              int first, Clock* clock) {
   wait_previous();
+  st = fresh(st);
+  rt = fresh(rt);
+  r = fresh(r);
+  z = fresh(z);
+  rsum_part = fresh(rsum_part);
   clock_start(clock);
   __shared__ double s_gsum[kFastCols];
   __shared__ int s_active[kFastCols];
@@ -1137,7 +1175,7 @@ k_dc_apply_t(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st,
         const int ik = __shfl_sync(0xffffffffu, id[k >> 2], 8 * (k & 3) + slot);
         const float pk = __shfl_sync(0xffffffffu, pe[k >> 2], 8 * (k & 3) + slot);
         if (src < left) {
-          const float4 rv = __ldg(reinterpret_cast<const float4*>(rg + (int64_t)ik * kFastCols));
+          const float4 rv = __ldca(reinterpret_cast<const float4*>(rg + (int64_t)ik * kFastCols));
           acc.x = fmaf(pk, rv.x, acc.x);
           acc.y = fmaf(pk, rv.y, acc.y);
           acc.z = fmaf(pk, rv.z, acc.z);

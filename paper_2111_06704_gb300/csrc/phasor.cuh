@@ -118,8 +118,8 @@ struct AxisPhasors {
 
   __device__ __forceinline__ double2 phasor(const double2* __restrict__ row, int h, int k,
                                             int l) const {
-    double2 a = __ldg(row + off[0] + abs(h)), b = __ldg(row + off[1] + abs(k)),
-            c = __ldg(row + off[2] + abs(l));
+    double2 a = __ldca(row + off[0] + abs(h)), b = __ldca(row + off[1] + abs(k)),
+            c = __ldca(row + off[2] + abs(l));
     if (h < 0) a.y = -a.y;
     if (k < 0) b.y = -b.y;
     if (l < 0) c.y = -c.y;

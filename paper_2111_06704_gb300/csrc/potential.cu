@@ -327,7 +327,7 @@ k_ion_sf_f64(const double2* __restrict__ axis, const AxisPhasors ap, int64_t coo
       if (t >= cnt) continue;
       const double2* row = tab + (size_t)(t0 + t) * ap.len;
       const int2 hk = s_hk[c];
-      double2 x = __ldg(row + ap.off[0] + abs(hk.x)), y = __ldg(row + ap.off[1] + abs(hk.y));
+      double2 x = __ldca(row + ap.off[0] + abs(hk.x)), y = __ldca(row + ap.off[1] + abs(hk.y));
       if (hk.x < 0) x.y = -x.y;
       if (hk.y < 0) y.y = -y.y;
       const double qt = q[t0 + t];
@@ -336,7 +336,7 @@ k_ion_sf_f64(const double2* __restrict__ axis, const AxisPhasors ap, int64_t coo
     __syncwarp();
 #pragma unroll 4
     for (int t = 0; t < cnt; ++t) {
-      const double2 z = __ldg(tab + (size_t)(t0 + t) * ap.len + ap.off[2] + en.l);
+      const double2 z = __ldca(tab + (size_t)(t0 + t) * ap.len + ap.off[2] + en.l);
       const double2 w = s_ab[warp][mine][t];
       ac = fma(w.x, z.x, ac);
       bd = fma(w.y, z.y, bd);
@@ -397,7 +397,7 @@ k_bsol_kspace_f64(const double* __restrict__ A, int n, int64_t lda, const double
 #pragma unroll
     for (int r = 0; r < kF64Frames; ++r) {
       if (r >= nf) break;
-      const double2 vv = __ldg(reinterpret_cast<const double2*>(v + (int64_t)(f0 + r) * lda + c));
+      const double2 vv = __ldca(reinterpret_cast<const double2*>(v + (int64_t)(f0 + r) * lda + c));
 #pragma unroll
       for (int i = 0; i < kF64Rows; ++i)
         acc[i][r] = fma(av[i].y, vv.y, fma(av[i].x, vv.x, acc[i][r]));
@@ -450,6 +450,7 @@ k_bsol_kspace_f32(const float* __restrict__ A, int64_t lda, const float2* __rest
   stamp_time(stamp);
   v = fresh(v);
   vhead = fresh(vhead);
+  bsol = fresh(bsol);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sub = warp % WS;
   const int row0 = (blockIdx.x * (kKsWarps / WS) + warp / WS) * kKsRows;
@@ -477,10 +478,10 @@ k_bsol_kspace_f32(const float* __restrict__ A, int64_t lda, const float2* __rest
       for (int p = 0; p < NP; ++p) {
         float va[4], vb[4];
         *reinterpret_cast<float4*>(va) =
-            __ldg(reinterpret_cast<const float4*>(v + frame[2 * p] * lda + c));
+            __ldca(reinterpret_cast<const float4*>(v + frame[2 * p] * lda + c));
         *reinterpret_cast<float4*>(vb) =
             NF == 1 ? *reinterpret_cast<float4*>(va)
-                    : __ldg(reinterpret_cast<const float4*>(v + frame[2 * p + 1] * lda + c));
+                    : __ldca(reinterpret_cast<const float4*>(v + frame[2 * p + 1] * lda + c));
 #pragma unroll
         for (int i = 0; i < kKsRows; ++i) {
           float2 s = make_float2(0.f, 0.f);
@@ -501,9 +502,9 @@ k_bsol_kspace_f32(const float* __restrict__ A, int64_t lda, const float2* __rest
       a[i] = __ldg(reinterpret_cast<const float4*>(Ahead + arow[i] * ldh + c));
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
-      const float4 x = __ldg(reinterpret_cast<const float4*>(vhead + frame[2 * p] * ldh + c));
+      const float4 x = __ldca(reinterpret_cast<const float4*>(vhead + frame[2 * p] * ldh + c));
       const float4 y =
-          NF == 1 ? x : __ldg(reinterpret_cast<const float4*>(vhead + frame[2 * p + 1] * ldh + c));
+          NF == 1 ? x : __ldca(reinterpret_cast<const float4*>(vhead + frame[2 * p + 1] * ldh + c));
 #pragma unroll
       for (int i = 0; i < kKsRows; ++i)
 #pragma unroll

@@ -30,11 +30,17 @@ __device__ __forceinline__ void end_after_previous(bool late) {
   if (late && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) wait_previous(false);
 }
 
-// p, for reads that must not move above the wait before (read-only loads may otherwise).
+// p, for what another kernel of the chain writes: nothing is read through the result before the
+// point of the call (after the wait).  Through a const __restrict__ parameter, or a __restrict__
+// one that the wait does not name, the compiler may move a load above the wait, and may take the
+// non-coherent path, which is for data that nothing writes while this kernel is resident; these
+// are still being written while it waits.  For the same reason such data are read by plain loads or
+// __ldca, never __ldg, which is for the constant operands (E, P, the tables).
 template <typename T>
 __device__ __forceinline__ T* fresh(T* p) {
-  asm volatile("" : "+l"(p)::"memory");
-  return p;
+  size_t g = __cvta_generic_to_global(p);  // (stays a global address for the compiler)
+  asm volatile("" : "+l"(g)::"memory");
+  return (T*)__cvta_global_to_generic(g);
 }
 
 template <typename... P, typename... A>

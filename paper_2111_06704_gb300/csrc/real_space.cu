@@ -360,8 +360,8 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
         }
       }
     } else {
-      const uint4 w0 = __ldg(reinterpret_cast<const uint4*>(ions + ion));
-      const int4 w1 = __ldg(reinterpret_cast<const int4*>(ions + ion) + 1);
+      const uint4 w0 = __ldca(reinterpret_cast<const uint4*>(ions + ion));
+      const int4 w1 = __ldca(reinterpret_cast<const int4*>(ions + ion) + 1);
       const uint32_t uI[3] = {w0.x, w0.y, w0.z};
       const int32_t lI[3] = {w1.x, w1.y, w1.z};
       const int32_t la[3] = {at.xl, at.yl, at.zl};
@@ -420,7 +420,7 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
   // a far image, in plain float from the fixed-point difference of the nearest image; one
   // that the screen's offsets took for far and this r^2 does not goes the near way
   auto evaluate_far = [&](uint32_t entry) {
-    const uint4 w = __ldg(reinterpret_cast<const uint4*>(ions + base0 + (entry & ((1u << kBits) - 1))));
+    const uint4 w = __ldca(reinterpret_cast<const uint4*>(ions + base0 + (entry & ((1u << kBits) - 1))));
     float d0 = (float)(int32_t)(ui[0] - w.x) * a.fs[0], d1 = (float)(int32_t)(ui[1] - w.y) * a.fs[1],
           d2 = (float)(int32_t)(ui[2] - w.z) * a.fs[2];
     float m2;
@@ -479,7 +479,7 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
         uint4 w = make_uint4(0u, 0u, 0u, 0u);
         bool in = lane < m;
         float dx[3];
-        if (in) w = __ldg(reinterpret_cast<const uint4*>(ions + t + lane));
+        if (in) w = __ldca(reinterpret_cast<const uint4*>(ions + t + lane));
         const uint32_t uI[3] = {w.x, w.y, w.z};
         float far2 = 0.f;
 #pragma unroll
@@ -523,7 +523,7 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
         }
       } else {
         for (int c = 0; c < m; ++c) {
-          const uint4 w = __ldg(reinterpret_cast<const uint4*>(ions + t + c));
+          const uint4 w = __ldca(reinterpret_cast<const uint4*>(ions + t + c));
           const float x = (float)(int32_t)(ui[0] - w.x) * a.fs[0];
           const float y = (float)(int32_t)(ui[1] - w.y) * a.fs[1];
           const float z = (float)(int32_t)(ui[2] - w.z) * a.fs[2];
