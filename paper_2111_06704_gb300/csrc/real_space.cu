@@ -124,7 +124,9 @@ __device__ __forceinline__ void split(double v, float& h, float& l) {
 constexpr int kPrepThreads = 128;
 
 // The ions' fixed-point coordinates (the phases of every k-vector use them), their records,
-// and the block's sums of q z and q for the dipole term and Q^sol: sums[frame][block].
+// and the block's sums of q z and q for the dipole term and Q^sol: sums[frame][block].  Fixed point
+// has no place for a coordinate that is not finite: the frame's sum of q z is NaN then, and so are
+// its b.
 __global__ void __launch_bounds__(kPrepThreads)
 k_ion_prepare(const double* __restrict__ ion_xyz, const double* __restrict__ ion_q, int n_ion,
               double lx, double ly, double lz, uint32_t* __restrict__ sion,
@@ -137,16 +139,16 @@ k_ion_prepare(const double* __restrict__ ion_xyz, const double* __restrict__ ion
   if (t < n_ion) {
     const size_t e = (size_t)f * n_ion + t;
     IonRec r;
-    const double z = ion_xyz[3 * e + 2], q = ion_q[e];
-    fixed64(ion_xyz[3 * e], lx, r.x, r.xl);
-    fixed64(ion_xyz[3 * e + 1], ly, r.y, r.yl);
+    const double x = ion_xyz[3 * e], y = ion_xyz[3 * e + 1], z = ion_xyz[3 * e + 2], q = ion_q[e];
+    fixed64(x, lx, r.x, r.xl);
+    fixed64(y, ly, r.y, r.yl);
     fixed64(z, lz, r.z, r.zl);
     split(q, r.qh, r.ql);
     sion[3 * e] = r.x;
     sion[3 * e + 1] = r.y;
     sion[3 * e + 2] = r.z;
     rec[e] = r;
-    qz = q * z;
+    qz = isfinite(x) && isfinite(y) && isfinite(z) ? q * z : nan("");
     qs = q;
   }
   for (int o = 16; o; o >>= 1) {
