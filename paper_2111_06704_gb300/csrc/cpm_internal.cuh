@@ -379,7 +379,8 @@ struct SolveArgs {
   const SysCol* sys = nullptr;  // ragged batch: device array [nrhs], one system per column
   bool ordered = false;          // one column: every sum in the build's fixed order
   bool timed = true;             // record the solve's device timings (events of the context)
-  // cluster path: an event to record right before its launch, and its iterations' time
+  // the tuner's: an event to record right before the first launch, and (cluster path) the
+  // iterations' time
   cudaEvent_t begin = nullptr;
   float* loop_ms = nullptr;
 };
