@@ -159,9 +159,10 @@ int copy_out(Ctx* c, void* dst, const void* dev, size_t bytes) {
                     "copy out");
 }
 
-// Per-axis phasor tables (FP64 storage): the layout of a point's entries, and how many
-// frames' ions are tabulated at a time so that the tables stay within kAxisBytes.
-constexpr size_t kAxisBytes = 512ull << 20;
+// Per-axis phasor tables (FP64 storage): the layout of a point's entries, and the points tabulated
+// at a time so that the tables stay within kAxisBytes, or, where that much memory cannot be had,
+// kAxisSmall (16,000 points of the 512-atom cell).
+constexpr size_t kAxisBytes = 512ull << 20, kAxisSmall = 32ull << 20;
 
 AxisPhasors axis_phasors(const Ctx* c) {
   AxisPhasors ap;
@@ -172,9 +173,29 @@ AxisPhasors axis_phasors(const Ctx* c) {
   return ap;
 }
 
-int axis_frames(const AxisPhasors& ap, int frames, int n_ion) {
-  const size_t per = (size_t)std::max(n_ion, 1) * ap.len * sizeof(double2);
-  return (int)std::max<size_t>(1, std::min<size_t>((size_t)frames, kAxisBytes / per));
+// Whole frames of n_ion points where one fits, else some of a frame's points.
+struct AxisChunk {
+  int frames, points;
+};
+
+AxisChunk axis_chunk(const AxisPhasors& ap, int frames, int n_ion, size_t bytes) {
+  const size_t points = std::max<size_t>(256, bytes / (ap.len * sizeof(double2)));
+  const size_t per = (size_t)std::max(n_ion, 1);
+  if (points < per) return {1, (int)points};
+  return {(int)std::min<size_t>((size_t)frames, points / per), (int)per};
+}
+
+// ws_pot for a call's usual form, or, where that much cannot be had, for its small one (not tried
+// again at every call: until the workspace is released or the next build).
+int reserve_potential(Ctx* c, size_t usual, size_t least, bool* small) {
+  *small = c->pot_refused && usual >= c->pot_refused && c->ws_pot.bytes < usual;
+  if (!*small) {
+    const int st = buf_reserve(c, &c->ws_pot, usual);
+    if (st != CPM_ENOMEM) return st;
+    c->pot_refused = usual;
+    *small = true;
+  }
+  return buf_reserve(c, &c->ws_pot, least);
 }
 
 Geometry geometry(const Ctx* c) {
@@ -365,6 +386,7 @@ void release_workspace(Ctx* c) {
                &c->ws_out0, &c->ws_out1, &c->ws_pot, &c->ws_guess, &c->ws_feat, &c->ws_grad, &c->ws_cluster,
                &c->tc_tiles};
   for (Buf* b : ws) buf_free(c, b);
+  c->pot_refused = 0;
   if (c->pinned) cudaFreeHost(c->pinned);
   c->pinned = nullptr;
   c->tc_tiles_nt = 0;
@@ -626,6 +648,7 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha) {
   c->shells_ready = false;
   c->gcd_m = 0;  // the electrodes' solves and S belong to the previous E
   c->smat_ready = false;
+  c->pot_refused = 0;
   cudaStream_t s = c->stream;
   const bool f64 = c->fp64();
   int st;
@@ -1024,17 +1047,28 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   const size_t ubytes = up((size_t)frames * std::max(n_ion, 1) * 3 * sizeof(uint32_t));
   int dev_sms = 1;
   cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, c->device);
-  const int nsplit = !c->A.ptr && !f64
-                         ? bsol_direct_splits(n, frames, c->mpad, c->kh, std::max(dev_sms, 1))
-                         : 1;
-  const size_t sbytes = nsplit > 1 ? (size_t)nsplit * kbytes : 0;
-  // FP64 storage: the ions' per-axis phasors, at most kAxisBytes of frames at a time
+  // The shares, the phasors tabulated at a time and the real-space part's lists are as many as
+  // serve the call best; where the memory for them cannot be had, one share, few phasors, no lists.
   const AxisPhasors ap = axis_phasors(c);
-  const int fchunk = axis_frames(ap, frames, n_ion);
-  const size_t abytes = f64 ? up((size_t)fchunk * std::max(n_ion, 1) * ap.len * sizeof(double2)) : 0;
-  const RealPlan rp = real_plan(n, frames, n_ion, geometry(c), f64, std::max(dev_sms, 1));
-  if ((st = buf_reserve(c, &c->ws_pot, vbytes + hbytes + kbytes + ubytes + sbytes + abytes + rp.bytes)))
-    return st;
+  int nsplit;
+  AxisChunk ck;
+  RealPlan rp;
+  size_t sbytes, abytes;
+  auto form = [&](bool small) {
+    nsplit = !c->A.ptr && !f64 && !small
+                 ? bsol_direct_splits(n, frames, c->mpad, c->kh, std::max(dev_sms, 1))
+                 : 1;
+    sbytes = nsplit > 1 ? (size_t)nsplit * kbytes : 0;
+    ck = f64 ? axis_chunk(ap, frames, n_ion, small ? kAxisSmall : kAxisBytes)
+             : AxisChunk{frames, std::max(n_ion, 1)};
+    abytes = f64 ? up((size_t)ck.frames * ck.points * ap.len * sizeof(double2)) : 0;
+    rp = real_plan(n, frames, n_ion, geometry(c), f64, std::max(dev_sms, 1), small);
+    return vbytes + hbytes + kbytes + ubytes + sbytes + abytes + rp.bytes;
+  };
+  const size_t least = form(true), usual = form(false);
+  bool small;
+  if ((st = reserve_potential(c, usual, least, &small))) return st;
+  if (small) form(true);
   if (!f64 && !c->turn.ptr) {
     if ((st = buf_alloc(c, &c->turn, 4096 * 4 * sizeof(float)))) return st;
     launch_turn_table(c->turn.ptr, s);
@@ -1056,7 +1090,7 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   }
   auto at = [&](int k) { return tm ? tm + k : nullptr; };
   // ion records (FP64: and axis phasors) -> real-space sums, and beside them structure factors
-  // -> k-space -> b; frames past the first chunk have their phasors and factors after that.
+  // -> k-space -> b; points past the first chunk have their phasors and factors after that.
   // 512 atoms, 200 ions, one frame: 74 -> 50 us in float storage (with the events between the
   // kernels gone), 116 -> 85 us in FP64; larger calls gain the kernels' last waves (26,600 atoms,
   // 16 frames of 5,000 ions 5.48 -> 5.11 ms)
@@ -1064,23 +1098,27 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
     launch_ion_prepare(dx, dq, frames, n_ion, geometry(c), sion, rp, rscratch, at(0), s);
   else if ((st = cuda_check(c, cudaMemsetAsync(v, 0, vbytes + hbytes, s), "v zero")))
     return st;
-  auto axis_frames_from = [&](int f0) {
-    launch_axis_phasors(dx + (size_t)f0 * n_ion * 3, nullptr,
-                        (int64_t)std::min(fchunk, frames - f0) * n_ion, c->p.box, ap, axis, s);
+  auto axis_from = [&](int f0, int i0) {  // (whole frames of all ions, or one frame's)
+    launch_axis_phasors(dx + ((size_t)f0 * n_ion + i0) * 3, nullptr,
+                        (int64_t)std::min(ck.frames, frames - f0) * std::min(ck.points, n_ion - i0),
+                        c->p.box, ap, axis, s);
   };
-  if (n_ion > 0 && f64) axis_frames_from(0);
+  if (n_ion > 0 && f64) axis_from(0, 0);
   launch_bsol_real((const double*)c->xyz.ptr, (const double*)c->alpha.ptr,
                    (const uint32_t*)c->sfix.ptr, c->atoms.ptr, c->htab.ptr, n, dx, dq, frames,
                    n_ion, geometry(c), f64, rp, rscratch, s);
-  for (int f0 = 0; n_ion > 0 && f0 < frames; f0 += f64 ? fchunk : frames) {
-    const int nf = f64 ? std::min(fchunk, frames - f0) : frames;
-    if (f0 > 0) axis_frames_from(f0);
-    launch_ion_structure_factor(f64, axis, ap, sion, n_ion, dq + (size_t)f0 * n_ion, nf, n_ion,
-                                SfList{c->sflist.ptr, c->n_sflist}, (const int*)c->hkl.ptr,
-                                (const double*)c->sqw.ptr, c->m, c->mpad, c->kh, c->turn.ptr,
-                                (char*)v + (size_t)f0 * 2 * c->mpad * c->esz(), vh,
-                                std::max(dev_sms, 1), f0 == 0, f0 == 0 ? at(1) : nullptr, s);
-  }
+  for (int f0 = 0; f0 < frames; f0 += ck.frames)
+    for (int i0 = 0; i0 < n_ion; i0 += ck.points) {
+      const int nf = std::min(ck.frames, frames - f0), ni = std::min(ck.points, n_ion - i0);
+      const bool first = f0 == 0 && i0 == 0;
+      if (!first) axis_from(f0, i0);
+      launch_ion_structure_factor(f64, axis, ap, sion, ni, dq + (size_t)f0 * n_ion + i0, n_ion, nf,
+                                  ni, i0 > 0, SfList{c->sflist.ptr, c->n_sflist},
+                                  (const int*)c->hkl.ptr, (const double*)c->sqw.ptr, c->m, c->mpad,
+                                  c->kh, c->turn.ptr,
+                                  (char*)v + (size_t)f0 * 2 * c->mpad * c->esz(), vh,
+                                  std::max(dev_sms, 1), first, first ? at(1) : nullptr, s);
+    }
   launch_bsol_kspace(f64, c->A.ptr, c->Ahead.ptr, n, c->mpad, c->kh, v, vh, frames, bk,
                      (const uint32_t*)c->sfix.ptr, (const int*)c->hkl.ptr,
                      (const double*)c->sqw.ptr, c->turn.ptr, nsplit, spart, std::max(dev_sms, 1),
@@ -1132,7 +1170,7 @@ int cpm_ion_forces(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   // FP64 storage takes its phasors from per-axis ones of the ions (at most kAxisBytes of
   // frames at a time) and of the electrode
   const AxisPhasors ap = axis_phasors(c);
-  const int fchunk = f64 ? axis_frames(ap, frames, n_ion) : frames;
+  const int fchunk = f64 ? axis_chunk(ap, frames, n_ion, kAxisBytes).frames : frames;
   int dev_sms = 1;
   cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, c->device);
   const ForceSplits sp = force_splits(f64, n, fchunk, n_ion, c->mpad, c->kh, std::max(dev_sms, 1));
@@ -1181,7 +1219,7 @@ int cpm_ion_forces(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
                       (double*)(base + orl), (double2*)(base + os), !f64, s);
     // the electrode's charge-weighted structure factors: the ions' kernel run over the
     // electrode atoms (the same coordinates every frame)
-    launch_ion_structure_factor(f64, ax_el, ap, (const uint32_t*)c->sfix.ptr, 0, fq, nf, n,
+    launch_ion_structure_factor(f64, ax_el, ap, (const uint32_t*)c->sfix.ptr, 0, fq, n, nf, n, false,
                                 SfList{c->sflist.ptr, c->n_sflist}, (const int*)c->hkl.ptr,
                                 (const double*)c->sqw.ptr, c->m, c->mpad, c->kh,
                                 c->turn.ptr, v, vh, std::max(dev_sms, 1), !f64, nullptr, s);

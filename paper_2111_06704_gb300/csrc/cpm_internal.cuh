@@ -162,6 +162,7 @@ struct Ctx {
   std::vector<int> kv_hkl;    // the k-vector table (host), made on the first build
   std::vector<double> kv_w;
   Buf ws_solve, ws_in0, ws_in1, ws_in2, ws_out0, ws_out1, ws_pot, ws_guess, ws_feat, ws_grad;
+  size_t pot_refused = 0;  // the smallest ws_pot that could not be had (0: none yet)
   void* pinned = nullptr;  // host memory the solves poll into (pinned_reserve)
   size_t pinned_bytes = 0;
   Buf ws_cluster;  // per-column results of the cluster-resident solve
@@ -280,14 +281,15 @@ void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
                          const double L[3], const AxisPhasors& ap, double2* out,
                          cudaStream_t s);
 // Structure factors of the points of `frames` frames, coord_stride points apart (0: every
-// frame has the same coordinates).  FP64 storage takes them from axis, float storage from
-// the fixed-point coordinates sion.  late: the kernel before is launched by launch_next and
+// frame has the same coordinates) and their charges charge_stride.  FP64 storage takes the points
+// from axis, float storage from the fixed-point coordinates sion; add (FP64): the sums are added to
+// those of the points before.  late: the kernel before is launched by launch_next and
 // waits for all that this one reads, so that the two may run side by side.  stamp (if not NULL):
 // the time at its start.
 void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhasors& ap,
                                  const uint32_t* sion, int64_t coord_stride,
-                                 const double* ion_q, int frames, int n_ion,
-                                 const SfList& kl, const int* hkl,
+                                 const double* ion_q, int64_t charge_stride, int frames, int n_ion,
+                                 bool add, const SfList& kl, const int* hkl,
                                  const double* sqw, int m, int mpad, int kh, const void* turn,
                                  void* v, void* vhead, int sms, bool late,
                                  unsigned long long* stamp, cudaStream_t s);
@@ -308,7 +310,9 @@ struct RealPlan {
   // scratch layout: ion records | block sums | partials | far terms | their counts
   size_t o_sums, o_part, o_far, o_far_count, bytes;
 };
-RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, bool fp64, int sms);
+// small: with the least scratch
+RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, bool fp64, int sms,
+                   bool small);
 size_t h_table_bytes();
 const void* h_table_host();     // erfc(sqrt s) / sqrt s, for a device copy
 size_t atom_record_bytes(int n);

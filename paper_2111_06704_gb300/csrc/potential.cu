@@ -95,7 +95,7 @@ __device__ __forceinline__ void sincos_t64x2(uint32_t p0, uint32_t p1, const flo
 // the rest of the grid), so its blocks always split the ions eight ways, and come first.
 __global__ void __launch_bounds__(kSfWarps * 32)
 k_ion_sf_f32(const uint32_t* __restrict__ sion, int64_t coord_stride,
-             const double* __restrict__ ion_q, int n_ion, const SfPair* __restrict__ pairs,
+             const double* __restrict__ ion_q, int64_t charge_stride, int n_ion, const SfPair* __restrict__ pairs,
              int npairs, const int* __restrict__ hkl, const double* __restrict__ sqw, int mpad,
              int kh, int tail_shares, int head_blocks, const float4* __restrict__ turn,
              float* __restrict__ vout, float2* __restrict__ vhead, bool late,
@@ -114,7 +114,7 @@ k_ion_sf_f32(const uint32_t* __restrict__ sion, int64_t coord_stride,
   const int shares = head ? kSfWarps : tail_shares;
   const int share = warp % shares, per = kSfWarps / shares;  // groups of 32 threads a block
   const uint32_t* fx = sion + (size_t)f * coord_stride * 3;
-  const double* q = ion_q + (size_t)f * n_ion;
+  const double* q = ion_q + (size_t)f * charge_stride;
   float* v = vout + (size_t)f * 2 * mpad;
   const int at = ((int)blockIdx.x - (head ? 0 : head_blocks)) * per * 32 +
                  (warp / shares) * 32 + lane;
@@ -292,7 +292,8 @@ constexpr int kSf64Batch = 8;  // points a warp takes at a time
 
 __global__ void __launch_bounds__(kSf64Warps * 32)
 k_ion_sf_f64(const double2* __restrict__ axis, const AxisPhasors ap, int64_t coord_stride,
-             const double* __restrict__ ion_q, int n_ion, const SfEntry* __restrict__ entries,
+             const double* __restrict__ ion_q, int64_t charge_stride, int n_ion, bool add,
+             const SfEntry* __restrict__ entries,
              int nentries, const double* __restrict__ sqw, int m, int mpad,
              double* __restrict__ vout, bool late, unsigned long long* stamp) {
   __shared__ double2 s_ab[kSf64Warps][32][kSf64Batch];
@@ -301,6 +302,7 @@ k_ion_sf_f64(const double2* __restrict__ axis, const AxisPhasors ap, int64_t coo
   if (!late) wait_previous(false);
   stamp_time(stamp);
   axis = fresh(axis);
+  vout = fresh(vout);
   const int f = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double* v = vout + (size_t)f * 2 * mpad;
@@ -317,7 +319,7 @@ k_ion_sf_f64(const double2* __restrict__ axis, const AxisPhasors ap, int64_t coo
   if (warp == 0) s_hk[mine] = make_int2(en.h, en.k);
   __syncthreads();
   const double2* tab = axis + (size_t)f * coord_stride * ap.len;
-  const double* q = ion_q + (size_t)f * n_ion;
+  const double* q = ion_q + (size_t)f * charge_stride;
   double ac = 0.0, bd = 0.0, ad = 0.0, bc = 0.0;
   for (int t0 = warp * kSf64Batch; t0 < n_ion; t0 += kSf64Warps * kSf64Batch) {
     const int cnt = min(kSf64Batch, n_ion - t0);
@@ -363,8 +365,9 @@ k_ion_sf_f64(const double2* __restrict__ axis, const AxisPhasors ap, int64_t coo
     if (k < 0) continue;
     const double w = sqw[k];
     const size_t kcol = 128 * (size_t)(k >> 6) + (k & 63);
-    v[kcol] = w * (u == 0 ? ac - bd : ac + bd);
-    v[kcol + 64] = w * (u == 0 ? ad + bc : bc - ad);
+    const double re = w * (u == 0 ? ac - bd : ac + bd), im = w * (u == 0 ? ad + bc : bc - ad);
+    v[kcol] = add ? v[kcol] + re : re;
+    v[kcol + 64] = add ? v[kcol + 64] + im : im;
   }
   end_after_previous(late);
 }
@@ -755,15 +758,15 @@ void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
 
 void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhasors& ap,
                                  const uint32_t* sion, int64_t coord_stride,
-                                 const double* ion_q, int frames, int n_ion,
-                                 const SfList& kl, const int* hkl,
+                                 const double* ion_q, int64_t charge_stride, int frames, int n_ion,
+                                 bool add, const SfList& kl, const int* hkl,
                                  const double* sqw, int m, int mpad, int kh, const void* turn,
                                  void* v, void* vhead, int sms, bool late,
                                  unsigned long long* stamp, cudaStream_t s) {
   if (fp64) {
     launch_next(k_ion_sf_f64, dim3(std::max(1, (kl.entries + 31) / 32), frames), kSf64Warps * 32, 0,
-                s, axis, ap, coord_stride, ion_q, n_ion, (const SfEntry*)kl.list, kl.entries, sqw, m,
-                mpad, (double*)v, late, stamp);
+                s, axis, ap, coord_stride, ion_q, charge_stride, n_ion, add, (const SfEntry*)kl.list,
+                kl.entries, sqw, m, mpad, (double*)v, late, stamp);
   } else {
     // warps of a block split the ions until the chip's warps are busy (24 resident an SM),
     // each with at least four blocks of eight ions, and, to even out the last wave, up to four
@@ -782,7 +785,7 @@ void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhaso
     }
     const int per = 32 * (kSfWarps / shares), hb = (kh + 31) / 32;
     launch_next(k_ion_sf_f32, dim3(hb + (npairs + per - 1) / per, frames), kSfWarps * 32, 0, s, sion,
-                coord_stride, ion_q, n_ion, pairs, npairs, hkl, sqw, mpad, kh, shares, hb,
+                coord_stride, ion_q, charge_stride, n_ion, pairs, npairs, hkl, sqw, mpad, kh, shares, hb,
                 (const float4*)turn, (float*)v, (float2*)vhead, late, stamp);
   }
 }

@@ -664,7 +664,8 @@ void launch_atom_records(const double* xyz, const double* alpha, int n, const Ge
 constexpr int kRealChainIons = 1200;
 constexpr size_t kRealFarBytes = (size_t)192 << 20;
 
-RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, bool fp64, int sms) {
+RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, bool fp64, int sms,
+                   bool small) {
   RealPlan p;
   const int64_t groups = (int64_t)((n + 31) / 32) * frames;
   p.shares = p.grid_shares = 1;
@@ -681,7 +682,7 @@ RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, bool fp64,
     const double mean = n_ion * (4.0 / 3.0 * kPi * geo.rc * geo.rc * geo.rc) /
                         (geo.L[0] * geo.L[1] * geo.L[2]);
     const double cap = 4.0 * mean / nsh + 16.0;
-    if (cap * nsh * frames * n * sizeof(float) <= (double)kRealFarBytes) {
+    if (!small && cap * nsh * frames * n * sizeof(float) <= (double)kRealFarBytes) {
       p.far_cap = (int)cap;
     } else {
       p.shares = p.grid_shares = 1;
