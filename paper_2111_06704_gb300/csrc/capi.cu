@@ -161,8 +161,8 @@ int copy_out(Ctx* c, void* dst, const void* dev, size_t bytes) {
 
 // Per-axis phasor tables (FP64 storage): the layout of a point's entries, and the points tabulated
 // at a time so that the tables stay within kAxisBytes, or, where that much memory cannot be had,
-// kAxisSmall (16,000 points of the 512-atom cell).
-constexpr size_t kAxisBytes = 512ull << 20, kAxisSmall = 32ull << 20;
+// kAxisSmall (3,600 points of the 512-atom cell).
+constexpr size_t kAxisBytes = 512ull << 20, kAxisSmall = 4ull << 20;
 
 AxisPhasors axis_phasors(const Ctx* c) {
   AxisPhasors ap;
@@ -1167,32 +1167,46 @@ int cpm_ion_forces(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
       (st = stage_out(c, &c->ws_out0, f_out, (size_t)frames * n_ion * 3 * sizeof(double),
                       (void**)&dout)))
     return st;
-  // FP64 storage takes its phasors from per-axis ones of the ions (at most kAxisBytes of
-  // frames at a time) and of the electrode
+  // FP64 storage takes its phasors from per-axis ones of the ions (at most kAxisBytes of them at a
+  // time: frames, or a frame's ions in parts) and of the electrode (all atoms at once, or, where
+  // the memory cannot be had, in parts whose structure factors are added)
   const AxisPhasors ap = axis_phasors(c);
-  const int fchunk = f64 ? axis_chunk(ap, frames, n_ion, kAxisBytes).frames : frames;
   int dev_sms = 1;
   cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, c->device);
-  const ForceSplits sp = force_splits(f64, n, fchunk, n_ion, c->mpad, c->kh, std::max(dev_sms, 1));
-  // scratch, for the frames of one pass: structure factors v [frames][2 mpad] (storage type) |
-  // v_head [frames][2 kh] | fixed-point ion coordinates [frames][n_ion][3] | the shares'
-  // gradients [k_total + real][frames][n_ion][3] and slab sums [real][frames] | per-axis
+  // scratch, for the ions of one pass: structure factors v [frames][2 mpad] (storage type) |
+  // v_head [frames][2 kh] | fixed-point ion coordinates [frames][ions][3] | the shares'
+  // gradients [k_total + real][frames][ions][3] and slab sums [real][frames] | per-axis
   // phasors of the ions and the electrode
-  size_t off = 0;
-  auto take = [&](size_t b) {
-    const size_t o = off;
-    off += (b + 255) & ~size_t(255);
-    return o;
+  AxisChunk ck;
+  int atoms;  // of the electrode's parts
+  ForceSplits sp;
+  size_t ov, oh, ou, ok, orl, os, oa, oe;
+  auto form = [&](bool small) {
+    size_t off = 0;
+    auto take = [&](size_t b) {
+      const size_t o = off;
+      off += (b + 255) & ~size_t(255);
+      return o;
+    };
+    const size_t axis_bytes = small ? kAxisSmall : kAxisBytes;
+    ck = f64 ? axis_chunk(ap, frames, n_ion, axis_bytes) : AxisChunk{frames, n_ion};
+    atoms = f64 && small ? axis_chunk(ap, 1, n, axis_bytes).points : n;
+    sp = force_splits(f64, n, ck.frames, ck.points, c->mpad, c->kh, std::max(dev_sms, 1));
+    const size_t ions = (size_t)ck.frames * ck.points, gbytes = ions * 3 * sizeof(double);
+    ov = take((size_t)ck.frames * 2 * c->mpad * c->esz());
+    oh = take((size_t)ck.frames * 2 * std::max(c->kh, 1) * sizeof(double));
+    ou = take(ions * 3 * sizeof(uint32_t));
+    ok = take(sp.k_total * gbytes);
+    orl = take(sp.real * gbytes);
+    os = take((size_t)sp.real * ck.frames * sizeof(double2));
+    oa = f64 ? take(ions * ap.len * sizeof(double2)) : 0;
+    oe = f64 ? take((size_t)atoms * ap.len * sizeof(double2)) : 0;
+    return off;
   };
-  const size_t gbytes = (size_t)fchunk * n_ion * 3 * sizeof(double);
-  const size_t ov = take((size_t)fchunk * 2 * c->mpad * c->esz()),
-               oh = take((size_t)fchunk * 2 * std::max(c->kh, 1) * sizeof(double)),
-               ou = take((size_t)fchunk * n_ion * 3 * sizeof(uint32_t)),
-               ok = take(sp.k_total * gbytes), orl = take(sp.real * gbytes),
-               os = take((size_t)sp.real * fchunk * sizeof(double2)),
-               oa = f64 ? take((size_t)fchunk * n_ion * ap.len * sizeof(double2)) : 0,
-               oe = f64 ? take((size_t)n * ap.len * sizeof(double2)) : 0;
-  if ((st = buf_reserve(c, &c->ws_pot, off))) return st;
+  const size_t least = form(true), usual = form(false);
+  bool small;
+  if ((st = reserve_potential(c, usual, least, &small))) return st;
+  if (small) form(true);
   if (!f64 && !c->turn.ptr) {
     if ((st = buf_alloc(c, &c->turn, 4096 * 4 * sizeof(float)))) return st;
     launch_turn_table(c->turn.ptr, s);
@@ -1202,33 +1216,44 @@ int cpm_ion_forces(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   void* vh = base + oh;
   uint32_t* sion = (uint32_t*)(base + ou);
   double2 *ax = (double2*)(base + oa), *ax_el = (double2*)(base + oe);
-  if (f64) launch_axis_phasors((const double*)c->xyz.ptr, nullptr, n, c->p.box, ap, ax_el, s);
-  for (int f0 = 0; f0 < frames; f0 += fchunk) {
-    const int nf = std::min(fchunk, frames - f0);
-    const double* fx = dx + (size_t)f0 * n_ion * 3;
+  auto electrode_from = [&](int a0) {
+    launch_axis_phasors((const double*)c->xyz.ptr + 3 * (size_t)a0, nullptr, std::min(atoms, n - a0),
+                        c->p.box, ap, ax_el, s);
+  };
+  if (f64 && atoms == n) electrode_from(0);
+  auto pass = [&](int f0, int i0) {  // (whole frames of all ions, or some of one frame's)
+    const int nf = std::min(ck.frames, frames - f0), ni = std::min(ck.points, n_ion - i0);
+    const size_t at = (size_t)f0 * n_ion + i0;
+    const double* fx = dx + at * 3;
     const double* fq = dqe + (size_t)f0 * n;
     // coordinates (FP64: and axis phasors) -> real-space shares, and beside them structure
     // factors -> k-space shares -> F.  FP64 factors come after: one block an SM, bound by the FP64
     // pipe; set up beside the real-space blocks, running or waiting, they crowd a few SMs (512
     // atoms: 88 us, 25 after)
-    launch_ion_fixed(fx, nf, n_ion, c->p.box, sion, s);
+    launch_ion_fixed(fx, nf, ni, c->p.box, sion, s);
     // (the forces' ion phases are those of the fixed-point coordinates in both storages)
-    if (f64) launch_axis_phasors(fx, sion, (int64_t)nf * n_ion, c->p.box, ap, ax, s);
+    if (f64) launch_axis_phasors(fx, sion, (int64_t)nf * ni, c->p.box, ap, ax, s);
     launch_force_real((const double*)c->xyz.ptr, (const double*)c->alpha.ptr,
-                      (const uint32_t*)c->sfix.ptr, n, fx, sion, nf, n_ion, fq, geometry(c), sp,
+                      (const uint32_t*)c->sfix.ptr, n, fx, sion, nf, ni, fq, geometry(c), sp,
                       (double*)(base + orl), (double2*)(base + os), !f64, s);
     // the electrode's charge-weighted structure factors: the ions' kernel run over the
     // electrode atoms (the same coordinates every frame)
-    launch_ion_structure_factor(f64, ax_el, ap, (const uint32_t*)c->sfix.ptr, 0, fq, n, nf, n, false,
-                                SfList{c->sflist.ptr, c->n_sflist}, (const int*)c->hkl.ptr,
-                                (const double*)c->sqw.ptr, c->m, c->mpad, c->kh,
-                                c->turn.ptr, v, vh, std::max(dev_sms, 1), !f64, nullptr, s);
-    launch_force_kspace_and_finish(f64, fx, dq + (size_t)f0 * n_ion, sion, nf, n_ion,
+    for (int a0 = 0; a0 < n; a0 += atoms) {
+      if (atoms < n) electrode_from(a0);
+      launch_ion_structure_factor(f64, ax_el, ap, (const uint32_t*)c->sfix.ptr, 0, fq + a0, n, nf,
+                                  std::min(atoms, n - a0), a0 > 0,
+                                  SfList{c->sflist.ptr, c->n_sflist}, (const int*)c->hkl.ptr,
+                                  (const double*)c->sqw.ptr, c->m, c->mpad, c->kh,
+                                  c->turn.ptr, v, vh, std::max(dev_sms, 1), !f64, nullptr, s);
+    }
+    launch_force_kspace_and_finish(f64, fx, dq + at, sion, nf, ni,
                                    (const int*)c->hkl.ptr, (const double*)c->sqw.ptr, c->mpad,
                                    c->kh, geometry(c), c->turn.ptr, v, vh, ax, ap, sp,
                                    (double*)(base + ok), (double*)(base + orl),
-                                   (double2*)(base + os), dout + (size_t)f0 * n_ion * 3, s);
-  }
+                                   (double2*)(base + os), dout + at * 3, s);
+  };
+  for (int f0 = 0; f0 < frames; f0 += ck.frames)
+    for (int i0 = 0; i0 < n_ion; i0 += ck.points) pass(f0, i0);
   if ((st = cuda_check(c, cudaGetLastError(), "ion forces"))) return st;
   if ((st = copy_out(c, f_out, dout, (size_t)frames * n_ion * 3 * sizeof(double)))) return st;
   return cuda_check(c, cudaStreamSynchronize(s), "ion forces sync");

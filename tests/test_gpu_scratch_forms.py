@@ -74,3 +74,16 @@ def test_potential(prec, cells, n_ion, frames, kw):
         return ctx.cpm_potential(xyz, q, el.chi)[0]
 
     _less_memory(prec, cells, call, **kw)
+
+
+@pytest.mark.parametrize("cells,n_ion,frames,kw", [
+    ((8, 8), 3000, 24, {}),
+    ((8, 5), 40011, 1, {}),  # one frame's ions in parts
+    ((26, 20), 7000, 3, {}),  # the electrode's atoms in parts
+])
+def test_forces(cells, n_ion, frames, kw):
+    def call(ctx, el):
+        xyz, q, qe = _ions(el, frames, n_ion)
+        return ctx.cpm_ion_forces(xyz, q, qe)
+
+    _less_memory("fp64", cells, call, **kw)
