@@ -693,8 +693,11 @@ int grad_async(cpm_ctx* c, const float* params, const float* norm, int bf16, int
                const AdamStep& adam) {
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-  const int blocks = (int)std::min<int64_t>((samples + kTs - 1) / kTs, std::max(sms, 1));
-  int st = buf_reserve(c, &c->ws_grad, (size_t)blocks * kPart * sizeof(double));
+  int blocks = (int)std::min<int64_t>((samples + kTs - 1) / kTs, std::max(sms, 1));
+  int st;  // (fewer blocks where the memory for their shares cannot be had)
+  while ((st = buf_reserve(c, &c->ws_grad, (size_t)blocks * kPart * sizeof(double))) ==
+             CPM_ENOMEM && blocks > 1)
+    blocks /= 2;
   if (!st) st = cuda_check(c, cudaFuncSetAttribute(k_mlp_grad,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)kGradSmem), "grad smem");

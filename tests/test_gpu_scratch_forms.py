@@ -9,6 +9,7 @@ import pytest
 
 from paper_2111_06704_gb300 import cpm
 from paper_2111_06704_gb300 import workloads as wl
+from paper_2111_06704_gb300.guess import LearnedGuess
 
 pytestmark = pytest.mark.gpu
 
@@ -87,3 +88,28 @@ def test_forces(cells, n_ion, frames, kw):
         return ctx.cpm_ion_forces(xyz, q, qe)
 
     _less_memory("fp64", cells, call, **kw)
+
+
+def test_gradient():
+    # blocks' shares of 84 KB each: as many blocks as the memory allows, the same sums to float
+    # rounding of the tiles' (1e-5 of a layer's largest entry: the bar of the gradient's tests)
+    el = wl.two_sheet_electrode(3, 2)
+    mem = Memory()
+    ctx = cpm.Context(el.box, rcut_dc=3.0,
+                      allocator=(mem.alloc, torch.cuda.caching_allocator_delete))
+    g = LearnedGuess(ctx, seed=3)
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    feat = torch.randn((30000, 32), generator=gen, device="cuda")
+    target = torch.randn(30000, generator=gen, device="cuda")
+    loss = g.gradient(feat, target)
+    ref = g.grad.clone()
+    ctx.cpm_release_workspace()
+    for mem.limit in (1 << 20, 100 << 10):
+        assert abs(g.gradient(feat, target) - loss) <= 1e-5 * loss
+        at = 0
+        for n in (2048, 64, 4096, 64, 4096, 64, 64, 1):
+            a, b = g.grad[at:at + n], ref[at:at + n]
+            assert (a - b).abs().max() <= 1e-5 * b.abs().max()
+            at += n
+        ctx.cpm_release_workspace()
+    ctx.close()
