@@ -309,13 +309,19 @@ k_mlp_forward(const float* __restrict__ params, const float* __restrict__ norm, 
 // the forward layers and the back-propagated ones in 8 samples x 4 units a thread (as
 // k_mlp_forward; the thread that made a pre-activation also meets its gradient, so silu'
 // stays in its registers), the weight gradients in 4 x 4 outputs over the tile's samples.
-// The weight gradients of a tile are float sums over its 128 samples, added to a float pair a
-// thread keeps over its tiles; blocks are added in FP64 in a fixed order.  Bound by FP32
+// The weight gradients of a tile (layers 1 to 3) are float sums over its 128 samples, added to a
+// float pair a thread keeps over its tiles; the biases' and the output weights' are float sums of a
+// thread's 8 samples a tile (registers are all taken).  A launch takes at most kGradTiles tiles a
+// block, and the next one adds to its blocks' shares in FP64: with one launch for 1,000 tiles a
+// block those sums, 8,000 terms long, were off by 6e-5 of a layer's largest entry where the samples
+// were alike.  (The same inside the kernel, every 32 tiles, cost 1% and more of any batch.)  Blocks
+// are added in FP64 in a fixed order.  Bound by FP32
 // multiply-adds (29,000 a sample; 8 warps an SM).  One thread a sample with scalar loads of
 // every operand and an atomic add per parameter and 128 samples took 3,702 us for 426,000
 // samples (8% of the chip's FP32 rate); this takes 781 us (the sigmoids' exponentials and
 // divisions issue as much as the products).
 constexpr int kGradThreads = 256;
+constexpr int kGradTiles = 32;
 constexpr int kPart = kP + 1;  // the parameters' gradients, the loss
 constexpr int oGW = kF * kH + 2 * kH * kH;   // WT1, WT2, WT3, then:
 constexpr int oGB = oGW + 2 * kH * kH;       // W2, W3 as given, then b1, b2, b3, W4, b4
@@ -370,7 +376,7 @@ __device__ __forceinline__ void tile_outer(const float* __restrict__ G,
 __global__ void __launch_bounds__(kGradThreads, 1)
 k_mlp_grad(const float* __restrict__ params, const float* __restrict__ norm, int bf16,
            int64_t samples, double inv_s, const float* __restrict__ feat,
-           const float* __restrict__ target, double* __restrict__ part) {
+           const float* __restrict__ target, double* __restrict__ part, int add) {
   extern __shared__ __align__(16) float gsm[];
   float *WT1 = gsm, *WT2 = WT1 + kF * kH, *WT3 = WT2 + kH * kH;
   float *W2 = gsm + oGW, *W3 = W2 + kH * kH, *bv = gsm + oGB;
@@ -506,17 +512,18 @@ k_mlp_grad(const float* __restrict__ params, const float* __restrict__ norm, int
   }
   // the block's sums: weight gradients from their threads, the others over the 16 sample groups
   double* out = part + (int64_t)blockIdx.x * kPart;
+  auto put = [&](int e, double x) { out[e] = add ? out[e] + x : x; };
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int e = (4 * ug + i) * kH + 4 * sg + j;
-      out[oW3 + e] = (double)h3[i][j] + (double)l3[i][j];
-      out[oW2 + e] = (double)h2[i][j] + (double)l2[i][j];
+      put(oW3 + e, (double)h3[i][j] + (double)l3[i][j]);
+      put(oW2 + e, (double)h2[i][j] + (double)l2[i][j]);
     }
 #pragma unroll
     for (int j = 0; j < 2; ++j)
-      out[oW1 + (4 * ug + i) * kF + 2 * sg + j] = (double)h1[i][j] + (double)l1[i][j];
+      put(oW1 + (4 * ug + i) * kF + 2 * sg + j, (double)h1[i][j] + (double)l1[i][j]);
   }
   __syncthreads();
   float* red = GA;  // [4][16 sample groups][64 units]
@@ -537,11 +544,11 @@ k_mlp_grad(const float* __restrict__ params, const float* __restrict__ norm, int
     const int arr = t >> 6, u = t & 63;
     double s = 0.0;
     for (int g = 0; g < 16; ++g) s += (double)red[(arr * 16 + g) * kH + u];
-    out[(arr == 0 ? ob1 : arr == 1 ? ob2 : arr == 2 ? ob3 : oW4) + u] = s;
+    put((arr == 0 ? ob1 : arr == 1 ? ob2 : arr == 2 ? ob3 : oW4) + u, s);
     if (t < 2) {
       s = 0.0;
       for (int g = 0; g < 16; ++g) s += red2[2 * g + t];
-      out[t == 0 ? ob4 : kP] = s;
+      put(t == 0 ? ob4 : kP, s);
     }
   }
 }
@@ -687,7 +694,8 @@ int features_async(cpm_ctx* c, int frames, const double* b, const double* b_prev
   return cuda_check(c, cudaGetLastError(), "features");
 }
 
-// Gradient, loss and, with adam.p, the Adam step: two launches on the context's stream.
+// Gradient, loss and, with adam.p, the Adam step, on the context's stream: two launches up to
+// kGradTiles tiles a block, one more for each as many.
 int grad_async(cpm_ctx* c, const float* params, const float* norm, int bf16, int64_t samples,
                const float* feat, const float* target, float* grad, double* loss,
                const AdamStep& adam) {
@@ -702,10 +710,12 @@ int grad_async(cpm_ctx* c, const float* params, const float* norm, int bf16, int
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)kGradSmem), "grad smem");
   if (st) return st;
-  (k_mlp_grad<<<blocks, kGradThreads, kGradSmem, c->stream>>>(
-       params, norm, bf16, samples, 1.0 / (double)samples, feat, target,
-       (double*)c->ws_grad.ptr),
-   note_launch());
+  const int64_t step = (int64_t)blocks * kGradTiles * kTs;
+  for (int64_t s0 = 0; s0 < samples; s0 += step)
+    (k_mlp_grad<<<blocks, kGradThreads, kGradSmem, c->stream>>>(
+         params, norm, bf16, std::min(step, samples - s0), 1.0 / (double)samples, feat + s0 * kF,
+         target + s0, (double*)c->ws_grad.ptr, s0 > 0),
+     note_launch());
   (k_grad_finish<<<(kPart + 31) / 32, 32 * kFinishSlices, 0, c->stream>>>(
        (const double*)c->ws_grad.ptr, blocks, grad, loss, adam),
    note_launch());
