@@ -69,12 +69,19 @@ int buf_reserve(Ctx* c, Buf* b, size_t bytes) {
   return buf_alloc(c, b, bytes);
 }
 
+constexpr size_t kPinnedKept = 64 << 10;
+
+void pinned_free(Ctx* c) {
+  if (c->pinned) cudaFreeHost(c->pinned);
+  c->pinned = nullptr;
+  c->pinned_bytes = 0;
+}
+
 int pinned_reserve(Ctx* c, size_t bytes) {
   if (c->pinned && c->pinned_bytes >= bytes) return CPM_OK;
   if (c->pinned) {
     cudaStreamSynchronize(c->stream);  // a copy into it may still be queued
-    cudaFreeHost(c->pinned);
-    c->pinned = nullptr;
+    pinned_free(c);
   }
   bytes = (bytes + 4095) & ~size_t(4095);
   if (cudaHostAlloc(&c->pinned, bytes, cudaHostAllocDefault) != cudaSuccess) {
@@ -387,8 +394,8 @@ void release_workspace(Ctx* c) {
                &c->tc_tiles};
   for (Buf* b : ws) buf_free(c, b);
   c->pot_refused = 0;
-  if (c->pinned) cudaFreeHost(c->pinned);
-  c->pinned = nullptr;
+  // (a few pages stay with the context: pinning them again costs more than a small call)
+  if (c->pinned_bytes > kPinnedKept) pinned_free(c);
   c->tc_tiles_nt = 0;
 }
 
@@ -513,6 +520,7 @@ int cpm_destroy(cpm_ctx* c) {
   if (!c) return CPM_EINVAL;
   cudaStreamSynchronize(c->stream);
   free_build(c);
+  pinned_free(c);
   cudaEventDestroy(c->ev_tc[0]);
   cudaEventDestroy(c->ev_tc[1]);
   cudaEventDestroy(c->ev_tc[2]);
