@@ -118,6 +118,8 @@ int cpm_batch_destroy(cpm_batch* b) {
   cudaStreamSynchronize(b->work.stream);
   Buf* all[] = {&b->cols, &b->pad_b, &b->pad_q, &b->pad_s, &b->work.ws_solve};
   for (Buf* x : all) buf_free(&b->work, x);
+  pinned_free(&b->work);
+  for (cudaEvent_t e : b->work.ev_pool) cudaEventDestroy(e);
   delete b;
   return CPM_OK;
 }

@@ -209,6 +209,7 @@ int buf_alloc(Ctx* c, Buf* b, size_t bytes);
 void buf_free(Ctx* c, Buf* b);
 int buf_reserve(Ctx* c, Buf* b, size_t bytes);  // grow-only
 int pinned_reserve(Ctx* c, size_t bytes);  // c->pinned, grow-only; CPM_ENOMEM leaves none
+void pinned_free(Ctx* c);
 int set_err(Ctx* c, int code, const std::string& msg);
 int cuda_check(Ctx* c, cudaError_t e, const char* what);
 // Where the array at p lives: 1 in device memory of the context's device (or managed
