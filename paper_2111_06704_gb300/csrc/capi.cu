@@ -1092,9 +1092,9 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
   // The kernels' own times (a start or an end each) into pinned host memory: events between
   // them would keep them apart.  No such memory: no times.
   unsigned long long* tm = nullptr;
-  if (pinned_reserve(c, 5 * sizeof(*tm)) == CPM_OK) {
+  if (pinned_reserve(c, 6 * sizeof(*tm)) == CPM_OK) {
     tm = (unsigned long long*)c->pinned;
-    std::fill(tm, tm + 5, 0ull);
+    std::fill(tm, tm + 6, 0ull);
   }
   auto at = [&](int k) { return tm ? tm + k : nullptr; };
   // ion records (FP64: and axis phasors) -> real-space sums, and beside them structure factors
@@ -1132,14 +1132,32 @@ int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
                      (const double*)c->sqw.ptr, c->turn.ptr, nsplit, spart, std::max(dev_sms, 1),
                      at(2), s);
   launch_bsol_finish((const double*)c->xyz.ptr, n, frames, n_ion, geometry(c), dchi, bk, db, dqs,
-                     rp, rscratch, at(3), s);
+                     rp, rscratch, at(3), at(5), s);
   if ((st = cuda_check(c, cudaGetLastError(), "potential kernels"))) return st;
+  unsigned over = 0;  // whether the real space's far terms outgrew their pool
+  if (rp.far_blocks > 0 && !tm &&
+      (st = cuda_check(c, cudaMemcpyAsync(&over, (char*)rscratch + rp.o_far_state + sizeof(over),
+                                          sizeof(over), cudaMemcpyDeviceToHost, s), "far terms")))
+    return st;
   if (qsol_out && n_ion == 0 &&
       (st = cuda_check(c, cudaMemsetAsync(dqs, 0, frames * sizeof(double), s), "qsol zero")))
     return st;
   if ((st = copy_out(c, b_out, db, (size_t)frames * n * sizeof(double)))) return st;
   if (qsol_out && (st = copy_out(c, qsol_out, dqs, (size_t)frames * sizeof(double)))) return st;
   if ((st = cuda_check(c, cudaStreamSynchronize(s), "potential sync"))) return st;
+  if (tm) over = (unsigned)tm[5];
+  if (over) {  // the real space again, the ions together
+    const RealPlan again = real_plan(n, frames, n_ion, geometry(c), f64, std::max(dev_sms, 1), true);
+    launch_bsol_real((const double*)c->xyz.ptr, (const double*)c->alpha.ptr,
+                     (const uint32_t*)c->sfix.ptr, c->atoms.ptr, c->htab.ptr, n, dx, dq, frames,
+                     n_ion, geometry(c), f64, again, rscratch, s);
+    launch_bsol_finish((const double*)c->xyz.ptr, n, frames, n_ion, geometry(c), dchi, bk, db, dqs,
+                       again, rscratch, nullptr, nullptr, s);
+    if ((st = cuda_check(c, cudaGetLastError(), "potential kernels")) ||
+        (st = copy_out(c, b_out, db, (size_t)frames * n * sizeof(double))) ||
+        (st = cuda_check(c, cudaStreamSynchronize(s), "potential sync")))
+      return st;
+  }
   c->t_pot_sf_ms = c->t_pot_kspace_ms = c->t_pot_real_ms = 0.f;
   if (tm) {
     auto ms = [&](int from, int to) {

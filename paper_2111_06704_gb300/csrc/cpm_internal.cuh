@@ -307,9 +307,11 @@ int bsol_direct_splits(int n, int frames, int mpad, int kh, int sms);
 struct RealPlan {
   int shares, grid_shares;      // shares of the ions within a block and over the grid
   int warps;                    // of a block
-  int far_cap;                  // far terms of an atom and share kept for the finish, or 0
-  // scratch layout: ion records | block sums | partials | far terms | their counts
-  size_t o_sums, o_part, o_far, o_far_count, bytes;
+  // far terms kept for the finish: blocks of them in the pool (0: none are), and of a warp at most
+  int far_blocks, far_row;
+  // scratch layout: ion records | block sums | partials | the pool | its state (blocks taken, more
+  // wanted than there are) | the warps' blocks | their lanes' counts
+  size_t o_sums, o_part, o_far, o_far_state, o_far_row, o_far_count, bytes;
 };
 // small: with the least scratch
 RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, bool fp64, int sms,
@@ -327,11 +329,12 @@ void launch_bsol_real(const double* xyz, const double* alpha, const uint32_t* sf
                       const void* atoms, const void* htab, int n, const double* ion_xyz,
                       const double* ion_q, int frames, int n_ion, const Geometry& geo, bool fp64,
                       const RealPlan& plan, void* scratch, cudaStream_t s);
-// stamp (if not NULL): the times at its start and end
+// stamp (if not NULL): the times at its start and end; over (if not NULL): whether far terms
+// outgrew their pool (b is wrong then)
 void launch_bsol_finish(const double* xyz, int n, int frames, int n_ion, const Geometry& geo,
                         const double* chi, const double* bsol_k, double* b_out, double* qsol,
                         const RealPlan& plan, void* scratch, unsigned long long* stamp,
-                        cudaStream_t s);
+                        unsigned long long* over, cudaStream_t s);
 
 // forces.cu
 struct ForceSplits {

@@ -130,10 +130,13 @@ constexpr int kPrepThreads = 128;
 __global__ void __launch_bounds__(kPrepThreads)
 k_ion_prepare(const double* __restrict__ ion_xyz, const double* __restrict__ ion_q, int n_ion,
               double lx, double ly, double lz, uint32_t* __restrict__ sion,
-              IonRec* __restrict__ rec, double2* __restrict__ sums, unsigned long long* stamp) {
+              IonRec* __restrict__ rec, double2* __restrict__ sums, unsigned* far_state,
+              unsigned long long* stamp) {
   __shared__ double2 red[kPrepThreads / 32];
   set_up_next();
   stamp_time(stamp);
+  if (far_state && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2)
+    far_state[threadIdx.x] = 0u;
   const int f = blockIdx.y, t = blockIdx.x * kPrepThreads + threadIdx.x;
   double qz = 0.0, qs = 0.0;
   if (t < n_ion) {
@@ -185,6 +188,7 @@ __global__ void k_atom_records(const double* __restrict__ xyz, const double* __r
 // ---- the sums ----------------------------------------------------------------------------
 
 constexpr int kMaxShifts = 64;
+constexpr int kFarTerms = 16;  // far terms of each lane that a block of the pool holds
 constexpr int kRealWarps = 8;
 constexpr int kListDepth = 72;  // pairs a lane can hold: fewer than 64 at a look, and at
 constexpr int kListStep = 8;    // most this many more before the next one
@@ -222,10 +226,13 @@ struct RealArgs {
   float shift[kMaxShifts][3];  // k L, the screen's
   signed char kshift[kMaxShifts][3];
   double* part;                // [gridDim.z][frames][n]
-  // far terms of a share in the ions' order, far_cap an atom (0: summed by the share):
-  float* far;                  // [share][frame][far_cap][n]
-  int* far_count;              // [share][frame][n]
-  int far_cap;
+  // far terms of a share in the ions' order (far_blocks 0: summed by the share), in blocks
+  // of a pool [far_blocks][kFarTerms][32] that a warp takes as its lists grow:
+  float* far;
+  unsigned* far_state;  // blocks taken, whether more were wanted than there are
+  int* far_row;         // [share][frame][group][far_len]: the warp's blocks
+  int* far_count;       // [share][frame][group][32]
+  int far_blocks, far_len;
 };
 
 // FP64 sum of one electrode-ion pair over every image within r_c.
@@ -266,7 +273,8 @@ __device__ __forceinline__ double pair_images(const double* ri, double ai, const
   return acc;
 }
 
-template <int kMode, bool kF64>
+// kPool: far terms go to the pool (float storage, listed images)
+template <int kMode, bool kF64, bool kPool>
 __global__ void __launch_bounds__(kRealWarps * 32)
 k_bsol_real(const __grid_constant__ RealArgs a) {
   constexpr int kBits = kIonBits<kMode>;
@@ -315,9 +323,10 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
   }
   float acch = 0.f, accl = 0.f, accf = 0.f;
   const int sh = blockIdx.z * a.shares + warp % a.shares;
-  const size_t at_share = (size_t)sh * gridDim.y + f;
-  float* far = a.far + at_share * a.far_cap * a.n + i;
-  int nfar = 0;
+  const size_t row = ((size_t)sh * gridDim.y + f) * ((a.n + 31) / 32) + grp;
+  int* mine = a.far_row + row * a.far_len;
+  float* far = nullptr;  // where this lane's next far term goes
+  int nfar = 0, have = 0;  // far terms of the lane, blocks of the warp
   double acc = 0.0;
   int cn = 0, cf = 0;  // near and far entries of this lane's list
   int base0 = 0;
@@ -438,8 +447,15 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
     if (m2 >= lane_far2 && m2 < a.cut2) {
       const float ir = rsqrtf(m2);  // 1 / r to ~2 ulp
       const float q = __uint_as_float(w.w), e = erfcf(a.gh * (m2 * ir)) * ir;
-      if (nfar < a.far_cap) far[(size_t)nfar++ * a.n] = q * e;
-      else accf += q * e;
+      if constexpr (kPool) {
+        if (nfar % kFarTerms == 0)
+          far = a.far + (size_t)mine[nfar / kFarTerms] * (kFarTerms * 32) + lane;
+        *far = q * e;
+        far += 32;
+        ++nfar;
+      } else {
+        accf += q * e;
+      }
     } else {
       evaluate(entry);
     }
@@ -451,6 +467,24 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
       if (k < cn) evaluate(list[warp][k][lane]);
     cn = 0;
     if constexpr (kFar) {
+      if constexpr (kPool) {  // blocks for what is listed
+        const int more = (__reduce_max_sync(0xffffffffu, nfar + cf) + kFarTerms - 1) / kFarTerms -
+                         have;
+        if (more > 0) {
+          unsigned b = 0;
+          if (lane == 0) {
+            b = atomicAdd(a.far_state, (unsigned)more);
+            if (b + more > (unsigned)a.far_blocks) {
+              a.far_state[1] = 1u;
+              b = ~0u;
+            }
+          }
+          b = __shfl_sync(0xffffffffu, b, 0);
+          for (int k = lane; k < more; k += 32) mine[have + k] = b == ~0u ? 0 : (int)b + k;
+          have += more;
+          __syncwarp();
+        }
+      }
       most = __reduce_max_sync(0xffffffffu, cf);
       for (int k = 1; k <= most; ++k)
         if (k <= cf) evaluate_far(list[warp][kListDepth - k][lane]);
@@ -550,7 +584,7 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
   drain();
   acc += (double)accf;
   acc += (double)acch + (double)accl;
-  if (a.far_cap > 0 && live) a.far_count[at_share * a.n + i] = nfar;
+  if (kPool && live) a.far_count[row * 32 + lane] = nfar;
   if (a.shares > 1) {  // the block's shares of a group, in share order
     red[warp][lane] = acc;
     __syncthreads();
@@ -563,9 +597,10 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
 struct FinishArgs {
   const double* part;  // [shares][frames][n] real-space sums
   int shares, n;
-  const float* far;  // far terms [far_shares][frame][far_cap][n] (far_cap 0: none)
-  const int* far_count;
-  int far_shares, far_cap;
+  const float* far;  // far terms of the shares (far_blocks 0: none)
+  const unsigned* far_state;
+  const int *far_row, *far_count;
+  int far_shares, far_blocks, far_len;
   const double2* sums;  // [frames][nsum] (sum q z, sum q)
   int nsum;
   const double* xyz;
@@ -573,6 +608,7 @@ struct FinishArgs {
   const double *chi, *bsol_k;
   double *b_out, *qsol;
   unsigned long long* stamp;  // start and end
+  unsigned long long* over;   // whether the far terms outgrew their pool
 };
 
 // b = chi - k_e (b^sol_k + real + dipole term), the real-space shares in share order; every warp
@@ -588,24 +624,26 @@ __global__ void __launch_bounds__(128) k_bsol_finish(const __grid_constant__ Fin
   double real = 0.0;
   if (i < a.n)
     for (int z = 0; z < a.shares; ++z) real += part[((size_t)z * gridDim.y + f) * a.n + i];
-  if (a.far_cap > 0 && i < a.n) {  // one float chain over the shares, as one warp adds them
-    const float* far = fresh(a.far);
-    const int* count = fresh(a.far_count);
+  if (a.far_blocks > 0 && i < a.n) {  // one float chain over the shares, as one warp adds them
+    const float* far = fresh(a.far) + lane;
+    const int *rows = fresh(a.far_row), *count = fresh(a.far_count);
     float c = 0.f;
     for (int z = 0; z < a.far_shares; ++z) {
-      const size_t at = (size_t)z * gridDim.y + f;
-      const float* t = far + at * a.far_cap * a.n + i;
-      const int m = count[at * a.n + i];
-      for (int k0 = 0; k0 < m; k0 += 16) {
-        float x[16];
+      const size_t row = ((size_t)z * gridDim.y + f) * ((a.n + 31) / 32) + (i >> 5);
+      const int m = count[row * 32 + lane];
+      for (int k0 = 0; k0 < m; k0 += kFarTerms) {
+        const float* t =
+            far + (size_t)rows[row * a.far_len + k0 / kFarTerms] * (kFarTerms * 32);
+        float x[kFarTerms];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) x[k] = k0 + k < m ? t[(size_t)(k0 + k) * a.n] : 0.f;
+        for (int k = 0; k < kFarTerms; ++k) x[k] = k0 + k < m ? t[k * 32] : 0.f;
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
+        for (int k = 0; k < kFarTerms; ++k)
           if (k0 + k < m) c += x[k];
       }
     }
     real += (double)c;
+    if (a.over && i == 0 && f == 0) *a.over = fresh(a.far_state)[1];
   }
   double qz = 0.0, qs = 0.0;
   for (int s = lane; s < a.nsum; s += 32) {
@@ -628,6 +666,27 @@ __global__ void __launch_bounds__(128) k_bsol_finish(const __grid_constant__ Fin
 }
 
 int prep_blocks(int n_ion) { return (n_ion + kPrepThreads - 1) / kPrepThreads; }
+
+// Shifts k with |k| <= m = floor((r_c + L / 2) / L) per direction (only k = 0 where L > 2 r_c):
+// every image within r_c of an atom, given the nearest one.  list: they fit the screen's.
+struct Shifts {
+  int m[3], total;
+  bool all_single, list;
+};
+
+Shifts whole_box_shifts(const Geometry& geo) {
+  Shifts sh;
+  sh.total = 1;
+  sh.all_single = true;
+  for (int u = 0; u < 3; ++u) {
+    const bool single = 2.0 * geo.rc < geo.L[u];
+    sh.all_single &= single;
+    sh.m[u] = single ? 0 : (int)floor((geo.rc + 0.5 * geo.L[u]) / geo.L[u]);
+    sh.total *= 2 * sh.m[u] + 1;
+  }
+  sh.list = sh.total <= kMaxShifts;
+  return sh;
+}
 
 }  // namespace
 
@@ -655,12 +714,17 @@ void launch_atom_records(const double* xyz, const double* alpha, int n, const Ge
 // Float storage adds an atom's far images in one float chain, in the ions' order; its rounding is
 // most of the real-space error where the ions are many (1e-9 of b at 5,000 ions in a small box),
 // and sums by shares would exchange it for another, so that b would move by as much with the
-// number of frames.  Above kRealChainIons the shares therefore leave their far terms in scratch,
-// four times the mean number of images within r_c of an atom (ions fill part of the box; a term
-// too many is added by its share), and the finish adds them in order.  Where that takes more
-// than kRealFarBytes the ions stay together, in blocks of fewer warps.  One frame of 2,000 ions, 320
-// atoms: 209 us a call so, 110 with sums by shares, 1,800 with the ions together; 5,341 atoms,
-// 5,000 ions, two frames: 963, 767 and 1,958.
+// number of frames.  Above kRealChainIons the shares therefore leave their far terms in scratch
+// and the finish adds them in order.  The warps take blocks of 16 terms a lane from one pool
+// as their lists grow: ions that are sorted in space give one share most of an atom's terms,
+// but not more of them (lists of a fixed length a share overflowed there, and the rest of the terms
+// was summed by the share).  The pool holds four times the mean number of images within r_c of
+// an atom (ions fill part of the box) and a block a warp.  Where that takes more than kRealFarBytes
+// the ions stay together, in blocks of fewer warps, and where a pool was too small after all
+// (ions in a small part of the box, and atoms in no order, so that every warp has a lane with all of
+// them) the caller sums them again that way.  One frame of 2,000 ions, 320 atoms: 178 us a call
+// (209 with lists of a fixed length, 110 with sums by shares, 1,800 with the ions together); 5,341
+// atoms, 5,000 ions, two frames: 750 (963, 767, 1,958).
 constexpr int kRealChainIons = 1200;
 constexpr size_t kRealFarBytes = (size_t)192 << 20;
 
@@ -670,20 +734,24 @@ RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, bool fp64,
   const int64_t groups = (int64_t)((n + 31) / 32) * frames;
   p.shares = p.grid_shares = 1;
   p.warps = kRealWarps;
-  p.far_cap = 0;
+  p.far_blocks = p.far_row = 0;
   while (p.shares < kRealWarps && groups * p.shares < 24 * (int64_t)sms) p.shares *= 2;
   const int64_t blocks = (groups * p.shares + kRealWarps - 1) / kRealWarps;
-  bool single = true;
-  for (int u = 0; u < 3; ++u) single &= 2.0 * geo.rc < geo.L[u];
+  const Shifts sh = whole_box_shifts(geo);
   p.grid_shares = (int)std::max<int64_t>(
-      1, std::min<int64_t>((sms + blocks - 1) / blocks, n_ion / ((single ? 32 : 8) * p.shares)));
+      1, std::min<int64_t>((sms + blocks - 1) / blocks,
+                           n_ion / ((sh.all_single ? 32 : 8) * p.shares)));
   if (!fp64 && n_ion > kRealChainIons && p.shares * p.grid_shares > 1) {
     const int nsh = p.shares * p.grid_shares;
     const double mean = n_ion * (4.0 / 3.0 * kPi * geo.rc * geo.rc * geo.rc) /
                         (geo.L[0] * geo.L[1] * geo.L[2]);
-    const double cap = 4.0 * mean / nsh + 16.0;
-    if (!small && cap * nsh * frames * n * sizeof(float) <= (double)kRealFarBytes) {
-      p.far_cap = (int)cap;
+    const double rows = (double)groups * nsh;
+    const int len = ((n_ion + nsh - 1) / nsh * sh.total + kFarTerms - 1) / kFarTerms;
+    const double pool = std::min(rows * len, rows * (4.0 * mean / nsh / kFarTerms + 1.0));
+    if (!small && pool * kFarTerms * 32 * sizeof(float) + rows * len * sizeof(int) <=
+                      (double)kRealFarBytes) {
+      p.far_blocks = (int)pool;
+      p.far_row = len;
     } else {
       p.shares = p.grid_shares = 1;
       p.warps =
@@ -694,9 +762,11 @@ RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, bool fp64,
   p.o_sums = up((size_t)frames * std::max(n_ion, 1) * sizeof(IonRec));
   p.o_part = p.o_sums + up((size_t)frames * std::max(prep_blocks(n_ion), 1) * sizeof(double2));
   p.o_far = p.o_part + up((size_t)p.grid_shares * frames * n * sizeof(double));
-  const size_t lists = (size_t)p.shares * p.grid_shares * frames * n;
-  p.o_far_count = p.o_far + up(lists * p.far_cap * sizeof(float));
-  p.bytes = p.o_far_count + (p.far_cap > 0 ? up(lists * sizeof(int)) : 0);
+  const size_t rows = (size_t)p.shares * p.grid_shares * groups;
+  p.o_far_state = p.o_far + up((size_t)p.far_blocks * kFarTerms * 32 * sizeof(float));
+  p.o_far_row = p.o_far_state + (p.far_blocks > 0 ? 256 : 0);
+  p.o_far_count = p.o_far_row + up(rows * p.far_row * sizeof(int));
+  p.bytes = p.o_far_count + (p.far_blocks > 0 ? up(rows * 32 * sizeof(int)) : 0);
   return p;
 }
 
@@ -705,7 +775,8 @@ void launch_ion_prepare(const double* ion_xyz, const double* ion_q, int frames, 
                         unsigned long long* stamp, cudaStream_t s) {
   (k_ion_prepare<<<dim3(prep_blocks(n_ion), frames), kPrepThreads, 0, s>>>(
        ion_xyz, ion_q, n_ion, geo.L[0], geo.L[1], geo.L[2], sion, (IonRec*)scratch,
-       (double2*)((char*)scratch + plan.o_sums), stamp),
+       (double2*)((char*)scratch + plan.o_sums),
+       plan.far_blocks > 0 ? (unsigned*)((char*)scratch + plan.o_far_state) : nullptr, stamp),
    note_launch());
 }
 
@@ -748,22 +819,17 @@ void launch_bsol_real(const double* xyz, const double* alpha, const uint32_t* sf
     }
   a.far2 = (float)(hi * hi);
   a.cut2 = (float)(a.rc2 * (1.0 - 1e-5));
-  // shifts k with |k| <= floor((r_c + L / 2) / L) per direction (only k = 0 where
-  // L > 2 r_c): every image within r_c of an atom, given the nearest one
-  int m[3], total = 1;
-  bool all_single = true;
   for (int u = 0; u < 3; ++u) {
     a.L[u] = geo.L[u];
     a.invL[u] = 1.0 / geo.L[u];
     a.single[u] = 2.0 * geo.rc < geo.L[u];
-    all_single &= a.single[u];
     a.fs[u] = (float)(geo.L[u] * 0x1p-32);
     pair(geo.L[u] * 0x1p-32, a.fsh[u], a.fsl[u]);
     a.reach[u] = (float)(0.5 * geo.L[u] - geo.rc) - 0.01f;
-    m[u] = a.single[u] ? 0 : (int)floor((geo.rc + 0.5 * geo.L[u]) / geo.L[u]);
-    total *= 2 * m[u] + 1;
   }
-  a.nshift = total <= kMaxShifts ? total : 0;
+  const Shifts sh = whole_box_shifts(geo);
+  const int* m = sh.m;
+  a.nshift = sh.list ? sh.total : 0;
   int k = 0;
   for (int x = -m[0]; a.nshift && x <= m[0]; ++x)
     for (int y = -m[1]; y <= m[1]; ++y)
@@ -776,27 +842,39 @@ void launch_bsol_real(const double* xyz, const double* alpha, const uint32_t* sf
       }
   a.part = (double*)((char*)scratch + plan.o_part);
   a.far = (float*)((char*)scratch + plan.o_far);
+  a.far_state = (unsigned*)((char*)scratch + plan.o_far_state);
+  a.far_row = (int*)((char*)scratch + plan.o_far_row);
   a.far_count = (int*)((char*)scratch + plan.o_far_count);
-  a.far_cap = plan.far_cap;
+  a.far_blocks = plan.far_blocks;
+  a.far_len = plan.far_row;
   const int groups = (n + 31) / 32, per = plan.warps / plan.shares;
   const dim3 grid((groups + per - 1) / per, frames, plan.grid_shares);
-  auto kernel = all_single ? (fp64 ? k_bsol_real<kSingleImage, true> : k_bsol_real<kSingleImage, false>)
-                : a.nshift ? (fp64 ? k_bsol_real<kShiftList, true> : k_bsol_real<kShiftList, false>)
-                           : k_bsol_real<kAllImages, true>;
+  const bool pool = plan.far_blocks > 0;
+  auto kernel = sh.all_single ? (fp64   ? k_bsol_real<kSingleImage, true, false>
+                                 : pool ? k_bsol_real<kSingleImage, false, true>
+                                        : k_bsol_real<kSingleImage, false, false>)
+                : sh.list     ? (fp64   ? k_bsol_real<kShiftList, true, false>
+                                 : pool ? k_bsol_real<kShiftList, false, true>
+                                        : k_bsol_real<kShiftList, false, false>)
+                              : k_bsol_real<kAllImages, true, false>;
   launch_next(kernel, grid, plan.warps * 32, 0, s, a);
 }
 
 void launch_bsol_finish(const double* xyz, int n, int frames, int n_ion, const Geometry& geo,
                         const double* chi, const double* bsol_k, double* b_out, double* qsol,
                         const RealPlan& plan, void* scratch, unsigned long long* stamp,
-                        cudaStream_t s) {
+                        unsigned long long* over, cudaStream_t s) {
   FinishArgs a;
   a.part = (const double*)((char*)scratch + plan.o_part);
   a.shares = plan.grid_shares;
   a.far = (const float*)((char*)scratch + plan.o_far);
+  a.far_state = (const unsigned*)((char*)scratch + plan.o_far_state);
+  a.far_row = (const int*)((char*)scratch + plan.o_far_row);
   a.far_count = (const int*)((char*)scratch + plan.o_far_count);
   a.far_shares = plan.shares * plan.grid_shares;
-  a.far_cap = plan.far_cap;
+  a.far_blocks = plan.far_blocks;
+  a.far_len = plan.far_row;
+  a.over = over;
   a.n = n;
   a.sums = (const double2*)((char*)scratch + plan.o_sums);
   a.nsum = prep_blocks(n_ion);

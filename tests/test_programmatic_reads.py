@@ -32,7 +32,8 @@ TAKES = {
     },
     "real_space.cu": {
         "k_bsol_real": ["a.ions"],
-        "k_bsol_finish": ["a.part", "a.sums", "a.bsol_k"],
+        "k_bsol_finish": ["a.part", "a.sums", "a.bsol_k", "a.far", "a.far_state", "a.far_row",
+                          "a.far_count"],
     },
     "forces.cu": {
         "k_force_kspace": ["sion", "v", "vhead"],
