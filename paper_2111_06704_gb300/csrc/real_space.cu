@@ -741,7 +741,8 @@ RealPlan real_plan(int n, int frames, int n_ion, const Geometry& geo, bool fp64,
   p.grid_shares = (int)std::max<int64_t>(
       1, std::min<int64_t>((sms + blocks - 1) / blocks,
                            n_ion / ((sh.all_single ? 32 : 8) * p.shares)));
-  if (!fp64 && n_ion > kRealChainIons && p.shares * p.grid_shares > 1) {
+  // (every image of a pair goes to FP64 sums where the shifts are not listed)
+  if (!fp64 && sh.list && n_ion > kRealChainIons && p.shares * p.grid_shares > 1) {
     const int nsh = p.shares * p.grid_shares;
     const double mean = n_ion * (4.0 / 3.0 * kPi * geo.rc * geo.rc * geo.rc) /
                         (geo.L[0] * geo.L[1] * geo.L[2]);

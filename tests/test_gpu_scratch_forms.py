@@ -113,3 +113,18 @@ def test_gradient():
             at += n
         ctx.cpm_release_workspace()
     ctx.close()
+
+
+def test_no_lists_where_images_are_not_listed():
+    # a box so small that every image of a pair is summed in FP64: no far terms, no pool for them
+    # (2,000 ions' records and factors are 0.3 MB; a pool was 30 MB)
+    el = wl.two_sheet_electrode(3, 2)
+    mem = Memory()
+    ctx = cpm.Context(el.box, precision=cpm.CPM_PREC_FP32, rcut_dc=3.0, rcut_real=30.0,
+                      allocator=(mem.alloc, torch.cuda.caching_allocator_delete))
+    ctx.cpm_build_E(el.xyz, el.alpha)
+    mem.asked.clear()
+    xyz, q, _ = _ions(el, 1, 2000)
+    ctx.cpm_potential(xyz, q, el.chi)
+    assert max(mem.asked) < 2 << 20
+    ctx.close()
