@@ -106,7 +106,7 @@ struct Ctx {
   Buf sqw;      // double [mpad]  sqrt(W_K), zero in the padding
   Buf flush;    // uint32 [(2*mpad/16 + 31)/32]: k-steps after which float partials flush
   int heavy_steps = 0;  // leading k-steps accumulated exactly in FP64
-  int kh = 0;           // head k-vectors with an FP64 operand copy (float storage only)
+  int kh = 0;           // head k-vectors with a float-pair operand copy (float storage only)
   Buf Ahead;            // float pairs [npad][2*kh] of the head columns, A's column layout
   Buf chunk_end;        // uint32 bit per K-block of 64 columns (tensor-core build)
   Buf kexp;             // int per K-block: FP16 plane scale exponent (tensor-core build)
@@ -282,11 +282,11 @@ void launch_axis_phasors(const double* xyz, const uint32_t* sfix, int64_t count,
                          const double L[3], const AxisPhasors& ap, double2* out,
                          cudaStream_t s);
 // Structure factors of the points of `frames` frames, coord_stride points apart (0: every
-// frame has the same coordinates) and their charges charge_stride.  FP64 storage takes the points
-// from axis, float storage from the fixed-point coordinates sion; add (FP64): the sums are added to
-// those of the points before.  late: the kernel before is launched by launch_next and
-// waits for all that this one reads, so that the two may run side by side.  stamp (if not NULL):
-// the time at its start.
+// frame has the same coordinates).  FP64 storage takes the points from axis, their charges
+// charge_stride apart, and adds the sums to those of the points before (add); float storage takes
+// all points of a frame at once, from the fixed-point coordinates sion.  late: the kernel before is
+// launched by launch_next and waits for all that this one reads, so that the two may run side by
+// side.  stamp (if not NULL): the time at its start.
 void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhasors& ap,
                                  const uint32_t* sion, int64_t coord_stride,
                                  const double* ion_q, int64_t charge_stride, int frames, int n_ion,

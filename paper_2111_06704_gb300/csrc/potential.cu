@@ -95,7 +95,7 @@ __device__ __forceinline__ void sincos_t64x2(uint32_t p0, uint32_t p1, const flo
 // the rest of the grid), so its blocks always split the ions eight ways, and come first.
 __global__ void __launch_bounds__(kSfWarps * 32)
 k_ion_sf_f32(const uint32_t* __restrict__ sion, int64_t coord_stride,
-             const double* __restrict__ ion_q, int64_t charge_stride, int n_ion, const SfPair* __restrict__ pairs,
+             const double* __restrict__ ion_q, int n_ion, const SfPair* __restrict__ pairs,
              int npairs, const int* __restrict__ hkl, const double* __restrict__ sqw, int mpad,
              int kh, int tail_shares, int head_blocks, const float4* __restrict__ turn,
              float* __restrict__ vout, float2* __restrict__ vhead, bool late,
@@ -114,7 +114,7 @@ k_ion_sf_f32(const uint32_t* __restrict__ sion, int64_t coord_stride,
   const int shares = head ? kSfWarps : tail_shares;
   const int share = warp % shares, per = kSfWarps / shares;  // groups of 32 threads a block
   const uint32_t* fx = sion + (size_t)f * coord_stride * 3;
-  const double* q = ion_q + (size_t)f * charge_stride;
+  const double* q = ion_q + (size_t)f * n_ion;
   float* v = vout + (size_t)f * 2 * mpad;
   const int at = ((int)blockIdx.x - (head ? 0 : head_blocks)) * per * 32 +
                  (warp / shares) * 32 + lane;
@@ -785,7 +785,7 @@ void launch_ion_structure_factor(bool fp64, const double2* axis, const AxisPhaso
     }
     const int per = 32 * (kSfWarps / shares), hb = (kh + 31) / 32;
     launch_next(k_ion_sf_f32, dim3(hb + (npairs + per - 1) / per, frames), kSfWarps * 32, 0, s, sion,
-                coord_stride, ion_q, charge_stride, n_ion, pairs, npairs, hkl, sqw, mpad, kh, shares, hb,
+                coord_stride, ion_q, n_ion, pairs, npairs, hkl, sqw, mpad, kh, shares, hb,
                 (const float4*)turn, (float*)v, (float2*)vhead, late, stamp);
   }
 }
