@@ -262,7 +262,7 @@ void kvector_table(const cpm_params& p, std::vector<int>& hkl, std::vector<doubl
 // per-block scales and accumulation chunks.
 struct KPlan {
   int heavy_steps = 0;  // leading 16-column k-steps of the head
-  int kh = 0;           // k-vectors of the b^sol contraction kept in FP64
+  int kh = 0;           // k-vectors of the b^sol contraction in float pairs
   int kb0 = 0, kb6 = 0, kb3 = 0, kb8 = 0, nkb = 0;  // tensor-core K-block regions
   std::vector<uint32_t> fmask;  // SIMT builds: k-steps after which float partials flush
   std::vector<uint32_t> cmask;  // tensor cores: K-blocks that end an accumulation chunk
@@ -300,7 +300,7 @@ void plan_kspace(const std::vector<double>& w, int mpad, int precision, KPlan& p
       while (h5 < nk && ws[h5] > 5e-3) ++h5;
       pl.heavy_steps = std::min(heavy, (h5 + 7) / 8 * 8);
     }
-    // head of the b^sol contraction kept in FP64: the heavy blocks, at least 256 and at
+    // head of the b^sol contraction, in float pairs: the heavy blocks, at least 256 and at
     // most 1024 k-vectors
     pl.kh = f64 ? 0 : std::min(mpad, std::max(256, std::min(1024, heavy / 8 * 64)));
     double cw = 0.0;

@@ -406,8 +406,7 @@ k_ek_simt(const T* __restrict__ A, int64_t lda, int ktot, T* __restrict__ E, int
 }
 
 // Head of the k-space sum in float-float arithmetic (lower-triangle 64 x 64 tiles, 4 x 4
-// outputs per thread): each FP64 operand value is split into a float pair a = ah + al,
-// and each term
+// outputs per thread): each operand value is a float pair a = ah + al, and each term
 //   a_i a_j = ah*bh (exact: rounded product plus its fma remainder) + ah*bl + al*bh
 // (al*bl is below 2^-48 of the product) is added to a float pair (hi, lo) per output
 // with an error-free two-sum.  About 11 float operations per term instead of one FP64
@@ -607,8 +606,8 @@ int launch_ek_simt(bool fp64, const void* A, int npad, int mpad, const double* x
   return cudaGetLastError() == cudaSuccess ? CPM_OK : CPM_ECUDA;
 }
 
-// FP64-accurate head of the k-space sum (the first ktot columns of the FP64 head operand,
-// row stride 2 kh, split into float pairs in hi/lo [npad][ktot]) plus the real-space,
+// Head of the k-space sum in float pairs (the first ktot columns of the head operand, float pairs
+// to 2^-48 of the FP64 phasors, row stride 2 kh; as planes in hi/lo [npad][ktot]) plus the real-space,
 // self and dipole terms, lower triangle, into Ehead as float pairs (hi, lo).
 int launch_ek_head_f64(const void* Ahead, int kh, int ktot, int npad, float* hi, float* lo,
                        const double* xyz, const double* alpha, int n, const Geometry& geo,

@@ -869,10 +869,12 @@ k_dc_apply(int n, int64_t ldv, int nrhs, const ColState* __restrict__ st,
 }
 
 // The same with each row's entries added in their order and the dots in that of 256-row blocks:
-// the build's solve for d (SolveArgs::ordered).  d and p_gap enter every later solve, and a
-// many-column solve, whose float matvec rounds at 1e-7, turns a change of p_gap's last bits
-// into 2e-9 of its charges; with its sums in one fixed order the build repeats to the last bit
-// whatever the per-column kernel above does.  32 rows a block: the eight warps load the rows'
+// the build's solve for d (SolveArgs::ordered).  Not more exact than the kernel above, and both
+// repeat to the last bit; but that one's order follows its shape (a warp or eight lanes a row, blocks
+// by the column count and the chip), and d and p_gap enter every later solve: a many-column
+// solve, whose float matvec rounds at 1e-7, turns a change of p_gap's last bits into 2e-9 of its
+// charges (its tolerance is 1e-6).  In this order, that of one thread a row, charges stay what
+// they were before the shapes were chosen so.  32 rows a block: the eight warps load the rows'
 // entries and the residuals they meet, coalesced, into shared memory, and one warp adds each
 // row's, a row a lane.  wpart[column][ldv] at 2 block; eight blocks make one of the solver's
 // partials (group_dot).
