@@ -180,8 +180,8 @@ int cpm_build_E(cpm_ctx* c, int n, const double* xyz, const double* alpha);
 int cpm_build_E_copy(cpm_ctx* dst, cpm_ctx* src);
 
 /* Frees the context's kept workspace: the E build's (above) and the solve and potential
- * workspaces, which later calls reserve again as needed.  The built E, P, d and the
- * operand A stay.  Waits for the context's stream first.  No counterpart in the paper:
+ * workspaces, which later calls reserve again as needed.  The built E, P, d, the
+ * operand A and up to 64 KB of pinned host memory stay.  Waits for the context's stream first.  No counterpart in the paper:
  * device-memory management of this library. */
 int cpm_release_workspace(cpm_ctx* c);
 
@@ -225,7 +225,10 @@ int cpm_plan_kspace(const cpm_params* p, cpm_kspace_plan* out, int* hkl, double*
  * the point-Gaussian coefficient alpha_i] + (4 pi/V) z_i sum_I q_I z_I (slab).
  * ion_xyz[frames*n_ion*3] (A), ion_q[frames*n_ion] (e), chi[n] (V, shared by all
  * frames).  b_out[frames*n] (V).  qsol_out[frames] (may be NULL) receives
- * Q^sol = sum_I q_I of each frame.  n_ion may be 0.
+ * Q^sol = sum_I q_I of each frame.  n_ion may be 0.  A coordinate that is NaN or infinite
+ * makes every b of its frame NaN.  Where the scratch that serves the call best cannot be
+ * had, it takes less and more time (CPM_ENOMEM where that cannot be had either), until
+ * cpm_release_workspace or the next build; so does cpm_ion_forces.
  */
 int cpm_potential(cpm_ctx* c, int frames, int n_ion, const double* ion_xyz,
                   const double* ion_q, const double* chi, double* b_out, double* qsol_out);
