@@ -273,9 +273,14 @@ __device__ __forceinline__ double pair_images(const double* ri, double ai, const
   return acc;
 }
 
-// kPool: far terms go to the pool (float storage, listed images)
+// kPool: far terms go to the pool (float storage, listed images).  Blocks an SM: three, where the
+// nearest image is all: in the 64 registers of a fourth the compiler leaves less of a warp's work
+// in flight, and grids of two or three blocks an SM are slower by up to 15% (12,094 atoms, 8 frames
+// of 4,000 ions 1,645 us a call, 1,434 so; many waves gain 1%).  Four for lists of shifts (512
+// atoms, 256 frames: 5,394 us a call with three, 5,186 so), but three with the pool, whose
+// grids are small.
 template <int kMode, bool kF64, bool kPool>
-__global__ void __launch_bounds__(kRealWarps * 32)
+__global__ void __launch_bounds__(kRealWarps * 32, kMode == kShiftList && !kPool ? 4 : 3)
 k_bsol_real(const __grid_constant__ RealArgs a) {
   constexpr int kBits = kIonBits<kMode>;
   constexpr bool kFar = !kF64;  // far images apart
@@ -541,7 +546,7 @@ k_bsol_real(const __grid_constant__ RealArgs a) {
         for (int c0 = 0; c0 < k; c0 += kListStep) {
           const int c1 = min(k, c0 + kListStep);
           look(c1 - c0);
-#pragma unroll 4
+#pragma unroll 2
           for (int c = c0; c < c1; ++c) {
             const float4 p = cand[warp][c];
             float x, y, z;
